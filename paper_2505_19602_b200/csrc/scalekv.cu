@@ -195,6 +195,8 @@ struct scalekv_ctx {
   cudaEvent_t ev_in[2] = {nullptr, nullptr}, ev_out[2] = {nullptr, nullptr}, ev_att[2] = {nullptr, nullptr};
   int set_layer[2] = {-1, -1};     // layer that last used a staging half (-1: unused)
   long long host_steps = 0;
+  const void *stage_ptr = nullptr; // the staging area of the last step and the size of its halves
+  size_t stage_half = 0;
   std::vector<int> page_table_host;
   // per layer state
   std::vector<int> next_scale;     // scale expected by the next append
@@ -869,16 +871,22 @@ scalekv_status scalekv_step_host(scalekv_ctx *ctx, int32_t layer, int32_t scale,
       CU(cudaEventCreateWithFlags(&ctx->ev_att[i], cudaEventDisableTiming));
     }
   }
-  // consecutive steps alternate between the two halves of the staging area
+  // Consecutive steps alternate between the two halves of the staging area: halves of the area, not of what this scale
+  // needs of it, so that a step of the next, larger scale does not reach into the half that the step before still uses.
   const int set = (int)(ctx->host_steps++ & 1);
-  char *dq = static_cast<char *>(staging) + (size_t)set * 4 * bytes, *dk = dq + bytes, *dv = dk + bytes, *dout = dv + bytes;
-  if (ctx->set_layer[set] >= 0) {
+  const size_t half = staging_bytes / 2 / 1024 * 1024;
+  char *dq = static_cast<char *>(staging) + (size_t)set * half, *dk = dq + bytes, *dv = dk + bytes, *dout = dv + bytes;
+  const bool other_area = ctx->stage_ptr != staging || ctx->stage_half != half;   // the halves of earlier steps lay elsewhere
+  for (int i = 0; i < 2; ++i) {
+    if (ctx->set_layer[i] < 0 || (i != set && !other_area)) continue;
     // the half's previous user must be through: its output copied out, its compress (which may read Q) done
-    CU(cudaStreamWaitEvent(ctx->s_h2d, ctx->ev_out[set], 0));
-    const int pl = ctx->set_layer[set];
+    CU(cudaStreamWaitEvent(ctx->s_h2d, ctx->ev_out[i], 0));
+    const int pl = ctx->set_layer[i];
     if (ctx->ev_compress_live[pl]) CU(cudaStreamWaitEvent(ctx->s_h2d, ctx->ev_compress[pl], 0));
-    else CU(cudaStreamWaitEvent(ctx->s_h2d, ctx->ev_att[set], 0));
+    else CU(cudaStreamWaitEvent(ctx->s_h2d, ctx->ev_att[i], 0));
   }
+  ctx->stage_ptr = staging;
+  ctx->stage_half = half;
   CU(cudaMemcpyAsync(dk, K_host, bytes, cudaMemcpyHostToDevice, ctx->s_h2d));
   CU(cudaMemcpyAsync(dv, V_host, bytes, cudaMemcpyHostToDevice, ctx->s_h2d));
   CU(cudaMemcpyAsync(dq, Q_host, bytes, cudaMemcpyHostToDevice, ctx->s_h2d));
