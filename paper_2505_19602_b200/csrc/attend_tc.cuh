@@ -1,17 +1,22 @@
 // Tensor-core attention over the paged store for bf16, head_dim 128 (Sec. 3.3, Eq. 5):
-// O = softmax(scale * Q K^T) V with online softmax.  One CTA owns up to two 128-query tiles (A, B)
-// of one slice and streams the slice's K/V pages once for both.
+// O = softmax(scale * Q K^T) V with online softmax.  A CTA's work is one of
+//   a pair   : two 128-query tiles (A, B) of one slice; every key tile is streamed once for both;
+//   a single : one 128-query tile.  A and B are then the same queries against the even and against the odd key tiles, and
+//              the two partial results are combined at the end.  A single takes 0.55 of a pair's time, so it serves a map's
+//              last odd tile, launches that do not fill the GPU with pairs, and a launch's last, partial wave (see
+//              AttendTc::launch).  Where singles leave SMs idle as well, the CTAs of a cluster share a single's key tiles
+//              and combine through distributed shared memory.
 //
 // Roles inside a CTA of 384 threads:
 //   warp 0 (one thread) : TMA producer.  The query tiles once; then per 128-key tile the K and V rows into
-//                         128B-swizzled shared memory: history tiles page by page through the slice's
-//                         page table, tiles of a not yet appended current map from the caller's tensors.
+//                         128B-swizzled shared memory: first the tiles of a not yet appended current map from the caller's
+//                         tensors (those loads need neither the cache length nor the page table and go out while the
+//                         length is still being read), then the history tiles page by page through the page table.
 //   warp 1 (one thread) : tcgen05.mma issuer; owns the TMEM allocation (512 columns: two S/P buffers
-//                         and two O accumulators).  With two query tiles the issue order is
-//                         S_A(0), S_B(0), then per key tile j  PV_A(j), S_A(j+1), PV_B(j), S_B(j+1): while one
+//                         and two O accumulators).  The issue order is
+//                         S_A(0), S_B(0), then per step j  PV_A(j), S_A(j+1), PV_B(j), S_B(j+1): while one
 //                         tile's softmax runs, the tensor pipe works for the other tile, and a tile's next S
-//                         product follows its PV product without a wait in between.  With one query tile the two S buffers
-//                         alternate and S(j+1) is issued ahead of PV(j).
+//                         product follows its PV product without a wait in between.
 //   warps 4-7, 8-11     : softmax, one warpgroup per query tile (warps 4-7 tile A, warps 8-11 tile B), one
 //                         thread per query row (TMEM lane), so that no row state is shared between threads and
 //                         the two tiles' chains  S -> softmax -> PV  run concurrently, each hiding the other's
@@ -25,21 +30,29 @@
 //                         P chunks already stored for this tile, the running sum and the O accumulator are
 //                         scaled down, and the exponentials taken ahead for the next chunk are taken again.  Threads that own a row of the observation window also
 //                         store that row's raw products (16-byte stores, key tile j in columns 128 j ..) for
-//                         the compress that follows.  At the end each warpgroup normalises its O tile, stages
-//                         it in the query tile's shared memory and one thread sends it out with TMA stores.
-//                         With a single query tile (n_k <= 128, or the last odd tile of a map) warps 4-7 serve
-//                         both S buffers and warps 8-11 idle.
+//                         the compress that follows.  At the end every warp normalises its rows of the O tile and sends
+//                         them out through its part of the query tile's shared memory; the two parts of a single are
+//                         merged on the way, a cluster's parts by all warps afterwards.
 //   warps 2-3           : append.  When the current map has not been copied into the store yet, its K/V
 //                         tiles come from the caller's tensors, and the CTA whose turn it is writes each
 //                         tile's rows from shared memory to the slice's pages (and their original
 //                         positions), so the copy costs no extra read and stays off the critical path.
+// What bounds it: a CTA's steps are two chains  S -> softmax -> P V  that take turns on the tensor pipe, 3 290 cycles per step
+// of a pair (2 048 at the tensor peak; 3 480 while the MMA warp still formed its descriptors between the arrival of P and the
+// issue).  Around the steps a CTA costs ~8 000 cycles: 3 400 to the first scores (4 440 before the queries and the first key
+// tile were requested ahead of the length, with the tensor maps' descriptors prefetched), ~2 000 from the last product to the
+// last row (the bulk stores and the wait for them took ~1 000 more), the launch of the next CTA 1 300.
+// 128 slices x 4 096 queries: 1 052 -> 1 030 us per launch.
 // Every mbarrier wait is bounded; a wait that gives up raises the sticky device status, sets a
 // CTA-wide abort flag and all roles fall through to the common exit where TMEM is released.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
 
-#include <cstdlib>
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
 #include <type_traits>
 #include <string>
 
@@ -61,14 +74,20 @@ constexpr uint32_t kHalfBytes = kTileBytes / 2;  // 64 head-dim columns = one 12
 constexpr uint32_t kOffQ = 0;                    // two query tiles (the dynamic shared memory must start 1024-byte aligned)
 constexpr uint32_t kOffRing = kOffQ + 2 * kTileBytes;
 constexpr uint32_t kOffBar = kOffRing + kStages * kTileBytes;
-constexpr uint32_t kSmemBytes = kOffBar + 256;
+constexpr uint32_t kOffStat = kOffBar + 256;     // a shared single's rows: reference and sum of part A (then of both parts), of part B
+constexpr uint32_t kSmemBytes = kOffStat + 2 * 128 * 8;
 static_assert(kSmemBytes <= 232448, "more shared memory than a CTA can have");
 // barrier slots (8 bytes each): one full/empty pair per ring stage, one S/P/PV barrier per S buffer or query tile
 enum { bQFull = 0, bFull = 1, bEmpty = bFull + kStages, bSFull = bEmpty + kStages, bPFull = bSFull + 2, bPvDone = bPFull + 2,
-       bFinal = bPvDone + 2, bOut = bFinal + 2, bPEarly = bOut + 2, bPvEarly = bPEarly + 2, bCount = bPvEarly + 2 };
+       bFinal = bPvDone + 2, bPEarly = bFinal + 2, bPvEarly = bPEarly + 2, bCount = bPvEarly + 2 };
 constexpr uint32_t kOffTmemSlot = 208;            // inside the barrier area, behind the barriers
 static_assert(bCount * 8 <= kOffTmemSlot, "barriers overlap the TMEM slot");
 static_assert(bCount <= 32, "one lane of the first warp initialises each barrier");
+constexpr int kMaxSplit = 8;                      // CTAs that may share a single's keys (portable cluster size)
+// where the CTAs of a cluster leave the parts of the rows that this one finishes (up to 128 + kMaxSplit - 1 rows of 512 bytes),
+// and their references and sums
+constexpr uint32_t kOffPartStat = kOffRing + (128 + kMaxSplit) * 512;
+static_assert(kOffPartStat + (128 + kMaxSplit) * 8 <= kOffRing + kStages * kTileBytes, "the parts have to fit the ring");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColO = 256;       // S/P buffers at 0 and 128, O accumulators at 256 and 384
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
@@ -120,6 +139,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   if (mbar_try(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, abort_flag, status);
 }
+// For a CTA that gives up: waits for a copy of its own that is still under way, whatever the status, a second at most.
+__device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  const unsigned long long t0 = globaltimer();
+  while (!mbar_try(bar, parity) && globaltimer() - t0 < kWaitLimitNs / 2) {}
+}
 // Self-test of the bounded wait (scalekv_selftest_wait): one warp waits, with the given limit, on a barrier
 // that nobody ever arrives at.  The wait must give up, raise the sticky status and return; a second warp that
 // polls the CTA's abort flag (also bounded) shows that the other roles of a CTA see the give-up.
@@ -162,18 +186,8 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm,
       : "memory");
 }
 
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap *tm, uint32_t src, int x, int y, int z, int w) {
-  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(tm), "r"(src), "r"(x), "r"(y),
-               "r"(z), "r"(w)
-               : "memory");
-}
-__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// waits until the bulk stores committed so far have READ their shared-memory source (the CTA may then leave; the
-// writes to global memory complete on their own)
-__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// orders this thread's shared-memory writes before later reads of the asynchronous (TMA) proxy
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
@@ -210,24 +224,6 @@ __device__ __forceinline__ void tc_mma_ss_x8(uint32_t d_tmem, uint32_t a_lo, uin
 // TS: A = P in TMEM (16 keys = 8 columns per step; a row's 128 bf16 values of P fill the first 64 columns of
 // its S buffer), B = V in shared memory as the MN-major operand (16 keys = 2048 B per step).
 __device__ __forceinline__ constexpr uint32_t p_col(int kk) { return (uint32_t)(kk * 8); }
-__device__ __forceinline__ void tc_mma_ts_x8(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
-                                             uint32_t accumulate_first) {
-  asm volatile(
-      "{\n\t.reg .pred e, pf, pt;\n\t.reg .b64 db;\n\t.reg .b32 at, bl;\n\t"
-      "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 pf, %5, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-      "mov.b64 db, {%2, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pf;\n\t"
-      "add.u32 at, %1, %6;\n\tadd.u32 bl, %2, 128;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, %7;\n\tadd.u32 bl, %2, 256;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, %8;\n\tadd.u32 bl, %2, 384;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, %9;\n\tadd.u32 bl, %2, 512;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, %10;\n\tadd.u32 bl, %2, 640;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, %11;\n\tadd.u32 bl, %2, 768;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, %12;\n\tadd.u32 bl, %2, 896;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "}" ::"r"(d_tmem),
-      "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first), "n"(p_col(1)), "n"(p_col(2)), "n"(p_col(3)), "n"(p_col(4)),
-      "n"(p_col(5)), "n"(p_col(6)), "n"(p_col(7))
-      : "memory");
-}
 // The first N of the eight steps (a_tmem and b_lo address the first of them).
 template <int N>
 __device__ __forceinline__ void tc_mma_ts_n(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
@@ -417,11 +413,23 @@ __device__ __noinline__ Raised raise_reference(int valid, float c, float m, floa
   return {m_new, l_run * f, sum, o_landed, 1};
 }
 
+// Division of numbers below 2^21 by a divisor below 2^21 the quick way (the remainder of 2^42 costs less than one quotient):
+// a CTA finds its item with three of these, and its first loads wait for it.
+struct Divisor {
+  unsigned long long mul;
+  int d;
+  static Divisor of(int d) { return {(1ull << 42) / (unsigned)d + 1, d}; }
+  __device__ __forceinline__ int div(int x) const { return (int)(((unsigned long long)(unsigned)x * mul) >> 42); }
+};
+
 struct Params {
   LayerView lv;
   TensorView O;
   float *lse;
   int n_k;
+  int n_pair;          // items [0, n_pair) walk the slices pair by pair, the others tile by tile
+  int cut_tile;        // tiles (of all slices) that the first n_pair items cover
+  Divisor per_pair, per_tile, per_heads;   // items of a slice pair by pair, tiles of a slice, heads
   float scale_log2e;   // softmax scale * log2(e)
   int box_rows;        // rows per K/V TMA box = min(page_tokens, 128)
   int fused_append;    // 1: the current map's K/V rows are still in the caller's tensors; read them there
@@ -436,13 +444,185 @@ struct Params {
   int win_pos[kMaxWindow];   // ascending raster indices of the window rows inside the current map
 };
 
+// rows that each CTA of a cluster finishes
+__device__ __forceinline__ int cluster_share(int n_k, int first_row, int n_split) { return (min(128, n_k - first_row) + n_split - 1) / n_split; }
+__device__ __forceinline__ uint32_t remote(uint32_t addr, int cta) {
+  uint32_t ra;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(cta));
+  return ra;
+}
+
+// The end of a softmax warp's work: its 32 rows of the O accumulator at o_addr, with references m and sums l, are normalised
+// and stored (have: there were keys for this tile).  A function of its own so that the sweep's registers are not allocated
+// around it.  window: this thread's row belongs to the observation window.
+__device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, uint32_t o_addr, int slice, int first_row, int qt, bool pair,
+                                         bool shared, bool have, int n_split, float m, float l, bool window) {
+  const int n_k = prm.n_k;
+  const int lane = threadIdx.x & 31, quarter = (threadIdx.x >> 5) & 3, row = quarter * 32 + lane;
+  // Output rows leave through shared memory, 32 columns of the warp's 32 rows at a time (128 of a row's 256 bytes there), so that a store instruction
+  // writes eight whole 64-byte pieces (a row written by its own thread straight from the registers touches 32 lines per
+  // instruction) and neither another warp nor an asynchronous copy has to be waited for.  16-byte pieces are permuted by
+  // the row's index against bank conflicts. 
+  const int b = prm.per_heads.div(slice), h = slice - b * prm.per_heads.d;
+  const int w0 = first_row + (pair ? qt * 128 : 0) + quarter * 32;       // the warp's first row
+  const int sub = lane >> 2, piece = lane & 3;
+  char *out = const_cast<char *>(prm.O.ptr) +
+              ((long long)b * prm.O.sb + (long long)h * prm.O.sh + (long long)(w0 + sub) * prm.O.st) * 2 + piece * 16;
+  auto slot = [](int r, int i) { return (uint32_t)r * 256 + (uint32_t)(((i ^ ((r >> 1) & 3)) + 4 * (r & 1)) << 4); };
+  auto emit = [&](const uint32_t *pk, uint32_t stage, int col) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + slot(lane, i)), "r"(pk[4 * i]),
+                   "r"(pk[4 * i + 1]), "r"(pk[4 * i + 2]), "r"(pk[4 * i + 3])
+                   : "memory");
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = 8 * i + sub;
+      uint4 val;
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
+                   : "r"(stage + slot(r, piece)) : "memory");
+      if (w0 + r < n_k) *reinterpret_cast<uint4 *>(out + i * prm.O.st * 16 + col * 2) = val;
+    }
+  };
+  auto row_sums = [&](float mr, float lr) {              // what is kept of a row besides its output
+    const float y = mr + log2f(lr);
+    if (prm.lse != nullptr && w0 + lane < n_k) prm.lse[(size_t)slice * n_k + w0 + lane] = y * 0.6931471805599453f;
+    if (window) {
+      int rank = 0;
+      for (int e = 0; e < prm.w; ++e)
+        if (prm.win_pos[e] == w0 + lane) rank = e;
+      prm.win_lse[(size_t)slice * prm.w + rank] = y;
+    }
+  };
+  if (!shared) {
+    if (have) {
+      const float inv = 1.f / l;
+      const uint32_t stage = base + kOffQ + qt * kTileBytes + quarter * 8192;    // (no product reads the query tile any more)
+      float o[2][32];
+      tc_ld32(o_addr, o[0]);
+#pragma unroll
+      for (int cc = 0; cc < kChunks; ++cc) {
+        uint32_t pk[16];
+        tc_wait_ld();
+        if (cc + 1 < kChunks) tc_ld32(o_addr + (cc + 1) * 32, o[(cc + 1) & 1]);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(o[cc & 1][2 * i] * inv, o[cc & 1][2 * i + 1] * inv);
+        emit(pk, stage + (cc & 1) * 128, cc * 32);
+      }
+      row_sums(m, l);
+    }
+  } else {
+    // ---- the two parts of a shared single are merged: each warpgroup takes half of the columns and hands the other one
+    // its own values of the other half (fp32, 16-byte pieces of a row permuted by its index).  A row's pieces are read and
+    // written by the threads of that row alone.
+    asm volatile("bar.sync 2, 256;" ::: "memory");         // no product reads the query tile any more
+    const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256, theirs = base + kOffQ + (qt ^ 1) * kTileBytes + row * 256;
+#pragma unroll 1
+    for (int cc = 0; cc < 2; ++cc) {
+      float o[32];
+      if (have) { tc_ld32(o_addr + (qt ^ 1) * 64 + cc * 32, o); tc_wait_ld(); }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float x0 = have ? o[4 * i] : 0.f, x1 = have ? o[4 * i + 1] : 0.f, x2 = have ? o[4 * i + 2] : 0.f, x3 = have ? o[4 * i + 3] : 0.f;
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(theirs + (uint32_t)((cc * 8 + (i ^ (row & 7))) << 4)), "f"(x0), "f"(x1),
+                     "f"(x2), "f"(x3)
+                     : "memory");
+      }
+    }
+    if (!have) { m = -INFINITY; l = 0.f; }
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(base + kOffStat + (uint32_t)(qt * 128 + row) * 8), "f"(m), "f"(l) : "memory");
+    asm volatile("bar.sync 2, 256;" ::: "memory");
+    float m2, l2;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(base + kOffStat + (uint32_t)((qt ^ 1) * 128 + row) * 8) : "memory");
+    const float M = fmaxf(m, m2);
+    float f1 = l > 0.f ? ex2(m - M) : 0.f, f2 = l2 > 0.f ? ex2(m2 - M) : 0.f;
+    const float both = l * f1 + l2 * f2;
+    // of a cluster the rows' owner: it gets this CTA's merged part, unnormalised, with its reference and sum
+    const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(row / own_rows, n_split - 1);   // (rows beyond the map go nowhere)
+    uint32_t dst = 0;
+    if (n_split == 1) {
+      f1 /= both; f2 /= both;
+    } else {
+      cluster_wait();                                     // every CTA of the cluster is through with its ring
+      dst = remote(base + kOffRing + (uint32_t)((int)blockIdx.z * own_rows + row - owner * own_rows) * 512, owner);
+      if (qt == 0 && first_row + row < n_k)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
+                         remote(base + kOffPartStat + (uint32_t)((int)blockIdx.z * own_rows + row - owner * own_rows) * 8, owner)),
+                     "f"(M), "f"(both)
+                     : "memory");
+    }
+#pragma unroll 1
+    for (int cc = 0; cc < 2; ++cc) {
+      float o[32];
+      uint32_t pk[16];
+      if (have) { tc_ld32(o_addr + qt * 64 + cc * 32, o); tc_wait_ld(); }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float x[4];
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
+                     : "r"(mine + (uint32_t)((cc * 8 + (i ^ (row & 7))) << 4)) : "memory");
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = (have ? o[4 * i + e] * f1 : 0.f) + x[e] * f2;
+        pk[2 * i] = pack_bf16(x[0], x[1]);
+        pk[2 * i + 1] = pack_bf16(x[2], x[3]);
+        if (n_split > 1 && first_row + row < n_k)
+          asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(((qt * 16 + cc * 8 + i) ^ (row & 31)) << 4)),
+                       "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3])
+                       : "memory");
+      }
+      __syncwarp();
+      if (n_split == 1) emit(pk, base + kOffQ + qt * kTileBytes + quarter * 8192 + cc * 128, qt * 64 + cc * 32);   // (where it has read)
+    }
+    if (n_split == 1 && qt == 0) row_sums(M, both);
+  }
+}
+
+// The end of a cluster's work: O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e with M the largest reference, for this CTA's
+// share of the rows, from the parts that the CTAs of the cluster have left here.  A warp takes a row at a time, a lane four
+// columns of it.
+__device__ __forceinline__ void finish_cluster(const Params &prm, uint32_t base, int slice, int q_first, int n_split) {
+  const int n_k = prm.n_k;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = prm.per_heads.div(slice), h = slice - b * prm.per_heads.d;
+  const int own_rows = cluster_share(n_k, q_first, n_split), r_lo = (int)blockIdx.z * own_rows, r_hi = min(r_lo + own_rows, min(128, n_k - q_first));
+  char *obase = const_cast<char *>(prm.O.ptr) + ((long long)b * prm.O.sb + (long long)h * prm.O.sh) * 2;
+  static_assert(kMaxWindow <= 64, "two window positions per lane");
+  const int wpos0 = prm.win_pos[lane] - q_first, wpos1 = prm.win_pos[lane + 32] - q_first;   // (unused ones are negative)
+#pragma unroll 2
+  for (int r = r_lo + warp; r < r_hi; r += kThreads / 32) {
+    const uint32_t src = base + kOffRing + (uint32_t)(r - r_lo) * 512 + (uint32_t)((lane ^ (r & 31)) << 4);
+    const uint32_t stat = base + kOffPartStat + (uint32_t)(r - r_lo) * 8;
+    float M = -INFINITY, sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 2
+    for (int e = 0; e < n_split; ++e) {
+      float me, le;
+      float4 x;
+      asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(me), "=f"(le) : "r"(stat + (uint32_t)(e * own_rows) * 8));
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(src + (uint32_t)(e * own_rows) * 512));
+      if (le > 0.f) {                                     // (a part without keys counts for nothing)
+        const float top = fmaxf(M, me), f0 = ex2(M - top), f = ex2(me - top);
+        M = top;
+        sum = sum * f0 + le * f;
+        a0 = a0 * f0 + x.x * f; a1 = a1 * f0 + x.y * f; a2 = a2 * f0 + x.z * f; a3 = a3 * f0 + x.w * f;
+      }
+    }
+    const float inv = 1.f / sum;
+    const int qi = q_first + r;
+    *reinterpret_cast<uint2 *>(obase + (long long)qi * prm.O.st * 2 + lane * 8) = make_uint2(pack_bf16(a0 * inv, a1 * inv), pack_bf16(a2 * inv, a3 * inv));
+    const float y = M + log2f(sum);
+    if (prm.lse != nullptr && lane == 0) prm.lse[(size_t)slice * n_k + qi] = y * 0.6931471805599453f;
+    if (wpos0 == r || wpos1 == r) prm.win_lse[(size_t)slice * prm.w + lane + (wpos0 == r ? 0 : 32)] = y;
+  }
+}
+
 // kWindow: the launch records the observation window's logits; the instance without that code serves the launches
 // that record nothing (its mere presence costs every warp's sweep 2-3 %).
 template <bool kWindow>
 __global__ void __launch_bounds__(kThreads, 1)
 attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKc,
-                 const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ CUtensorMap tmO, const Params prm) {
+                 const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ Params prm) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   uint8_t *base_ptr = smem_raw;
@@ -453,22 +633,28 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const LayerView &lv = prm.lv;
-  const int slice = blockIdx.y;
-  const int b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int n_k = prm.n_k;
-  const int q_first = blockIdx.x * 256;                  // first query row of tile A
-  const bool single = q_first + 128 >= n_k;              // tile B would be empty
+  // This CTA's queries: slice by slice, so that CTAs that run together share a slice's K and V in L2, first pair by pair
+  // (a slice's last odd tile is a single), then, behind the first n_pair items, tile by tile.
+  const int tiles = (n_k + 127) >> 7;                    // query tiles of a slice
+  const int e = (int)blockIdx.x - prm.n_pair;
+  const int at = e < 0 ? (int)blockIdx.x : prm.cut_tile + e;
+  const int slice = e < 0 ? prm.per_pair.div(at) : prm.per_tile.div(at);
+  const int q_tile = e < 0 ? 2 * (at - slice * prm.per_pair.d) : at - slice * prm.per_tile.d;
+  const bool pair = e < 0 && q_tile + 1 < tiles;
+  const int b = prm.per_heads.div(slice), h = slice - b * prm.per_heads.d;
+  const int q_first = q_tile * 128;                      // first query row of tile A
+  const int n_split = gridDim.z;                         // CTAs (of a cluster) that share this item's keys
   // What needs no global memory comes first: the lanes of warp 0 initialise one barrier each, warp 1 allocates the
-  // TMEM.  When the launch allows it (programmatic stream serialisation) this part runs while the kernel before this
+  // TMEM, warp 2 fetches the tensor maps' descriptors.  When the launch allows it (programmatic stream serialisation) this part runs while the kernel before this
   // one in the stream is still finishing; `griddepcontrol.wait` then holds every thread until that kernel's writes
   // - cache lengths, page tables, pages, the status word - are visible.  The grid behind this one may come up as
   // soon as all of this grid's CTAs are running.
   if (warp == 0) {
     if (lane < bCount) {
-      // arrivals per phase: a ring stage is released by the MMA warp's commit and the two append warps; P, early P and
-      // the staged output tile are announced by one lane of each of the four warps of a softmax warpgroup
-      const bool four = (lane >= bPFull && lane < bPFull + 2) || (lane >= bPEarly && lane < bPEarly + 2) ||
-                        (lane >= bOut && lane < bOut + 2);
+      // arrivals per phase: a ring stage is released by the MMA warp's commit and the two append warps; P and early P
+      // are announced by one lane of each of the four warps of a softmax warpgroup
+      const bool four = (lane >= bPFull && lane < bPFull + 2) || (lane >= bPEarly && lane < bPEarly + 2);
       const bool three = lane >= bEmpty && lane < bEmpty + kStages;
       mbar_init(bar(lane), four ? 4u : (three ? 3u : 1u));
     }
@@ -477,40 +663,61 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + kOffBar + kOffTmemSlot), "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else if (warp == 2 && lane < 5) {
+    const CUtensorMap *tm = lane == 0 ? &tmQ : (lane == 1 ? &tmKc : (lane == 2 ? &tmVc : (lane == 3 ? &tmK : &tmV)));
+    asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
   }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int hist = lv.hist_len[slice];
-  const int L = hist + n_k;
-  // key tiles: Th from the pages (all of them unless the current map still waits in the caller's
-  // tensors), then Tc of the current map; each source ends in a ragged tile
   const bool fused = prm.fused_append != 0;
-  const int Th = ((fused ? hist : L) + 127) >> 7;
-  const int Tc = fused ? (n_k + 127) >> 7 : 0;
-  const int T = Th + Tc;
-  auto tile_valid = [&](int j) {   // number of real keys in tile j
-    const int rest = j < Th ? (fused ? hist : L) - j * 128 : n_k - (j - Th) * 128;
-    return rest < 128 ? rest : 128;
-  };
   int *status = lv.status;
-  // Set-up, one rendezvous for everything.  Warp 0: its first lane decides for the whole CTA whether it runs at all
-  // (one thread, because the status word may change between two threads' reads, and a CTA of which only a part
-  // left would go on with barriers and TMEM nobody set up): an earlier CTA gave up - do not pile on; swizzled
-  // tiles need the alignment, and a slice must not outgrow its page table - report, do not fault.  Meanwhile the
-  // warp's lanes initialise one barrier each.  Warp 1 allocates the TMEM.  Everybody but warp 0 then waits on a
-  // named barrier for the barriers, the decision and the allocation; warp 0 (the TMA producer) needs neither the
-  // TMEM address nor anybody else: it only announces its part and goes on to issue the first loads while the
-  // allocation is still under way.
+  // Set-up, one rendezvous for everything.  Warp 0 asks for the slice's length, sends the first loads on their way - the
+  // queries and, unless the keys are split over a cluster, the first K tile of a current map in the caller's tensors -
+  // and then decides for the whole CTA whether it runs at all (one thread, because the status word may change between two
+  // threads' reads, and a CTA of which only a part left would go on with barriers and TMEM nobody set up): an earlier CTA
+  // gave up - do not pile on; swizzled tiles need the alignment, and a slice must not outgrow its page table - report,
+  // do not fault.  Everybody but warp 0 then waits on a named barrier for the barriers, the length, the decision and the
+  // TMEM allocation; warp 0 needs nobody: it goes on to issue loads.
   volatile int *leave_slot = reinterpret_cast<volatile int *>(base_ptr + kOffBar + kOffTmemSlot + 8);
-  int leave = 0;
+  volatile int *hist_slot = reinterpret_cast<volatile int *>(base_ptr + kOffBar + kOffTmemSlot + 12);
+  volatile int *item_slot = hist_slot + 1;               // slice and first query row, for the end of the softmax warps' work
+  int leave = 0, hist = 0;
+  const int Tc = fused ? tiles : 0;                      // key tiles of a current map outside the pages
+  const int early = n_split == 1 && Tc > 0 ? 1 : 0;       // ring tiles that are loaded right away
+  // ring tile t (2 i is K, 2 i + 1 is V of the i-th key tile), which belongs to key tile c of the current map
+  auto load_map_tile = [&](int t, int c) {               // one lane
+    const int st = t % kStages;
+    const CUtensorMap *tc = (t & 1) ? &tmVc : &tmKc;
+    const uint32_t dst = base + kOffRing + st * kTileBytes;
+    mbar_expect_tx(bar(bFull + st), kTileBytes);
+    tma_load_4d(dst, tc, 0, c * 128, h, b, bar(bFull + st));
+    tma_load_4d(dst + kHalfBytes, tc, 64, c * 128, h, b, bar(bFull + st));
+  };
   if (warp == 0) {
     if (lane == 0) {
-      if (*reinterpret_cast<volatile int *>(status) != 0) leave = 1;
-      else if ((base & 1023u) || L > (lv.pages_per_slice << lv.page_shift)) { atomicExch(status, kDevCheck); leave = 1; }
+      const int len = *reinterpret_cast<volatile int *>(lv.hist_len + slice), st = *reinterpret_cast<volatile int *>(status);
+      if (!(base & 1023u)) {
+        const int nq = pair ? 2 : 1;
+        mbar_expect_tx(bar(bQFull), nq * kTileBytes);
+        for (int t = 0; t < nq; ++t) {
+          tma_load_4d(base + kOffQ + t * kTileBytes, &tmQ, 0, q_first + t * 128, h, b, bar(bQFull));
+          tma_load_4d(base + kOffQ + t * kTileBytes + kHalfBytes, &tmQ, 64, q_first + t * 128, h, b, bar(bQFull));
+          if (t == 0 && early > 0) load_map_tile(0, 0);
+        }
+      }
+      hist = len;
+      if (st != 0) leave = 1;
+      else if ((base & 1023u) || hist + n_k > (lv.pages_per_slice << lv.page_shift)) { atomicExch(status, kDevCheck); leave = 1; }
       *abort_flag = 0;
       *leave_slot = leave;
+      *hist_slot = hist;
+      item_slot[0] = slice;
+      item_slot[1] = q_first;
+      // the length that the next scale finds unless a compress of this one evicts
+      if (!leave && q_tile == 0 && blockIdx.z == 0) lv.next_len[slice] = hist + n_k;
     }
     leave = __shfl_sync(0xffffffffu, leave, 0);
+    hist = __shfl_sync(0xffffffffu, hist, 0);
     __syncwarp();
     __threadfence_block();
     asm volatile("bar.arrive 1, %0;" ::"n"(kThreads) : "memory");
@@ -519,183 +726,155 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
     tc_fence_after();
     leave = *leave_slot;
+    hist = *hist_slot;
   }
-  if (leave) {
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kTmemCols) : "memory");
-    return;
-  }
+  // Key tiles: Tc of the current map when it still waits in the caller's tensors, then Th of the pages; each source ends in a
+  // ragged tile.  This CTA streams the tiles lo .. lo + nt - 1.
+  const int rows_h = fused ? hist : hist + n_k;          // entries in the pages
+  const int Th = (rows_h + 127) >> 7;
+  const int lo = (Tc + Th) * (int)blockIdx.z / n_split;
+  const int nt = leave ? 0 : (Tc + Th) * ((int)blockIdx.z + 1) / n_split - lo;
+  auto tile_valid = [&](int i) {   // number of real keys in tile i
+    const int rest = i < Tc ? n_k - i * 128 : rows_h - (i - Tc) * 128;
+    return rest < 128 ? rest : 128;
+  };
+  // A single's key tiles are shared by A and B - unless they are so few that the combination would cost more than it gives:
+  // then A takes them all.
+  const bool shared = !pair && (n_split > 1 || nt > 2);
+  // key tiles that the softmax of tile A / B sees
+  auto n_steps = [&](int qt) { return shared ? (nt + 1 - qt) >> 1 : (pair || qt == 0 ? nt : 0); };
   const uint32_t tmem = warp == 0 ? 0u : *tmem_slot;
 
   if (warp < 4) {
   if (warp == 0) {
-    {
-      // ---------------------------------------------------------------- TMA producer
-      // (the whole warp walks the loop so that addresses stay warp-uniform; one lane issues)
-      const int nq = single ? 1 : 2;
-      if (elect_one()) {
-        mbar_expect_tx(bar(bQFull), nq * kTileBytes);
-        for (int t = 0; t < nq; ++t) {
-          tma_load_4d(base + kOffQ + t * kTileBytes, &tmQ, 0, q_first + t * 128, h, b, bar(bQFull));
-          tma_load_4d(base + kOffQ + t * kTileBytes + kHalfBytes, &tmQ, 64, q_first + t * 128, h, b, bar(bQFull));
-        }
-      }
-      const int R = prm.box_rows;
-      const int last_page = fused ? (hist > 0 ? (hist - 1) >> lv.page_shift : 0) : (L - 1) >> lv.page_shift;
-      const int *pt = lv.page_table + (size_t)slice * lv.pages_per_slice;
-      bool ok = true;
-      // ring tile t = 2 j is K_j, t = 2 j + 1 is V_j
-      for (int t = 0; t < 2 * T && ok; ++t) {
-        const int st = t % kStages, j = t >> 1;
-        ok = mbar_wait_warp(bar(bEmpty + st), ((t / kStages) & 1) ^ 1, abort_flag, status);
-        if (!ok) break;
+    // ---------------------------------------------------------------- TMA producer
+    // (the whole warp walks the loop so that addresses stay warp-uniform; one lane issues)
+    const int R = prm.box_rows;
+    const int last_page = rows_h > 0 ? (rows_h - 1) >> lv.page_shift : 0;
+    const int *pt = lv.page_table + (size_t)slice * lv.pages_per_slice;
+    bool ok = nt > 0;
+    int t = early;
+    for (; t < 2 * nt && ok; ++t) {
+      const int st = t % kStages, i = lo + (t >> 1);
+      ok = mbar_wait_warp(bar(bEmpty + st), ((t / kStages) & 1) ^ 1, abort_flag, status);
+      if (!ok) break;
+      if (i < Tc) {
+        if (elect_one()) load_map_tile(t, i);
+      } else if (elect_one()) {
         const CUtensorMap *tm = (t & 1) ? &tmV : &tmK;
-        if (j >= Th) {
-          if (elect_one()) {
-            const CUtensorMap *tc = (t & 1) ? &tmVc : &tmKc;
-            const uint32_t dst = base + kOffRing + st * kTileBytes;
-            mbar_expect_tx(bar(bFull + st), kTileBytes);
-            tma_load_4d(dst, tc, 0, (j - Th) * 128, h, b, bar(bFull + st));
-            tma_load_4d(dst + kHalfBytes, tc, 64, (j - Th) * 128, h, b, bar(bFull + st));
-          }
-        } else if (elect_one()) {
-          mbar_expect_tx(bar(bFull + st), kTileBytes);
-          for (int r0 = 0; r0 < 128; r0 += R) {
-            const int slot = j * 128 + r0;
-            int lp = slot >> lv.page_shift;
-            lp = lp > last_page ? last_page : lp;
-            const int row = (__ldg(pt + lp) << lv.page_shift) + (slot & lv.page_mask);
-            const uint32_t dst = base + kOffRing + st * kTileBytes + r0 * 128;
-            tma_load_2d(dst, tm, 0, row, bar(bFull + st));
-            tma_load_2d(dst + kHalfBytes, tm, 64, row, bar(bFull + st));
-          }
+        mbar_expect_tx(bar(bFull + st), kTileBytes);
+        for (int r0 = 0; r0 < 128; r0 += R) {
+          const int slot = (i - Tc) * 128 + r0;
+          int lp = slot >> lv.page_shift;
+          lp = lp > last_page ? last_page : lp;
+          const int row = (__ldg(pt + lp) << lv.page_shift) + (slot & lv.page_mask);
+          const uint32_t dst = base + kOffRing + st * kTileBytes + r0 * 128;
+          tma_load_2d(dst, tm, 0, row, bar(bFull + st));
+          tma_load_2d(dst + kHalfBytes, tm, 64, row, bar(bFull + st));
         }
-        __syncwarp();
       }
+      __syncwarp();
     }
+    if (!ok && !(base & 1023u)) {
+      // this CTA gives up or has no keys: nothing may land in its shared memory once that is used for something else or gone
+      mbar_drain(bar(bQFull), 0);
+      for (int k = t > kStages ? t - kStages : 0; k < t; ++k) mbar_drain(bar(bFull + k % kStages), (k / kStages) & 1);
+    }
+    if (n_split > 1) cluster_arrive();
   } else if (warp == 1) {
-    {
-      // ---------------------------------------------------------------- MMA issuer
-      // (the whole warp walks the loop and waits; one elected lane issues the MMAs and commits)
-      constexpr uint32_t idesc_qk = instr_desc(false);
-      constexpr uint32_t idesc_pv = instr_desc(true);
-      bool ok = mbar_wait_warp(bar(bQFull), 0, abort_flag, status);
-      // S buffer `buf` = Q tile `qt` times K tile j (transposed)
-      constexpr uint32_t dhi = desc_hi(1024);
-      const bool leader = elect_one();
-      const uint32_t q_lo[2] = {desc_lo(base + kOffQ, 16), desc_lo(base + kOffQ + kTileBytes, 16)};
-      auto issue_s = [&](int j, int qt, int buf) {
-        const uint32_t a_lo = q_lo[qt], b_lo = desc_lo(base + kOffRing + ((2 * j) % kStages) * kTileBytes, 16);
-        const uint32_t d = tmem + kColS + buf * 128;
-        tc_mma_ss_x8(d, a_lo, b_lo, dhi, idesc_qk);
-        if (leader) tc_commit(bar(bSFull + buf));
-        __syncwarp();
-      };
-      // O of tile `qt` += P (bf16 pairs in the first 32 columns of each half of S buffer `buf`) times V tile t
-      auto issue_pv = [&](int t, int qt, int buf, uint32_t p_parity, bool release_v) -> bool {
-        const int vt = 2 * t + 1, vs = vt % kStages;
-        if (!mbar_wait_warp(bar(bFull + vs), (vt / kStages) & 1, abort_flag, status)) return false;
-        if (!mbar_wait_warp(bar(bPFull + buf), p_parity, abort_flag, status)) return false;
+    // ---------------------------------------------------------------- MMA issuer
+    // (the whole warp walks the loop and waits; one elected lane issues the MMAs and commits)
+    constexpr uint32_t idesc_qk = instr_desc(false);
+    constexpr uint32_t idesc_pv = instr_desc(true);
+    constexpr uint32_t dhi = desc_hi(1024);
+    const bool leader = elect_one();
+    const uint32_t q_lo[2] = {desc_lo(base + kOffQ, 16), desc_lo(base + kOffQ + (pair ? kTileBytes : 0u), 16)};
+    // ring tile of tile qt's K in step j (its V is the next one): a pair's tiles share it, a single's take turns
+    auto ring_k = [&](int j, int qt) { return shared ? 4 * j + 2 * qt : 2 * j; };
+    auto ring_full = [&](int t) { return mbar_wait_warp(bar(bFull + t % kStages), (t / kStages) & 1, abort_flag, status); };
+    // A tile's chain is  sweep -> PV(j) -> S(j+1) -> sweep ..., so between the moment a tile's P is complete
+    // and the issue of its next S product this warp does nothing but issue: the operands of both products
+    // are waited for beforehand (they arrive long before P does), the two products go out back to back, and the
+    // commits follow them.
+    auto k_desc = [&](int kt) { return desc_lo(base + kOffRing + (kt % kStages) * kTileBytes, 16); };
+    auto mma_s = [&](uint32_t kd, int qt) { tc_mma_ss_x8(tmem + kColS + qt * 128, q_lo[qt], kd, dhi, idesc_qk); };
+    constexpr int kEarlySteps = 2 * kEarlyChunks;      // a chunk of 32 keys is two steps of 16
+    auto mma_pv_early = [&](uint32_t vd, int qt, bool accumulate) {
+      tc_mma_ts_n<kEarlySteps>(tmem + kColO + qt * 128, tmem + kColS + qt * 128, vd, dhi, idesc_pv, accumulate ? 1u : 0u);
+    };
+    auto mma_pv_rest = [&](uint32_t vd, int qt) {
+      tc_mma_ts_n<8 - kEarlySteps>(tmem + kColO + qt * 128, tmem + kColS + qt * 128 + p_col(kEarlySteps), vd + 128 * kEarlySteps, dhi,
+                                   idesc_pv, 1u);
+    };
+    const int steps[2] = {n_steps(0), n_steps(1)};
+    bool ok = nt > 0 && mbar_wait_warp(bar(bQFull), 0, abort_flag, status);
+    for (int qt = 0; qt < 2 && ok && steps[qt] > 0; ++qt) {
+      const int kt = ring_k(0, qt);
+      ok = ring_full(kt);
+      if (!ok) break;
+      tc_fence_after();
+      mma_s(k_desc(kt), qt);
+      if (leader) {
+        tc_commit(bar(bSFull + qt));
+        if (!pair || qt == 1) tc_commit(bar(bEmpty + kt % kStages));
+      }
+      __syncwarp();
+    }
+    for (int j = 0; j < steps[0] && ok; ++j) {
+      for (int qt = 0; qt < 2 && ok; ++qt) {
+        if (j >= steps[qt]) break;
+        const bool more = j + 1 < steps[qt];
+        const int vt = ring_k(j, qt) + 1, kt = ring_k(j + 1, qt);
+        const uint32_t vd = desc_lo(base + kOffRing + (vt % kStages) * kTileBytes, kHalfBytes), kd = k_desc(kt);
+        const uint32_t v_empty = bar(bEmpty + vt % kStages), k_empty = bar(bEmpty + kt % kStages);
+        ok = ring_full(vt) && mbar_wait_warp(bar(bPEarly + qt), j & 1, abort_flag, status);
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t b_lo = desc_lo(base + kOffRing + vs * kTileBytes, kHalfBytes);
-        const uint32_t d = tmem + kColO + qt * 128, a = tmem + kColS + buf * 128;
-        const uint32_t acc0 = t > 0 ? 1u : 0u;
-        tc_mma_ts_x8(d, a, b_lo, dhi, idesc_pv, acc0);
-        if (leader) {
-          tc_commit(bar(bPvDone + qt));
-          if (release_v) tc_commit(bar(bEmpty + vs));
-        }
+        mma_pv_early(vd, qt, j > 0);
+        if (leader) tc_commit(bar(bPvEarly + qt));
         __syncwarp();
-        return true;
-      };
-      if (!single) {
-        // A tile's chain is  sweep -> PV(j) -> S(j+1) -> sweep ..., so between the moment a tile's P is complete
-        // and the issue of its next S product this warp does nothing but issue: the operands of both products
-        // are waited for beforehand (they arrive long before P does), the two products go out back to back, and the
-        // commits follow them.
-        auto ring_full = [&](int t) { return mbar_wait_warp(bar(bFull + t % kStages), (t / kStages) & 1, abort_flag, status); };
-        auto mma_s = [&](int j, int qt) {
-          tc_mma_ss_x8(tmem + kColS + qt * 128, q_lo[qt], desc_lo(base + kOffRing + ((2 * j) % kStages) * kTileBytes, 16), dhi, idesc_qk);
-        };
-        constexpr int kEarlySteps = 2 * kEarlyChunks;      // a chunk of 32 keys is two steps of 16
-        auto mma_pv_early = [&](int j, int qt) {
-          tc_mma_ts_n<kEarlySteps>(tmem + kColO + qt * 128, tmem + kColS + qt * 128,
-                                   desc_lo(base + kOffRing + ((2 * j + 1) % kStages) * kTileBytes, kHalfBytes), dhi, idesc_pv,
-                                   j > 0 ? 1u : 0u);
-        };
-        auto mma_pv_rest = [&](int j, int qt) {
-          tc_mma_ts_n<8 - kEarlySteps>(tmem + kColO + qt * 128, tmem + kColS + qt * 128 + p_col(kEarlySteps),
-                                       desc_lo(base + kOffRing + ((2 * j + 1) % kStages) * kTileBytes, kHalfBytes) + 128 * kEarlySteps,
-                                       dhi, idesc_pv, 1u);
-        };
-        ok = ok && ring_full(0);
-        if (ok) {
-          tc_fence_after();
-          mma_s(0, 0);
-          if (leader) tc_commit(bar(bSFull + 0));
-          __syncwarp();
-          mma_s(0, 1);
-          if (leader) { tc_commit(bar(bSFull + 1)); tc_commit(bar(bEmpty + 0)); }
-          __syncwarp();
-        }
-        for (int j = 0; j < T && ok; ++j) {
-          const bool more = j + 1 < T;
-          ok = ring_full(2 * j + 1) && (!more || ring_full(2 * j + 2));
-          for (int qt = 0; qt < 2 && ok; ++qt) {
-            ok = mbar_wait_warp(bar(bPEarly + qt), j & 1, abort_flag, status);
-            if (!ok) break;
-            tc_fence_after();
-            mma_pv_early(j, qt);
-            if (leader) tc_commit(bar(bPvEarly + qt));
-            __syncwarp();
-            ok = mbar_wait_warp(bar(bPFull + qt), j & 1, abort_flag, status);
-            if (!ok) break;
-            tc_fence_after();
-            mma_pv_rest(j, qt);
-            if (more) mma_s(j + 1, qt);
-            if (leader) {
-              // after the last key tile the tile's one-shot barrier for the epilogue instead of an S barrier:
-              // tile A normalises and stores its rows while tile B is still in its last sweep
-              tc_commit(bar((more ? bSFull : bFinal) + qt));
-              tc_commit(bar(bPvDone + qt));
-              if (qt == 1) {
-                tc_commit(bar(bEmpty + (2 * j + 1) % kStages));
-                if (more) tc_commit(bar(bEmpty + (2 * j + 2) % kStages));
-              }
-            }
-            __syncwarp();
+        ok = (!more || ring_full(kt)) && mbar_wait_warp(bar(bPFull + qt), j & 1, abort_flag, status);
+        if (!ok) break;
+        tc_fence_after();
+        mma_pv_rest(vd, qt);
+        if (more) mma_s(kd, qt);
+        if (leader) {
+          // after the last key tile the tile's one-shot barrier for the epilogue instead of an S barrier:
+          // tile A normalises and stores its rows while tile B is still in its last sweep
+          tc_commit(bar((more ? bSFull : bFinal) + qt));
+          tc_commit(bar(bPvDone + qt));
+          if (!pair || qt == 1) {
+            tc_commit(v_empty);
+            if (more) tc_commit(k_empty);
           }
         }
-      } else {
-        for (int j = 0; j < T && ok; ++j) {
-          ok = mbar_wait_warp(bar(bFull + (2 * j) % kStages), ((2 * j) / kStages) & 1, abort_flag, status);
-          if (!ok) break;
-          tc_fence_after();
-          issue_s(j, 0, j & 1);
-          if (leader) tc_commit(bar(bEmpty + (2 * j) % kStages));
-          if (j > 0) ok = issue_pv(j - 1, 0, (j - 1) & 1, ((j - 1) >> 1) & 1, true);
-        }
-        if (ok) ok = issue_pv(T - 1, 0, (T - 1) & 1, ((T - 1) >> 1) & 1, true);
-        if (ok && leader) tc_commit(bar(bFinal + 0));
+        __syncwarp();
       }
     }
+    if (n_split > 1) cluster_arrive();
   } else {
     // ------------------------------------------------------------------ append (warps 2 and 3)
     // Every ring tile is waited for and released, so that the empty barrier's phases stay in step;
-    // only current-map tiles whose turn falls on this CTA are copied: rows [0, valid) of the tile go
-    // to slots hist + 128 (j - Th) + r of the slice, un-swizzled, 16 bytes per thread and step.
+    // current-map tiles whose turn falls on this item are copied: rows [0, valid) of a tile go
+    // to slots hist + 128 i + r of the slice, un-swizzled, 16 bytes per thread and step.
+    // A tile that is copied holds its ring stage for a while, so no CTA gets two in a row: the items of a slice that is
+    // walked pair by pair take turns.  In a slice that is walked tile by tile (or partly so) an item copies its own tiles.
+    const bool turns = slice * prm.per_pair.d + prm.per_pair.d <= prm.n_pair;
     const int u = (warp - 2) * 32 + lane;
     const int chunk = u & 15, rsub = u >> 4;
     const uint32_t src_off = (uint32_t)(chunk >> 3) * kHalfBytes;
     bool ok = true;
-    for (int t = 0; t < 2 * T && ok; ++t) {
-      const int st = t % kStages, j = t >> 1;
+    for (int t = 0; t < 2 * nt && ok; ++t) {
+      const int st = t % kStages, i = lo + (t >> 1);
       ok = mbar_wait_warp(bar(bFull + st), (t / kStages) & 1, abort_flag, status);
       if (!ok) break;
-      if (prm.copy_in && j >= Th && (j - Th) % (int)gridDim.x == (int)blockIdx.x) {
-        const int first = (j - Th) * 128;
-        const int nvalid = tile_valid(j);
+      if (prm.copy_in && i < Tc &&
+          (turns ? i - prm.per_pair.div(i) * prm.per_pair.d == q_tile >> 1 : i == q_tile || (pair && i == q_tile + 1))) {
+        const int first = i * 128;
+        const int nvalid = tile_valid(i);
         char *pool = (t & 1) ? lv.v_pool : lv.k_pool;
         const uint32_t tile = base + kOffRing + st * kTileBytes + src_off;
+#pragma unroll 4
         for (int r = rsub; r < nvalid; r += 4) {
           uint4 val;
           const uint32_t addr = tile + r * 128 + (((chunk & 7) ^ (r & 7)) << 4);
@@ -708,6 +887,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(bEmpty + st));
     }
+    if (n_split > 1) cluster_arrive();
   }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue
@@ -717,29 +897,30 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
     const float c = prm.scale_log2e;
     const uint64_t c2 = pack2(c, c);
-    const bool active = qt == 0 || !single;      // with one query tile the second warpgroup has nothing to do
+    const int my_first = q_first + (pair ? qt * 128 : 0);   // first query row of this warpgroup's tile
     float m = -INFINITY, l = 0.f;
-    // window row of this thread (rank in the window, or -1) and whether its warp has any
-    int wrank = -1;
+    // where this thread's row of the observation window is recorded (nullptr: it owns none), and whether its warp owns any
+    float *win_row = nullptr;
     bool wwarp = false;
-    if (kWindow && prm.win_logits != nullptr && active) {
-      const int qi = q_first + qt * 128 + row;
+    if (kWindow) {
+      int rank = -1;
       for (int e = 0; e < prm.w; ++e)
-        if (prm.win_pos[e] == qi) wrank = e;
-      wwarp = __any_sync(0xffffffffu, wrank >= 0);
+        if (prm.win_pos[e] == my_first + row) rank = e;
+      if (rank >= 0) win_row = prm.win_logits + ((size_t)slice * prm.w + rank) * prm.ld_l;
+      wwarp = __any_sync(0xffffffffu, rank >= 0);
     }
-    // (the window row's address is taken once: inside the sweep it would cost 64-bit arithmetic in every chunk)
-    float *win_row = wrank >= 0 ? prm.win_logits + ((size_t)slice * prm.w + wrank) * prm.ld_l : nullptr;
     const uint32_t o_addr = lane_addr + kColO + qt * 128;
     bool ok = true;
-    for (int j = 0; j < T && ok && active; ++j) {
-      const int buf = single ? (j & 1) : qt;
-      const uint32_t par = single ? ((j >> 1) & 1) : (j & 1);
-      ok = mbar_wait_warp(bar(bSFull + buf), par, abort_flag, status);
+    const int steps = n_steps(qt);
+    const uint32_t s_addr = lane_addr + kColS + qt * 128;
+    for (int j = 0; j < steps && ok; ++j) {
+      const int i_tile = lo + (shared ? 2 * j + qt : j);
+      const int valid = tile_valid(i_tile);      // real keys: < 128 only in a ragged tile
+      // the tile's first column of the window row (taken here: the one thread that stores it is what its tile waits for)
+      float *win_dst = kWindow ? win_row + (i_tile < Tc ? i_tile + Th : i_tile - Tc) * 128 : nullptr;
+      ok = mbar_wait_warp(bar(bSFull + qt), j & 1, abort_flag, status);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t s_addr = lane_addr + kColS + buf * 128;
-      const int valid = tile_valid(j);           // < 128 only in a ragged tile
       int o_landed = 0;                          // the previous PV product of this tile has been waited for
       // The sweep is software-pipelined over the chunks: while chunk cc is summed, packed, checked and stored
       // ("back"), the exponentials of chunk cc + 1 ("front": x = s c - m and 2^x, in place in the chunk's registers)
@@ -749,13 +930,13 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       float v[2][32];
       auto log_window = [&](const float *x, int cc) {
         // The row's raw products go out as they are (the score kernel applies the softmax scale), 32
-        // columns as eight 16-byte stores, at column 128 j + ...: key tile j owns columns [128 j, 128 j + 128)
-        // of a logit row, so the current map starts at the next multiple of 128 behind the history and
+        // columns as eight 16-byte stores: every key tile owns 128 columns of a logit row, the history's tiles before
+        // the current map's, so the current map starts at the next multiple of 128 behind the history and
         // every store is aligned.  Columns of a ragged tile beyond its keys hold finite values nobody reads.
-        if (wrank >= 0) {
-          float4 *dst = reinterpret_cast<float4 *>(win_row + (j * 128 + cc * 32));
+        if (win_row != nullptr) {
+          float4 *dst = reinterpret_cast<float4 *>(win_dst + cc * 32);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) dst[i] = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+          for (int v4 = 0; v4 < 8; ++v4) dst[v4] = make_float4(x[4 * v4], x[4 * v4 + 1], x[4 * v4 + 2], x[4 * v4 + 3]);
         }
         __syncwarp();   // the tcgen05 instructions that follow want the warp converged
       };
@@ -817,7 +998,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         if (__any_sync(0xffffffffu, !(lt <= 8192.f))) {
           // Once the early chunks' P is with the tensor core, their product has to land before O is scaled, and only
           // the later chunks' P is still this thread's to scale.
-          const bool late = !single && cc >= kEarlyChunks;
+          const bool late = cc >= kEarlyChunks;
           const Raised r = raise_reference(vc, c, m, l, s_addr, cc, late ? kEarlyChunks : 0, o_addr, (late || j > 0) ? 1 : 0,
                                            late ? (o_landed == 2) : (o_landed >= 1), bar((late ? bPvEarly : bPvDone) + qt),
                                            (late ? j : j - 1) & 1, abort_flag, status);
@@ -835,12 +1016,12 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           tc_st16(s_addr + cc * 16, pk);
           l += lt;
         }
-        if (!single && cc == kEarlyChunks - 1) {
+        if (cc == kEarlyChunks - 1) {
           // P of the first chunks is complete: that part of the PV product may start under the rest of the sweep
           tc_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(bPEarly + buf));
+          if (lane == 0) mbar_arrive(bar(bPEarly + qt));
         }
         if (cc + 2 < kChunks) tc_wait_ld();
       }
@@ -860,63 +1041,28 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       tc_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(bPFull + buf));
+      if (lane == 0) mbar_arrive(bar(bPFull + qt));
     }
-    if (ok && active) {
+    if (ok && steps > 0) {
       // a barrier that completes exactly once, after the last PV product: the per-tile PV barrier will
       // not do, a parity wait cannot tell phases two apart and this warp may be that far behind it
       ok = mbar_wait_warp(bar(bFinal + qt), 0, abort_flag, status);
     }
-    if (ok && active) {
-      tc_fence_after();
-      const float inv = 1.f / l;
-      const int qi = q_first + qt * 128 + row;
-      // The normalised rows go to the query tile's shared memory (no product reads it any more) in the layout
-      // of a TMA box - two halves of 64 columns, rows of 128 bytes, 128-byte swizzle - and one thread sends the
-      // tile out with two bulk tensor stores: a row written by its own thread straight to global memory costs a
-      // 128-byte line per lane and store instruction.  The tensor map clips the rows beyond n_k.
-      const uint32_t stage = base + kOffQ + qt * kTileBytes + row * 128;
-      float o[2][32];
-      tc_ld32(o_addr, o[0]);
-#pragma unroll
-      for (int cc = 0; cc < kChunks; ++cc) {
-        tc_wait_ld();
-        if (cc + 1 < kChunks) tc_ld32(o_addr + (cc + 1) * 32, o[(cc + 1) & 1]);
-        const float *oc = o[cc & 1];
-#pragma unroll
-        for (int v4 = 0; v4 < 4; ++v4) {
-          const uint32_t wx = pack_bf16(oc[8 * v4 + 0] * inv, oc[8 * v4 + 1] * inv);
-          const uint32_t wy = pack_bf16(oc[8 * v4 + 2] * inv, oc[8 * v4 + 3] * inv);
-          const uint32_t wz = pack_bf16(oc[8 * v4 + 4] * inv, oc[8 * v4 + 5] * inv);
-          const uint32_t ww = pack_bf16(oc[8 * v4 + 6] * inv, oc[8 * v4 + 7] * inv);
-          const uint32_t addr = stage + (uint32_t)(cc >> 1) * kHalfBytes + ((uint32_t)(((cc & 1) * 4 + v4) ^ (row & 7)) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(wx), "r"(wy), "r"(wz), "r"(ww) : "memory");
-        }
-      }
-      fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(bOut + qt));
-      if (quarter == 0) {
-        // one warp waits until all rows of the tile are staged; one of its lanes issues the stores
-        ok = mbar_wait_warp(bar(bOut + qt), 0, abort_flag, status);
-        if (ok && elect_one()) {
-          const uint32_t src = base + kOffQ + qt * kTileBytes;
-          tma_store_4d(&tmO, src, 0, q_first + qt * 128, h, b);
-          tma_store_4d(&tmO, src + kHalfBytes, 64, q_first + qt * 128, h, b);
-          tma_store_commit();
-        }
-        __syncwarp();
-      }
-      if (prm.lse != nullptr && qi < n_k) prm.lse[(size_t)slice * n_k + qi] = (m + log2f(l)) * 0.6931471805599453f;
-      if (kWindow && wrank >= 0) prm.win_lse[(size_t)slice * prm.w + wrank] = m + log2f(l);
-    }
-    if (quarter == 0) tma_store_wait_read();   // (a lane that issued nothing has nothing to wait for)
+    if (n_split > 1) cluster_arrive();                     // this CTA's ring is free (as far as this warp knows)
+    tc_fence_after();
+    finish_rows(prm, base, o_addr, item_slot[0], item_slot[1], qt, pair, shared, ok && steps > 0, n_split, m, l, kWindow && win_row != nullptr);
     tc_fence_before();
   }
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kTmemCols) : "memory");
+  }
+  if (n_split > 1) {
+    if (warp < 4) cluster_wait();
+    cluster_arrive();
+    cluster_wait();
+    if (!leave) finish_cluster(prm, base, item_slot[0], item_slot[1], n_split);
   }
 }
 
@@ -931,6 +1077,42 @@ struct AttendTc {
   CUtensorMap tmK, tmV;
   bool on = false;
   int box_rows = 128;
+  int n_sm = 148;
+  int max_clusters[tc::kMaxSplit + 1] = {0};   // clusters of c CTAs that fit the device at once
+
+  static const void *kernel(bool window) {
+    return window ? (const void *)tc::attend_tc_kernel<true> : (const void *)tc::attend_tc_kernel<false>;
+  }
+
+  // How a launch is cut.  Measured on a B200 (148 SMs), us per launch, averaged over a layer with a long and three with a short
+  // cache, against one CTA for every pair or odd tile, the odd ones by a single warpgroup:
+  //   16 slices, singles (split over clusters up to 400 queries): 256 / 400 / 576 / 1024 queries 22.0 -> 18.7, 26.8 -> 21.5,
+  //   30.3 -> 22.5, 37.3 -> 29.6;  below three key tiles neither sharing nor splitting pays (13-15 us either way);
+  //   128 slices x 1024 queries (512 pairs, 3.5 waves), the last 68 pairs as 136 singles: 135 -> 122.
+  // n_pair: items that are walked pair by pair; items: all of them; split: CTAs that share an item's keys.
+  struct Cut { int n_pair, items, split; };
+  Cut cut(int tiles, int slices, int key_tiles) const {
+    constexpr float kJoin = 0.9f;      // what combining over a cluster costs, in steps (of two key tiles) of a single
+    const int pairs = tiles / 2 * slices, odd = tiles % 2 * slices;
+    auto steps = [&](int split) { const int per = (key_tiles + split - 1) / split; return (float)((per + 1) / 2); };
+    if (2 * pairs + odd <= n_sm) {
+      // every query tile finds an SM of its own: singles, their keys shared by as many CTAs as pay and fit
+      const int items = 2 * pairs + odd;
+      int split = 1;
+      float best = steps(1);
+      for (int c = 2; c <= tc::kMaxSplit && c <= key_tiles; ++c)
+        if (items <= max_clusters[c] && steps(c) + kJoin < best) { best = steps(c) + kJoin; split = c; }
+      return {0, items, split};
+    }
+    // Pairs.  They run in waves, more or less; where a last wave would leave more than half of the SMs idle its items are
+    // worked on tile by tile, which needs twice as many SMs for 0.55 of the time.
+    const int items = pairs + odd, last = items % n_sm;
+    if (2 * last <= n_sm) {
+      const int per = (tiles + 1) / 2, first = items - last;          // the tiles from item `first` on
+      return {first, first + tiles * slices - (first / per * tiles + 2 * (first % per)), 1};
+    }
+    return {items, items, 1};
+  }
 
   bool init(int dtype, int head_dim, void *k_pool, void *v_pool, long long n_pages, int page_tokens, std::string &err) {
     on = false;
@@ -953,12 +1135,40 @@ struct AttendTc {
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) { err = "cuTensorMapEncodeTiled(pool) failed with code " + std::to_string((int)r); return false; }
     }
-    if (cudaFuncSetAttribute(tc::attend_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(tc::attend_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes) != cudaSuccess) {
-      err = "cannot raise the dynamic shared memory limit";
-      return false;
+    for (bool window : {false, true})
+      if (cudaFuncSetAttribute(kernel(window), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes) != cudaSuccess) {
+        err = "cannot raise the dynamic shared memory limit";
+        return false;
+      }
+    return on = read_device(err);
+  }
+
+  // What a launch has to know about the device.  The number of clusters of every size that run at once (a cluster has to fit
+  // one GPC) takes the runtime about a millisecond to tell, so it is asked once per device.
+  bool read_device(std::string &err) {
+    struct Device { int n_sm = 0, clusters[tc::kMaxSplit + 1] = {0}; };
+    static std::mutex lock;
+    static std::map<int, Device> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { err = "no current device"; return false; }
+    std::lock_guard<std::mutex> hold(lock);
+    Device &d = known[dev];
+    if (d.n_sm == 0) {
+      int n = 0;
+      if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { err = "cannot read the number of SMs"; return false; }
+      for (int c = 2; c <= tc::kMaxSplit; ++c) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        cfg.gridDim = dim3(1, 1, c); cfg.blockDim = dim3(tc::kThreads); cfg.dynamicSmemBytes = tc::kSmemBytes;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = c;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&d.clusters[c], kernel(true), &cfg) != cudaSuccess) { cudaGetLastError(); d.clusters[c] = 0; }
+      }
+      d.n_sm = n;
     }
-    on = true;
+    n_sm = d.n_sm;
+    std::copy(d.clusters, d.clusters + tc::kMaxSplit + 1, max_clusters);
     return true;
   }
   bool enabled() const { return on; }
@@ -978,14 +1188,14 @@ struct AttendTc {
 
   // Kc / Vc: the current map's K and V when they have not been copied into the store yet (the kernel
   // reads them there and copies them in), else nullptr.
+  // hist: entries before the current map (an upper bound over the slices); only sizes the launch.
   // win_logits / win_pos / w: where to record the window rows' logits (nullptr: do not).
   bool launch(const LayerView &lv, const TensorView &Q, const TensorView &O, float *lse, int n_k, const TensorView *Kc,
-              const TensorView *Vc, bool copy_in, int n_prev, float scale, float *win_logits, float *win_lse, int ld_l, const int *win_pos, int w,
+              const TensorView *Vc, bool copy_in, int hist, int n_prev, float scale, float *win_logits, float *win_lse, int ld_l, const int *win_pos, int w,
               cudaStream_t stream, std::string &err) {
-    CUtensorMap tmQ, tmKc, tmVc, tmO;
+    CUtensorMap tmQ, tmKc, tmVc;
     const int B = lv.n_slices / lv.n_heads;
     if (!map_rows(&tmQ, Q, n_k, lv.n_heads, B, "Q", err)) return false;
-    if (!map_rows(&tmO, O, n_k, lv.n_heads, B, "O", err)) return false;
     const bool fused = Kc != nullptr && Vc != nullptr;
     if (fused) {
       if (!map_rows(&tmKc, *Kc, n_k, lv.n_heads, B, "K", err) || !map_rows(&tmVc, *Vc, n_k, lv.n_heads, B, "V", err)) return false;
@@ -1005,20 +1215,27 @@ struct AttendTc {
     prm.ld_l = ld_l;
     prm.w = win_logits ? w : 0;
     for (int e = 0; e < kMaxWindow; ++e) prm.win_pos[e] = (win_logits && e < w) ? win_pos[e] : -1;
-    dim3 grid((n_k + 255) / 256, lv.n_slices);
+    const int tiles = (n_k + 127) / 128;
+    const Cut how = cut(tiles, lv.n_slices, fused ? (hist + 127) / 128 + tiles : (hist + n_k + 127) / 128);
+    const int per = (tiles + 1) / 2;
+    prm.n_pair = how.n_pair;
+    prm.cut_tile = how.n_pair / per * tiles + 2 * (how.n_pair % per);
+    prm.per_pair = tc::Divisor::of(per); prm.per_tile = tc::Divisor::of(tiles); prm.per_heads = tc::Divisor::of(lv.n_heads);
     // programmatic stream serialisation: the kernel's set-up may overlap the end of the kernel before it in the stream
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
+    cfg.gridDim = dim3(how.items, 1, how.split);
     cfg.blockDim = dim3(tc::kThreads);
     cfg.dynamicSmemBytes = tc::kSmemBytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = (unsigned)how.split;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t launched = win_logits ? cudaLaunchKernelEx(&cfg, tc::attend_tc_kernel<true>, tmQ, tmK, tmV, tmKc, tmVc, tmO, prm)
-                                            : cudaLaunchKernelEx(&cfg, tc::attend_tc_kernel<false>, tmQ, tmK, tmV, tmKc, tmVc, tmO, prm);
+    cfg.numAttrs = how.split > 1 ? 2 : 1;
+    void *args[] = {&tmQ, &tmK, &tmV, &tmKc, &tmVc, &prm};
+    const cudaError_t launched = cudaLaunchKernelExC(&cfg, kernel(win_logits != nullptr), args);
     if (launched != cudaSuccess) {
       err = "attend: kernel launch failed";
       return false;

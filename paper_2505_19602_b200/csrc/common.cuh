@@ -21,6 +21,7 @@ struct LayerView {
   int *pos_pool;           // [n_pages][page_tokens] original positions
   const int *page_table;   // [n_slices][pages_per_slice]
   int *hist_len;           // [n_slices] entries held before the current map
+  int *next_len;           // [n_slices] entries held after it: what the next scale finds in hist_len
   int *status;             // sticky device status word
   int pages_per_slice;
   int page_shift, page_mask;

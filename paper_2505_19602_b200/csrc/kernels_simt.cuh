@@ -59,10 +59,10 @@ __global__ void __launch_bounds__(256) append_kernel(LayerView lv, TensorView K,
   }
 }
 
-// hist_len += n_k for a current map that no compress has consumed.
+// The length after a current map that was neither attended nor compressed (attend writes it itself).
 __global__ void commit_kernel(LayerView lv, int n_k) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < lv.n_slices) lv.hist_len[s] += n_k;
+  if (s < lv.n_slices) lv.next_len[s] = lv.hist_len[s] + n_k;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(256) attend_simt_kernel(LayerView lv, TensorVi
     for (int e = 0; e < VN; ++e) Qs[r * LD + c * VN + e] = v[e];
   }
   if (tid < BM) { m_s[tid] = -INFINITY; l_s[tid] = 0.f; }
+  if (blockIdx.x == 0 && tid == 0) lv.next_len[slice] = L;     // unless a compress of this scale evicts
 
   float acc[4][NJ];
 #pragma unroll
@@ -728,8 +729,7 @@ __global__ void __launch_bounds__(256) compact_kernel(LayerView lv, const int *k
       }
     }
   }
-  // no CTA of this kernel reads the length (the keep list's length is kept_count)
-  if (do_pos_cta && threadIdx.x == 0) lv.hist_len[slice] = kept;
+  if (do_pos_cta && threadIdx.x == 0) lv.next_len[slice] = kept;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(1024) compress_fused_kernel(LayerView lv, Wind
     for (int c0 = lo; c0 < kept; c0 += C) __syncthreads();     // keeps the barrier count of the working threads
   }
   if (tid == 0) {
-    lv.hist_len[slice] = kept;
+    lv.next_len[slice] = kept;
     kept_count[slice] = kept;
   }
 }

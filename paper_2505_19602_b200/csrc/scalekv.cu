@@ -162,7 +162,8 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
   p.off_v = o; o = align_up(o + (size_t)p.n_pages * p.P * row_bytes, 1024);
   p.off_pos = o; o = align_up(o + (size_t)p.n_pages * p.P * 4, 1024);
   p.off_pt = o; o = align_up(o + pt * 4, 1024);
-  p.off_len = o; o = align_up(o + (size_t)p.n_layers * p.n_slices * 4, 1024);
+  // lengths before the even and before the odd scales: a scale's kernels read the one and write the other
+  p.off_len = o; o = align_up(o + 2 * (size_t)p.n_layers * p.n_slices * 4, 1024);
   p.off_status = o; o = align_up(o + 256, 1024);
   p.pool_bytes = o;
   o = 0;
@@ -203,6 +204,7 @@ struct scalekv_ctx {
   std::vector<int> hist;           // entries before the current map (uniform over slices)
   std::vector<int> pending;        // n_k of an appended, not yet committed current map (0 = none)
   std::vector<int> attended;       // attend ran for the pending map
+  std::vector<char> attend_marked; // ... and ev_attend was recorded behind it
   std::vector<char> in_store;      // the pending map's rows have been copied into the pages
   std::vector<char> logits_padded; // attend recorded the logits while the current map was still outside the store
   std::vector<int> logits_of;      // scale whose window logits attend recorded for this layer (-1: none)
@@ -245,6 +247,15 @@ scalekv_status fail(scalekv_ctx *c, scalekv_status st, const char *fmt, ...) {
     if (e_ != cudaSuccess) return fail(ctx, SCALEKV_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
   } while (0)
 
+// The device's per-slice lengths of layer l as they stand before scale k.  They are kept twice, for even and odd scales:
+// the kernels of scale k read the one copy and write the other - attend hist + n_k, an evicting compress the number of
+// survivors - so a scale that evicts nothing needs no kernel of its own to commit its map, and no kernel reads a word
+// that another CTA of its grid writes.
+int *lengths_before(scalekv_ctx *c, int l, int k) {
+  const Plan &p = c->plan;
+  return reinterpret_cast<int *>(c->pool + p.off_len) + ((size_t)(k & 1) * p.n_layers + l) * p.n_slices;
+}
+
 LayerView layer_view(scalekv_ctx *c, int l) {
   const Plan &p = c->plan;
   LayerView lv;
@@ -252,7 +263,9 @@ LayerView layer_view(scalekv_ctx *c, int l) {
   lv.v_pool = c->pool + p.off_v;
   lv.pos_pool = reinterpret_cast<int *>(c->pool + p.off_pos);
   lv.page_table = reinterpret_cast<const int *>(c->pool + p.off_pt) + p.layers[l].page_table_off;
-  lv.hist_len = reinterpret_cast<int *>(c->pool + p.off_len) + (size_t)l * p.n_slices;
+  const int scale = c->pending[l] ? c->next_scale[l] - 1 : c->next_scale[l];      // the scale being worked on
+  lv.hist_len = lengths_before(c, l, scale);
+  lv.next_len = lengths_before(c, l, scale + 1);
   lv.status = reinterpret_cast<int *>(c->pool + p.off_status);
   lv.pages_per_slice = p.layers[l].total_pages;
   lv.page_shift = p.page_shift;
@@ -350,7 +363,7 @@ scalekv_status commit_pending(scalekv_ctx *ctx, int l, cudaStream_t s) {
   if (L > p.layers[l].persist_pages * p.P && p.layers[l].persist_pages < p.layers[l].total_pages)
     return fail(ctx, SCALEKV_ERR_CAPACITY, "layer %d: %d entries kept without compress exceed the persistent capacity %d",
                 l, L, p.layers[l].persist_pages * p.P);
-  {
+  if (!ctx->attended[l]) {      // (an attend has left the new length already)
     Scope sc(ctx, s, kOther);
     commit_kernel<<<(p.n_slices + 255) / 256, 256, 0, s>>>(layer_view(ctx, l), ctx->pending[l]);
   }
@@ -442,12 +455,13 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
     return bail(SCALEKV_ERR_CUDA);
   // pages start out as zeros: tiles are loaded whole, and rows beyond a slice's length must be finite
   if (cudaMemset(ctx->pool + p.off_k, 0, p.off_pos - p.off_k) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
-  if (cudaMemset(ctx->pool + p.off_len, 0, (size_t)p.n_layers * p.n_slices * 4) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
+  if (cudaMemset(ctx->pool + p.off_len, 0, 2 * (size_t)p.n_layers * p.n_slices * 4) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
   if (cudaMemset(ctx->pool + p.off_status, 0, 256) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
   ctx->next_scale.assign(p.n_layers, 0);
   ctx->hist.assign(p.n_layers, 0);
   ctx->pending.assign(p.n_layers, 0);
   ctx->attended.assign(p.n_layers, 0);
+  ctx->attend_marked.assign(p.n_layers, 0);
   ctx->in_store.assign(p.n_layers, 1);
   ctx->logits_of.assign(p.n_layers, -1);
   ctx->logits_padded.assign(p.n_layers, 0);
@@ -508,7 +522,7 @@ scalekv_status scalekv_reset(scalekv_ctx *ctx) {
     CU(cudaEventRecord(ctx->ev_compress[0], ctx->s_side));
     CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_compress[0], 0));
   }
-  CU(cudaMemsetAsync(ctx->pool + p.off_len, 0, (size_t)p.n_layers * p.n_slices * 4, ctx->s_main));
+  CU(cudaMemsetAsync(ctx->pool + p.off_len, 0, 2 * (size_t)p.n_layers * p.n_slices * 4, ctx->s_main));
   if (ctx->s_side != ctx->s_main) {
     // later side-stream work must not overtake the reset
     CU(cudaEventRecord(ctx->ev_attend[0], ctx->s_main));
@@ -640,7 +654,7 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
                       ? nullptr
                       : reinterpret_cast<float *>(ctx->ws + p.off_logits) + (size_t)(layer % kSets) * p.logits_elems;
       float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
-      if (!ctx->tc.launch(lv, tview(Q), tview(O), lse, nk, fused ? &kc : nullptr, fused ? &vc : nullptr, fused && copy, p.N[k],
+      if (!ctx->tc.launch(lv, tview(Q), tview(O), lse, nk, fused ? &kc : nullptr, fused ? &vc : nullptr, fused && copy, ctx->hist[layer], p.N[k],
                           ctx->scale, wl, wlse, p.ld_l, win.data(), (int)win.size(), ctx->s_main, e))
         return fail(ctx, SCALEKV_ERR_CUDA, "attend launch: %s", e.c_str());
       if (copy) ctx->in_store[layer] = 1;
@@ -657,7 +671,11 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
     }
   }
   ctx->attended[layer] = 1;
-  if (ctx->s_side != ctx->s_main) CU(cudaEventRecord(ctx->ev_attend[layer], ctx->s_main));
+  // a compress that may evict will wait for this point of stream_main
+  const int table = p.budgets[(size_t)layer * p.K + ctx->next_scale[layer] - 1];
+  const bool mark = ctx->s_side != ctx->s_main && table != SCALEKV_KEEP_ALL && ctx->hist[layer] + nk > table;
+  if (mark) CU(cudaEventRecord(ctx->ev_attend[layer], ctx->s_main));
+  ctx->attend_marked[layer] = mark;
   return check_launch(ctx, "attend");
 }
 
@@ -749,8 +767,9 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     st = materialize(ctx, layer);
     if (st != SCALEKV_OK) return st;
   }
+  if (!evict && ctx->attended[layer]) return commit_pending(ctx, layer, ctx->s_main);      // nothing to launch
   if (s != ctx->s_main) {
-    if (!ctx->attended[layer] || copy_now) CU(cudaEventRecord(ctx->ev_attend[layer], ctx->s_main));
+    if (!ctx->attended[layer] || copy_now || !ctx->attend_marked[layer]) CU(cudaEventRecord(ctx->ev_attend[layer], ctx->s_main));
     CU(cudaStreamWaitEvent(s, ctx->ev_attend[layer], 0));
   }
   if (!evict) {
@@ -773,7 +792,10 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
       const int ow = ctx->set_owner[layer % kSets];
       if (ow >= 0 && ow != layer) {
         ctx->logits_of[ow] = -1;
-        if (s != ctx->s_main && ctx->attended[ow]) CU(cudaStreamWaitEvent(s, ctx->ev_attend[ow], 0));
+        if (s != ctx->s_main && ctx->attended[ow]) {
+          if (!ctx->attend_marked[ow]) CU(cudaEventRecord(ctx->ev_attend[ow], ctx->s_main));
+          CU(cudaStreamWaitEvent(s, ctx->ev_attend[ow], 0));
+        }
       }
     }
     if (!recorded) {
@@ -1011,8 +1033,7 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   std::vector<double> host(2 + 2 * (size_t)p.n_slices);
   std::vector<int> len(p.n_slices);
   CU(cudaMemcpyAsync(host.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, ctx->s_main));
-  CU(cudaMemcpyAsync(len.data(), ctx->pool + p.off_len + (size_t)layer * p.n_slices * 4, (size_t)p.n_slices * 4,
-                     cudaMemcpyDeviceToHost, ctx->s_main));
+  CU(cudaMemcpyAsync(len.data(), layer_view(ctx, layer).hist_len, (size_t)p.n_slices * 4, cudaMemcpyDeviceToHost, ctx->s_main));
   CU(cudaStreamSynchronize(ctx->s_main));
   const double cnt = (double)rows * p.n_slices;
   *car = host[0] / cnt;
@@ -1146,6 +1167,12 @@ scalekv_status scalekv_selftest_wait(scalekv_ctx *ctx, int32_t limit_ms, int32_t
 scalekv_status scalekv_join(scalekv_ctx *ctx) {
   if (!ctx) return SCALEKV_ERR_INVALID_ARG;
   if (ctx->s_side != ctx->s_main && ctx->side_dirty) {   // (nothing enqueued there since the last join: nothing to wait for)
+    // A capture of steps that evicted nothing has not taken the side stream in: what is pending there (it was sent behind
+    // a reset, say) is not the capture's, and must not be joined by it.
+    cudaStreamCaptureStatus cap_main = cudaStreamCaptureStatusNone, cap_side = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing(ctx->s_main, &cap_main));
+    CU(cudaStreamIsCapturing(ctx->s_side, &cap_side));
+    if (cap_main != cudaStreamCaptureStatusNone && cap_side == cudaStreamCaptureStatusNone) return SCALEKV_OK;
     CU(cudaEventRecord(ctx->ev_join, ctx->s_side));
     CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_join, 0));
     // stream_main is now behind every compress enqueued so far: later appends need not wait for them again
@@ -1175,7 +1202,7 @@ scalekv_status scalekv_lengths(scalekv_ctx *ctx, int32_t layer, int32_t *len_hos
   if (layer < 0 || layer >= p.n_layers) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "layer %d out of range", layer);
   scalekv_status st = scalekv_sync(ctx);
   if (st != SCALEKV_OK) return st;
-  CU(cudaMemcpy(len_host, ctx->pool + p.off_len + (size_t)layer * p.n_slices * 4, (size_t)p.n_slices * 4, cudaMemcpyDeviceToHost));
+  CU(cudaMemcpy(len_host, layer_view(ctx, layer).hist_len, (size_t)p.n_slices * 4, cudaMemcpyDeviceToHost));
   for (int s = 0; s < p.n_slices; ++s) len_host[s] += ctx->pending[layer];
   return SCALEKV_OK;
 }
@@ -1192,7 +1219,7 @@ scalekv_status scalekv_export_slice(scalekv_ctx *ctx, int32_t layer, int32_t b, 
   if (st != SCALEKV_OK) return st;
   const int slice = b * p.H + h;
   int hist = 0;
-  CU(cudaMemcpy(&hist, ctx->pool + p.off_len + ((size_t)layer * p.n_slices + slice) * 4, 4, cudaMemcpyDeviceToHost));
+  CU(cudaMemcpy(&hist, layer_view(ctx, layer).hist_len + slice, 4, cudaMemcpyDeviceToHost));
   const int L = hist + (ctx->map_lost[layer] ? 0 : ctx->pending[layer]);   // a given-up last map is not exported
   *len = L;
   if (L > cap) return fail(ctx, SCALEKV_ERR_CAPACITY, "slice holds %d entries, cap is %d", L, cap);

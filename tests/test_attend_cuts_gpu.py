@@ -1,0 +1,35 @@
+"""How the tensor-core attention cuts a launch: pairs of query tiles, single tiles whose keys the two warpgroups share, single
+tiles whose keys a cluster of CTAs shares, and launches whose last items are worked on tile by tile."""
+import pytest
+import torch
+
+from oracle import scalekv_oracle as orc
+from paper_2505_19602_b200 import binding
+from parity_util import ParityRun
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch,heads,sides,budget", [
+    (1, 1, (1, 11, 12, 16, 37), 40),       # one slice: clusters of up to 8 CTAs, rows that do not divide among them
+    (1, 3, (2, 16, 17, 29), -1),           # full cache: 128 + 1 rows, odd numbers of key tiles
+    (1, 16, (3, 9, 33), 70),               # 144 single tiles: every SM has one, nothing is left to split
+    (7, 10, (2, 12, 25), 150),             # 70 slices x 5 tiles: 210 items, the last 62 tile by tile from inside a slice
+    (5, 15, (1, 18), 25),                  # 75 slices x 3 tiles: 150 items, one whole slice tile by tile
+    (6, 16, (2, 20), 30),                  # 96 slices x 4 tiles: 192 pairs, the last 44 tile by tile
+    (4, 16, (1, 8, 20), 30),               # 64 slices x 4 tiles: 128 pairs, no more than one wave
+])
+def test_every_way_of_cutting_a_launch(batch, heads, sides, budget):
+    n = orc.scale_token_counts(sides)
+    B, H, d = batch, heads, 128
+    gen = torch.Generator().manual_seed(91)
+    data = [tuple(torch.randn(B, H, nk, d, generator=gen).to(torch.bfloat16) for _ in range(3)) for nk in n]
+    slices = [(0, b, h) for b in range(B) for h in range(H)]
+    followed = slices if len(slices) <= 3 else slices[:2] + slices[len(slices) * 2 // 3:][:2] + slices[-3:]
+    for run in ("run", "run_pipelined"):   # with the map's rows copied by the attention kernel, and left to the compress
+        budgets = [[budget] * len(sides)]
+        kv = binding.ScaleKV(1, B, H, d, "bf16", sides, sides, budgets)
+        p = ParityRun(kv, "bf16", sides, budgets, lambda l, k: data[k], lambda k: orc.window_centroids(sides[k], sides[k], 16),
+                      followed, compress_last=True)
+        getattr(p, run)()
+        kv.close()
