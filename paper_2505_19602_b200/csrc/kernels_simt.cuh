@@ -485,11 +485,8 @@ __global__ void __launch_bounds__(1024) row_lse_kernel(LayerView lv, WindowArg w
 // ------------------------------------------------------------------------------------------
 // select: per-slice top-k' of the non-window entries by key (Sec. 3.3), one CTA of 1024 threads per
 // slice with the slice's keys in shared memory (with pool > 1 a candidate's key is first replaced by
-// its importance averaged over the neighbouring entries):
-//   radix select of the k'-th largest key, 8 bits per pass, warp-aggregated histogram updates; then
-//   the ordered emit of the ascending slot list of survivors (selected U window); ties at the
-//   threshold go to the lowest slots = lowest original positions.  Every thread owns a run of
-//   consecutive entries, so two block scans order the whole list.  Deterministic.
+// its importance averaged over the neighbouring entries); see select_and_emit.  Ties at the threshold go to the lowest
+// slots = lowest original positions.  Deterministic.
 // Dynamic shared memory: 4 * ld_s bytes of keys.
 // ------------------------------------------------------------------------------------------
 constexpr int kMaxHeadBudgets = 128;
@@ -503,121 +500,133 @@ __global__ void head_budget_kernel(HeadBudgets hb, int n_heads, int n_slices, in
   if (s < n_slices) slice_budget[s] = hb.v[s % n_heads];
 }
 // Shared state of one selection (static shared memory of the calling kernel).
+constexpr int kSelectBins = 2048;
 struct SelectShared {
-  int hist[256];
+  int hist[kSelectBins];
   int warp_sums[33];
-  uint32_t prefix;
-  int remaining;
+  int keeps[32], ties[32];
+  int bin, need, in_bin, n_cand, n_ties;
+  uint32_t tie_key;
 };
 
-// The selection proper, run by a whole CTA of 1024 threads: key[0 .. L) (shared or global memory) -> out[] = the
+// The selection proper, run by a whole CTA of NT threads: key[0 .. L) (shared or global memory) -> out[] = the
 // ascending slots of the survivors (the `budget` largest keys, equal keys by lowest slot, plus every sentinel
-// entry).  Returns the number of survivors; *kprime_plus_win receives the count the rule demands.
-__device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int budget, int *out, SelectShared &sh,
+// entry).  Returns the number of survivors; *kprime_plus_win receives the count the rule demands.  Keys other than the
+// sentinel are below 2^(shift + 11); out has room for L entries and serves as scratch before it is written.
+//   A histogram over the keys' upper 11 bits says in which bin the budget runs out; when the bin holds no more keys than there
+//   are threads they are gathered and every one is ranked against all, else the next 11 bits decide in the same way.
+//   The emit gives every warp a run of consecutive entries and orders them by ballots, twice: to count, and behind one
+//   exclusive sum over the warps to write.
+// What bounds it is the latency of its rounds of block barriers.  Four 8-bit radix passes with warp-aggregated updates and
+// three block scans took 11 000 cycles for 265 entries and 23 000 for 4 248 (1 024 threads).
+template <int NT>
+__device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int budget, int shift, int *out, SelectShared &sh,
                                                 int *kprime_plus_win) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  int n_win_local = 0;
-  for (int i = tid; i < L; i += 1024) n_win_local += (key[i] == kWindowKey) ? 1 : 0;
-  int n_win;
-  block_exclusive_scan(n_win_local, sh.warp_sums, &n_win);
-  const int cand = L - n_win;
-  const int kprime = (budget < 0 || budget > cand) ? cand : budget;
-  *kprime_plus_win = kprime + n_win;
-
-  // radix select of the kprime-th largest key
-  uint32_t threshold = 0;
-  int n_ties_taken = 0;       // how many entries equal to the threshold are kept
-  if (kprime > 0 && kprime < cand) {
-    if (tid == 0) { sh.prefix = 0; sh.remaining = kprime; }
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      const uint32_t mask_hi = pass == 0 ? 0u : (0xFFFFFFFFu << (shift + 8));
-      if (tid < 256) sh.hist[tid] = 0;
-      __syncthreads();
-      const uint32_t prefix = sh.prefix;
-      for (int i0 = 0; i0 < L; i0 += 1024) {
-        const int i = i0 + tid;
-        const uint32_t k = i < L ? key[i] : kWindowKey;
-        const bool in = (k != kWindowKey) && ((k & mask_hi) == prefix);
-        const uint32_t digit = in ? ((k >> shift) & 0xFFu) : 256u;
-        // one shared-memory atomic per distinct digit in the warp
-        const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-        if (in && lane == (__ffs(peers) - 1)) atomicAdd(&sh.hist[digit], __popc(peers));
-      }
-      __syncthreads();
-      if (tid < 32) {
-        // digits 255 .. 0 in descending order, 8 per lane; find where the running count reaches `rem`
-        int c[8], tot = 0;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) { c[e] = sh.hist[255 - (lane * 8 + e)]; tot += c[e]; }
-        int incl = tot;
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += t;
-        }
-        const int rem = sh.remaining;
-        const int before = incl - tot;
-        __syncwarp();
-        if (before < rem && incl >= rem) {
-          int dsel = 0, r = rem - before;
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (r > 0) {
-              if (c[e] >= r) { dsel = 255 - (lane * 8 + e); sh.remaining = r; r = 0; }
-              else r -= c[e];
-            }
-          }
-          sh.prefix = prefix | ((uint32_t)dsel << shift);
-        }
-      }
-      __syncthreads();
-    }
-    threshold = sh.prefix;
-    n_ties_taken = sh.remaining;
-  }
-  const bool keep_all = (kprime >= cand);
-  const bool keep_none = (kprime == 0);
-
-  // ordered emit: thread t owns entries [t * E, (t + 1) * E)
-  const int E = (L + 1023) >> 10;
-  const int i_lo = tid * E, i_hi = (i_lo + E < L) ? i_lo + E : L;
-  int n_tie = 0;
-  for (int i = i_lo; i < i_hi; ++i) {
-    const uint32_t k = key[i];
-    n_tie += (k != kWindowKey && !keep_all && !keep_none && k == threshold) ? 1 : 0;
-  }
-  int tie_total, keep_total;
-  int tie_rank = block_exclusive_scan(n_tie, sh.warp_sums, &tie_total);
-  int n_keep = 0;
-  {
-    int tr = tie_rank;
-    for (int i = i_lo; i < i_hi; ++i) {
+  constexpr int NW = NT / 32, PER = kSelectBins / NT;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int kprime = 0;
+  uint32_t above_min = kWindowKey, tie_key = kWindowKey;     // the smallest key of which every entry stays; the key of which
+  int n_ties = 0;                                            // the first n_ties entries stay as well
+  uint32_t prefix = 0;                                       // the keys in question: those with key >> above_shift == prefix
+  for (int above_shift = shift + 11, s = shift, need = 0;; above_shift = s, s = s > 11 ? s - 11 : 0) {
+    const bool first = above_shift == shift + 11;
+    for (int i = tid; i < kSelectBins; i += NT) sh.hist[i] = 0;
+    if (tid == 0) sh.n_cand = 0;
+    __syncthreads();
+    for (int i = tid; i < L; i += NT) {
       const uint32_t k = key[i];
-      bool keep = (k == kWindowKey);
-      if (!keep) {
-        if (keep_all) keep = true;
-        else if (!keep_none) {
-          if (k > threshold) keep = true;
-          else if (k == threshold) { keep = tr < n_ties_taken; ++tr; }
+      if (k != kWindowKey && (k >> above_shift) == prefix) atomicAdd(&sh.hist[(k >> s) - (prefix << (above_shift - s))], 1);
+    }
+    __syncthreads();
+    // thread t counts the bins 2047 - PER t, .. downwards, so that the exclusive sum is what lies above them
+    int c[PER], mine = 0, all;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) { c[e] = sh.hist[kSelectBins - 1 - (tid * PER + e)]; mine += c[e]; }
+    const int above = block_exclusive_scan(mine, sh.warp_sums, &all);
+    if (first) {
+      kprime = (budget < 0 || budget > all) ? all : budget;
+      *kprime_plus_win = kprime + (L - all);
+      if (kprime == all) above_min = 0;
+      if (kprime == 0 || kprime == all) break;
+      need = kprime;
+    }
+    if (above < need && above + mine >= need) {
+      int r = need - above;
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        if (r > 0) {
+          if (c[e] >= r) { sh.bin = kSelectBins - 1 - (tid * PER + e); sh.need = r; sh.in_bin = c[e]; r = 0; }
+          else r -= c[e];
         }
       }
-      n_keep += keep ? 1 : 0;
     }
-  }
-  int oidx = block_exclusive_scan(n_keep, sh.warp_sums, &keep_total);
-  for (int i = i_lo; i < i_hi; ++i) {
-    const uint32_t k = key[i];
-    bool keep = (k == kWindowKey);
-    if (!keep) {
-      if (keep_all) keep = true;
-      else if (!keep_none) {
-        if (k > threshold) keep = true;
-        else if (k == threshold) { keep = tie_rank < n_ties_taken; ++tie_rank; }
+    __syncthreads();
+    prefix = (prefix << (above_shift - s)) + (uint32_t)sh.bin;
+    need = sh.need;
+    const int m = sh.in_bin;
+    if (m == need) {                             // the whole bin stays
+      above_min = prefix << s;
+      break;
+    }
+    if (s == 0) {                                // equal keys
+      tie_key = prefix;
+      n_ties = need;
+      above_min = prefix + 1;
+      break;
+    }
+    if (m <= NT) {
+      for (int i = tid; i < L; i += NT) {
+        const uint32_t k = key[i];
+        if (k != kWindowKey && (k >> s) == prefix) out[atomicAdd(&sh.n_cand, 1)] = (int)k;
       }
+      __syncthreads();
+      const int v = tid < m ? out[tid] : -1;     // (keys are below 2^31)
+      int gt = 0, ge = 0;
+      if (wid * 32 < m) {
+#pragma unroll 8
+        for (int i = 0; i < m; ++i) {
+          const int o = out[i];
+          gt += o > v;
+          ge += o >= v;
+        }
+      }
+      if (tid < m && gt < need && ge >= need) { sh.tie_key = (uint32_t)v; sh.n_ties = need - gt; }   // (equal keys write the same)
+      __syncthreads();                           // (and the candidates have been read: out may be written)
+      tie_key = sh.tie_key;
+      n_ties = sh.n_ties;
+      above_min = tie_key + 1;
+      break;
     }
-    if (keep) out[oidx++] = i;
   }
-  return keep_total;
+
+  // ordered emit: warp w owns entries [w * run, (w + 1) * run)
+  const int run = ((L + NW - 1) / NW + 31) & ~31, lo = wid * run, hi = min(lo + run, L);
+  const uint32_t lower = (1u << lane) - 1u;
+  int n_keep = 0, n_tie = 0;
+  for (int i0 = lo; i0 < hi; i0 += 32) {
+    const int i = i0 + lane;
+    const uint32_t k = i < hi ? key[i] : 0u;
+    n_keep += __popc(__ballot_sync(0xffffffffu, i < hi && (k >= above_min || k == kWindowKey)));
+    n_tie += __popc(__ballot_sync(0xffffffffu, i < hi && k == tie_key && k != kWindowKey));
+  }
+  if (lane == 0) { sh.keeps[wid] = n_keep; sh.ties[wid] = n_tie; }
+  __syncthreads();
+  const int keeps = lane < NW ? sh.keeps[lane] : 0, ties = lane < NW ? sh.ties[lane] : 0;
+  const int total = __reduce_add_sync(0xffffffffu, keeps) + min(__reduce_add_sync(0xffffffffu, ties), n_ties);
+  int tie_at = __reduce_add_sync(0xffffffffu, lane < wid ? ties : 0);
+  int at = __reduce_add_sync(0xffffffffu, lane < wid ? keeps : 0) + min(tie_at, n_ties);
+  for (int i0 = lo; i0 < hi; i0 += 32) {
+    const int i = i0 + lane;
+    const uint32_t k = i < hi ? key[i] : 0u;
+    const bool tie = i < hi && k == tie_key && k != kWindowKey;
+    const uint32_t tied = __ballot_sync(0xffffffffu, tie);
+    const bool keep = (i < hi && (k >= above_min || k == kWindowKey)) || (tie && tie_at + __popc(tied & lower) < n_ties);
+    const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+    if (keep) out[at + __popc(kept & lower)] = i;
+    at += __popc(kept);
+    tie_at += __popc(tied);
+  }
+  return total;
 }
 
 // The importance averaged over `pool` neighbouring entries (zeros beyond both ends), summed in slot order.
@@ -634,7 +643,7 @@ __device__ __forceinline__ uint32_t pooled_key(const float *sc, int i, int L, in
 // that is selected from the global key array as it stands (with pool > 1 the pooled keys are first written back
 // there), every pass streaming the keys through L2.
 __global__ void __launch_bounds__(1024) select_kernel(LayerView lv, WindowArg wa, int budget, const int *slice_budget, uint32_t *keys,
-                                                      const float *scores, int pool, int ld_s, int in_smem, int *keep_list,
+                                                      const float *scores, int pool, int ld_s, int in_smem, int shift, int *keep_list,
                                                       int *kept_count) {
   extern __shared__ uint32_t key_sm[];         // [L] when in_smem
   __shared__ SelectShared sh;
@@ -655,7 +664,7 @@ __global__ void __launch_bounds__(1024) select_kernel(LayerView lv, WindowArg wa
   __syncthreads();
   if (slice_budget != nullptr) budget = slice_budget[slice];
   int want;
-  const int keep_total = select_and_emit(in_smem ? key_sm : gkey, L, budget, out, sh, &want);
+  const int keep_total = select_and_emit<1024>(in_smem ? key_sm : gkey, L, budget, shift, out, sh, &want);
   if (tid == 0) {
     kept_count[slice] = keep_total;
     // the count rule of the selection: k' candidates and every sentinel entry survive
@@ -734,144 +743,162 @@ __global__ void __launch_bounds__(256) compact_kernel(LayerView lv, const int *k
 
 // ------------------------------------------------------------------------------------------
 // compress in one launch (Sec. 3.3, "KV Cache Selection"): importance, selection and pruning of one slice by one
-// CTA of 1024 threads, the phases separated by block barriers - what score_kernel, select_kernel and
+// CTA of 512 threads, the phases separated by block barriers - what score_kernel, select_kernel and
 // compact_kernel do in three launches, for every slice whose keys and keep list fit in shared memory.
 //   phase 1  policy 0: s_i = (1/w) sum_j 2^(y_ji * logit_scale - lse_j) from the window rows' logits (see
-//            score_kernel) -> scores (global, kept for inspection and for the pooling) and radix keys (shared);
+//            score_kernel), two neighbouring columns per thread -> scores (global, kept for inspection) and radix keys
+//            (shared); the window entries, whose slots follow from the map's place behind the history, get the sentinel.
 //            policy 1: keys from the original positions (see recent_keys_kernel).
-//   phase 2  select_and_emit: radix select in shared memory, ascending keep list in shared memory.
+//   phase 2  select_and_emit, ascending keep list in shared memory.
 //   phase 3  slot j <- old slot keep[j] for K, V and pos, in chunks: every thread loads its 8 16-byte pieces of
-//            the chunk, block barrier, stores them (keep[j] >= j, see compact_kernel); the untouched prefix is skipped.
+//            the chunk, block barrier, stores them.  keep is ascending and keep[j] >= j: within a chunk every source is read
+//            before any destination is written, and the sources of later chunks lie beyond every earlier destination.  The
+//            untouched prefix is skipped.
 // ext.on: the current map has not been copied into the pages (a one-call step whose attend left it in the caller's
 // tensors): entries hist .. L-1 are rows of those tensors, phase 3 reads the survivors among them there and every kept
 // row of the map is written, whatever its index.
-// Dynamic shared memory: 4 * (2 * ld_s + pages_per_slice) bytes.  grid = n_slices.
+// Few slices: the gridDim.y CTAs of a cluster find the same keep list and move a share of every row's columns each.
+// What bounds it: for short keep lists the latency of the phases, which 512 threads (so that two slices can share an SM) and
+// fewer rounds of barriers cut; for long ones the memory system: an SM stores 32 bytes per cycle (17 cycles per row, 22
+// measured for loads and stores of 16 slices), and 128 slices at once move at the HBM's rate (42 cycles per row = 5.9 TB/s).
+// Dynamic shared memory: 4 * (2 * ld_s + pages_per_slice) bytes.  grid (n_slices, shares).
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) compress_fused_kernel(LayerView lv, WindowArg wa, int policy, int n_sink,
-                                                              const float *logits, const float *lse, int ld_l, float logit_scale,
-                                                              int tile_padded, int budget, const int *slice_budget, int pool,
-                                                              float *scores, int ld_s, int *kept_count, ExternalMap ext) {
-  extern __shared__ uint32_t fsm[];
-  uint32_t *key = fsm;                                   // [ld_s]
-  int *list = reinterpret_cast<int *>(fsm + ld_s);       // [ld_s]
-  int *pt = list + ld_s;                                 // [pages_per_slice]
+constexpr int kCompressThreads = 512;
+
+__global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(LayerView lv, WindowArg wa, int policy, int n_sink,
+                                                                          const float *logits, const float *lse, int ld_l,
+                                                                          float logit_scale, int tile_padded, int budget,
+                                                                          const int *slice_budget, int pool, int shift, float *scores,
+                                                                          int ld_s, int *kept_count, ExternalMap ext) {
+  constexpr int NT = kCompressThreads;
+  extern __shared__ __align__(16) uint32_t fsm[];
+  int *list = reinterpret_cast<int *>(fsm);              // [ld_s]
+  uint32_t *key = fsm + ld_s;                            // [ld_s]
+  int *pt = list + 2 * ld_s;                             // [pages_per_slice]
   __shared__ SelectShared sh;
   __shared__ float lse_row[kMaxWindow];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int slice = blockIdx.x;
-  const int dev_status = *reinterpret_cast<volatile int *>(lv.status);
-  const int hist = lv.hist_len[slice];
+  const int share = blockIdx.y, shares = gridDim.y;
+  const int w = wa.w;
+  const int dev_status = *reinterpret_cast<volatile int *>(lv.status);      // (all of this is under way before any of it is needed)
+  const int hist = *reinterpret_cast<volatile int *>(lv.hist_len + slice);
+  if (slice_budget != nullptr) budget = slice_budget[slice];
+  for (int i = tid; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(lv.page_table + (size_t)slice * lv.pages_per_slice + i);
+  if (policy == 0 && tid < w) lse_row[tid] = lse[(size_t)slice * w + tid];
   if (dev_status != 0) return;                 // an earlier kernel reported a failed check: leave the store alone
   const int L = hist + wa.n_k;
-  const int w = wa.w;
-  for (int i = tid; i < lv.pages_per_slice; i += 1024) pt[i] = __ldg(lv.page_table + (size_t)slice * lv.pages_per_slice + i);
-  if (policy == 0 && tid < w) lse_row[tid] = lse[(size_t)slice * w + tid];
   __syncthreads();
   auto row_of = [&](int slot) { return ((size_t)pt[slot >> lv.page_shift] << lv.page_shift) + (size_t)(slot & lv.page_mask); };
-  // With ext.on the current map (entries hist .. L-1) is not in the pages: entry i is row i - hist of the caller's
-  // tensors and its original position follows from its index.
-  auto pos_of = [&](int i) { return (ext.on && i >= hist) ? wa.n_prev + (i - hist) : lv.pos_pool[row_of(i)]; };
   const long long ext_base = ext.on ? (long long)(slice / lv.n_heads) * ext.sb + (long long)(slice % lv.n_heads) * ext.sh : 0;
 
   // ---- phase 1: keys
-  float *sc_out = scores + (size_t)slice * ld_s;
   if (policy == 0) {
-    const int pad = tile_padded ? ((((hist + 127) >> 7) << 7) - hist) : 0;     // the current map starts at a multiple of 128 columns
+    float *sc_out = scores + (size_t)slice * ld_s;
+    // columns of a logit row: the history's, then the current map's from map_col on
+    const int map_col = tile_padded ? (hist + 127) & ~127 : hist, cols = map_col + wa.n_k;
     const float inv_w = 1.f / (float)w;
-    for (int i = tid; i < L; i += 1024) {
-      const float *y = logits + (size_t)slice * w * ld_l + (i >= hist ? i + pad : i);
-      float sc = 0.f;
+    const float *y = logits + (size_t)slice * w * ld_l;
+    for (int c0 = tid * 2; c0 < cols; c0 += NT * 2) {
+      float s0 = 0.f, s1 = 0.f;
       int j = 0;
-      for (; j + 8 <= w; j += 8) {
-        float t[8];
+      for (; j + 16 <= w; j += 16) {             // (a window of 16: one round of loads)
+        float2 t[16];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) t[e] = __ldg(y + (size_t)(j + e) * ld_l);
+        for (int e = 0; e < 16; ++e) t[e] = __ldg(reinterpret_cast<const float2 *>(y + (size_t)(j + e) * ld_l + c0));
 #pragma unroll
-        for (int e = 0; e < 8; ++e) sc += exp2f(fmaf(t[e], logit_scale, -lse_row[j + e]));
+        for (int e = 0; e < 16; ++e) {
+          s0 += exp2f(fmaf(t[e].x, logit_scale, -lse_row[j + e]));
+          s1 += exp2f(fmaf(t[e].y, logit_scale, -lse_row[j + e]));
+        }
       }
-      for (; j < w; ++j) sc += exp2f(fmaf(__ldg(y + (size_t)j * ld_l), logit_scale, -lse_row[j]));
-      sc *= inv_w;
-      sc_out[i] = sc;
-      const bool win = is_window_pos(wa, pos_of(i));
-      key[i] = win ? kWindowKey : (__float_as_uint(sc) & 0x7FFFFFFFu);
+#pragma unroll 4
+      for (; j < w; ++j) {
+        const float2 t = __ldg(reinterpret_cast<const float2 *>(y + (size_t)j * ld_l + c0));
+        s0 += exp2f(fmaf(t.x, logit_scale, -lse_row[j]));
+        s1 += exp2f(fmaf(t.y, logit_scale, -lse_row[j]));
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int col = c0 + e;
+        const int i = col < hist ? col : (col >= map_col && col < cols ? col - map_col + hist : -1);   // (the padding between them is nobody's)
+        if (i >= 0) {
+          const float sc = (e == 0 ? s0 : s1) * inv_w;
+          if (share == 0) sc_out[i] = sc;
+          key[i] = __float_as_uint(sc) & 0x7FFFFFFFu;
+        }
+      }
     }
+    __syncthreads();
     if (pool > 1) {
-      __syncthreads();                         // this CTA's scores are visible to all of its threads
-      for (int i = tid; i < L; i += 1024)
-        if (key[i] != kWindowKey) list[i] = (int)pooled_key(sc_out, i, L, pool);
+      for (int i = tid; i < L; i += NT) list[i] = (int)pooled_key(reinterpret_cast<const float *>(key), i, L, pool);
       __syncthreads();
-      for (int i = tid; i < L; i += 1024)
-        if (key[i] != kWindowKey) key[i] = (uint32_t)list[i];
+      for (int i = tid; i < L; i += NT) key[i] = (uint32_t)list[i];
+      __syncthreads();
     }
+    if (tid < w) key[hist + (wa.all ? tid : wa.pos[tid])] = kWindowKey;
   } else {
-    for (int i = tid; i < L; i += 1024) {
-      const int pos = pos_of(i);
+    for (int i = tid; i < L; i += NT) {
+      const int pos = i >= hist ? wa.n_prev + (i - hist) : lv.pos_pool[row_of(i)];
       key[i] = pos < n_sink ? kWindowKey : (uint32_t)pos + 1u;
     }
   }
   __syncthreads();
+  if (shares > 1) {                            // positions of this slice are read above and written below, by different CTAs
+    asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  }
 
   // ---- phase 2: selection
-  if (slice_budget != nullptr) budget = slice_budget[slice];
   int want;
-  const int kept = select_and_emit(key, L, budget, list, sh, &want);
+  const int kept = select_and_emit<NT>(key, L, budget, shift, list, sh, &want);
   if (kept != want) {                          // the count rule of the selection (block-uniform)
     if (tid == 0) atomicExch(lv.status, kDevCheck);
     return;
   }
   __syncthreads();
 
-  // ---- phase 3: in-place gather of K, V and pos
-  const int ppr = lv.row_bytes >> 4;           // 16-byte pieces per row
-  const int per_row = 2 * ppr;                 // K pieces, then V pieces
-  const int r_step = 1024 / per_row;           // rows per sweep of the CTA
-  const int C = 8 * r_step;                    // rows per chunk
+  // ---- phase 3: in-place gather of K, V and pos (a row of K or V is 256 bytes for either data type)
   int lo = 0, hi = kept;                       // first j with keep[j] != j
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
     if (list[mid] == mid) lo = mid + 1; else hi = mid;
   }
   if (ext.on && lo > hist) lo = hist;          // kept rows of the current map are not where they belong yet, whatever their index
-  const int r_in = tid / per_row, c = tid % per_row;
-  const char *ext_ptr = c < ppr ? ext.k : ext.v;
-  char *pool_ptr = c < ppr ? lv.k_pool : lv.v_pool;
-  const int piece = c < ppr ? c : c - ppr;
-  const bool pos_thread = c == 0;
-  if (r_in < r_step) {
-    for (int c0 = lo; c0 < kept; c0 += C) {
-      uint4 buf[8];
-      int pv[8];
+  const int pieces = 32 / shares;              // of a row's 32 16-byte pieces (16 of K, 16 of V); the lanes of a warp take `shares` rows
+  const int piece = share * pieces + lane % pieces;
+  const char *ext_ptr = (piece < 16 ? ext.k : ext.v) + (piece & 15) * 16;
+  char *pool_ptr = (piece < 16 ? lv.k_pool : lv.v_pool) + (piece & 15) * 16;
+  const int r_in = wid * shares + lane / pieces, r_step = NT / 32 * shares;
+  const int C = 8 * r_step;                    // rows per chunk, at most one per thread
+  for (int c0 = lo; c0 < kept; c0 += C) {
+    uint4 buf[8];
+    int pos = 0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = c0 + r_in + u * r_step;
-        if (j < kept) {
-          const int src = list[j];
-          if (ext.on && src >= hist) {
-            const long long e = (ext_base + (long long)(src - hist) * ext.st) * ext.esize;
-            buf[u] = __ldg(reinterpret_cast<const uint4 *>(ext_ptr + e) + piece);
-            if (pos_thread) pv[u] = wa.n_prev + (src - hist);
-          } else {
-            const size_t row = row_of(src);
-            buf[u] = reinterpret_cast<const uint4 *>(pool_ptr + row * lv.row_bytes)[piece];
-            if (pos_thread) pv[u] = lv.pos_pool[row];
-          }
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = c0 + r_in + u * r_step;
-        if (j < kept) {
-          const size_t row = row_of(j);
-          reinterpret_cast<uint4 *>(pool_ptr + row * lv.row_bytes)[piece] = buf[u];
-          if (pos_thread) lv.pos_pool[row] = pv[u];
-        }
+    for (int u = 0; u < 8; ++u) {
+      const int j = c0 + r_in + u * r_step;
+      if (j < kept) {
+        const int src = list[j];
+        const char *from = ext.on && src >= hist ? ext_ptr + (ext_base + (long long)(src - hist) * ext.st) * ext.esize
+                                                 : pool_ptr + row_of(src) * 256;
+        buf[u] = __ldcg(reinterpret_cast<const uint4 *>(from));
       }
     }
-  } else {
-    for (int c0 = lo; c0 < kept; c0 += C) __syncthreads();     // keeps the barrier count of the working threads
+    const int jp = c0 + tid;
+    const bool has_pos = share == 0 && tid < C && jp < kept;
+    if (has_pos) {
+      const int src = list[jp];
+      pos = ext.on && src >= hist ? wa.n_prev + (src - hist) : lv.pos_pool[row_of(src)];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = c0 + r_in + u * r_step;
+      if (j < kept) *reinterpret_cast<uint4 *>(pool_ptr + row_of(j) * 256) = buf[u];
+    }
+    if (has_pos) lv.pos_pool[row_of(jp)] = pos;
   }
-  if (tid == 0) {
+  if (tid == 0 && share == 0) {
     lv.next_len[slice] = kept;
     kept_count[slice] = kept;
   }

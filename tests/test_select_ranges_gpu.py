@@ -1,0 +1,61 @@
+"""The selection's histogram levels, its ranking and its ties, and the pruning by one CTA or a cluster per slice."""
+import pytest
+import torch
+
+from oracle import scalekv_oracle as orc
+from paper_2505_19602_b200 import binding
+from parity_util import ParityRun
+
+pytestmark = pytest.mark.gpu
+
+
+def levels_inputs(B, H, d, n, distinct, seed):
+    """Queries of one direction and keys with `distinct` different products with it (1: every entry ties with every other)."""
+    def fn(layer, scale):
+        g = torch.Generator().manual_seed(seed * 100 + scale)
+        Q = torch.zeros(B, H, n[scale], d)
+        Q[..., 0] = 1.0
+        K = 0.1 * torch.randn(B, H, n[scale], d, generator=g)
+        K[..., 0] = torch.randint(0, distinct, (B, H, n[scale]), generator=g).float() * 0.25
+        V = torch.randn(B, H, n[scale], d, generator=g)
+        return tuple(t.to(torch.bfloat16) for t in (Q, K, V))
+    return fn
+
+
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("heads", [1, 17])                 # a cluster of two CTAs per slice, one CTA per slice
+@pytest.mark.parametrize("distinct,budget", [
+    (1, 1),        # all keys equal, more of them than there are threads: the last level runs out of bits
+    (1, 700),
+    (2, 900),      # two keys: whole bins stay, or the tie runs through one
+    (300, 500),    # a bin with repeated keys, ranked
+])
+def test_ties_at_every_level(distinct, budget, heads, separate):
+    sides = (2, 40, 13)
+    n = orc.scale_token_counts(sides)
+    budgets = [[budget] * len(sides)]
+    kv = binding.ScaleKV(1, 1, heads, 128, "bf16", sides, sides, budgets)
+    run = ParityRun(kv, "bf16", sides, budgets, levels_inputs(1, heads, 128, n, distinct, 3),
+                    lambda k: orc.window_centroids(sides[k], sides[k], 16), sorted({(0, 0, 0), (0, 0, heads - 1)}), compress_last=True,
+                    max_rows=32)
+    run.separate_kernels = separate
+    run.run()
+    assert run.resyncs == 0 and run.evictions >= 2
+    kv.close()
+
+
+@pytest.mark.parametrize("heads", [2, 17])
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("budget", [5, 129, 2100])         # around the sinks, a chunk of rows, everything but a few
+def test_positional_rule_over_long_slices(budget, separate, heads):
+    sides = (20, 42, 3)
+    n = orc.scale_token_counts(sides)
+    budgets = [[budget] * len(sides)]
+    g = torch.Generator().manual_seed(8)
+    data = [tuple(torch.randn(1, heads, nk, 128, generator=g).to(torch.bfloat16) for _ in range(3)) for nk in n]
+    kv = binding.ScaleKV(1, 1, heads, 128, "bf16", sides, sides, budgets)
+    run = ParityRun(kv, "bf16", sides, budgets, lambda l, k: data[k], lambda k: None, sorted({(0, 0, 0), (0, 0, heads - 1)}),
+                    compress_last=True, max_rows=16)
+    run.policy, run.n_sink, run.separate_kernels = "recent", 4, separate
+    run.run()
+    kv.close()
