@@ -142,8 +142,9 @@ def _i32_array(values):
 
 def tensor_arg(t: torch.Tensor) -> scalekv_tensor:
     """[B, H, n, d] tensor -> view with element strides; the last axis must be contiguous."""
-    assert t.dim() == 4 and t.stride(3) == 1, "expected [B, H, n, d] with contiguous head_dim"
-    return scalekv_tensor(t.data_ptr(), t.stride(0), t.stride(1), t.stride(2))
+    s = t.stride()
+    assert len(s) == 4 and s[3] == 1, "expected [B, H, n, d] with contiguous head_dim"
+    return scalekv_tensor(t.data_ptr(), s[0], s[1], s[2])
 
 
 # ---- host-only helpers ----------------------------------------------------------------------
@@ -393,7 +394,8 @@ class ScaleKV:
         cs, ts, ns = (C.c_double * n)(), (C.c_double * n)(), (C.c_double * n)()
         self._check(self.lib.scalekv_layer_stats_ex(self.ctx, layer, tensor_arg(Q), topk_prime, query_stride,
                                                     C.byref(car), C.byref(htk), cs, ts, ns))
-        shape = lambda a: [[a[b * self.n_heads + h] for h in range(self.n_heads)] for b in range(self.batch)]
+        H = self.n_heads
+        shape = lambda a: [a[b * H:(b + 1) * H] for b in range(self.batch)]
         return car.value, htk.value, shape(cs), shape(ts), shape(ns)
 
     def scalekv_lengths(self, layer):

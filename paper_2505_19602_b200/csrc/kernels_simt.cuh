@@ -918,6 +918,8 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
 // the GPU: with one split the block adds its rows' c_i and t_i to the accumulators itself; with several every
 // CTA writes, per row, (maximum, normaliser, current mass, K' largest logits) to `partial` and
 // layer_stats_merge_kernel combines the splits.
+// acc: per slice the sums of c_i and t_i over the sampled rows, and the slice's length.
+// (This kernel serves f32 and K' > 16; see stats_mma_kernel.)
 // grid (ceil(n_rows / 64), n_slices, n_split); dynamic shared memory: layer_stats_smem_bytes<D>(K').
 // ------------------------------------------------------------------------------------------
 template <int D> __host__ __device__ constexpr size_t layer_stats_smem_bytes(int topk) {
@@ -936,11 +938,8 @@ __device__ __forceinline__ void stats_block_accumulate(float c_i, float t_i, dou
   if (tid == 0) {
     float cs = 0.f, ts = 0.f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { cs += red_c[w]; ts += red_t[w]; }   // fixed order
-    atomicAdd(&acc[0], (double)cs);
-    atomicAdd(&acc[1], (double)ts);
-    // the same sums per slice, behind the two totals
-    atomicAdd(&acc[2 + 2 * blockIdx.y], (double)cs);
-    atomicAdd(&acc[3 + 2 * blockIdx.y], (double)ts);
+    atomicAdd(&acc[3 * blockIdx.y], (double)cs);
+    atomicAdd(&acc[3 * blockIdx.y + 1], (double)ts);
   }
 }
 
@@ -961,6 +960,7 @@ __global__ void __launch_bounds__(256) layer_stats_kernel(LayerView lv, TensorVi
   const int slice = blockIdx.y;
   const int b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int L = lv.hist_len[slice] + n_k;
+  if (tid == 0 && blockIdx.x == 0 && blockIdx.z == 0) acc[3 * slice + 2] = (double)L;
   const int r0 = blockIdx.x * 64;
   const int Kp = topk_prime;
   const int n_split = gridDim.z;
@@ -1137,6 +1137,282 @@ __global__ void __launch_bounds__(64) layer_stats_merge_kernel(const float *part
   float c_i = 0.f, t_i = 0.f;
   if (blockIdx.x * 64 + row < n_rows) { c_i = cur / z; t_i = tsum / z; }
   stats_block_accumulate(c_i, t_i, acc, red_c, red_t);
+}
+
+// ------------------------------------------------------------------------------------------
+// layer statistics, bf16 x 128 and K' <= 16.  The same quantities as above; a CTA of 256 threads owns 64 sampled rows of one
+// slice and a range of its keys in tiles of 64.  Warp (wr, wc) takes rows 16 wr .. and keys 32 wc .. of a tile by tensor-core
+// products (m16n8k16), and every thread keeps, for the two rows of which it holds scores, its own maximum, normaliser,
+// current-map mass and descending list of the 16 largest history logits in registers: nothing is exchanged before the end,
+// when the four lanes and two warps of a row, and in a second kernel the key ranges, merge their lists pair by pair.
+// Entries hist .. L-1 of a slice are the current map.  Logits are kept in base 2.
+// The work is small (a calibration pass of one image: 70 GF, 0.3 G weights); what bounds it is the instructions per weight - an
+// exponential, an insertion where a list grows - and, at the small scales, the latency of a call.  Tensor-core products by
+// m16n8k16 leave the scores in registers and are a tenth of that time, so a TMEM pipeline would not shorten it.
+// One layer's 13 scales, one image, 16 slices: 2 048 us with the kernels above, 485 us here (4 096 queries, every 16th of them,
+// 10 521 keys: 921 + 19 -> 111 + 16 us); a call at the small scales 67 -> 32 us, sums in page-locked memory among the causes.
+// grid (ceil(n_rows / 64), n_slices, n_split); static shared memory: two K tiles and the query tile.
+// ------------------------------------------------------------------------------------------
+constexpr int kTop = 16;
+constexpr float kNoMax = -1e30f;         // a finite stand-in for -inf, so that differences of maxima are numbers
+
+__device__ __forceinline__ float pow2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void order(float &a, float &b) {
+  const float hi = fmaxf(a, b);
+  b = fminf(a, b);
+  a = hi;
+}
+// eight values into descending order (odd-even merge sort)
+__device__ __forceinline__ void sort8(float *v) {
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) order(v[i], v[i + 1]);
+#pragma unroll
+  for (int i = 0; i < 8; i += 4) { order(v[i], v[i + 2]); order(v[i + 1], v[i + 3]); order(v[i + 1], v[i + 2]); }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) order(v[i], v[i + 4]);
+  order(v[2], v[4]); order(v[3], v[5]);
+  order(v[1], v[2]); order(v[3], v[4]); order(v[5], v[6]);
+}
+// a bitonic list into descending order
+__device__ __forceinline__ void order_bitonic(float *a) {
+#pragma unroll
+  for (int d = kTop / 2; d > 0; d >>= 1)
+#pragma unroll
+    for (int i = 0; i < kTop; ++i)
+      if ((i & d) == 0) order(a[i], a[i + d]);
+}
+// the kTop largest of two descending lists, descending
+__device__ __forceinline__ void merge_top(float *a, const float *b) {
+#pragma unroll
+  for (int i = 0; i < kTop; ++i) a[i] = fmaxf(a[i], b[kTop - 1 - i]);
+  order_bitonic(a);
+}
+struct RowStats {
+  float m, z, cur, top[kTop];
+  __device__ __forceinline__ void clear() {
+    m = kNoMax; z = 0.f; cur = 0.f;
+#pragma unroll
+    for (int i = 0; i < kTop; ++i) top[i] = -INFINITY;
+  }
+  __device__ __forceinline__ void merge(float m2, float z2, float cur2, const float *top2) {
+    const float mm = fmaxf(m, m2), f = pow2(m - mm), f2 = pow2(m2 - mm);
+    z = z * f + z2 * f2;
+    cur = cur * f + cur2 * f2;
+    m = mm;
+    merge_top(top, top2);
+  }
+  // with the lane `mask` away
+  __device__ __forceinline__ void merge_lane(int mask) {
+    float t[kTop];
+#pragma unroll
+    for (int i = 0; i < kTop; ++i) t[i] = __shfl_xor_sync(0xffffffffu, top[i], mask);
+    const float m2 = __shfl_xor_sync(0xffffffffu, m, mask), z2 = __shfl_xor_sync(0xffffffffu, z, mask);
+    const float cur2 = __shfl_xor_sync(0xffffffffu, cur, mask);
+    merge(m2, z2, cur2, t);
+  }
+};
+constexpr int kStatsRec16 = 4 + kTop;    // floats per (split, row) record: m, z, cur, unused, the list
+
+__global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorView Q, int n_k, int stride, int n_rows, float scale_log2e,
+                                                           float *partial) {
+  __shared__ __align__(128) uint8_t sm[3 * 64 * 256];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wr = warp & 3, wc = warp >> 2;
+  const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int hist = lv.hist_len[slice], L = hist + n_k;
+  const int r0 = blockIdx.x * 64;
+  const int tiles = (L + 63) >> 6, n_split = gridDim.z;
+  const int t_lo = (int)((long long)tiles * blockIdx.z / n_split), t_hi = (int)((long long)tiles * (blockIdx.z + 1) / n_split);
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
+  // 16-byte piece c of row r of a 64 x 256-byte tile
+  auto at = [&](int tile, int r, int c) { return base + (uint32_t)(tile * 16384 + r * 256 + ((c ^ (r & 7)) << 4)); };
+  auto fetch = [&](int t) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = u * 16 + (tid >> 4), c = tid & 15, slot = t * 64 + r;
+      if (slot < L)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at(t & 1, r, c)), "l"(lv.k_pool + slot_row(lv, slice, slot) * 256 + c * 16) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = u * 16 + (tid >> 4), c = tid & 15;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r0 + r < n_rows) v = reinterpret_cast<const uint4 *>(row_ptr<__nv_bfloat16>(Q, b, h, (r0 + r) * stride))[c];
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at(2, r, c)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+  }
+  if (t_lo < t_hi) fetch(t_lo);
+  __syncthreads();
+  uint32_t qa[8][4];                     // the warp's 16 query rows, 8 steps of 16 columns
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(qa[k][0]), "=r"(qa[k][1]), "=r"(qa[k][2]), "=r"(qa[k][3])
+                 : "r"(at(2, wr * 16 + (lane & 15), 2 * k + (lane >> 4))));
+  RowStats st[2];
+  st[0].clear();
+  st[1].clear();
+  const bool idle = r0 + wr * 16 >= n_rows;            // (such a warp only helps to load)
+  for (int t = t_lo; t < t_hi; ++t) {
+    if (t + 1 < t_hi) fetch(t + 1); else asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    if (idle) { __syncthreads(); continue; }
+    float acc[4][4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+#pragma unroll
+      for (int n = 0; n < 4; n += 2) {
+        uint32_t kb[4];                  // two groups of 8 keys, each with both halves of the 16 columns
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(kb[0]), "=r"(kb[1]), "=r"(kb[2]), "=r"(kb[3])
+                     : "r"(at(t & 1, wc * 32 + n * 8 + (lane & 7) + ((lane >> 4) << 3), 2 * k + ((lane >> 3) & 1))));
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                       : "+f"(acc[n + g][0]), "+f"(acc[n + g][1]), "+f"(acc[n + g][2]), "+f"(acc[n + g][3])
+                       : "r"(qa[k][0]), "r"(qa[k][1]), "r"(qa[k][2]), "r"(qa[k][3]), "r"(kb[2 * g]), "r"(kb[2 * g + 1]));
+      }
+    }
+    // acc[n][2 i + e] belongs to row lane / 4 + 8 i and key 8 n + 2 (lane % 4) + e of the warp's part
+    const int j0 = t * 64 + wc * 32 + 2 * (lane & 3);
+    const bool ragged = t * 64 + 64 > L, any_hist = t * 64 < hist, any_cur = t * 64 + 64 > hist;     // (the same for all threads)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      RowStats &s = st[i];
+      float y[8], mx = kNoMax;
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float v = acc[n][2 * i + e] * scale_log2e;
+          if (ragged && j0 + 8 * n + e >= L) v = -INFINITY;
+          y[2 * n + e] = v;
+          mx = fmaxf(mx, v);
+        }
+      const float m_new = fmaxf(s.m, mx), f = pow2(s.m - m_new);
+      float sum = 0.f, cur = 0.f;
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float p = pow2(y[2 * n + e] - m_new);
+          sum += p;
+          if (any_cur && j0 + 8 * n + e >= hist) cur += p;
+        }
+      s.z = s.z * f + sum;
+      s.cur = s.cur * f + cur;
+      s.m = m_new;
+      if (any_hist) {
+        float top = -INFINITY;
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            if (any_cur && j0 + 8 * n + e >= hist) y[2 * n + e] = -INFINITY;
+            top = fmaxf(top, y[2 * n + e]);
+          }
+        if (__any_sync(0xffffffffu, top > s.top[kTop - 1])) {        // eight at a time: 14 operations a weight, 32 one by one
+          sort8(y);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) s.top[8 + q] = fmaxf(s.top[8 + q], y[7 - q]);
+          order_bitonic(s.top);
+        }
+      }
+    }
+    __syncthreads();                     // the tile has been read: its buffer is the next but one's
+  }
+  // the four lanes of a row, then its two warps
+  float *ex = reinterpret_cast<float *>(sm);           // [64][kStatsRec16]: the K tiles are done with
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    st[i].merge_lane(1);
+    st[i].merge_lane(2);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    float *e = ex + (wr * 16 + 8 * i + (lane >> 2)) * kStatsRec16;
+    if (wc == 1 && (lane & 3) == 0) {
+      e[0] = st[i].m; e[1] = st[i].z; e[2] = st[i].cur;
+#pragma unroll
+      for (int q = 0; q < kTop; ++q) e[4 + q] = st[i].top[q];
+    }
+  }
+  __syncthreads();
+  if (wc == 0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int row = wr * 16 + 8 * i + (lane >> 2);
+      const float *e = ex + row * kStatsRec16;
+      float t2[kTop];
+#pragma unroll
+      for (int q = 0; q < kTop; ++q) t2[q] = e[4 + q];
+      st[i].merge(e[0], e[1], e[2], t2);
+      if ((lane & 3) == 0 && r0 + row < n_rows) {
+        float4 *rec = reinterpret_cast<float4 *>(partial + (((size_t)slice * n_rows + r0 + row) * n_split + blockIdx.z) * kStatsRec16);
+        rec[0] = make_float4(st[i].m, st[i].z, st[i].cur, 0.f);
+#pragma unroll
+        for (int q = 0; q < kTop / 4; ++q) rec[1 + q] = make_float4(st[i].top[4 * q], st[i].top[4 * q + 1], st[i].top[4 * q + 2], st[i].top[4 * q + 3]);
+      }
+    }
+  }
+}
+
+// Merges the key ranges' records of stats_mma_kernel and sums c_i and t_i over a slice's rows in a fixed order: sixteen lanes
+// per row, a record each.  grid n_slices, 1024 threads.  acc as above (host memory: the caller reads it when the stream is
+// through); also writes the length the next scale finds.
+__global__ void __launch_bounds__(1024) stats_sum_kernel(LayerView lv, const float *partial, int n_split, int n_rows, int n_k, int topk_prime,
+                                                        double *acc) {
+  __shared__ double red[2][64];
+  const int tid = threadIdx.x, l = tid & 15, slice = blockIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int L = lv.hist_len[slice] + n_k;
+  double c_sum = 0.0, t_sum = 0.0;
+  for (int row0 = 0; row0 < n_rows; row0 += 64) {
+    const int row = row0 + (tid >> 4);
+    RowStats st;
+    st.clear();
+    if (row < n_rows && l < n_split) {
+      const float4 *rec = reinterpret_cast<const float4 *>(partial + (((size_t)slice * n_rows + row) * n_split + l) * kStatsRec16);
+      const float4 r = rec[0];
+      st.m = r.x; st.z = r.y; st.cur = r.z;
+#pragma unroll
+      for (int q = 0; q < kTop / 4; ++q) {
+        const float4 v = rec[1 + q];
+        st.top[4 * q] = v.x; st.top[4 * q + 1] = v.y; st.top[4 * q + 2] = v.z; st.top[4 * q + 3] = v.w;
+      }
+    }
+    for (int d = 1; d < n_split; d <<= 1) st.merge_lane(d);
+    if (l == 0 && row < n_rows) {
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < kTop; ++q)
+        if (q < topk_prime) t += pow2(st.top[q] - st.m);
+      c_sum += (double)(st.cur / st.z);
+      t_sum += (double)(t / st.z);
+    }
+  }
+  if (l == 0) { red[0][tid >> 4] = c_sum; red[1][tid >> 4] = t_sum; }
+  __syncthreads();
+  if (tid < 64) {                        // one warp sums the c_i, one the t_i
+    double v = red[tid >> 5][tid & 31] + red[tid >> 5][(tid & 31) + 32];
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if ((tid & 31) == 0) acc[3 * slice + (tid >> 5)] = v;
+  }
+  if (tid == 64) {
+    acc[3 * slice + 2] = (double)L;
+    lv.next_len[slice] = L;
+  }
 }
 
 }  // namespace scalekv

@@ -175,7 +175,7 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
   p.off_keep = o; o = align_up(o + (size_t)p.n_slices * p.ld_s * 4, 1024);
   p.off_kept = o; o = align_up(o + (size_t)p.n_slices * 4, 1024);
   p.off_hbud = o; o = align_up(o + (size_t)p.n_slices * 4, 1024);
-  p.off_acc = o; o = align_up(o + 16 + (size_t)p.n_slices * 16, 1024);
+  p.off_acc = o; o = align_up(o + 16 + (size_t)p.n_slices * 24, 1024);
   p.off_stats = o; o = align_up(o + (size_t)kStatsMaxCtas * 64 * kStatsRec * 4, 1024);   // key-range partials of layer_stats
   p.ws_bytes = o;
   return SCALEKV_OK;
@@ -196,6 +196,8 @@ struct scalekv_ctx {
   cudaEvent_t ev_in[2] = {nullptr, nullptr}, ev_out[2] = {nullptr, nullptr}, ev_att[2] = {nullptr, nullptr};
   int set_layer[2] = {-1, -1};     // layer that last used a staging half (-1: unused)
   long long host_steps = 0;
+  // layer_stats only: the sums arrive in page-locked memory of the library's own (host, created at the first call)
+  double *stats_host = nullptr, *stats_host_dev = nullptr;
   const void *stage_ptr = nullptr; // the staging area of the last step and the size of its halves
   size_t stage_half = 0;
   std::vector<int> page_table_host;
@@ -205,6 +207,7 @@ struct scalekv_ctx {
   std::vector<int> pending;        // n_k of an appended, not yet committed current map (0 = none)
   std::vector<int> attended;       // attend ran for the pending map
   std::vector<char> attend_marked; // ... and ev_attend was recorded behind it
+  std::vector<char> len_written;   // a kernel of the pending map has left the length the next scale finds
   std::vector<char> in_store;      // the pending map's rows have been copied into the pages
   std::vector<char> logits_padded; // attend recorded the logits while the current map was still outside the store
   std::vector<int> logits_of;      // scale whose window logits attend recorded for this layer (-1: none)
@@ -363,7 +366,7 @@ scalekv_status commit_pending(scalekv_ctx *ctx, int l, cudaStream_t s) {
   if (L > p.layers[l].persist_pages * p.P && p.layers[l].persist_pages < p.layers[l].total_pages)
     return fail(ctx, SCALEKV_ERR_CAPACITY, "layer %d: %d entries kept without compress exceed the persistent capacity %d",
                 l, L, p.layers[l].persist_pages * p.P);
-  if (!ctx->attended[l]) {      // (an attend has left the new length already)
+  if (!ctx->len_written[l]) {   // (attend and the statistics leave the new length themselves)
     Scope sc(ctx, s, kOther);
     commit_kernel<<<(p.n_slices + 255) / 256, 256, 0, s>>>(layer_view(ctx, l), ctx->pending[l]);
   }
@@ -462,6 +465,7 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
   ctx->pending.assign(p.n_layers, 0);
   ctx->attended.assign(p.n_layers, 0);
   ctx->attend_marked.assign(p.n_layers, 0);
+  ctx->len_written.assign(p.n_layers, 0);
   ctx->in_store.assign(p.n_layers, 1);
   ctx->logits_of.assign(p.n_layers, -1);
   ctx->logits_padded.assign(p.n_layers, 0);
@@ -554,6 +558,7 @@ scalekv_status scalekv_destroy(scalekv_ctx *ctx) {
     if (ctx->ev_out[i]) cudaEventDestroy(ctx->ev_out[i]);
     if (ctx->ev_att[i]) cudaEventDestroy(ctx->ev_att[i]);
   }
+  if (ctx->stats_host) cudaFreeHost(ctx->stats_host);
   for (auto e : ctx->ev_attend) cudaEventDestroy(e);
   for (auto e : ctx->ev_compress) cudaEventDestroy(e);
   for (auto e : ctx->event_pool) cudaEventDestroy(e);
@@ -613,6 +618,7 @@ scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, sc
   }
   ctx->pending[layer] = nk;
   ctx->attended[layer] = 0;
+  ctx->len_written[layer] = 0;
   ctx->next_scale[layer] = scale + 1;
   ctx->set_owner[par] = layer;
   return check_launch(ctx, "append");
@@ -671,6 +677,7 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
     }
   }
   ctx->attended[layer] = 1;
+  ctx->len_written[layer] = 1;
   // a compress that may evict will wait for this point of stream_main
   const int table = p.budgets[(size_t)layer * p.K + ctx->next_scale[layer] - 1];
   const bool mark = ctx->s_side != ctx->s_main && table != SCALEKV_KEEP_ALL && ctx->hist[layer] + nk > table;
@@ -1024,45 +1031,83 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   const int k = ctx->next_scale[layer] - 1;
   const int rows = (nk + query_stride - 1) / query_stride;
   double *acc = reinterpret_cast<double *>(ctx->ws + p.off_acc);
-  const size_t acc_bytes = 16 + (size_t)p.n_slices * 16;
-  CU(cudaMemsetAsync(acc, 0, acc_bytes, ctx->s_main));
+  const size_t acc_bytes = (size_t)p.n_slices * 24;
   // few slices and few sampled rows leave most SMs idle: split every slice's keys over enough CTAs to fill them
   const int row_blocks = (rows + 63) / 64;
   const int tiles = (ctx->hist[layer] + nk + 63) / 64;
   int n_split = 1;
   while (n_split < 16 && row_blocks * p.n_slices * n_split * 2 <= kStatsMaxCtas && n_split * 2 <= tiles) n_split *= 2;
   float *partial = reinterpret_cast<float *>(ctx->ws + p.off_stats);
-  {
+  // The tensor-core kernel: two CTAs per SM and no second wave (256 rows x 16 slices: 4 key ranges against 8).
+  // (The records of a launch with very many rows may outgrow the scratch: then the other kernel.)
+  const int mma_split = std::max(1, std::min({16, 2 * ctx->tc.n_sm / (row_blocks * p.n_slices), tiles}));
+  const bool tensor = ctx->dtype == SCALEKV_BF16 && topk_prime <= kTop &&
+                      (size_t)p.n_slices * rows * mma_split * kStatsRec16 <= (size_t)kStatsMaxCtas * 64 * kStatsRec;
+  const LayerView lv = layer_view(ctx, layer);
+  const double *sums;                                    // per slice: sums of c_i and t_i over the rows, length
+  std::vector<double> copied;
+  if (tensor) {
+    if (!ctx->stats_host) {
+      CU(cudaHostAlloc(reinterpret_cast<void **>(&ctx->stats_host), acc_bytes, cudaHostAllocMapped));
+      CU(cudaHostGetDevicePointer(reinterpret_cast<void **>(&ctx->stats_host_dev), ctx->stats_host, 0));
+    }
+    // (programmatic launches: a kernel comes up while the one before it ends)
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.stream = ctx->s_main;
+    {
+      Scope sc(ctx, ctx->s_main, kOther);
+      cfg.gridDim = dim3(row_blocks, p.n_slices, mma_split);
+      cfg.blockDim = dim3(256);
+      CU(cudaLaunchKernelEx(&cfg, stats_mma_kernel, lv, tview(Q), nk, query_stride, rows, ctx->scale * 1.4426950408889634f, partial));
+    }
     Scope sc(ctx, ctx->s_main, kOther);
-    dim3 grid(row_blocks, p.n_slices, n_split);
-    if (ctx->dtype == SCALEKV_BF16)
-      layer_stats_kernel<__nv_bfloat16, 128><<<grid, 256, layer_stats_smem_bytes<128>(topk_prime), ctx->s_main>>>(
-          layer_view(ctx, layer), tview(Q), nk, p.N[k], query_stride, rows, topk_prime, ctx->scale, acc, partial);
-    else
-      layer_stats_kernel<float, 64><<<grid, 256, layer_stats_smem_bytes<64>(topk_prime), ctx->s_main>>>(
-          layer_view(ctx, layer), tview(Q), nk, p.N[k], query_stride, rows, topk_prime, ctx->scale, acc, partial);
-  }
-  if (n_split > 1) {
-    Scope sc(ctx, ctx->s_main, kOther);
-    layer_stats_merge_kernel<<<dim3(row_blocks, p.n_slices), 64, 0, ctx->s_main>>>(partial, n_split, rows, topk_prime, acc);
+    cfg.gridDim = dim3(p.n_slices);
+    cfg.blockDim = dim3(1024);
+    CU(cudaLaunchKernelEx(&cfg, stats_sum_kernel, lv, (const float *)partial, mma_split, rows, nk, topk_prime, ctx->stats_host_dev));
+    sums = ctx->stats_host;
+    ctx->len_written[layer] = 1;
+  } else {
+    CU(cudaMemsetAsync(acc, 0, acc_bytes, ctx->s_main));
+    {
+      Scope sc(ctx, ctx->s_main, kOther);
+      dim3 grid(row_blocks, p.n_slices, n_split);
+      if (ctx->dtype == SCALEKV_BF16)
+        layer_stats_kernel<__nv_bfloat16, 128><<<grid, 256, layer_stats_smem_bytes<128>(topk_prime), ctx->s_main>>>(
+            lv, tview(Q), nk, p.N[k], query_stride, rows, topk_prime, ctx->scale, acc, partial);
+      else
+        layer_stats_kernel<float, 64><<<grid, 256, layer_stats_smem_bytes<64>(topk_prime), ctx->s_main>>>(
+            lv, tview(Q), nk, p.N[k], query_stride, rows, topk_prime, ctx->scale, acc, partial);
+    }
+    if (n_split > 1) {
+      Scope sc(ctx, ctx->s_main, kOther);
+      layer_stats_merge_kernel<<<dim3(row_blocks, p.n_slices), 64, 0, ctx->s_main>>>(partial, n_split, rows, topk_prime, acc);
+    }
   }
   scalekv_status st = check_launch(ctx, "layer_stats");
   if (st != SCALEKV_OK) return st;
-  std::vector<double> host(2 + 2 * (size_t)p.n_slices);
-  std::vector<int> len(p.n_slices);
-  CU(cudaMemcpyAsync(host.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, ctx->s_main));
-  CU(cudaMemcpyAsync(len.data(), layer_view(ctx, layer).hist_len, (size_t)p.n_slices * 4, cudaMemcpyDeviceToHost, ctx->s_main));
+  if (!tensor) {
+    copied.resize(3 * (size_t)p.n_slices);
+    sums = copied.data();
+    CU(cudaMemcpyAsync(copied.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, ctx->s_main));
+  }
   CU(cudaStreamSynchronize(ctx->s_main));
-  const double cnt = (double)rows * p.n_slices;
-  *car = host[0] / cnt;
-  *htk = host[1] / cnt;
+  double c_all = 0.0, t_all = 0.0;
   for (int s = 0; s < p.n_slices; ++s) {
-    const double c_s = host[2 + 2 * s] / rows, t_s = host[3 + 2 * s] / rows;
+    c_all += sums[3 * s];
+    t_all += sums[3 * s + 1];
+    const double c_s = sums[3 * s] / rows, t_s = sums[3 * s + 1] / rows;
     if (car_slices) car_slices[s] = c_s;
     if (htk_slices) htk_slices[s] = t_s;
-    // the stored length does not count the map just appended until a compress commits it
-    if (nca_slices) nca_slices[s] = c_s * (double)(len[s] + nk) / (double)nk;
+    if (nca_slices) nca_slices[s] = c_s * sums[3 * s + 2] / (double)nk;
   }
+  const double cnt = (double)rows * p.n_slices;
+  *car = c_all / cnt;
+  *htk = t_all / cnt;
   return SCALEKV_OK;
 }
 
