@@ -66,10 +66,222 @@ __global__ void commit_kernel(LayerView lv, int n_k) {
 }
 
 // ------------------------------------------------------------------------------------------
-// attend (SIMT): O = softmax(scale * Q K^T) V with online softmax, fp32 FMA (Eq. 5).
-// grid (ceil(n_k / 64), n_slices), 256 threads.  A block owns 64 query rows and streams the
-// slice's cache in tiles of 64 entries; thread (ty, tx) owns rows ty + 16 i, columns tx + 16 j.
+// attend, f32 x 64: O = softmax(scale * Q K^T) V with online softmax, fp32 FMA throughout (Eq. 5; the 1e-4 bound on outputs
+// rules TF32 out).  A CTA of 128 threads owns 64 query rows of one slice and streams its keys in tiles of 64; thread (ty, tx) owns
+// rows ty + 8 i and the keys (then the output columns) of tx, so that a warp only reads P that it has written itself.
+//   S  : keys tx + 16 j, packed multiply-adds over pairs of columns, operands as 16-byte loads from rows of 272 bytes: the
+//        two query rows of a warp's load are broadcasts and the 16 key rows meet no bank twice.
+//   P V: columns 4 tx .., packed over pairs of columns, P as 16-byte loads of four keys.
+// 12 loads feed 64 packed multiply-adds of 2 cycles each in both products, so the FMA pipe is what bounds them; K arrives
+// under P V and V under S (asynchronous copies, 70 KB of shared memory, three CTAs per SM to cover the barriers between).
+// 16 slices, us per launch averaged over four layers, 64/144/256/400/576/1024/1600 queries: 22.8/40.6/61/85/120/244/479 with 4 x 4
+// register tiles and scalar operands of P V, 15.9/18.7/26/54/92/188/365 here (FMA pipe 55 % busy: 2.3 warps per scheduler do
+// not cover the loads' latency, and the accumulators leave no registers for more).
+// Few CTAs: gridDim.z CTAs of a cluster share a slice's keys; each then combines a share of the rows,
+// O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e, reading the parts through distributed shared memory.
+// grid (ceil(n_k / 64), n_slices, split); dynamic shared memory kAttendF32Smem.
 // ------------------------------------------------------------------------------------------
+constexpr int kF32Ld = 68;                                  // floats per row of a tile
+constexpr int kF32Tile = 64 * kF32Ld;
+constexpr int kAttendF32Smem = (4 * kF32Tile + 2 * 64) * 4;
+constexpr int kF32MaxSplit = 8;
+
+__device__ __forceinline__ uint64_t pair_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t pair_mul(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t pair_of(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 pair_parts(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
+__global__ void __launch_bounds__(128, 3) attend_f32_kernel(LayerView lv, TensorView Q, TensorView O, float *lse, int n_k, float scale_log2e) {
+  extern __shared__ __align__(16) float sm_f32[];
+  float *Qs = sm_f32, *Ks = Qs + kF32Tile, *Vs = Ks + kF32Tile, *Ps = Vs + kF32Tile;
+  float *m_s = Ps + kF32Tile, *l_s = m_s + 64;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
+  const int q0 = blockIdx.x * 64;
+  const int L = lv.hist_len[slice] + n_k;
+  if (blockIdx.x == 0 && blockIdx.z == 0 && tid == 0) lv.next_len[slice] = L;     // unless a compress of this scale evicts
+  const int n_split = gridDim.z, tiles = (L + 63) >> 6;
+  const int t_lo = tiles * (int)blockIdx.z / n_split, t_hi = tiles * ((int)blockIdx.z + 1) / n_split;
+  auto fetch = [&](float *tile, const char *pool, int t) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int r = u * 8 + (tid >> 4), c = tid & 15, slot = t * 64 + r;
+      float *dst = tile + r * kF32Ld + c * 4;
+      if (slot < L)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                     "l"(pool + slot_row(lv, slice, slot) * 256 + c * 16)
+                     : "memory");
+      else
+        *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (t_lo < t_hi) fetch(Ks, lv.k_pool, t_lo);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int r = u * 8 + (tid >> 4), c = tid & 15;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (q0 + r < n_k) v = reinterpret_cast<const float4 *>(row_ptr<float>(Q, b, h, q0 + r))[c];
+    *reinterpret_cast<float4 *>(Qs + r * kF32Ld + c * 4) = v;
+  }
+  uint64_t o[8][2];
+  float m[8], l[8];                       // l: this thread's keys only
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { o[i][0] = o[i][1] = 0ull; m[i] = -1e30f; l[i] = 0.f; }
+  const float *qrow = Qs + ty * kF32Ld, *krow = Ks + tx * kF32Ld, *vcol = Vs + tx * 4;
+  float *prow = Ps + ty * kF32Ld;
+
+  for (int t = t_lo; t < t_hi; ++t) {
+    fetch(Vs, lv.v_pool, t);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();                      // K of this tile (and at first Q) is there
+    uint64_t s2[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s2[i][j] = 0ull;
+#pragma unroll 4
+    for (int c = 0; c < 64; c += 4) {
+      ulonglong2 k[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const ulonglong2 *>(krow + 16 * j * kF32Ld + c);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(qrow + 8 * i * kF32Ld + c);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s2[i][j] = pair_fma(q.x, k[j].x, s2[i][j]);
+          s2[i][j] = pair_fma(q.y, k[j].y, s2[i][j]);
+        }
+      }
+    }
+    __syncthreads();                      // everybody has read K
+    if (t + 1 < t_hi) fetch(Ks, lv.k_pool, t + 1); else asm volatile("cp.async.commit_group;" ::: "memory");
+    const int valid = L - t * 64;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float y[4], mx = m[i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 e = pair_parts(s2[i][j]);
+        y[j] = tx + 16 * j < valid ? (e.x + e.y) * scale_log2e : -INFINITY;
+        mx = fmaxf(mx, y[j]);
+      }
+#pragma unroll
+      for (int d = 8; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+      const float f = exp2f(m[i] - mx);
+      m[i] = mx;
+      l[i] *= f;
+      const uint64_t ff = pair_of(f, f);
+      o[i][0] = pair_mul(o[i][0], ff);
+      o[i][1] = pair_mul(o[i][1], ff);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float p = exp2f(y[j] - mx);
+        l[i] += p;
+        prow[8 * i * kF32Ld + tx + 16 * j] = p;
+      }
+    }
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();                      // V is there (and P, which only this warp reads)
+#pragma unroll 4
+    for (int c = 0; c < 64; c += 4) {
+      ulonglong2 v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = *reinterpret_cast<const ulonglong2 *>(vcol + (c + e) * kF32Ld);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 p = *reinterpret_cast<const float4 *>(prow + 8 * i * kF32Ld + c);
+        const uint64_t p0 = pair_of(p.x, p.x), p1 = pair_of(p.y, p.y), p2 = pair_of(p.z, p.z), p3 = pair_of(p.w, p.w);
+        o[i][0] = pair_fma(p0, v[0].x, o[i][0]);
+        o[i][1] = pair_fma(p0, v[0].y, o[i][1]);
+        o[i][0] = pair_fma(p1, v[1].x, o[i][0]);
+        o[i][1] = pair_fma(p1, v[1].y, o[i][1]);
+        o[i][0] = pair_fma(p2, v[2].x, o[i][0]);
+        o[i][1] = pair_fma(p2, v[2].y, o[i][1]);
+        o[i][0] = pair_fma(p3, v[3].x, o[i][0]);
+        o[i][1] = pair_fma(p3, v[3].y, o[i][1]);
+      }
+    }
+    __syncthreads();                      // everybody has read V
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], d);
+
+  if (n_split == 1) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = q0 + ty + 8 * i;
+      if (r >= n_k) continue;
+      const float inv = 1.f / l[i];
+      const float2 x = pair_parts(o[i][0]), y = pair_parts(o[i][1]);
+      *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, r)) + tx * 4) = make_float4(x.x * inv, x.y * inv, y.x * inv, y.y * inv);
+      if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + r] = (m[i] + log2f(l[i])) * 0.6931471805599453f;
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    *reinterpret_cast<ulonglong2 *>(prow + 8 * i * kF32Ld + tx * 4) = make_ulonglong2(o[i][0], o[i][1]);
+    if (tx == 0) { m_s[ty + 8 * i] = m[i]; l_s[ty + 8 * i] = l[i]; }
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  auto peer = [&](const float *p, int cta) {
+    uint32_t ra;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(cta));
+    return ra;
+  };
+  const int r_lo = 64 * (int)blockIdx.z / n_split, r_hi = min(64 * ((int)blockIdx.z + 1) / n_split, n_k - q0);
+  for (int r = r_lo + ty; r < r_hi; r += 8) {
+    float4 x[kF32MaxSplit];
+    float me[kF32MaxSplit], le[kF32MaxSplit], M = -1e30f;
+#pragma unroll
+    for (int e = 0; e < kF32MaxSplit; ++e) {
+      x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      me[e] = -1e30f; le[e] = 0.f;
+      if (e < n_split) {
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(me[e]) : "r"(peer(m_s + r, e)));
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(le[e]) : "r"(peer(l_s + r, e)));
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[e].x), "=f"(x[e].y), "=f"(x[e].z), "=f"(x[e].w)
+                     : "r"(peer(Ps + r * kF32Ld + tx * 4, e)));
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < kF32MaxSplit; ++e) M = fmaxf(M, me[e]);
+    float sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+    for (int e = 0; e < kF32MaxSplit; ++e) {
+      const float f = exp2f(me[e] - M);
+      sum = fmaf(f, le[e], sum);
+      a0 = fmaf(f, x[e].x, a0); a1 = fmaf(f, x[e].y, a1); a2 = fmaf(f, x[e].z, a2); a3 = fmaf(f, x[e].w, a3);
+    }
+    const float inv = 1.f / sum;
+    *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, q0 + r)) + tx * 4) = make_float4(a0 * inv, a1 * inv, a2 * inv, a3 * inv);
+    if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + q0 + r] = (M + log2f(sum)) * 0.6931471805599453f;
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 template <typename T, int D>
 __device__ __forceinline__ void load_tile_rows(float *dst, int ld, const LayerView &lv, const char *pool, int slice,
                                                int j0, int L) {
@@ -87,140 +299,6 @@ __device__ __forceinline__ void load_tile_rows(float *dst, int ld, const LayerVi
     }
 #pragma unroll
     for (int e = 0; e < VN; ++e) dst[r * ld + c * VN + e] = v[e];
-  }
-}
-
-template <typename T, int D>
-__global__ void __launch_bounds__(256) attend_simt_kernel(LayerView lv, TensorView Q, TensorView O, float *lse, int n_k,
-                                                          float scale) {
-  constexpr int BM = 64, BN = 64, LD = D + 4, LDS = BN + 1;
-  constexpr int CH = D * (int)sizeof(T) / 16;
-  constexpr int VN = Vec16<T>::N;
-  constexpr int NJ = D / 16;
-  extern __shared__ float smem[];
-  float *Qs = smem;
-  float *KVs = Qs + BM * LD;
-  float *Ss = KVs + BN * LD;
-  float *m_s = Ss + BM * LDS;
-  float *l_s = m_s + BM;
-  float *a_s = l_s + BM;
-
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int slice = blockIdx.y;
-  const int b = slice / lv.n_heads, h = slice % lv.n_heads;
-  const int q0 = blockIdx.x * BM;
-  const int L = lv.hist_len[slice] + n_k;
-
-  for (int idx = tid; idx < BM * CH; idx += 256) {
-    const int r = idx / CH, c = idx % CH;
-    float v[VN];
-    if (q0 + r < n_k) {
-      Vec16<T>::load(row_ptr<T>(Q, b, h, q0 + r) + c * VN, v);
-    } else {
-#pragma unroll
-      for (int e = 0; e < VN; ++e) v[e] = 0.f;
-    }
-#pragma unroll
-    for (int e = 0; e < VN; ++e) Qs[r * LD + c * VN + e] = v[e];
-  }
-  if (tid < BM) { m_s[tid] = -INFINITY; l_s[tid] = 0.f; }
-  if (blockIdx.x == 0 && tid == 0) lv.next_len[slice] = L;     // unless a compress of this scale evicts
-
-  float acc[4][NJ];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) acc[i][j] = 0.f;
-
-  for (int j0 = 0; j0 < L; j0 += BN) {
-    __syncthreads();
-    load_tile_rows<T, D>(KVs, LD, lv, lv.k_pool, slice, j0, L);
-    __syncthreads();
-    float s[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-    for (int c = 0; c < D; c += 4) {
-      float4 q[4], k[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const float4 *>(&Qs[(ty + 16 * i) * LD + c]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const float4 *>(&KVs[(tx + 16 * j) * LD + c]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s[i][j] = fmaf(q[i].x, k[j].x, s[i][j]);
-          s[i][j] = fmaf(q[i].y, k[j].y, s[i][j]);
-          s[i][j] = fmaf(q[i].z, k[j].z, s[i][j]);
-          s[i][j] = fmaf(q[i].w, k[j].w, s[i][j]);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        Ss[(ty + 16 * i) * LDS + tx + 16 * j] = (j0 + tx + 16 * j < L) ? s[i][j] * scale : -INFINITY;
-    __syncthreads();
-    // K tile is consumed: bring V in while the rows are normalised
-    load_tile_rows<T, D>(KVs, LD, lv, lv.v_pool, slice, j0, L);
-    {
-      const int row = tid >> 2, part = tid & 3;
-      float *srow = Ss + row * LDS + part * 16;
-      float mx = -INFINITY;
-#pragma unroll
-      for (int e = 0; e < 16; ++e) mx = fmaxf(mx, srow[e]);
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      const float m_old = m_s[row];
-      const float m_new = fmaxf(m_old, mx);
-      float sum = 0.f;
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        float p = expf(srow[e] - m_new);
-        srow[e] = p;
-        sum += p;
-      }
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-      __syncwarp();
-      if (part == 0) {
-        const float a = expf(m_old - m_new);
-        a_s[row] = a;
-        m_s[row] = m_new;
-        l_s[row] = l_s[row] * a + sum;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float a = a_s[ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) acc[i][j] *= a;
-    }
-    for (int kk = 0; kk < BN; ++kk) {
-      float p[4], v[NJ];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = Ss[(ty + 16 * i) * LDS + kk];
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) v[j] = KVs[kk * LD + tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) acc[i][j] = fmaf(p[i], v[j], acc[i][j]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = ty + 16 * i;
-    if (q0 + r >= n_k) continue;
-    const float inv = 1.f / l_s[r];
-    T *orow = const_cast<T *>(row_ptr<T>(O, b, h, q0 + r));
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) orow[tx + 16 * j] = from_float<T>(acc[i][j] * inv);
-    if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + q0 + r] = m_s[r] + logf(l_s[r]);
   }
 }
 
@@ -293,27 +371,6 @@ __global__ void __launch_bounds__(256) score_logits_kernel(LayerView lv, TensorV
       if (col < L) logits[((size_t)slice * wa.w + r) * ld_l + col] = s[i][j] * (scale * 1.4426950408889634f);
     }
   }
-}
-
-__device__ __forceinline__ float block_reduce_max(float v, float *red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  float r = red[0];
-  for (int i = 1; i < nw; ++i) r = fmaxf(r, red[i]);
-  return r;
-}
-__device__ __forceinline__ float block_reduce_sum(float v, float *red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  float r = 0.f;
-  for (int i = 0; i < nw; ++i) r += red[i];   // fixed order: deterministic
-  return r;
 }
 
 // ------------------------------------------------------------------------------------------

@@ -186,6 +186,7 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
 struct scalekv_ctx {
   Plan plan;
   int device = 0;
+  int n_sm = 148;
   int dtype = 0;
   float scale = 0.f;
   char *pool = nullptr, *ws = nullptr;
@@ -442,6 +443,7 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, cfg->device);
   if (major != 10) return bail(SCALEKV_ERR_UNSUPPORTED);
+  cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
   // page tables: persistent pages first, then the transient set the layer shares (layer mod kSets)
   ctx->page_table_host.resize(p.pt_elems);
   for (int l = 0; l < p.n_layers; ++l) {
@@ -483,12 +485,11 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
     // kernels cannot take is refused here and not at its first launch
     bool ok = true;
     if (cfg->dtype == SCALEKV_BF16) {
-      ok = ok && set_smem(attend_simt_kernel<__nv_bfloat16, 128>, (64 * 132 * 2 + 64 * 65 + 192) * 4);
       ok = ok && set_smem(score_logits_kernel<__nv_bfloat16, 128>, 2 * 64 * 132 * 4);
       ok = ok && set_smem(layer_stats_kernel<__nv_bfloat16, 128>, layer_stats_smem_bytes<128>(64));
     } else {
       ok = ok && set_smem(layer_stats_kernel<float, 64>, layer_stats_smem_bytes<64>(64));
-      ok = ok && set_smem(attend_simt_kernel<float, 64>, (64 * 68 * 2 + 64 * 65 + 192) * 4);
+      ok = ok && set_smem(attend_f32_kernel, kAttendF32Smem);
       ok = ok && set_smem(score_logits_kernel<float, 64>, 2 * 64 * 68 * 4);
     }
     // select and compact stage a slice in shared memory when it fits and work from global memory when it does not
@@ -667,13 +668,20 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       ctx->logits_of[layer] = wl ? k : -1;
       ctx->logits_padded[layer] = fused ? 1 : 0;
     } else {
-      dim3 grid((nk + 63) / 64, p.n_slices);
-      if (ctx->dtype == SCALEKV_BF16)
-        attend_simt_kernel<__nv_bfloat16, 128><<<grid, 256, (64 * 132 * 2 + 64 * 65 + 192) * 4, ctx->s_main>>>(
-            lv, tview(Q), tview(O), lse, nk, ctx->scale);
-      else
-        attend_simt_kernel<float, 64><<<grid, 256, (64 * 68 * 2 + 64 * 65 + 192) * 4, ctx->s_main>>>(
-            lv, tview(Q), tview(O), lse, nk, ctx->scale);
+      // CTAs that share a slice's keys: as many as fit beside each other (three per SM) and find a tile each
+      const int ctas = (nk + 63) / 64 * p.n_slices, tiles = (ctx->hist[layer] + nk + 63) / 64;
+      const int split = std::max(1, std::min({kF32MaxSplit, 3 * ctx->n_sm / ctas, tiles}));
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr[1];
+      cfg.gridDim = dim3((nk + 63) / 64, p.n_slices, split);
+      cfg.blockDim = dim3(128);
+      cfg.dynamicSmemBytes = kAttendF32Smem;
+      cfg.stream = ctx->s_main;
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)split;
+      cfg.attrs = attr;
+      cfg.numAttrs = split > 1 ? 1 : 0;
+      CU(cudaLaunchKernelEx(&cfg, attend_f32_kernel, lv, tview(Q), tview(O), lse, nk, ctx->scale * 1.4426950408889634f));
     }
   }
   ctx->attended[layer] = 1;
@@ -1040,7 +1048,7 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   float *partial = reinterpret_cast<float *>(ctx->ws + p.off_stats);
   // The tensor-core kernel: two CTAs per SM and no second wave (256 rows x 16 slices: 4 key ranges against 8).
   // (The records of a launch with very many rows may outgrow the scratch: then the other kernel.)
-  const int mma_split = std::max(1, std::min({16, 2 * ctx->tc.n_sm / (row_blocks * p.n_slices), tiles}));
+  const int mma_split = std::max(1, std::min({16, 2 * ctx->n_sm / (row_blocks * p.n_slices), tiles}));
   const bool tensor = ctx->dtype == SCALEKV_BF16 && topk_prime <= kTop &&
                       (size_t)p.n_slices * rows * mma_split * kStatsRec16 <= (size_t)kStatsMaxCtas * 64 * kStatsRec;
   const LayerView lv = layer_view(ctx, layer);
