@@ -1,4 +1,5 @@
-"""ctypes binding of libscalekv.so: argument marshalling only.
+"""Binding of libscalekv.so: argument marshalling only.  The hot calls go through a small native module (csrc/call.cpp) that
+reads the tensors and calls the library; everything else is ctypes.
 
 Function names equal the C ABI's (include/scalekv.h).  PyTorch provides device memory and
 streams; every step of the path runs inside the library's CUDA kernels.  There is no CPU
@@ -16,6 +17,8 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libscalekv.so")
 SOURCES = [os.path.join(_HERE, "csrc", f) for f in ("scalekv.cu", "select_static.cu", "kernels_simt.cuh", "attend_tc.cuh", "common.cuh")]
 HEADER = os.path.join(os.path.dirname(_HERE), "include", "scalekv.h")
+CALL_PATH = os.path.join(_HERE, "_scalekv_call.so")
+CALL_SOURCE = os.path.join(_HERE, "csrc", "call.cpp")
 
 KEEP_ALL = -1
 MAX_WINDOW = 64
@@ -54,7 +57,9 @@ class scalekv_tensor(C.Structure):
 
 
 def build_library(force=False, verbose=False):
-    """Compiles the CUDA sources for sm_100a into libscalekv.so (in-tree) when out of date."""
+    """Compiles the CUDA sources for sm_100a into libscalekv.so, and the native module of the hot calls (both in-tree), when out
+    of date."""
+    build_call(force, verbose)
     if not force and os.path.exists(LIB_PATH):
         newest = max(os.path.getmtime(p) for p in SOURCES + [HEADER] if os.path.exists(p))
         if os.path.getmtime(LIB_PATH) >= newest:
@@ -71,7 +76,43 @@ def build_library(force=False, verbose=False):
     return LIB_PATH
 
 
+def build_call(force=False, verbose=False):
+    """Compiles the native module of the hot calls against PyTorch's headers."""
+    if not force and os.path.exists(CALL_PATH) and os.path.getmtime(CALL_PATH) >= max(os.path.getmtime(CALL_SOURCE), os.path.getmtime(HEADER)):
+        return CALL_PATH
+    import sysconfig
+
+    from torch.utils import cpp_extension
+
+    libs = cpp_extension.library_paths()
+    cmd = ["g++", "-O2", "-shared", "-fPIC", "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *(f"-isystem{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_path("include")]), CALL_SOURCE, "-o", CALL_PATH,
+           *(f"-L{d}" for d in libs), *(f"-Wl,-rpath,{d}" for d in libs), "-lc10", "-ltorch_cpu", "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    if verbose:
+        print(res.stderr)
+    return CALL_PATH
+
+
 _lib = None
+_call = None
+
+
+def load_call():
+    """The native module of the hot calls (built when missing)."""
+    global _call
+    if _call is None:
+        import importlib.machinery
+        import importlib.util
+
+        if not os.path.exists(CALL_PATH):
+            build_call()
+        loader = importlib.machinery.ExtensionFileLoader("_scalekv_call", CALL_PATH)
+        _call = importlib.util.module_from_spec(importlib.util.spec_from_loader("_scalekv_call", loader))
+        loader.exec_module(_call)
+    return _call
 
 
 def load_library():
@@ -246,6 +287,9 @@ class ScaleKV:
         if not torch.cuda.is_available():
             raise RuntimeError("ScaleKV needs a CUDA device (sm_100a); there is no CPU path")
         self.lib = load_library()
+        self._call = load_call()
+        self._fn = {f: C.cast(getattr(self.lib, "scalekv_" + f), C.c_void_p).value
+                    for f in ("step", "step_ex", "append", "attend", "compress_ex")}
         self.device = torch.device("cuda", device)
         self.n_layers, self.batch, self.n_heads, self.head_dim = n_layers, batch, n_heads, head_dim
         self.dtype = {"bf16": BF16, "f32": F32, BF16: BF16, F32: F32}[dtype]
@@ -284,6 +328,7 @@ class ScaleKV:
         st = self.lib.scalekv_init(C.byref(cfg), C.byref(self.ctx))
         if st:
             raise ScaleKVError(st, "scalekv_init")
+        self._handle = self.ctx.value
         self.cfg = cfg
 
     # -- plumbing
@@ -295,6 +340,7 @@ class ScaleKV:
         if getattr(self, "ctx", None) and self.ctx.value:
             self.lib.scalekv_destroy(self.ctx)
             self.ctx = C.c_void_p(None)
+            self._handle = 0
 
     def __del__(self):
         try:
@@ -307,48 +353,47 @@ class ScaleKV:
         self._check(self.lib.scalekv_reset(self.ctx))
 
     def scalekv_append(self, layer, scale, K, V):
-        self._check(self.lib.scalekv_append(self.ctx, layer, scale, tensor_arg(K), tensor_arg(V)))
+        self._check(self._call.append(self._fn["append"], self._handle, layer, scale, K, V))
 
     def scalekv_attend(self, layer, Q, O=None, lse=None):
         if O is None:
             O = torch.empty_like(Q)
-        self._check(self.lib.scalekv_attend(self.ctx, layer, tensor_arg(Q), tensor_arg(O),
-                                            None if lse is None else lse.data_ptr()))
+        self._check(self._call.attend(self._fn["attend"], self._handle, layer, Q, O, lse))
         return O
 
-    def scalekv_compress(self, layer, Qw, window_pos=None, qw_is_full_map=False):
+    @staticmethod
+    def _window(window_pos):
+        """(array or None, its address, its length) of a window given as a sequence, as a prepared array or not at all."""
         if window_pos is None:
-            self._check(self.lib.scalekv_compress(self.ctx, layer, tensor_arg(Qw), 0, None, int(qw_is_full_map)))
-        else:
-            wp = _i32_array(window_pos)
-            self._check(self.lib.scalekv_compress(self.ctx, layer, tensor_arg(Qw), len(window_pos), wp, int(qw_is_full_map)))
+            return None, 0, 0
+        wp = window_pos if isinstance(window_pos, C.Array) else _i32_array(window_pos)
+        return wp, C.addressof(wp), len(wp)
+
+    def scalekv_compress(self, layer, Qw, window_pos=None, qw_is_full_map=False):
+        wp, at, w = self._window(window_pos)
+        self._check(self._call.compress_ex(self._fn["compress_ex"], self._handle, layer, Qw, w, at, int(qw_is_full_map), 0))
+
+    @staticmethod
+    def _select_opts(policy, pool_kernel, n_sink, head_shared, head_budgets, separate_kernels):
+        hb = _i32_array(head_budgets) if head_budgets is not None else None
+        return scalekv_select_opts({"score": 0, "recent": 1}[policy], pool_kernel, n_sink, int(head_shared), hb, int(separate_kernels))
 
     def scalekv_compress_ex(self, layer, Qw=None, window_pos=None, qw_is_full_map=False, policy="score", pool_kernel=1,
                             n_sink=0, head_shared=False, head_budgets=None, separate_kernels=False):
         """scalekv_compress with a selection variant: policy "score" (optionally pooled) or "recent"."""
-        hb = _i32_array(head_budgets) if head_budgets is not None else None
-        opts = scalekv_select_opts({"score": 0, "recent": 1}[policy], pool_kernel, n_sink, int(head_shared), hb,
-                                   int(separate_kernels))
-        q = tensor_arg(Qw) if Qw is not None else scalekv_tensor(None, 0, 0, 0)
-        if window_pos is None:
-            wp, w = None, 0
-        else:
-            wp, w = _i32_array(window_pos), len(window_pos)
-        self._check(self.lib.scalekv_compress_ex(self.ctx, layer, q, w, wp, int(qw_is_full_map), C.byref(opts)))
+        opts = self._select_opts(policy, pool_kernel, n_sink, head_shared, head_budgets, separate_kernels)
+        wp, at, w = self._window(window_pos)
+        self._check(self._call.compress_ex(self._fn["compress_ex"], self._handle, layer, Qw, w, at, int(qw_is_full_map),
+                                           C.addressof(opts)))
 
     def scalekv_step(self, layer, scale, Q, K, V, O, window_pos=None, whole_map=False, lse=None):
         """append + attend + compress (window rows taken from Q) in one call; window_pos None and not whole_map: no compress.
         window_pos may be a prepared ctypes int32 array (see window_array)."""
         if whole_map:
-            w, wp = -1, None
-        elif window_pos is None:
-            w, wp = 0, None
+            wp, at, w = None, 0, -1
         else:
-            wp = window_pos if isinstance(window_pos, C.Array) else _i32_array(window_pos)
-            w = len(wp)
-        lp = C.cast(lse.data_ptr(), C.POINTER(C.c_float)) if lse is not None else None
-        self._check(self.lib.scalekv_step(self.ctx, layer, scale, tensor_arg(Q), tensor_arg(K), tensor_arg(V), tensor_arg(O),
-                                          lp, w, wp))
+            wp, at, w = self._window(window_pos)
+        self._check(self._call.step(self._fn["step"], self._handle, layer, scale, Q, K, V, O, lse, w, at))
 
     @staticmethod
     def window_array(window_pos):
@@ -358,17 +403,10 @@ class ScaleKV:
     def scalekv_step_ex(self, layer, scale, Q, K, V, O, compress=True, window_pos=None, lse=None, policy="score", pool_kernel=1,
                         n_sink=0, head_shared=False, head_budgets=None, separate_kernels=False):
         """append + attend + scalekv_compress_ex (Q as the full current map) in one call; compress=False: no compress."""
-        hb = _i32_array(head_budgets) if head_budgets is not None else None
-        opts = scalekv_select_opts({"score": 0, "recent": 1}[policy], pool_kernel, n_sink, int(head_shared), hb,
-                                   int(separate_kernels))
-        if window_pos is None:
-            wp, w = None, 0
-        else:
-            wp = window_pos if isinstance(window_pos, C.Array) else _i32_array(window_pos)
-            w = len(wp)
-        lp = C.cast(lse.data_ptr(), C.POINTER(C.c_float)) if lse is not None else None
-        self._check(self.lib.scalekv_step_ex(self.ctx, layer, scale, tensor_arg(Q), tensor_arg(K), tensor_arg(V), tensor_arg(O),
-                                             lp, int(bool(compress)), w, wp, C.byref(opts)))
+        opts = self._select_opts(policy, pool_kernel, n_sink, head_shared, head_budgets, separate_kernels)
+        wp, at, w = self._window(window_pos)
+        self._check(self._call.step_ex(self._fn["step_ex"], self._handle, layer, scale, Q, K, V, O, lse, int(bool(compress)), w, at,
+                                       C.addressof(opts)))
 
     def scalekv_step_host(self, layer, scale, Qh, Kh, Vh, Oh, staging, window_pos=None, whole_map=False):
         if whole_map:

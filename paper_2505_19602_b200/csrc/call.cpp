@@ -1,0 +1,122 @@
+// The hot calls of the C ABI for Python callers: tensors are read through PyTorch's C++ interface and handed to the function
+// whose address the binding passes, in one native call.  Building four ctypes structures and converting them took 3.1 us
+// of the 11 us that a step costs the host; the small scales are bound by that.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/scalekv.h"
+
+namespace {
+
+// [B, H, n, d] tensor -> view with element strides; the last axis must be contiguous
+bool view(PyObject *obj, scalekv_tensor *out) {
+  if (!THPVariable_Check(obj)) {
+    PyErr_SetString(PyExc_TypeError, "expected a tensor");
+    return false;
+  }
+  const at::Tensor &t = THPVariable_Unpack(obj);
+  if (t.dim() != 4 || t.stride(3) != 1) {
+    PyErr_SetString(PyExc_AssertionError, "expected [B, H, n, d] with contiguous head_dim");
+    return false;
+  }
+  out->ptr = t.data_ptr();
+  out->stride_b = t.stride(0);
+  out->stride_h = t.stride(1);
+  out->stride_t = t.stride(2);
+  return true;
+}
+
+// None or a tensor of floats
+bool floats(PyObject *obj, float **out) {
+  *out = nullptr;
+  if (obj == Py_None) return true;
+  if (!THPVariable_Check(obj)) {
+    PyErr_SetString(PyExc_TypeError, "expected a tensor or None");
+    return false;
+  }
+  *out = static_cast<float *>(THPVariable_Unpack(obj).data_ptr());
+  return true;
+}
+
+template <typename T> T address(PyObject *obj) { return reinterpret_cast<T>(PyLong_AsVoidPtr(obj)); }
+
+bool arguments(Py_ssize_t n, Py_ssize_t want) {
+  if (n == want) return true;
+  PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
+  return false;
+}
+
+#define CALL(expr)            \
+  int st;                     \
+  if (PyErr_Occurred()) return nullptr; \
+  Py_BEGIN_ALLOW_THREADS      \
+  st = (int)(expr);           \
+  Py_END_ALLOW_THREADS        \
+  return PyLong_FromLong(st)
+
+// step(function, ctx, layer, scale, Q, K, V, O, lse, w, window address)
+PyObject *step(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  scalekv_tensor q, k, v, o;
+  float *lse;
+  if (!arguments(n, 11) || !view(a[4], &q) || !view(a[5], &k) || !view(a[6], &v) || !view(a[7], &o) || !floats(a[8], &lse)) return nullptr;
+  const auto fn = address<decltype(&scalekv_step)>(a[0]);
+  const auto ctx = address<scalekv_ctx *>(a[1]);
+  const int layer = (int)PyLong_AsLong(a[2]), scale = (int)PyLong_AsLong(a[3]), w = (int)PyLong_AsLong(a[9]);
+  const auto window = address<const int32_t *>(a[10]);
+  CALL(fn(ctx, layer, scale, q, k, v, o, lse, w, window));
+}
+
+// step_ex(function, ctx, layer, scale, Q, K, V, O, lse, compress, w, window address, options address)
+PyObject *step_ex(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  scalekv_tensor q, k, v, o;
+  float *lse;
+  if (!arguments(n, 13) || !view(a[4], &q) || !view(a[5], &k) || !view(a[6], &v) || !view(a[7], &o) || !floats(a[8], &lse)) return nullptr;
+  const auto fn = address<decltype(&scalekv_step_ex)>(a[0]);
+  const auto ctx = address<scalekv_ctx *>(a[1]);
+  const int layer = (int)PyLong_AsLong(a[2]), scale = (int)PyLong_AsLong(a[3]), compress = (int)PyLong_AsLong(a[9]), w = (int)PyLong_AsLong(a[10]);
+  const auto window = address<const int32_t *>(a[11]);
+  const auto opts = address<const scalekv_select_opts *>(a[12]);
+  CALL(fn(ctx, layer, scale, q, k, v, o, lse, compress, w, window, opts));
+}
+
+// append(function, ctx, layer, scale, K, V)
+PyObject *append(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  scalekv_tensor k, v;
+  if (!arguments(n, 6) || !view(a[4], &k) || !view(a[5], &v)) return nullptr;
+  const auto fn = address<decltype(&scalekv_append)>(a[0]);
+  const auto ctx = address<scalekv_ctx *>(a[1]);
+  const int layer = (int)PyLong_AsLong(a[2]), scale = (int)PyLong_AsLong(a[3]);
+  CALL(fn(ctx, layer, scale, k, v));
+}
+
+// attend(function, ctx, layer, Q, O, lse)
+PyObject *attend(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  scalekv_tensor q, o;
+  float *lse;
+  if (!arguments(n, 6) || !view(a[3], &q) || !view(a[4], &o) || !floats(a[5], &lse)) return nullptr;
+  const auto fn = address<decltype(&scalekv_attend)>(a[0]);
+  const auto ctx = address<scalekv_ctx *>(a[1]);
+  const int layer = (int)PyLong_AsLong(a[2]);
+  CALL(fn(ctx, layer, q, o, lse));
+}
+
+// compress_ex(function, ctx, layer, Qw or None, w, window address, full map, options address)
+PyObject *compress_ex(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  scalekv_tensor q = {nullptr, 0, 0, 0};
+  if (!arguments(n, 8) || (a[3] != Py_None && !view(a[3], &q))) return nullptr;
+  const auto fn = address<decltype(&scalekv_compress_ex)>(a[0]);
+  const auto ctx = address<scalekv_ctx *>(a[1]);
+  const int layer = (int)PyLong_AsLong(a[2]), w = (int)PyLong_AsLong(a[4]), full = (int)PyLong_AsLong(a[6]);
+  const auto window = address<const int32_t *>(a[5]);
+  const auto opts = address<const scalekv_select_opts *>(a[7]);
+  CALL(fn(ctx, layer, q, w, window, full, opts));
+}
+
+#define METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {METHOD(step), METHOD(step_ex), METHOD(append), METHOD(attend), METHOD(compress_ex), {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_scalekv_call", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__scalekv_call() { return PyModule_Create(&module); }
