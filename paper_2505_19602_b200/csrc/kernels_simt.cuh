@@ -1201,14 +1201,16 @@ __global__ void __launch_bounds__(64) layer_stats_merge_kernel(const float *part
 // slice and a range of its keys in tiles of 64.  Warp (wr, wc) takes rows 16 wr .. and keys 32 wc .. of a tile by tensor-core
 // products (m16n8k16), and every thread keeps, for the two rows of which it holds scores, its own maximum, normaliser,
 // current-map mass and descending list of the 16 largest history logits in registers: nothing is exchanged before the end,
-// when the four lanes and two warps of a row, and in a second kernel the key ranges, merge their lists pair by pair.
+// when the four lanes and two warps of a row, and in the CTA that finishes last the key ranges, merge their lists pair by pair.
 // Entries hist .. L-1 of a slice are the current map.  Logits are kept in base 2.
 // The work is small (a calibration pass of one image: 70 GF, 0.3 G weights); what bounds it is the instructions per weight - an
 // exponential, an insertion where a list grows - and, at the small scales, the latency of a call.  Tensor-core products by
 // m16n8k16 leave the scores in registers and are a tenth of that time, so a TMEM pipeline would not shorten it.
 // One layer's 13 scales, one image, 16 slices: 2 048 us with the kernels above, 485 us here (4 096 queries, every 16th of them,
 // 10 521 keys: 921 + 19 -> 111 + 16 us); a call at the small scales 67 -> 32 us, sums in page-locked memory among the causes.
-// grid (ceil(n_rows / 64), n_slices, n_split); static shared memory: two K tiles and the query tile.
+// sums (host memory: the caller reads it when the stream is through): per slice and block of rows the sums of c_i and t_i, then
+// the slices' lengths.  counters: one per slice and block of rows, zero before and after.
+// grid (ceil(n_rows / 64), n_slices, n_split <= 16); static shared memory: two K tiles and the query tile.
 // ------------------------------------------------------------------------------------------
 constexpr int kTop = 16;
 constexpr float kNoMax = -1e30f;         // a finite stand-in for -inf, so that differences of maxima are numbers
@@ -1274,8 +1276,8 @@ struct RowStats {
 };
 constexpr int kStatsRec16 = 4 + kTop;    // floats per (split, row) record: m, z, cur, unused, the list
 
-__global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorView Q, int n_k, int stride, int n_rows, float scale_log2e,
-                                                           float *partial) {
+__global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorView Q, int n_k, int stride, int n_rows, int topk_prime,
+                                                           float scale_log2e, float *partial, int *counters, double *sums) {
   __shared__ __align__(128) uint8_t sm[3 * 64 * 256];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wr = warp & 3, wc = warp >> 2;
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
@@ -1423,52 +1425,58 @@ __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorV
       }
     }
   }
-}
-
-// Merges the key ranges' records of stats_mma_kernel and sums c_i and t_i over a slice's rows in a fixed order: sixteen lanes
-// per row, a record each.  grid n_slices, 1024 threads.  acc as above (host memory: the caller reads it when the stream is
-// through); also writes the length the next scale finds.
-__global__ void __launch_bounds__(1024) stats_sum_kernel(LayerView lv, const float *partial, int n_split, int n_rows, int n_k, int topk_prime,
-                                                        double *acc) {
-  __shared__ double red[2][64];
-  const int tid = threadIdx.x, l = tid & 15, slice = blockIdx.x;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int L = lv.hist_len[slice] + n_k;
+  // The CTA that finishes a block of rows last merges the key ranges' records, sixteen lanes per row, a record each, and sums
+  // c_i and t_i over the rows in a fixed order.
+  int *last = reinterpret_cast<int *>(sm);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    int *count = counters + (size_t)slice * gridDim.x + blockIdx.x;
+    const int before = atomicAdd(count, 1);
+    *last = before == n_split - 1;
+    if (before == n_split - 1) *count = 0;             // as the next launch wants to find it
+  }
+  __syncthreads();
+  if (!*last) return;
+  __threadfence();
+  const int l = tid & 15, n_here = min(64, n_rows - r0);
   double c_sum = 0.0, t_sum = 0.0;
-  for (int row0 = 0; row0 < n_rows; row0 += 64) {
+  for (int row0 = 0; row0 < n_here; row0 += 16) {
     const int row = row0 + (tid >> 4);
-    RowStats st;
-    st.clear();
-    if (row < n_rows && l < n_split) {
-      const float4 *rec = reinterpret_cast<const float4 *>(partial + (((size_t)slice * n_rows + row) * n_split + l) * kStatsRec16);
-      const float4 r = rec[0];
-      st.m = r.x; st.z = r.y; st.cur = r.z;
+    RowStats &s = st[0];
+    s.clear();
+    if (row < n_here && l < n_split) {
+      const float4 *rec = reinterpret_cast<const float4 *>(partial + (((size_t)slice * n_rows + r0 + row) * n_split + l) * kStatsRec16);
+      const float4 r = __ldcg(rec);
+      s.m = r.x; s.z = r.y; s.cur = r.z;
 #pragma unroll
       for (int q = 0; q < kTop / 4; ++q) {
-        const float4 v = rec[1 + q];
-        st.top[4 * q] = v.x; st.top[4 * q + 1] = v.y; st.top[4 * q + 2] = v.z; st.top[4 * q + 3] = v.w;
+        const float4 v = __ldcg(rec + 1 + q);
+        s.top[4 * q] = v.x; s.top[4 * q + 1] = v.y; s.top[4 * q + 2] = v.z; s.top[4 * q + 3] = v.w;
       }
     }
-    for (int d = 1; d < n_split; d <<= 1) st.merge_lane(d);
-    if (l == 0 && row < n_rows) {
+    for (int d = 1; d < n_split; d <<= 1) s.merge_lane(d);
+    if (l == 0 && row < n_here) {
       float t = 0.f;
 #pragma unroll
       for (int q = 0; q < kTop; ++q)
-        if (q < topk_prime) t += pow2(st.top[q] - st.m);
-      c_sum += (double)(st.cur / st.z);
-      t_sum += (double)(t / st.z);
+        if (q < topk_prime) t += pow2(s.top[q] - s.m);
+      c_sum += (double)(s.cur / s.z);
+      t_sum += (double)(t / s.z);
     }
   }
-  if (l == 0) { red[0][tid >> 4] = c_sum; red[1][tid >> 4] = t_sum; }
+  double *red = reinterpret_cast<double *>(sm + 64);   // [2][16]
+  if (l == 0) { red[tid >> 4] = c_sum; red[16 + (tid >> 4)] = t_sum; }
   __syncthreads();
-  if (tid < 64) {                        // one warp sums the c_i, one the t_i
-    double v = red[tid >> 5][tid & 31] + red[tid >> 5][(tid & 31) + 32];
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    if ((tid & 31) == 0) acc[3 * slice + (tid >> 5)] = v;
+  if (tid < 32) {                        // half a warp sums the c_i, half the t_i
+    double v = red[tid];
+    for (int d = 8; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    double *out = sums + ((size_t)slice * gridDim.x + blockIdx.x) * 2;
+    if (l == 0) out[tid >> 4] = v;
   }
-  if (tid == 64) {
-    acc[3 * slice + 2] = (double)L;
-    lv.next_len[slice] = L;
+  if (blockIdx.x == 0 && tid == 32) {
+    sums[(size_t)2 * gridDim.x * gridDim.y + slice] = (double)L;
+    lv.next_len[slice] = L;              // what the next scale finds
   }
 }
 

@@ -59,7 +59,7 @@ struct Plan {
   size_t off_k, off_v, off_pos, off_pt, off_len, off_status, pool_bytes;
   size_t pt_elems, logits_elems;
   // workspace layout
-  size_t off_logits, off_wlse, off_scores, off_keys, off_keep, off_kept, off_hbud, off_acc, off_stats, ws_bytes;
+  size_t off_logits, off_wlse, off_scores, off_keys, off_keep, off_kept, off_hbud, off_acc, off_count, off_stats, ws_bytes;
 };
 
 // Raster indices of the observation window of an h x w map (see scalekv_window_centroids).
@@ -176,6 +176,7 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
   p.off_kept = o; o = align_up(o + (size_t)p.n_slices * 4, 1024);
   p.off_hbud = o; o = align_up(o + (size_t)p.n_slices * 4, 1024);
   p.off_acc = o; o = align_up(o + 16 + (size_t)p.n_slices * 24, 1024);
+  p.off_count = o; o = align_up(o + (size_t)p.n_slices * ((p.n_max + 63) / 64) * 4, 1024);
   p.off_stats = o; o = align_up(o + (size_t)kStatsMaxCtas * 64 * kStatsRec * 4, 1024);   // key-range partials of layer_stats
   p.ws_bytes = o;
   return SCALEKV_OK;
@@ -199,6 +200,7 @@ struct scalekv_ctx {
   long long host_steps = 0;
   // layer_stats only: the sums arrive in page-locked memory of the library's own (host, created at the first call)
   double *stats_host = nullptr, *stats_host_dev = nullptr;
+  size_t stats_host_doubles = 0;
   const void *stage_ptr = nullptr; // the staging area of the last step and the size of its halves
   size_t stage_half = 0;
   std::vector<int> page_table_host;
@@ -1052,14 +1054,18 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   const bool tensor = ctx->dtype == SCALEKV_BF16 && topk_prime <= kTop &&
                       (size_t)p.n_slices * rows * mma_split * kStatsRec16 <= (size_t)kStatsMaxCtas * 64 * kStatsRec;
   const LayerView lv = layer_view(ctx, layer);
-  const double *sums;                                    // per slice: sums of c_i and t_i over the rows, length
+  const double *sums;      // sums of c_i and t_i over the rows and lengths: see the kernels
   std::vector<double> copied;
   if (tensor) {
-    if (!ctx->stats_host) {
-      CU(cudaHostAlloc(reinterpret_cast<void **>(&ctx->stats_host), acc_bytes, cudaHostAllocMapped));
+    const size_t need = (size_t)p.n_slices * (2 * row_blocks + 1);
+    if (ctx->stats_host_doubles < need) {      // (at the first call, sized for every row of the largest map)
+      const size_t most = (size_t)p.n_slices * (2 * ((p.n_max + 63) / 64) + 1);
+      CU(cudaHostAlloc(reinterpret_cast<void **>(&ctx->stats_host), most * sizeof(double), cudaHostAllocMapped));
       CU(cudaHostGetDevicePointer(reinterpret_cast<void **>(&ctx->stats_host_dev), ctx->stats_host, 0));
+      ctx->stats_host_doubles = most;
+      CU(cudaMemsetAsync(ctx->ws + p.off_count, 0, (size_t)p.n_slices * ((p.n_max + 63) / 64) * 4, ctx->s_main));
     }
-    // (programmatic launches: a kernel comes up while the one before it ends)
+    // (a programmatic launch: the kernel comes up while the one before it ends)
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1067,16 +1073,11 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.stream = ctx->s_main;
-    {
-      Scope sc(ctx, ctx->s_main, kOther);
-      cfg.gridDim = dim3(row_blocks, p.n_slices, mma_split);
-      cfg.blockDim = dim3(256);
-      CU(cudaLaunchKernelEx(&cfg, stats_mma_kernel, lv, tview(Q), nk, query_stride, rows, ctx->scale * 1.4426950408889634f, partial));
-    }
+    cfg.gridDim = dim3(row_blocks, p.n_slices, mma_split);
+    cfg.blockDim = dim3(256);
     Scope sc(ctx, ctx->s_main, kOther);
-    cfg.gridDim = dim3(p.n_slices);
-    cfg.blockDim = dim3(1024);
-    CU(cudaLaunchKernelEx(&cfg, stats_sum_kernel, lv, (const float *)partial, mma_split, rows, nk, topk_prime, ctx->stats_host_dev));
+    CU(cudaLaunchKernelEx(&cfg, stats_mma_kernel, lv, tview(Q), nk, query_stride, rows, topk_prime, ctx->scale * 1.4426950408889634f, partial,
+                          reinterpret_cast<int *>(ctx->ws + p.off_count), ctx->stats_host_dev));
     sums = ctx->stats_host;
     ctx->len_written[layer] = 1;
   } else {
@@ -1106,12 +1107,22 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   CU(cudaStreamSynchronize(ctx->s_main));
   double c_all = 0.0, t_all = 0.0;
   for (int s = 0; s < p.n_slices; ++s) {
-    c_all += sums[3 * s];
-    t_all += sums[3 * s + 1];
-    const double c_s = sums[3 * s] / rows, t_s = sums[3 * s + 1] / rows;
+    double c_sum = 0.0, t_sum = 0.0, len;
+    if (tensor) {
+      for (int i = 0; i < row_blocks; ++i) {
+        c_sum += sums[2 * ((size_t)s * row_blocks + i)];
+        t_sum += sums[2 * ((size_t)s * row_blocks + i) + 1];
+      }
+      len = sums[(size_t)2 * row_blocks * p.n_slices + s];
+    } else {
+      c_sum = sums[3 * s]; t_sum = sums[3 * s + 1]; len = sums[3 * s + 2];
+    }
+    c_all += c_sum;
+    t_all += t_sum;
+    const double c_s = c_sum / rows, t_s = t_sum / rows;
     if (car_slices) car_slices[s] = c_s;
     if (htk_slices) htk_slices[s] = t_s;
-    if (nca_slices) nca_slices[s] = c_s * sums[3 * s + 2] / (double)nk;
+    if (nca_slices) nca_slices[s] = c_s * len / (double)nk;
   }
   const double cnt = (double)rows * p.n_slices;
   *car = c_all / cnt;
