@@ -67,23 +67,21 @@ __global__ void commit_kernel(LayerView lv, int n_k) {
 
 // ------------------------------------------------------------------------------------------
 // attend, f32 x 64: O = softmax(scale * Q K^T) V with online softmax, fp32 FMA throughout (Eq. 5; the 1e-4 bound on outputs
-// rules TF32 out).  A CTA of 128 threads owns 64 query rows of one slice and streams its keys in tiles of 64; thread (ty, tx) owns
-// rows ty + 8 i and the keys (then the output columns) of tx, so that a warp only reads P that it has written itself.
-//   S  : keys tx + 16 j, packed multiply-adds over pairs of columns, operands as 16-byte loads from rows of 272 bytes: the
-//        two query rows of a warp's load are broadcasts and the 16 key rows meet no bank twice.
-//   P V: columns 4 tx .., packed over pairs of columns, P as 16-byte loads of four keys.
-// 12 loads feed 64 packed multiply-adds of 2 cycles each in both products, so the FMA pipe is what bounds them; K arrives
-// under P V and V under S (asynchronous copies, 70 KB of shared memory, three CTAs per SM to cover the barriers between).
-// 16 slices, us per launch averaged over four layers, 64/144/256/400/576/1024/1600 queries: 22.8/40.6/61/85/120/244/479 with 4 x 4
-// register tiles and scalar operands of P V, 15.9/18.7/26/54/92/188/365 here (FMA pipe 55 % busy: 2.3 warps per scheduler do
-// not cover the loads' latency, and the accumulators leave no registers for more).
-// Few CTAs: gridDim.z CTAs of a cluster share a slice's keys; each then combines a share of the rows,
+// rules TF32 out).  A CTA of 256 threads owns 128 query rows of one slice and streams its keys in tiles of 64; thread (ty, tx) owns
+// rows 8 ty .. 8 ty + 7 and keys, then output columns, 4 tx .. 4 tx + 3, all accumulators packed over pairs of rows.  Q, K and P
+// lie transposed in shared memory, so that both products read, per key column (per key), 8 rows and 4 keys (columns) with three
+// 16-byte loads for 16 packed multiply-adds of 2 cycles each: the FMA pipe bounds them.  Packing over the rows keeps the scores
+// in 32 registers (over columns they take 64), so that 16 warps of an SM cover the latencies.  K arrives (asynchronous
+// copies) under P V and is transposed from there, V arrives under S; a warp only reads P that it has written itself.
+// gridDim.z CTAs of a cluster share a slice's keys; each then combines a share of the rows,
 // O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e, reading the parts through distributed shared memory.
-// grid (ceil(n_k / 64), n_slices, split); dynamic shared memory kAttendF32Smem.
+// 16 slices, us per launch averaged over four layers, 64/144/256/400/576/1024/1600 queries: 22.8/40.6/61/85/120/244/479 with
+// 4 x 4 register tiles and scalar operands of P V, 15.3/18.8/26/54/93/187/363 with 64 rows per CTA packed over columns (FMA pipe
+// 55 % busy, 2.3 warps per scheduler), 17/21.6/29/51/84/169/330 here (68 %, shared-memory wavefronts 65 %).
+// grid (ceil(n_k / 128), n_slices, split); dynamic shared memory kAttendF32Smem (two CTAs per SM).
 // ------------------------------------------------------------------------------------------
-constexpr int kF32Ld = 68;                                  // floats per row of a tile
-constexpr int kF32Tile = 64 * kF32Ld;
-constexpr int kAttendF32Smem = (4 * kF32Tile + 2 * 64) * 4;
+constexpr int kF32Rows = 128;
+constexpr int kAttendF32Smem = (64 * kF32Rows + 3 * 64 * 64 + 64 * kF32Rows) * 4;
 constexpr int kF32MaxSplit = 8;
 
 __device__ __forceinline__ uint64_t pair_fma(uint64_t a, uint64_t b, uint64_t c) {
@@ -107,119 +105,139 @@ __device__ __forceinline__ float2 pair_parts(uint64_t v) {
   return r;
 }
 
-__global__ void __launch_bounds__(128, 3) attend_f32_kernel(LayerView lv, TensorView Q, TensorView O, float *lse, int n_k, float scale_log2e) {
+__global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, TensorView Q, TensorView O, float *lse, int n_k, float scale_log2e) {
   extern __shared__ __align__(16) float sm_f32[];
-  float *Qs = sm_f32, *Ks = Qs + kF32Tile, *Vs = Ks + kF32Tile, *Ps = Vs + kF32Tile;
-  float *m_s = Ps + kF32Tile, *l_s = m_s + 64;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  float *Qt = sm_f32;                     // [column][row]
+  float *Kt = Qt + 64 * kF32Rows;         // [column][key]
+  float *Kr = Kt + 64 * 64;               // [key][column], as it arrives; chunks permuted by the key
+  float *Vs = Kr + 64 * 64;               // [key][column]
+  float *Pt = Vs + 64 * 64;               // [key][row], chunks permuted by the key
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ty = tid >> 4, tx = tid & 15;
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
-  const int q0 = blockIdx.x * 64;
+  const int q0 = blockIdx.x * kF32Rows;
   const int L = lv.hist_len[slice] + n_k;
   if (blockIdx.x == 0 && blockIdx.z == 0 && tid == 0) lv.next_len[slice] = L;     // unless a compress of this scale evicts
   const int n_split = gridDim.z, tiles = (L + 63) >> 6;
   const int t_lo = tiles * (int)blockIdx.z / n_split, t_hi = tiles * ((int)blockIdx.z + 1) / n_split;
-  auto fetch = [&](float *tile, const char *pool, int t) {
+  auto fetch = [&](float *tile, const char *pool, int t, bool permute) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int r = u * 8 + (tid >> 4), c = tid & 15, slot = t * 64 + r;
-      float *dst = tile + r * kF32Ld + c * 4;
+    for (int u = 0; u < 4; ++u) {
+      const int r = u * 16 + ty, slot = t * 64 + r;
+      float *dst = tile + r * 64 + (permute ? tx ^ (r & 7) : tx) * 4;
       if (slot < L)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-                     "l"(pool + slot_row(lv, slice, slot) * 256 + c * 16)
+                     "l"(pool + slot_row(lv, slice, slot) * 256 + tx * 16)
                      : "memory");
       else
         *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (t_lo < t_hi) fetch(Ks, lv.k_pool, t_lo);
+  if (t_lo < t_hi) fetch(Kr, lv.k_pool, t_lo, true);
+  // Q: a warp transposes 32 rows, four columns at a time
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
-    const int r = u * 8 + (tid >> 4), c = tid & 15;
+    const int r = (warp & 3) * 32 + lane, c = (warp >> 2) * 8 + u;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (q0 + r < n_k) v = reinterpret_cast<const float4 *>(row_ptr<float>(Q, b, h, q0 + r))[c];
-    *reinterpret_cast<float4 *>(Qs + r * kF32Ld + c * 4) = v;
+    Qt[(4 * c + 0) * kF32Rows + r] = v.x;
+    Qt[(4 * c + 1) * kF32Rows + r] = v.y;
+    Qt[(4 * c + 2) * kF32Rows + r] = v.z;
+    Qt[(4 * c + 3) * kF32Rows + r] = v.w;
   }
-  uint64_t o[8][2];
+  uint64_t o[4][4];                       // [pair of rows][column]
   float m[8], l[8];                       // l: this thread's keys only
 #pragma unroll
-  for (int i = 0; i < 8; ++i) { o[i][0] = o[i][1] = 0ull; m[i] = -1e30f; l[i] = 0.f; }
-  const float *qrow = Qs + ty * kF32Ld, *krow = Ks + tx * kF32Ld, *vcol = Vs + tx * 4;
-  float *prow = Ps + ty * kF32Ld;
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[i][j] = 0ull;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { m[i] = -1e30f; l[i] = 0.f; }
+  // one step of either product: 8 rows (two 16-byte loads) times 4 keys or columns
+  auto step = [&](uint64_t (&acc)[4][4], const float *a0, const float *a1, const float *bv) {
+    const ulonglong2 r0 = *reinterpret_cast<const ulonglong2 *>(a0), r1 = *reinterpret_cast<const ulonglong2 *>(a1);
+    const float4 x = *reinterpret_cast<const float4 *>(bv);
+    const uint64_t rows[4] = {r0.x, r0.y, r1.x, r1.y};
+    const uint64_t cols[4] = {pair_of(x.x, x.x), pair_of(x.y, x.y), pair_of(x.z, x.z), pair_of(x.w, x.w)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = pair_fma(rows[i], cols[j], acc[i][j]);
+  };
 
   for (int t = t_lo; t < t_hi; ++t) {
-    fetch(Vs, lv.v_pool, t);
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();                      // K of this tile (and at first Q) is there
-    uint64_t s2[8][4];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                      // K has arrived (and V has been read)
+    fetch(Vs, lv.v_pool, t, false);
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int u = 0; u < 4; ++u) {         // a warp transposes 32 keys, four columns at a time
+      const int r = (warp & 1) * 32 + lane, c = (warp >> 1) * 4 + u;
+      const float4 v = *reinterpret_cast<const float4 *>(Kr + r * 64 + (c ^ (r & 7)) * 4);
+      Kt[(4 * c + 0) * 64 + r] = v.x;
+      Kt[(4 * c + 1) * 64 + r] = v.y;
+      Kt[(4 * c + 2) * 64 + r] = v.z;
+      Kt[(4 * c + 3) * 64 + r] = v.w;
+    }
+    __syncthreads();
+    if (t + 1 < t_hi) fetch(Kr, lv.k_pool, t + 1, true); else asm volatile("cp.async.commit_group;" ::: "memory");
+    uint64_t s2[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) s2[i][j] = 0ull;
 #pragma unroll 4
-    for (int c = 0; c < 64; c += 4) {
-      ulonglong2 k[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const ulonglong2 *>(krow + 16 * j * kF32Ld + c);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(qrow + 8 * i * kF32Ld + c);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s2[i][j] = pair_fma(q.x, k[j].x, s2[i][j]);
-          s2[i][j] = pair_fma(q.y, k[j].y, s2[i][j]);
-        }
-      }
-    }
-    __syncthreads();                      // everybody has read K
-    if (t + 1 < t_hi) fetch(Ks, lv.k_pool, t + 1); else asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int c = 0; c < 64; ++c) step(s2, Qt + c * kF32Rows + ty * 8, Qt + c * kF32Rows + ty * 8 + 4, Kt + c * 64 + tx * 4);
     const int valid = L - t * 64;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      float y[4], mx = m[i];
+    for (int i = 0; i < 4; ++i) {
+      float y[2][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float2 e = pair_parts(s2[i][j]);
-        y[j] = tx + 16 * j < valid ? (e.x + e.y) * scale_log2e : -INFINITY;
-        mx = fmaxf(mx, y[j]);
+        const bool real = tx * 4 + j < valid;
+        y[0][j] = real ? e.x * scale_log2e : -INFINITY;
+        y[1][j] = real ? e.y * scale_log2e : -INFINITY;
       }
+      float f[2];
 #pragma unroll
-      for (int d = 8; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-      const float f = exp2f(m[i] - mx);
-      m[i] = mx;
-      l[i] *= f;
-      const uint64_t ff = pair_of(f, f);
-      o[i][0] = pair_mul(o[i][0], ff);
-      o[i][1] = pair_mul(o[i][1], ff);
+      for (int r = 0; r < 2; ++r) {
+        const int q = 2 * i + r;
+        float mx = fmaxf(fmaxf(y[r][0], y[r][1]), fmaxf(y[r][2], y[r][3]));
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+        mx = fmaxf(mx, m[q]);
+        f[r] = exp2f(m[q] - mx);
+        m[q] = mx;
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          y[r][j] = exp2f(y[r][j] - mx);
+          sum += y[r][j];
+        }
+        l[q] = l[q] * f[r] + sum;
+      }
+      const uint64_t ff = pair_of(f[0], f[1]);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float p = exp2f(y[j] - mx);
-        l[i] += p;
-        prow[8 * i * kF32Ld + tx + 16 * j] = p;
+        o[i][j] = pair_mul(o[i][j], ff);
+        s2[i][j] = pair_of(y[0][j], y[1][j]);
       }
     }
+    // P of key 4 tx + j: rows 8 ty .. as two chunks, permuted by the key's group of four
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int half = 0; half < 2; ++half)
+        *reinterpret_cast<ulonglong2 *>(Pt + (tx * 4 + j) * kF32Rows + ((ty * 2 + half) ^ (tx & 7)) * 4) =
+            make_ulonglong2(s2[2 * half][j], s2[2 * half + 1][j]);
     asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();                      // V is there (and P, which only this warp reads)
+    __syncthreads();                      // V has arrived
 #pragma unroll 4
-    for (int c = 0; c < 64; c += 4) {
-      ulonglong2 v[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = *reinterpret_cast<const ulonglong2 *>(vcol + (c + e) * kF32Ld);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 p = *reinterpret_cast<const float4 *>(prow + 8 * i * kF32Ld + c);
-        const uint64_t p0 = pair_of(p.x, p.x), p1 = pair_of(p.y, p.y), p2 = pair_of(p.z, p.z), p3 = pair_of(p.w, p.w);
-        o[i][0] = pair_fma(p0, v[0].x, o[i][0]);
-        o[i][1] = pair_fma(p0, v[0].y, o[i][1]);
-        o[i][0] = pair_fma(p1, v[1].x, o[i][0]);
-        o[i][1] = pair_fma(p1, v[1].y, o[i][1]);
-        o[i][0] = pair_fma(p2, v[2].x, o[i][0]);
-        o[i][1] = pair_fma(p2, v[2].y, o[i][1]);
-        o[i][0] = pair_fma(p3, v[3].x, o[i][0]);
-        o[i][1] = pair_fma(p3, v[3].y, o[i][1]);
-      }
+    for (int k = 0; k < 64; ++k) {
+      const float *p = Pt + k * kF32Rows;
+      const int x = (k >> 2) & 7;
+      step(o, p + ((ty * 2) ^ x) * 4, p + ((ty * 2 + 1) ^ x) * 4, Vs + k * 64 + tx * 4);
     }
-    __syncthreads();                      // everybody has read V
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i)
@@ -229,19 +247,33 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(LayerView lv, Tensor
   if (n_split == 1) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int r = q0 + ty + 8 * i;
+      const int r = q0 + ty * 8 + i;
       if (r >= n_k) continue;
       const float inv = 1.f / l[i];
-      const float2 x = pair_parts(o[i][0]), y = pair_parts(o[i][1]);
-      *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, r)) + tx * 4) = make_float4(x.x * inv, x.y * inv, y.x * inv, y.y * inv);
+      float x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 e = pair_parts(o[i >> 1][j]);
+        x[j] = ((i & 1) ? e.y : e.x) * inv;
+      }
+      *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, r)) + tx * 4) = make_float4(x[0], x[1], x[2], x[3]);
       if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + r] = (m[i] + log2f(l[i])) * 0.6931471805599453f;
     }
     return;
   }
+  // the parts: rows of 64 columns where Q was, references and sums where K was
+  __syncthreads();
+  float *part = Qt, *m_s = Kt, *l_s = Kt + kF32Rows;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    *reinterpret_cast<ulonglong2 *>(prow + 8 * i * kF32Ld + tx * 4) = make_ulonglong2(o[i][0], o[i][1]);
-    if (tx == 0) { m_s[ty + 8 * i] = m[i]; l_s[ty + 8 * i] = l[i]; }
+    float x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 e = pair_parts(o[i >> 1][j]);
+      x[j] = (i & 1) ? e.y : e.x;
+    }
+    *reinterpret_cast<float4 *>(part + (ty * 8 + i) * 64 + tx * 4) = make_float4(x[0], x[1], x[2], x[3]);
+    if (tx == 0) { m_s[ty * 8 + i] = m[i]; l_s[ty * 8 + i] = l[i]; }
   }
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
@@ -250,8 +282,9 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(LayerView lv, Tensor
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(cta));
     return ra;
   };
-  const int r_lo = 64 * (int)blockIdx.z / n_split, r_hi = min(64 * ((int)blockIdx.z + 1) / n_split, n_k - q0);
-  for (int r = r_lo + ty; r < r_hi; r += 8) {
+  const int rows = min(kF32Rows, n_k - q0);
+  const int r_lo = rows * (int)blockIdx.z / n_split, r_hi = rows * ((int)blockIdx.z + 1) / n_split;
+  for (int r = r_lo + ty; r < r_hi; r += 16) {
     float4 x[kF32MaxSplit];
     float me[kF32MaxSplit], le[kF32MaxSplit], M = -1e30f;
 #pragma unroll
@@ -262,7 +295,7 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(LayerView lv, Tensor
         asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(me[e]) : "r"(peer(m_s + r, e)));
         asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(le[e]) : "r"(peer(l_s + r, e)));
         asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[e].x), "=f"(x[e].y), "=f"(x[e].z), "=f"(x[e].w)
-                     : "r"(peer(Ps + r * kF32Ld + tx * 4, e)));
+                     : "r"(peer(part + r * 64 + tx * 4, e)));
       }
     }
 #pragma unroll

@@ -670,13 +670,16 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       ctx->logits_of[layer] = wl ? k : -1;
       ctx->logits_padded[layer] = fused ? 1 : 0;
     } else {
-      // CTAs that share a slice's keys: as many as fit beside each other (three per SM) and find a tile each
-      const int ctas = (nk + 63) / 64 * p.n_slices, tiles = (ctx->hist[layer] + nk + 63) / 64;
-      const int split = std::max(1, std::min({kF32MaxSplit, 3 * ctx->n_sm / ctas, tiles}));
+      // CTAs that share a slice's keys: so that the SM with the most work has as little of it as possible
+      const int blocks = (nk + kF32Rows - 1) / kF32Rows, ctas = blocks * p.n_slices, tiles = (ctx->hist[layer] + nk + 63) / 64;
+      int split = 1;
+      auto load = [&](int c) { return (float)((ctas * c + ctx->n_sm - 1) / ctx->n_sm) * ((float)((tiles + c - 1) / c) + 1.5f); };   // in key tiles; a CTA costs 1.5 more
+      for (int c = 2; c <= kF32MaxSplit && c <= tiles; ++c)
+        if (load(c) < load(split)) split = c;
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[1];
-      cfg.gridDim = dim3((nk + 63) / 64, p.n_slices, split);
-      cfg.blockDim = dim3(128);
+      cfg.gridDim = dim3(blocks, p.n_slices, split);
+      cfg.blockDim = dim3(256);
       cfg.dynamicSmemBytes = kAttendF32Smem;
       cfg.stream = ctx->s_main;
       attr[0].id = cudaLaunchAttributeClusterDimension;
