@@ -648,8 +648,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   // What needs no global memory comes first: the lanes of warp 0 initialise one barrier each, warp 1 allocates the
   // TMEM, warp 2 fetches the tensor maps' descriptors.  When the launch allows it (programmatic stream serialisation) this part runs while the kernel before this
   // one in the stream is still finishing; `griddepcontrol.wait` then holds every thread until that kernel's writes
-  // - cache lengths, page tables, pages, the status word - are visible.  The grid behind this one may come up as
-  // soon as all of this grid's CTAs are running.
+  // - cache lengths, page tables, pages, the status word - are visible.  (The grid behind this one comes up when every
+  // CTA of this grid has issued its last products: see there.)
   if (warp == 0) {
     if (lane < bCount) {
       // arrivals per phase: a ring stage is released by the MMA warp's commit and the two append warps; P and early P
@@ -667,7 +667,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const CUtensorMap *tm = lane == 0 ? &tmQ : (lane == 1 ? &tmKc : (lane == 2 ? &tmVc : (lane == 3 ? &tmK : &tmV)));
     asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const bool fused = prm.fused_append != 0;
   int *status = lv.status;
@@ -851,6 +850,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         __syncwarp();
       }
     }
+    // Now the next grid of the stream may come up: its set-up runs under this grid's epilogues.  Not earlier: its CTAs
+    // would sit and wait on every SM that this grid leaves free, and the compress of the layer before, on the other stream,
+    // would find none (a graph of 32 layers with compresses, us per layer and step, trigger at the start -> here: 16 slices
+    // x 576 / 784 / 1024 queries 36.8 -> 26.7, 54.1 -> 46.6, 77.7 -> 71.0, without any compress work 24.6, 46.8, 57.1).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (n_split > 1) cluster_arrive();
   } else {
     // ------------------------------------------------------------------ append (warps 2 and 3)

@@ -847,11 +847,10 @@ __global__ void __launch_bounds__(256) compact_kernel(LayerView lv, const int *k
 // ext.on: the current map has not been copied into the pages (a one-call step whose attend left it in the caller's
 // tensors): entries hist .. L-1 are rows of those tensors, phase 3 reads the survivors among them there and every kept
 // row of the map is written, whatever its index.
-// Few slices: the gridDim.y CTAs of a cluster find the same keep list and move a share of every row's columns each.
 // What bounds it: for short keep lists the latency of the phases, which 512 threads (so that two slices can share an SM) and
 // fewer rounds of barriers cut; for long ones the memory system: an SM stores 32 bytes per cycle (17 cycles per row, 22
 // measured for loads and stores of 16 slices), and 128 slices at once move at the HBM's rate (42 cycles per row = 5.9 TB/s).
-// Dynamic shared memory: 4 * (2 * ld_s + pages_per_slice) bytes.  grid (n_slices, shares).
+// Dynamic shared memory: 4 * (2 * ld_s + pages_per_slice) bytes.  grid (n_slices).
 // ------------------------------------------------------------------------------------------
 constexpr int kCompressThreads = 512;
 
@@ -869,7 +868,6 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   __shared__ float lse_row[kMaxWindow];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int slice = blockIdx.x;
-  const int share = blockIdx.y, shares = gridDim.y;
   const int w = wa.w;
   const int dev_status = *reinterpret_cast<volatile int *>(lv.status);      // (all of this is under way before any of it is needed)
   const int hist = *reinterpret_cast<volatile int *>(lv.hist_len + slice);
@@ -914,7 +912,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
         const int i = col < hist ? col : (col >= map_col && col < cols ? col - map_col + hist : -1);   // (the padding between them is nobody's)
         if (i >= 0) {
           const float sc = (e == 0 ? s0 : s1) * inv_w;
-          if (share == 0) sc_out[i] = sc;
+          sc_out[i] = sc;
           key[i] = __float_as_uint(sc) & 0x7FFFFFFFu;
         }
       }
@@ -934,10 +932,6 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
     }
   }
   __syncthreads();
-  if (shares > 1) {                            // positions of this slice are read above and written below, by different CTAs
-    asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-  }
 
   // ---- phase 2: selection
   int want;
@@ -955,18 +949,16 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
     if (list[mid] == mid) lo = mid + 1; else hi = mid;
   }
   if (ext.on && lo > hist) lo = hist;          // kept rows of the current map are not where they belong yet, whatever their index
-  const int pieces = 32 / shares;              // of a row's 32 16-byte pieces (16 of K, 16 of V); the lanes of a warp take `shares` rows
-  const int piece = share * pieces + lane % pieces;
+  const int piece = lane;                      // of a row's 32 16-byte pieces (16 of K, 16 of V)
   const char *ext_ptr = (piece < 16 ? ext.k : ext.v) + (piece & 15) * 16;
   char *pool_ptr = (piece < 16 ? lv.k_pool : lv.v_pool) + (piece & 15) * 16;
-  const int r_in = wid * shares + lane / pieces, r_step = NT / 32 * shares;
-  const int C = 8 * r_step;                    // rows per chunk, at most one per thread
+  constexpr int kRows = NT / 32, C = 8 * kRows;  // rows per chunk, at most one per thread
   for (int c0 = lo; c0 < kept; c0 += C) {
     uint4 buf[8];
     int pos = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int j = c0 + r_in + u * r_step;
+      const int j = c0 + wid + u * kRows;
       if (j < kept) {
         const int src = list[j];
         const char *from = ext.on && src >= hist ? ext_ptr + (ext_base + (long long)(src - hist) * ext.st) * ext.esize
@@ -975,7 +967,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
       }
     }
     const int jp = c0 + tid;
-    const bool has_pos = share == 0 && tid < C && jp < kept;
+    const bool has_pos = tid < C && jp < kept;
     if (has_pos) {
       const int src = list[jp];
       pos = ext.on && src >= hist ? wa.n_prev + (src - hist) : lv.pos_pool[row_of(src)];
@@ -983,12 +975,12 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int j = c0 + r_in + u * r_step;
+      const int j = c0 + wid + u * kRows;
       if (j < kept) *reinterpret_cast<uint4 *>(pool_ptr + row_of(j) * 256) = buf[u];
     }
     if (has_pos) lv.pos_pool[row_of(jp)] = pos;
   }
-  if (tid == 0 && share == 0) {
+  if (tid == 0) {
     lv.next_len[slice] = kept;
     kept_count[slice] = kept;
   }

@@ -855,23 +855,13 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
         ext.on = 1; ext.k = kc.ptr; ext.v = vc.ptr; ext.sb = kc.sb; ext.sh = kc.sh; ext.st = kc.st; ext.esize = p.esize;
         if (vc.sb != kc.sb || vc.sh != kc.sh || vc.st != kc.st) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "K and V of a map must have the same strides");
       }
-      // Few slices leave most SMs idle: then a cluster of two CTAs moves a slice (16 slices, 1 944 of 4 248 entries kept: 35 -> 25 us).
-      // Not more of them, and not for more slices: every CTA keeps an attention CTA of the layers that follow off its SM
-      // (pass of one image, 32 layers, called layer by layer: 13.3 ms with one CTA per slice, 13.5 with two, 13.8 with four;
-      // replayed from a graph 12.7, 12.6, 12.5; 32 slices: 3.51 ms against 3.71 with four).
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute attr[1];
-      const unsigned shares = p.n_slices <= 16 ? 2 : 1;
-      cfg.gridDim = dim3(p.n_slices, shares);
-      cfg.blockDim = dim3(kCompressThreads);
-      cfg.dynamicSmemBytes = ctx->fused_smem;
-      cfg.stream = s;
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = shares; attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = shares > 1 ? 1 : 0;
-      CU(cudaLaunchKernelEx(&cfg, compress_fused_kernel, lv, wa, recent ? 1 : 0, n_sink, (const float *)logits, (const float *)wlse, p.ld_l,
-                            logit_scale, tile_padded, budget, (const int *)slice_budget, pool, shift, scores, p.ld_s, kept, ext));
+      // One CTA per slice, however few the slices: every CTA keeps an attention CTA of the layers that follow off its SM,
+      // and a compress that is quicker alone is slower among them (16 slices, 1 944 of 4 248 entries kept, by one CTA, a
+      // cluster of two or of four: alone 35, 25, 20 us; a pass of one image, 32 layers, 13.31, 13.57, 13.87 ms called layer
+      // by layer, replayed from a graph 12.30, 12.47, 12.5).
+      compress_fused_kernel<<<p.n_slices, kCompressThreads, ctx->fused_smem, s>>>(lv, wa, recent ? 1 : 0, n_sink, logits, wlse, p.ld_l,
+                                                                                 logit_scale, tile_padded, budget, slice_budget, pool,
+                                                                                 shift, scores, p.ld_s, kept, ext);
       if (external) ctx->in_store[layer] = 1;
     } else {
       if (!recent) {

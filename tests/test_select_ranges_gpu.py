@@ -1,4 +1,4 @@
-"""The selection's histogram levels, its ranking and its ties, and the pruning by one CTA or a cluster per slice."""
+"""The selection's histogram levels, its ranking and its ties, and the pruning."""
 import pytest
 import torch
 
@@ -23,7 +23,7 @@ def levels_inputs(B, H, d, n, distinct, seed):
 
 
 @pytest.mark.parametrize("separate", [False, True])
-@pytest.mark.parametrize("heads", [1, 17])                 # a cluster of two CTAs per slice, one CTA per slice
+@pytest.mark.parametrize("heads", [1, 17])
 @pytest.mark.parametrize("distinct,budget", [
     (1, 1),        # all keys equal, more of them than there are threads: the last level runs out of bits
     (1, 700),
