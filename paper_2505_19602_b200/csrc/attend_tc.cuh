@@ -74,7 +74,7 @@ constexpr uint32_t kHalfBytes = kTileBytes / 2;  // 64 head-dim columns = one 12
 constexpr uint32_t kOffQ = 0;                    // two query tiles (the dynamic shared memory must start 1024-byte aligned)
 constexpr uint32_t kOffRing = kOffQ + 2 * kTileBytes;
 constexpr uint32_t kOffBar = kOffRing + kStages * kTileBytes;
-constexpr uint32_t kOffStat = kOffBar + 256;     // a shared single's rows: reference and sum of part A (then of both parts), of part B
+constexpr uint32_t kOffStat = kOffBar + 256;     // a shared single's rows: reference and sum of part A, of part B
 constexpr uint32_t kSmemBytes = kOffStat + 2 * 128 * 8;
 static_assert(kSmemBytes <= 232448, "more shared memory than a CTA can have");
 // barrier slots (8 bytes each): one full/empty pair per ring stage, one S/P/PV barrier per S buffer or query tile
@@ -187,6 +187,8 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm,
 }
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+// (orders nothing, and so does not wait for this thread's stores)
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
@@ -327,6 +329,11 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -444,8 +451,11 @@ struct Params {
   int win_pos[kMaxWindow];   // ascending raster indices of the window rows inside the current map
 };
 
+// a / b for 0 <= a < 256 and 0 < b <= 128 (the true quotient of a + 1/2 is 1 / 256 or more from any integer, the approximate
+// one a few units in the last place from the true one)
+__device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
 // rows that each CTA of a cluster finishes
-__device__ __forceinline__ int cluster_share(int n_k, int first_row, int n_split) { return (min(128, n_k - first_row) + n_split - 1) / n_split; }
+__device__ __forceinline__ int cluster_share(int n_k, int first_row, int n_split) { return small_div(min(128, n_k - first_row) + n_split - 1, n_split); }
 __device__ __forceinline__ uint32_t remote(uint32_t addr, int cta) {
   uint32_t ra;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(cta));
@@ -485,15 +495,18 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
       if (w0 + r < n_k) *reinterpret_cast<uint4 *>(out + i * prm.O.st * 16 + col * 2) = val;
     }
   };
+  auto window_rank = [&] {
+    int rank = -1;
+    if (window)
+      for (int e = 0; e < prm.w; ++e)
+        if (prm.win_pos[e] == w0 + lane) rank = e;
+    return rank;
+  };
   auto row_sums = [&](float mr, float lr) {              // what is kept of a row besides its output
     const float y = mr + log2f(lr);
     if (prm.lse != nullptr && w0 + lane < n_k) prm.lse[(size_t)slice * n_k + w0 + lane] = y * 0.6931471805599453f;
-    if (window) {
-      int rank = 0;
-      for (int e = 0; e < prm.w; ++e)
-        if (prm.win_pos[e] == w0 + lane) rank = e;
-      prm.win_lse[(size_t)slice * prm.w + rank] = y;
-    }
+    const int rank = window_rank();
+    if (rank >= 0) prm.win_lse[(size_t)slice * prm.w + rank] = y;
   };
   if (!shared) {
     if (have) {
@@ -513,106 +526,144 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
       row_sums(m, l);
     }
   } else {
-    // ---- the two parts of a shared single are merged: each warpgroup takes half of the columns and hands the other one
-    // its own values of the other half (fp32, 16-byte pieces of a row permuted by its index).  A row's pieces are read and
-    // written by the threads of that row alone.
-    asm volatile("bar.sync 2, 256;" ::: "memory");         // no product reads the query tile any more
-    const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256, theirs = base + kOffQ + (qt ^ 1) * kTileBytes + row * 256;
-#pragma unroll 1
-    for (int cc = 0; cc < 2; ++cc) {
-      float o[32];
-      if (have) { tc_ld32(o_addr + (qt ^ 1) * 64 + cc * 32, o); tc_wait_ld(); }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float x0 = have ? o[4 * i] : 0.f, x1 = have ? o[4 * i + 1] : 0.f, x2 = have ? o[4 * i + 2] : 0.f, x3 = have ? o[4 * i + 3] : 0.f;
-        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(theirs + (uint32_t)((cc * 8 + (i ^ (row & 7))) << 4)), "f"(x0), "f"(x1),
-                     "f"(x2), "f"(x3)
-                     : "memory");
-      }
-    }
+    // ---- the two parts of a shared single are merged, half of the columns by each warpgroup: the rows of both lie in the
+    // same TMEM lanes, so all that is handed over are the references and sums.  Here and in finish_cluster every instruction
+    // runs once or twice per launch, so the code is kept short and what a row needs alone is worked out before the rendezvous
+    // (with the parts handed over in shared memory, one row at a time per warp in finish_cluster and pushes of single pieces, a
+    // step of 16 slices x 144 / 256 / 400 / 576 queries took 13.7 / 14.3 / 16.9 / 19.1 us; now 10.7 / 11.3 / 14.4 / 18.4).
     if (!have) { m = -INFINITY; l = 0.f; }
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(base + kOffStat + (uint32_t)(qt * 128 + row) * 8), "f"(m), "f"(l) : "memory");
-    asm volatile("bar.sync 2, 256;" ::: "memory");
+    // of a cluster the rows' owner: it gets this CTA's merged part, unnormalised, with its reference and sum
+    const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(small_div(row, own_rows), n_split - 1);   // (rows beyond the map go nowhere)
+    const int at = (int)blockIdx.z * own_rows + row - owner * own_rows;      // and the row's place there
+    const uint32_t dst = n_split > 1 ? remote(base + kOffRing + (uint32_t)at * 512 + (uint32_t)qt * 256, owner) : 0;
+    const int rank = window_rank();
+    tc_fence_before();
+    asm volatile("bar.sync 2, 256;" ::: "memory");         // both accumulators are complete, no product reads the query tile any more
+    tc_fence_after();
     float m2, l2;
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(base + kOffStat + (uint32_t)((qt ^ 1) * 128 + row) * 8) : "memory");
     const float M = fmaxf(m, m2);
     float f1 = l > 0.f ? ex2(m - M) : 0.f, f2 = l2 > 0.f ? ex2(m2 - M) : 0.f;
     const float both = l * f1 + l2 * f2;
-    // of a cluster the rows' owner: it gets this CTA's merged part, unnormalised, with its reference and sum
-    const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(row / own_rows, n_split - 1);   // (rows beyond the map go nowhere)
-    uint32_t dst = 0;
-    if (n_split == 1) {
-      f1 /= both; f2 /= both;
-    } else {
-      cluster_wait();                                     // every CTA of the cluster is through with its ring
-      dst = remote(base + kOffRing + (uint32_t)((int)blockIdx.z * own_rows + row - owner * own_rows) * 512, owner);
-      if (qt == 0 && first_row + row < n_k)
-        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
-                         remote(base + kOffPartStat + (uint32_t)((int)blockIdx.z * own_rows + row - owner * own_rows) * 8, owner)),
-                     "f"(M), "f"(both)
-                     : "memory");
-    }
+    if (n_split == 1) { const float inv = 1.f / both; f1 *= inv; f2 *= inv; }
+    const bool none1 = !__any_sync(0xffffffffu, l > 0.f), none2 = !__any_sync(0xffffffffu, l2 > 0.f);   // a part without keys left garbage
+    const uint64_t ff1 = pack2(f1, f1), ff2 = pack2(f2, f2);
+    // (of a cluster) the warpgroup's half of the row, 16-byte pieces permuted by its index
+    const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256;
 #pragma unroll 1
     for (int cc = 0; cc < 2; ++cc) {
-      float o[32];
+      float o[32], other[32];
       uint32_t pk[16];
-      if (have) { tc_ld32(o_addr + qt * 64 + cc * 32, o); tc_wait_ld(); }
+      tc_ld32(o_addr + qt * 64 + cc * 32, o);
+      tc_ld32((qt == 0 ? o_addr + 128 : o_addr - 128) + qt * 64 + cc * 32, other);
+      tc_wait_ld();
+      if (none1) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        float x[4];
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
-                     : "r"(mine + (uint32_t)((cc * 8 + (i ^ (row & 7))) << 4)) : "memory");
+        for (int i = 0; i < 32; ++i) o[i] = 0.f;
+      }
+      if (none2) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x[e] = (have ? o[4 * i + e] * f1 : 0.f) + x[e] * f2;
-        pk[2 * i] = pack_bf16(x[0], x[1]);
-        pk[2 * i + 1] = pack_bf16(x[2], x[3]);
-        if (n_split > 1 && first_row + row < n_k)
-          asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(((qt * 16 + cc * 8 + i) ^ (row & 31)) << 4)),
-                       "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3])
-                       : "memory");
+        for (int i = 0; i < 32; ++i) other[i] = 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        unpack2(fma2(pack2(o[2 * i], o[2 * i + 1]), ff1, mul2(pack2(other[2 * i], other[2 * i + 1]), ff2)), o[2 * i], o[2 * i + 1]);
+        pk[i] = pack_bf16(o[2 * i], o[2 * i + 1]);
+      }
+      if (n_split > 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((cc * 8 + (i ^ (row & 7))) << 4)), "f"(o[4 * i]),
+                       "f"(o[4 * i + 1]), "f"(o[4 * i + 2]), "f"(o[4 * i + 3]) : "memory");
       }
       __syncwarp();
       if (n_split == 1) emit(pk, base + kOffQ + qt * kTileBytes + quarter * 8192 + cc * 128, qt * 64 + cc * 32);   // (where it has read)
     }
-    if (n_split == 1 && qt == 0) row_sums(M, both);
+    if (n_split > 1) {
+      // Off to the owners: 256 contiguous bytes (this warpgroup's half of a row) by 16 lanes at a time; stores of 16-byte
+      // pieces of 32 rows travel between SMs piece by piece.
+      cluster_wait();                                     // every CTA of the cluster is through with its ring
+      if (qt == 0 && first_row + row < n_k)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(remote(base + kOffPartStat + (uint32_t)at * 8, owner)), "f"(M), "f"(both)
+                     : "memory");
+      const int half = lane >> 4, p16 = lane & 15;
+#pragma unroll 8
+      for (int e = 0; e < 16; ++e) {
+        const int r = 2 * e + half;
+        const uint32_t to = __shfl_sync(0xffffffffu, dst, r) + (uint32_t)p16 * 16;
+        float4 x;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
+                     : "r"(mine + (uint32_t)((r - lane) * 256) + (uint32_t)((p16 ^ (r & 7)) << 4)) : "memory");
+        if (w0 + r < n_k)
+          asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(to), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
+      }
+      __syncwarp();
+      if (qt == 0)                                        // (for the row's owner to find after the cluster's barrier)
+        asm volatile("st.shared.s32 [%0], %1;" ::"r"(mine), "r"(rank) : "memory");
+    } else if (qt == 0) {
+      row_sums(M, both);
+    }
   }
 }
 
 // The end of a cluster's work: O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e with M the largest reference, for this CTA's
-// share of the rows, from the parts that the CTAs of the cluster have left here.  A warp takes a row at a time, a lane four
-// columns of it.
+// share of the rows, from the parts that the CTAs of the cluster have left here.  A warp takes four rows at a time, a lane
+// 16 columns of one.
 __device__ __forceinline__ void finish_cluster(const Params &prm, uint32_t base, int slice, int q_first, int n_split) {
   const int n_k = prm.n_k;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = prm.per_heads.div(slice), h = slice - b * prm.per_heads.d;
   const int own_rows = cluster_share(n_k, q_first, n_split), r_lo = (int)blockIdx.z * own_rows, r_hi = min(r_lo + own_rows, min(128, n_k - q_first));
   char *obase = const_cast<char *>(prm.O.ptr) + ((long long)b * prm.O.sb + (long long)h * prm.O.sh) * 2;
-  static_assert(kMaxWindow <= 64, "two window positions per lane");
-  const int wpos0 = prm.win_pos[lane] - q_first, wpos1 = prm.win_pos[lane + 32] - q_first;   // (unused ones are negative)
-#pragma unroll 2
-  for (int r = r_lo + warp; r < r_hi; r += kThreads / 32) {
-    const uint32_t src = base + kOffRing + (uint32_t)(r - r_lo) * 512 + (uint32_t)((lane ^ (r & 31)) << 4);
-    const uint32_t stat = base + kOffPartStat + (uint32_t)(r - r_lo) * 8;
-    float M = -INFINITY, sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 2
+  static_assert(kMaxSplit == 8, "eight lanes weigh the parts of a row");
+  const int sub = lane >> 3, part = lane & 7;
+#pragma unroll 1                                           // (code that runs once costs its fetching: no copies of it)
+  for (int r0 = r_lo + warp * 4; r0 < r_hi; r0 += kThreads / 8) {
+    const bool live = r0 + sub < r_hi;
+    const int r = live ? r0 + sub : r0, at = r - r_lo;
+    // lane e of a row weighs part e (a part without keys counts for nothing: it left zeros)
+    float m = -INFINITY, sum = 0.f;
+    if (part < n_split)
+      asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m), "=f"(sum) : "r"(base + kOffPartStat + (uint32_t)(part * own_rows + at) * 8));
+    float M = m;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float weight = sum > 0.f ? ex2(m - M) : 0.f;
+    sum *= weight;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    float a[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a[i] = 0.f;
+    const uint32_t src = base + kOffRing + (uint32_t)at * 512 + (uint32_t)part * 16;
+#pragma unroll 1
     for (int e = 0; e < n_split; ++e) {
-      float me, le;
-      float4 x;
-      asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(me), "=f"(le) : "r"(stat + (uint32_t)(e * own_rows) * 8));
-      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(src + (uint32_t)(e * own_rows) * 512));
-      if (le > 0.f) {                                     // (a part without keys counts for nothing)
-        const float top = fmaxf(M, me), f0 = ex2(M - top), f = ex2(me - top);
-        M = top;
-        sum = sum * f0 + le * f;
-        a0 = a0 * f0 + x.x * f; a1 = a1 * f0 + x.y * f; a2 = a2 * f0 + x.z * f; a3 = a3 * f0 + x.w * f;
+      const float f = __shfl_sync(0xffffffffu, weight, sub * 8 + e);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float4 x;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
+                     : "r"(src + (uint32_t)(e * own_rows) * 512 + i * 128));
+        a[4 * i] = fmaf(x.x, f, a[4 * i]); a[4 * i + 1] = fmaf(x.y, f, a[4 * i + 1]);
+        a[4 * i + 2] = fmaf(x.z, f, a[4 * i + 2]); a[4 * i + 3] = fmaf(x.w, f, a[4 * i + 3]);
       }
     }
-    const float inv = 1.f / sum;
-    const int qi = q_first + r;
-    *reinterpret_cast<uint2 *>(obase + (long long)qi * prm.O.st * 2 + lane * 8) = make_uint2(pack_bf16(a0 * inv, a1 * inv), pack_bf16(a2 * inv, a3 * inv));
-    const float y = M + log2f(sum);
-    if (prm.lse != nullptr && lane == 0) prm.lse[(size_t)slice * n_k + qi] = y * 0.6931471805599453f;
-    if (wpos0 == r || wpos1 == r) prm.win_lse[(size_t)slice * prm.w + lane + (wpos0 == r ? 0 : 32)] = y;
+    if (live) {
+      const float inv = 1.f / sum;
+      const int qi = q_first + r;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<uint2 *>(obase + (long long)qi * prm.O.st * 2 + part * 8 + i * 64) =
+            make_uint2(pack_bf16(a[4 * i] * inv, a[4 * i + 1] * inv), pack_bf16(a[4 * i + 2] * inv, a[4 * i + 3] * inv));
+      if (part == 0) {
+        const float y = M + log2f(sum);
+        if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + qi] = y * 0.6931471805599453f;
+        int rank;
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(rank) : "r"(base + kOffQ + (uint32_t)r * 256));
+        if ((unsigned)rank < (unsigned)prm.w) prm.win_lse[(size_t)slice * prm.w + rank] = y;
+      }
+    }
   }
 }
 
@@ -1052,7 +1103,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       // not do, a parity wait cannot tell phases two apart and this warp may be that far behind it
       ok = mbar_wait_warp(bar(bFinal + qt), 0, abort_flag, status);
     }
-    if (n_split > 1) cluster_arrive();                     // this CTA's ring is free (as far as this warp knows)
+    if (n_split > 1) cluster_arrive_relaxed();             // this CTA's ring is free (this warp has never touched it)
     tc_fence_after();
     finish_rows(prm, base, o_addr, item_slot[0], item_slot[1], qt, pair, shared, ok && steps > 0, n_split, m, l, kWindow && win_row != nullptr);
     tc_fence_before();
@@ -1090,8 +1141,8 @@ struct AttendTc {
 
   // How a launch is cut.  Measured on a B200 (148 SMs), us per launch, averaged over a layer with a long and three with a short
   // cache, against one CTA for every pair or odd tile, the odd ones by a single warpgroup:
-  //   16 slices, singles (split over clusters up to 400 queries): 256 / 400 / 576 / 1024 queries 22.0 -> 18.7, 26.8 -> 21.5,
-  //   30.3 -> 22.5, 37.3 -> 29.6;  below three key tiles neither sharing nor splitting pays (13-15 us either way);
+  //   16 slices, singles (split over clusters up to 400 queries): 256 / 400 / 576 / 1024 queries 22.0 -> 15.4, 26.8 -> 18.6,
+  //   30.3 -> 22.6, 37.3 -> 29.3;  below three key tiles neither sharing nor splitting pays (13-15 us either way);
   //   128 slices x 1024 queries (512 pairs, 3.5 waves), the last 68 pairs as 136 singles: 135 -> 122.
   // n_pair: items that are walked pair by pair; items: all of them; split: CTAs that share an item's keys.
   struct Cut { int n_pair, items, split; };
