@@ -78,7 +78,7 @@ constexpr uint32_t kOffStat = kOffBar + 256;     // a shared single's rows: refe
 constexpr uint32_t kSmemBytes = kOffStat + 2 * 128 * 8;
 static_assert(kSmemBytes <= 232448, "more shared memory than a CTA can have");
 // barrier slots (8 bytes each): one full/empty pair per ring stage, one S/P/PV barrier per S buffer or query tile
-enum { bQFull = 0, bFull = 1, bEmpty = bFull + kStages, bSFull = bEmpty + kStages, bPFull = bSFull + 2, bPvDone = bPFull + 2,
+enum { bQFull = 0, bFull = 2, bEmpty = bFull + kStages, bSFull = bEmpty + kStages, bPFull = bSFull + 2, bPvDone = bPFull + 2,
        bFinal = bPvDone + 2, bPEarly = bFinal + 2, bPvEarly = bPEarly + 2, bCount = bPvEarly + 2 };
 constexpr uint32_t kOffTmemSlot = 208;            // inside the barrier area, behind the barriers
 static_assert(bCount * 8 <= kOffTmemSlot, "barriers overlap the TMEM slot");
@@ -748,10 +748,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       const int len = *reinterpret_cast<volatile int *>(lv.hist_len + slice), st = *reinterpret_cast<volatile int *>(status);
       if (!(base & 1023u)) {
         const int nq = pair ? 2 : 1;
-        mbar_expect_tx(bar(bQFull), nq * kTileBytes);
-        for (int t = 0; t < nq; ++t) {
-          tma_load_4d(base + kOffQ + t * kTileBytes, &tmQ, 0, q_first + t * 128, h, b, bar(bQFull));
-          tma_load_4d(base + kOffQ + t * kTileBytes + kHalfBytes, &tmQ, 64, q_first + t * 128, h, b, bar(bQFull));
+        for (int t = 0; t < nq; ++t) {                     // (tile A's first product need not wait for B's queries)
+          mbar_expect_tx(bar(bQFull + t), kTileBytes);
+          tma_load_4d(base + kOffQ + t * kTileBytes, &tmQ, 0, q_first + t * 128, h, b, bar(bQFull + t));
+          tma_load_4d(base + kOffQ + t * kTileBytes + kHalfBytes, &tmQ, 64, q_first + t * 128, h, b, bar(bQFull + t));
           if (t == 0 && early > 0) load_map_tile(0, 0);
         }
       }
@@ -828,6 +828,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (!ok && !(base & 1023u)) {
       // this CTA gives up or has no keys: nothing may land in its shared memory once that is used for something else or gone
       mbar_drain(bar(bQFull), 0);
+      if (pair) mbar_drain(bar(bQFull + 1), 0);
       for (int k = t > kStages ? t - kStages : 0; k < t; ++k) mbar_drain(bar(bFull + k % kStages), (k / kStages) & 1);
     }
     if (n_split > 1) cluster_arrive();
@@ -857,10 +858,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                                    idesc_pv, 1u);
     };
     const int steps[2] = {n_steps(0), n_steps(1)};
-    bool ok = nt > 0 && mbar_wait_warp(bar(bQFull), 0, abort_flag, status);
+    bool ok = nt > 0;
     for (int qt = 0; qt < 2 && ok && steps[qt] > 0; ++qt) {
       const int kt = ring_k(0, qt);
-      ok = ring_full(kt);
+      ok = mbar_wait_warp(bar(bQFull + (pair ? qt : 0)), 0, abort_flag, status) && ring_full(kt);
       if (!ok) break;
       tc_fence_after();
       mma_s(k_desc(kt), qt);
