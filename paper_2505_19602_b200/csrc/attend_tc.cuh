@@ -789,8 +789,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     return rest < 128 ? rest : 128;
   };
   // A single's key tiles are shared by A and B - unless they are so few that the combination would cost more than it gives:
-  // then A takes them all.
-  const bool shared = !pair && (n_split > 1 || nt > 2);
+  // then A takes them all.  Two tiles are shared in small launches only (us per layer and step, 36 queries behind 21 entries,
+  // A alone / shared: 16 slices 7.6 / 6.7, 32 slices 8.2 / 7.4, 64 slices 9.0 / 8.8, 96 slices 9.5 / 10.4, 128 slices 10.6 / 10.9).
+  const bool shared = !pair && (n_split > 1 || nt > (gridDim.x <= 64 ? 1 : 2));
   // key tiles that the softmax of tile A / B sees
   auto n_steps = [&](int qt) { return shared ? (nt + 1 - qt) >> 1 : (pair || qt == 0 ? nt : 0); };
   const uint32_t tmem = warp == 0 ? 0u : *tmem_slot;
@@ -1143,7 +1144,7 @@ struct AttendTc {
   // How a launch is cut.  Measured on a B200 (148 SMs), us per launch, averaged over a layer with a long and three with a short
   // cache, against one CTA for every pair or odd tile, the odd ones by a single warpgroup:
   //   16 slices, singles (split over clusters up to 400 queries): 256 / 400 / 576 / 1024 queries 22.0 -> 15.4, 26.8 -> 18.6,
-  //   30.3 -> 22.6, 37.3 -> 29.3;  below three key tiles neither sharing nor splitting pays (13-15 us either way);
+  //   30.3 -> 22.6, 37.3 -> 29.3;  two key tiles are not worth splitting;
   //   128 slices x 1024 queries (512 pairs, 3.5 waves), the last 68 pairs as 136 singles: 135 -> 122.
   // n_pair: items that are walked pair by pair; items: all of them; split: CTAs that share an item's keys.
   struct Cut { int n_pair, items, split; };

@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     (5, 15, (1, 18), 25),                  # 75 slices x 3 tiles: 150 items, one whole slice tile by tile
     (6, 16, (2, 20), 30),                  # 96 slices x 4 tiles: 192 pairs, the last 44 tile by tile
     (4, 16, (1, 8, 20), 30),               # 64 slices x 4 tiles: 128 pairs, no more than one wave
+    (4, 16, (2, 8, 11), -1),               # 64 single tiles with two key tiles: shared by the two warpgroups
+    (5, 13, (2, 8, 11), -1),               # 65: one warpgroup takes both
 ])
 def test_every_way_of_cutting_a_launch(batch, heads, sides, budget):
     n = orc.scale_token_counts(sides)
