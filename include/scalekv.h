@@ -161,7 +161,7 @@ scalekv_status scalekv_attend(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Q,
  *               ascending, identical for every slice.  NULL means the window is the whole current
  *               map (w = n_k; requires n_k <= SCALEKV_MAX_WINDOW and a dense Qw of n_k rows).
  * k^l is budgets[layer][scale] of the scale last appended.  If nothing can be evicted the call
- * only commits the lengths.  Runs on stream_side after this layer's attend. */
+ * changes nothing on the device.  Runs on stream_side after this layer's attend. */
 scalekv_status scalekv_compress(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Qw, int32_t w,
                                 const int32_t *window_pos, int32_t qw_is_full_map);
 

@@ -1,6 +1,5 @@
-// SIMT kernels of the ScaleKV hot path: append, fp32-FMA attention (the f32 x 64 configuration
-// and the reference path for bf16), observation-window scoring, segmented radix top-k, in-place
-// gather-compaction and the offline layer statistics.
+// Kernels of the ScaleKV hot path beside the tensor-core attention: append, fp32-FMA attention (the f32 x 64 configuration),
+// observation-window scoring, per-slice top-k, in-place gather-compaction and the offline layer statistics.
 #pragma once
 #include "common.cuh"
 
