@@ -826,12 +826,13 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     }
     if (!recorded) {
       // this writes the logit buffer of the layer's set: if another layer of that set has appended since, what
-      // its attend recorded there is lost (its compress scores from K too), and its attend must be through first
+      // its attends recorded there is lost (its compress scores from K too), and they must be through first - whatever state
+      // that layer is in by now: a compress that evicted nothing, or an append behind it, leaves an attend in flight
       const int ow = ctx->set_owner[layer % kSets];
       if (ow >= 0 && ow != layer) {
         ctx->logits_of[ow] = -1;
-        if (s != ctx->s_main && ctx->attended[ow]) {
-          if (!ctx->attend_marked[ow]) CU(cudaEventRecord(ctx->ev_attend[ow], ctx->s_main));
+        if (s != ctx->s_main) {
+          if (!ctx->attended[ow] || !ctx->attend_marked[ow]) CU(cudaEventRecord(ctx->ev_attend[ow], ctx->s_main));
           CU(cudaStreamWaitEvent(s, ctx->ev_attend[ow], 0));
         }
       }

@@ -40,3 +40,38 @@ def test_overlapped_compresses_change_nothing(layers, budget_of):
     for k in range(len(SIDES)):
         for l in range(layers):
             assert torch.equal(beside[k][l], alone[k][l]), (k, l)
+
+
+# Layers 0 and 4 share their logit buffer.  Layer 0 scores from K, into that buffer, because layer 4 has appended in between:
+# "kept": while the attend of layer 4, whose compress has evicted nothing, may still record there
+def _shared_buffer_pass(order, data, windows, sides, side_stream):
+    kv = binding.ScaleKV(5, 4, 16, 128, "bf16", sides, sides, [[5] * len(sides)] * 4 + [[-1] * len(sides)], page_tokens=4096,
+                         side_stream=side_stream)
+    out = []
+    torch.cuda.synchronize()
+    for k in range(len(sides)):
+        O = [torch.empty_like(Q) for Q, _, _ in data[k]]
+        append = lambda l: kv.scalekv_append(l, k, *data[k][l > 0][1:])
+        attend = lambda l: kv.scalekv_attend(l, data[k][l > 0][0], O[l > 0])
+        compress = lambda l: kv.scalekv_compress(l, data[k][l > 0][0], windows[k], qw_is_full_map=True)
+        append(0), attend(0), append(4)
+        if order == "kept":
+            attend(4), compress(4), compress(0)
+        out.append(O)
+    kv.scalekv_join()
+    kv.scalekv_sync()
+    kept = [kv.scalekv_export_slice(l, b, h) for l in (0, 4) for b in range(4) for h in range(16)]
+    kv.close()
+    return [o for O in out for o in O] + kept
+
+
+@pytest.mark.parametrize("order", ["kept"])
+def test_layers_that_share_a_logit_buffer_wait_for_each_other(order):
+    sides = (8, 32, 40)
+    gen = torch.Generator(device="cuda").manual_seed(29)
+    data = [[tuple(torch.randn(4, 16, a * a, 128, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+             for _ in range(2)] for a in sides]
+    windows = [orc.window_centroids(a, a, 16) for a in sides]
+    beside, alone = (_shared_buffer_pass(order, data, windows, sides, s) for s in (True, False))
+    for x, y in zip(beside, alone, strict=True):
+        assert torch.equal(x, y)
