@@ -229,6 +229,7 @@ struct scalekv_ctx {
   size_t fused_smem = 0;
   bool side_dirty = false;         // stream_side has work that stream_main has not joined yet
   int set_owner[kSets] = {-1, -1, -1, -1};   // layer that last appended into each transient page set / logit buffer
+  int set_compressed[kSets] = {-1, -1, -1, -1};   // layer whose compress on stream_side last used the set's logit buffer
   int64_t launches = 0;
   int scores_len = 0;              // length of the score vectors left by the last evicting compress
   bool profile = false;            // launches are bracketed by events
@@ -681,6 +682,13 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
                       ? nullptr
                       : reinterpret_cast<float *>(ctx->ws + p.off_logits) + (size_t)(layer % kSets) * p.logits_elems;
       float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
+      // What it records goes where a compress of another layer of the set may still score: append has waited for this layer's
+      // and the owner's compresses, not for one that was called behind it.
+      const int cl = ctx->set_compressed[layer % kSets];
+      if (wl && cl >= 0 && ctx->ev_compress_live[cl] && ctx->compress_no[cl] > ctx->main_behind) {
+        CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_compress[cl], 0));
+        ctx->main_behind = ctx->compress_no[cl];
+      }
       if (!ctx->tc.launch(lv, tview(Q), tview(O), lse, nk, fused ? &kc : nullptr, fused ? &vc : nullptr, fused && copy, ctx->hist[layer], p.N[k],
                           ctx->scale, wl, wlse, p.ld_l, win.data(), (int)win.size(), ctx->s_main, e))
         return fail(ctx, SCALEKV_ERR_CUDA, "attend launch: %s", e.c_str());
@@ -916,6 +924,7 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     ctx->ev_compress_live[layer] = 1;
     ctx->compress_no[layer] = ++ctx->side_compresses;
     ctx->layer_of_no[ctx->side_compresses % kSets] = layer;
+    ctx->set_compressed[layer % kSets] = layer;
   }
   return SCALEKV_OK;
 }

@@ -44,9 +44,10 @@ def test_overlapped_compresses_change_nothing(layers, budget_of):
 
 # Layers 0 and 4 share their logit buffer.  Layer 0 scores from K, into that buffer, because layer 4 has appended in between:
 # "kept": while the attend of layer 4, whose compress has evicted nothing, may still record there
+# "late": and layer 4 only attends then
 def _shared_buffer_pass(order, data, windows, sides, side_stream):
-    kv = binding.ScaleKV(5, 4, 16, 128, "bf16", sides, sides, [[5] * len(sides)] * 4 + [[-1] * len(sides)], page_tokens=4096,
-                         side_stream=side_stream)
+    budgets = [[5] * len(sides)] * 4 + [[-1 if order == "kept" else 5] * len(sides)]
+    kv = binding.ScaleKV(5, 4, 16, 128, "bf16", sides, sides, budgets, page_tokens=4096, side_stream=side_stream)
     out = []
     torch.cuda.synchronize()
     for k in range(len(sides)):
@@ -57,6 +58,8 @@ def _shared_buffer_pass(order, data, windows, sides, side_stream):
         append(0), attend(0), append(4)
         if order == "kept":
             attend(4), compress(4), compress(0)
+        else:
+            compress(0), attend(4), compress(4)
         out.append(O)
     kv.scalekv_join()
     kv.scalekv_sync()
@@ -65,7 +68,7 @@ def _shared_buffer_pass(order, data, windows, sides, side_stream):
     return [o for O in out for o in O] + kept
 
 
-@pytest.mark.parametrize("order", ["kept"])
+@pytest.mark.parametrize("order", ["kept", "late"])
 def test_layers_that_share_a_logit_buffer_wait_for_each_other(order):
     sides = (8, 32, 40)
     gen = torch.Generator(device="cuda").manual_seed(29)
