@@ -124,7 +124,7 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
       }
     }
   p.layers.resize(p.n_layers);
-  int trans_max = 0, len_max = 0;
+  int trans_max = 0, room = 0;
   size_t pt = 0;
   long long page = 0;
   for (int l = 0; l < p.n_layers; ++l) {
@@ -147,15 +147,18 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
     lp.first_page = (int)page;
     page += (long long)p.n_slices * lp.persist_pages;
     trans_max = std::max(trans_max, lp.total_pages - lp.persist_pages);
-    len_max = std::max(len_max, lp.max_len);
+    room = std::max(room, lp.total_pages * p.P);
   }
   p.trans_pages_per_slice = trans_max;
   for (int t = 0; t < kSets; ++t) { p.trans_first[t] = (int)page; page += (long long)p.n_slices * trans_max; }
   if (page > 0x7fffffffLL / p.P) { err = "store too large for 32-bit row indices"; return SCALEKV_ERR_CAPACITY; }
   p.n_pages = page;
   p.pt_elems = pt;
-  p.ld_s = (int)align_up((size_t)len_max, 64);
-  p.ld_l = (int)align_up((size_t)len_max + 256, 64);
+  // Keys, scores and keep lists have room for what a slice's pages hold, not only for the lengths that the budgets lead to: a scale
+  // whose compress was skipped, or sinks beyond the budget, make a slice longer than that, and append accepts it up to its pages.
+  // A logit row holds the history's and the map's tiles of 128, both rounded up.
+  p.ld_s = (int)align_up((size_t)room, 64);
+  p.ld_l = p.ld_s + 256;
   const size_t row_bytes = (size_t)p.d * p.esize;
   size_t o = 0;
   p.off_k = o; o = align_up(o + (size_t)p.n_pages * p.P * row_bytes, 1024);

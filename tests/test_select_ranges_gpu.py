@@ -59,3 +59,38 @@ def test_positional_rule_over_long_slices(budget, separate, heads):
     run.policy, run.n_sink, run.separate_kernels = "recent", 4, separate
     run.run()
     kv.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f32", 64)])
+@pytest.mark.parametrize("how", ["skipped", "sinks"])
+def test_slices_longer_than_their_budgets_lead_to(how, dtype, d):
+    """Pages hold more than the budgets' plan needs, and append accepts what they hold: the first scale is never compressed, or its
+    100 sinks outnumber the budget of 10."""
+    sides, page = (10, 11, 4), 512
+    n = orc.scale_token_counts(sides)
+    budgets = [[10] * len(sides)]
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator().manual_seed(41)
+    kv = binding.ScaleKV(1, 1, 2, d, dtype, sides, sides, budgets, page_tokens=page)
+    caches = [orc.SliceCache(n, d) for _ in range(2)]
+    for k, nk in enumerate(n):
+        Q, K, V = (torch.randn(1, 2, nk, d, generator=g).to(dt) for _ in range(3))
+        Qd, Kd, Vd = Q.cuda(), K.cuda(), V.cuda()
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, Kd, Vd)
+        O = kv.scalekv_attend(0, Qd)
+        window = orc.window_centroids(sides[k], sides[k], 16)
+        if k > 0:
+            kv.scalekv_compress(0, Qd, window, qw_is_full_map=True)
+        elif how == "sinks":
+            kv.scalekv_compress_ex(0, Qd, policy="recent", n_sink=100)      # all of them: nothing is evicted
+        kv.scalekv_sync()
+        for h in range(2):
+            c = caches[h]
+            c.append(K[0, h].double().numpy(), V[0, h].double().numpy())
+            want, _ = c.attend(Q[0, h].double().numpy())
+            assert abs(want - O[0, h].double().cpu().numpy()).max() <= (2e-2 if dtype == "bf16" else 1e-4)
+            if k > 0:
+                pos, _ = c.compress(Q[0, h].double().numpy()[window], window, budgets[0][k])
+                assert (kv.scalekv_export_slice(0, 0, h).numpy() == pos).all()
+    kv.close()
