@@ -36,10 +36,7 @@ __global__ void __launch_bounds__(256) append_kernel(LayerView lv, TensorView K,
   const int b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int ppr = lv.row_bytes >> 4;  // 16-byte pieces per row
   const int hist = lv.hist_len[slice];
-  if (hist + n_k > (lv.pages_per_slice << lv.page_shift)) {      // would outgrow the page table: report, do not fault
-    if (threadIdx.x == 0) atomicExch(lv.status, kDevCheck);
-    return;
-  }
+  if (outgrown(lv, hist + n_k)) return;
   const int rows_per_step = 256 / ppr;
   const int r_in = threadIdx.x / ppr, c = threadIdx.x % ppr;
   const int i0 = blockIdx.x * 64;
@@ -115,6 +112,7 @@ __global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, Tensor
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int q0 = blockIdx.x * kF32Rows;
   const int L = lv.hist_len[slice] + n_k;
+  if (outgrown(lv, L)) return;
   if (blockIdx.x == 0 && blockIdx.z == 0 && tid == 0) lv.next_len[slice] = L;     // unless a compress of this scale evicts
   const int n_split = gridDim.z, tiles = (L + 63) >> 6;
   const int t_lo = tiles * (int)blockIdx.z / n_split, t_hi = tiles * ((int)blockIdx.z + 1) / n_split;
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(256) score_logits_kernel(LayerView lv, TensorV
   const int b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int L = lv.hist_len[slice] + wa.n_k;
   const int j0 = blockIdx.x * 64;
-  if (j0 >= L) return;
+  if (outgrown(lv, L) || j0 >= L) return;
   for (int idx = tid; idx < 64 * CH; idx += 256) {
     const int r = idx / CH, c = idx % CH;
     float v[VN];
@@ -452,7 +450,7 @@ __global__ void __launch_bounds__(256) score_kernel(LayerView lv, WindowArg wa, 
   const int hist = lv.hist_len[slice];
   const int L = hist + wa.n_k;
   const int i = blockIdx.x * 256 + threadIdx.x;
-  if (blockIdx.x * 256 >= L) return;
+  if (outgrown(lv, L) || blockIdx.x * 256 >= L) return;
   const int w = wa.w;
   if (threadIdx.x < w) lse_row[threadIdx.x] = lse[(size_t)slice * w + threadIdx.x];
   __syncthreads();
@@ -486,7 +484,7 @@ __global__ void __launch_bounds__(256) head_mean_kernel(LayerView lv, WindowArg 
   const int L = lv.hist_len[s0] + wa.n_k;
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (blockIdx.x == 0 && threadIdx.x < H && lv.hist_len[s0 + threadIdx.x] + wa.n_k != L) atomicExch(lv.status, kDevCheck);
-  if (i >= L) return;
+  if (outgrown(lv, L) || i >= L) return;
   const int pos = lv.pos_pool[slot_row(lv, s0, i)];
   float sum = 0.f;
   bool same = true;
@@ -510,7 +508,7 @@ __global__ void __launch_bounds__(256) recent_keys_kernel(LayerView lv, int n_k,
   const int slice = blockIdx.y;
   const int L = lv.hist_len[slice] + n_k;
   const int i = blockIdx.x * 256 + threadIdx.x;
-  if (i >= L) return;
+  if (outgrown(lv, L) || i >= L) return;
   const int pos = lv.pos_pool[slot_row(lv, slice, i)];
   keys[(size_t)slice * ld_s + i] = pos < n_sink ? kWindowKey : (uint32_t)pos + 1u;
 }
@@ -523,6 +521,7 @@ __global__ void __launch_bounds__(1024) row_lse_kernel(LayerView lv, WindowArg w
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int slice = blockIdx.x;
   const int L = lv.hist_len[slice] + wa.n_k;
+  if (outgrown(lv, L)) return;
   const int w = wa.w;
   const float *y = logits + (size_t)slice * w * ld_l;
   for (int g0 = 0; g0 < w; g0 += 16) {
@@ -740,7 +739,7 @@ __global__ void __launch_bounds__(1024) select_kernel(LayerView lv, WindowArg wa
   const int slice = blockIdx.x;
   const int dev_status = *reinterpret_cast<volatile int *>(lv.status);   // both loads in flight before the test
   const int L = lv.hist_len[slice] + wa.n_k;
-  if (dev_status != 0) return;                 // an earlier kernel reported a failed check: leave the store alone
+  if (dev_status != 0 || outgrown(lv, L)) return;   // a failed check, an earlier kernel's or this one's: leave the store alone
   int *out = keep_list + (size_t)slice * ld_s;
   uint32_t *gkey = keys + (size_t)slice * ld_s;
   const float *sc = scores + (size_t)slice * ld_s;
@@ -873,8 +872,8 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   if (slice_budget != nullptr) budget = slice_budget[slice];
   for (int i = tid; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(lv.page_table + (size_t)slice * lv.pages_per_slice + i);
   if (policy == 0 && tid < w) lse_row[tid] = lse[(size_t)slice * w + tid];
-  if (dev_status != 0) return;                 // an earlier kernel reported a failed check: leave the store alone
   const int L = hist + wa.n_k;
+  if (dev_status != 0 || outgrown(lv, L)) return;   // a failed check, an earlier kernel's or this one's: leave the store alone
   __syncthreads();
   auto row_of = [&](int slot) { return ((size_t)pt[slot >> lv.page_shift] << lv.page_shift) + (size_t)(slot & lv.page_mask); };
   const long long ext_base = ext.on ? (long long)(slice / lv.n_heads) * ext.sb + (long long)(slice % lv.n_heads) * ext.sh : 0;
@@ -1041,6 +1040,7 @@ __global__ void __launch_bounds__(256) layer_stats_kernel(LayerView lv, TensorVi
   const int slice = blockIdx.y;
   const int b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int L = lv.hist_len[slice] + n_k;
+  if (outgrown(lv, L)) return;
   if (tid == 0 && blockIdx.x == 0 && blockIdx.z == 0) acc[3 * slice + 2] = (double)L;
   const int r0 = blockIdx.x * 64;
   const int Kp = topk_prime;
@@ -1308,6 +1308,10 @@ __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorV
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int hist = lv.hist_len[slice], L = hist + n_k;
+  if (outgrown(lv, L)) {
+    if (tid < 2) sums[((size_t)slice * gridDim.x + blockIdx.x) * 2 + tid] = NAN;      // (not what an earlier call left there)
+    return;
+  }
   const int r0 = blockIdx.x * 64;
   const int tiles = (L + 63) >> 6, n_split = gridDim.z;
   const int t_lo = (int)((long long)tiles * blockIdx.z / n_split), t_hi = (int)((long long)tiles * (blockIdx.z + 1) / n_split);

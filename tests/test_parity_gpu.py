@@ -723,6 +723,30 @@ def test_head_shared_importance_refuses_heads_that_diverged():
     kv.close()
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_calls_behind_a_refused_selection_stay_inside_the_store(dtype):
+    """The host goes on with the compressed lengths, the device with the uncompressed ones, which the next map's entries take beyond
+    the pages: every kernel that follows leaves instead of looking slots up there, and the error stands at the next sync."""
+    sides, heads, d = (2, 5, 9, 14), 3, 128 if dtype == "bf16" else 64
+    kv = binding.ScaleKV(1, 1, heads, d, dtype, sides, sides, [[10] * len(sides)], page_tokens=16)
+    g = torch.Generator(device="cuda").manual_seed(43)
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(1, heads, a * a, d, generator=g, device="cuda", dtype=kv.torch_dtype) for _ in range(3))
+        window = orc.window_centroids(a, a, 16)
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        kv.scalekv_attend(0, Q)
+        if k == 3:
+            kv.scalekv_layer_stats_ex(0, Q, 16, 1)
+            kv.scalekv_layer_stats_ex(0, Q, 20, 1)
+        # the heads part at scale 1; their common selection is refused at scale 2
+        kv.scalekv_compress_ex(0, Q, window, qw_is_full_map=True, head_shared=k == 2, separate_kernels=k == 3)
+    with pytest.raises(binding.ScaleKVError) as e:
+        kv.scalekv_sync()
+    assert e.value.status == binding.STATUS_NAMES.index("DEVICE_CHECK")
+    kv.close()
+
+
 @pytest.mark.parametrize("policy", ["score", "recent"])
 def test_per_head_budgets_leave_a_ragged_store(policy):
     """scalekv_compress_ex with head_budgets: every head prunes to its own budget (0 keeps only the
