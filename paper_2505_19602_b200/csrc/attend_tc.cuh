@@ -710,6 +710,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       mbar_init(bar(lane), four ? 4u : (three ? 3u : 1u));
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncwarp();                                        // lane 0 is about to use barriers that other lanes have initialised
   } else if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + kOffBar + kOffTmemSlot), "r"(kTmemCols)
                  : "memory");
