@@ -50,6 +50,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <map>
 #include <mutex>
@@ -1034,8 +1035,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       tc_wait_ld();
       if (kWindow && wwarp) { log_window(v[0], 0); log_window(v[1], 1); }
       if (j == 0) {
-        // no reference yet: the largest of the row's first 32 products serves (column 0 of the first tile
-        // always holds a key, so it is finite); a later chunk that exceeds the band raises it like any other
+        // no reference yet: the largest of the row's first 32 products serves; a later chunk that exceeds the band raises it
+        // like any other.  Where all 32 are -inf (masked keys) it is the lowest number: differences from it are numbers.
         float mt = -INFINITY;
 #pragma unroll
         for (int i = 0; i < 32; i += 2) {
@@ -1043,7 +1044,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           const float e1 = (i + 1 < valid) ? v[0][i + 1] : -INFINITY;
           mt = max3(mt, e0, e1);
         }
-        m = mt * c;
+        m = fmaxf(mt * c, -FLT_MAX);
       }
       front(v[0], valid, masked);
 #pragma unroll

@@ -35,3 +35,27 @@ def test_every_way_of_cutting_a_launch(batch, heads, sides, budget):
                       followed, compress_last=True)
         getattr(p, run)()
         kv.close()
+
+
+@pytest.mark.parametrize("batch,heads", [(1, 16), (4, 15), (8, 16)])      # clusters, singles, pairs
+@pytest.mark.parametrize("first", [0, 128, 256])                          # the masked keys open a tile of the map: every part's first
+def test_keys_masked_with_minus_infinity(first, batch, heads):
+    """32 keys at the head of a tile whose products are -inf: no weight, whichever part of the keys starts with them."""
+    sides, d = (8, 18), 128
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    kv = binding.ScaleKV(1, batch, heads, d, "bf16", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    keys, values = [], []
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(batch, heads, a * a, d, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+        Q[..., 0] = 1.0
+        if k == 1:
+            K[:, :, first: first + 32, 0] = -float("inf")
+        keys.append(K), values.append(V)
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        O = kv.scalekv_attend(0, Q)
+        kv.scalekv_sync()
+        S = Q.double() @ torch.cat(keys, 2).double().transpose(2, 3) / d ** 0.5
+        want = S.softmax(-1) @ torch.cat(values, 2).double()
+        assert (O.double() - want).abs().max().item() <= 2e-2
+    kv.close()
