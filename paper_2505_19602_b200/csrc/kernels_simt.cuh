@@ -1,6 +1,8 @@
 // Kernels of the ScaleKV hot path beside the tensor-core attention: append, fp32-FMA attention (the f32 x 64 configuration),
 // observation-window scoring, per-slice top-k, in-place gather-compaction and the offline layer statistics.
 #pragma once
+#include <cfloat>
+
 #include "common.cuh"
 
 namespace scalekv {
@@ -79,6 +81,7 @@ __global__ void commit_kernel(LayerView lv, int n_k) {
 constexpr int kF32Rows = 128;
 constexpr int kAttendF32Smem = (64 * kF32Rows + 3 * 64 * 64 + 64 * kF32Rows) * 4;
 constexpr int kF32MaxSplit = 8;
+constexpr float kNoMax = -FLT_MAX;       // a finite stand-in for -inf, so that differences of maxima are numbers; no finite score lies below
 
 __device__ __forceinline__ uint64_t pair_fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
@@ -149,7 +152,7 @@ __global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, Tensor
 #pragma unroll
     for (int j = 0; j < 4; ++j) o[i][j] = 0ull;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) { m[i] = -1e30f; l[i] = 0.f; }
+  for (int i = 0; i < 8; ++i) { m[i] = kNoMax; l[i] = 0.f; }
   // one step of either product: 8 rows (two 16-byte loads) times 4 keys or columns
   auto step = [&](uint64_t (&acc)[4][4], const float *a0, const float *a1, const float *bv) {
     const ulonglong2 r0 = *reinterpret_cast<const ulonglong2 *>(a0), r1 = *reinterpret_cast<const ulonglong2 *>(a1);
@@ -283,11 +286,11 @@ __global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, Tensor
   const int r_lo = rows * (int)blockIdx.z / n_split, r_hi = rows * ((int)blockIdx.z + 1) / n_split;
   for (int r = r_lo + ty; r < r_hi; r += 16) {
     float4 x[kF32MaxSplit];
-    float me[kF32MaxSplit], le[kF32MaxSplit], M = -1e30f;
+    float me[kF32MaxSplit], le[kF32MaxSplit], M = kNoMax;
 #pragma unroll
     for (int e = 0; e < kF32MaxSplit; ++e) {
       x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-      me[e] = -1e30f; le[e] = 0.f;
+      me[e] = kNoMax; le[e] = 0.f;
       if (e < n_split) {
         asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(me[e]) : "r"(peer(m_s + r, e)));
         asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(le[e]) : "r"(peer(l_s + r, e)));
@@ -1237,7 +1240,6 @@ __global__ void __launch_bounds__(64) layer_stats_merge_kernel(const float *part
 // grid (ceil(n_rows / 64), n_slices, n_split <= 16); static shared memory: two K tiles and the query tile.
 // ------------------------------------------------------------------------------------------
 constexpr int kTop = 16;
-constexpr float kNoMax = -1e30f;         // a finite stand-in for -inf, so that differences of maxima are numbers
 
 __device__ __forceinline__ float pow2(float x) {
   float y;

@@ -25,3 +25,23 @@ def test_f32_attention_matches_oracle(batch, heads, sides, budget):
                     sorted({(0, 0, 0), (0, batch - 1, heads - 1)}), compress_last=True).run()
     assert run.compared == len(sides) * len(run.slices)
     kv.close()
+
+
+@pytest.mark.parametrize("heads", [1, 40])             # keys shared by a cluster, and not
+def test_f32_rows_of_scores_near_the_lowest_number(heads):
+    """Every score near the type's lowest value: they differ by less than it resolves, so all keys weigh the same."""
+    sides = (3, 17)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    kv = binding.ScaleKV(1, 1, heads, 64, "f32", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    values = []
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(1, heads, a * a, 64, generator=g, device="cuda") for _ in range(3))
+        Q[..., 0], K[..., 0] = 1.0, -3e38
+        values.append(V)
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        O = kv.scalekv_attend(0, Q)
+        kv.scalekv_sync()
+        want = torch.cat(values, 2).mean(2, keepdim=True)
+        assert (O - want).abs().max().item() <= 1e-5
+    kv.close()

@@ -45,3 +45,20 @@ def test_statistics_match_the_oracle(heads, topk, stride, sides):
         assert abs(car - np.mean(want_c)) <= 1e-4 * abs(car) and abs(htk - np.mean(want_t)) <= 1e-4 * abs(htk) + 1e-7
         assert kv.scalekv_lengths(0) == [[sum(n[:k + 1])] * heads]
     kv.close()
+
+
+def test_rows_of_scores_near_the_lowest_number():
+    """Every score near the type's lowest value: they differ by less than it resolves, so all entries weigh the same."""
+    sides, heads, d, topk = (4, 9), 3, 128, 16
+    n = orc.scale_token_counts(sides)
+    g = torch.Generator(device="cuda").manual_seed(19)
+    kv = binding.ScaleKV(1, 1, heads, d, "bf16", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    for k, nk in enumerate(n):
+        Q, K, V = (torch.randn(1, heads, nk, d, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+        Q[..., 0], K[..., 0] = 1.0, -3e38
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        _, _, cs, ts, _ = kv.scalekv_layer_stats_ex(0, Q, topk, 1)
+        L = sum(n[: k + 1])
+        assert np.allclose(cs, nk / L, rtol=1e-5) and np.allclose(ts, min(topk, L - nk) / L, rtol=1e-5, atol=1e-7)
+    kv.close()
