@@ -3,11 +3,25 @@
 // of the 11 us that a step costs the host; the small scales are bound by that.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+
+#include <exception>
 
 #include "../../include/scalekv.h"
 
 namespace {
+
+// A C++ exception (a sparse tensor has no strides, a wrapped one no memory) becomes the Python one that the tensor's own method
+// raises: none may cross the interpreter's C frames.
+template <typename F> bool guarded(F read) {
+  try {
+    return read();
+  } catch (...) {
+    torch::translate_exception_to_python(std::current_exception());
+    return false;
+  }
+}
 
 // [B, H, n, d] tensor -> view with element strides; the last axis must be contiguous
 bool view(PyObject *obj, scalekv_tensor *out) {
@@ -15,16 +29,18 @@ bool view(PyObject *obj, scalekv_tensor *out) {
     PyErr_SetString(PyExc_TypeError, "expected a tensor");
     return false;
   }
-  const at::Tensor &t = THPVariable_Unpack(obj);
-  if (t.dim() != 4 || t.stride(3) != 1) {
-    PyErr_SetString(PyExc_AssertionError, "expected [B, H, n, d] with contiguous head_dim");
-    return false;
-  }
-  out->ptr = t.data_ptr();
-  out->stride_b = t.stride(0);
-  out->stride_h = t.stride(1);
-  out->stride_t = t.stride(2);
-  return true;
+  return guarded([&] {
+    const at::Tensor &t = THPVariable_Unpack(obj);
+    if (t.dim() != 4 || t.stride(3) != 1) {
+      PyErr_SetString(PyExc_AssertionError, "expected [B, H, n, d] with contiguous head_dim");
+      return false;
+    }
+    out->ptr = t.data_ptr();
+    out->stride_b = t.stride(0);
+    out->stride_h = t.stride(1);
+    out->stride_t = t.stride(2);
+    return true;
+  });
 }
 
 // None or a tensor of floats
@@ -35,8 +51,10 @@ bool floats(PyObject *obj, float **out) {
     PyErr_SetString(PyExc_TypeError, "expected a tensor or None");
     return false;
   }
-  *out = static_cast<float *>(THPVariable_Unpack(obj).data_ptr());
-  return true;
+  return guarded([&] {
+    *out = static_cast<float *>(THPVariable_Unpack(obj).data_ptr());
+    return true;
+  });
 }
 
 template <typename T> T address(PyObject *obj) { return reinterpret_cast<T>(PyLong_AsVoidPtr(obj)); }

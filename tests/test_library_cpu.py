@@ -133,3 +133,32 @@ def test_pass_work_counts_what_a_one_call_step_leaves_out():
     assert full["attend_min_bytes"] == kv_q_o + logits + appended
     assert step["attend_min_bytes"] == kv_q_o + logits                        # scale 0 evicts, scale 1 is the last
     assert full["compress_bytes"] == step["compress_bytes"] and step["compress_launches"] == 1
+
+
+# ---- the native module of the hot calls, driven with a stand-in for the library's function
+@pytest.fixture
+def native():
+    import torch
+
+    seen = []
+    kind = C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_int32, C.c_int32, binding.scalekv_tensor, binding.scalekv_tensor)
+
+    def append(ctx, layer, scale, K, V):
+        seen.append((layer, scale, [(t.ptr, t.stride_b, t.stride_h, t.stride_t) for t in (K, V)]))
+        return 7
+
+    fn = kind(append)
+    return binding.load_call(), C.cast(fn, C.c_void_p).value, seen, fn, torch.arange(240.0).reshape(2, 3, 5, 8)
+
+
+def test_native_call_raises_what_the_tensor_raises(native):
+    import torch
+
+    call, fn, seen, _, t = native
+    with pytest.raises(RuntimeError):
+        call.attend(fn, 0, 0, t, t, torch.zeros(2, 3).to_sparse())
+    with pytest.raises(RuntimeError):
+        torch.func.vmap(lambda k: call.append(fn, 0, 0, 0, k, k))(t.unsqueeze(0))
+    with pytest.raises(AssertionError):
+        call.append(fn, 0, 0, 0, t.transpose(2, 3), t)
+    assert not seen
