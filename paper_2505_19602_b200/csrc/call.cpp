@@ -23,18 +23,36 @@ template <typename F> bool guarded(F read) {
   }
 }
 
-// [B, H, n, d] tensor -> view with element strides; the last axis must be contiguous
+// obj.name() or, with an index, obj.name(index)
+bool ask(PyObject *obj, const char *name, int index, long long *out) {
+  PyObject *r = index < 0 ? PyObject_CallMethod(obj, name, nullptr) : PyObject_CallMethod(obj, name, "i", index);
+  if (!r) return false;
+  *out = (long long)(intptr_t)PyLong_AsVoidPtr(r);
+  Py_DECREF(r);
+  return !PyErr_Occurred();
+}
+
+bool bad_shape() {
+  PyErr_SetString(PyExc_AssertionError, "expected [B, H, n, d] with contiguous head_dim");
+  return false;
+}
+
+// [B, H, n, d] tensor -> view with element strides; the last axis must be contiguous.  Anything else that has a tensor's dim(),
+// stride(i) and data_ptr() is asked for them (a subclass of Tensor may have its own).
 bool view(PyObject *obj, scalekv_tensor *out) {
-  if (!THPVariable_Check(obj)) {
-    PyErr_SetString(PyExc_TypeError, "expected a tensor");
-    return false;
+  if (!THPVariable_CheckExact(obj)) {
+    long long dim, last, ptr, sb, sh, st;
+    if (!ask(obj, "dim", -1, &dim)) return false;
+    if (dim != 4) return bad_shape();
+    if (!ask(obj, "stride", 3, &last)) return false;
+    if (last != 1) return bad_shape();
+    if (!ask(obj, "data_ptr", -1, &ptr) || !ask(obj, "stride", 0, &sb) || !ask(obj, "stride", 1, &sh) || !ask(obj, "stride", 2, &st)) return false;
+    *out = {reinterpret_cast<const void *>((intptr_t)ptr), sb, sh, st};
+    return true;
   }
   return guarded([&] {
     const at::Tensor &t = THPVariable_Unpack(obj);
-    if (t.dim() != 4 || t.stride(3) != 1) {
-      PyErr_SetString(PyExc_AssertionError, "expected [B, H, n, d] with contiguous head_dim");
-      return false;
-    }
+    if (t.dim() != 4 || t.stride(3) != 1) return bad_shape();
     out->ptr = t.data_ptr();
     out->stride_b = t.stride(0);
     out->stride_h = t.stride(1);
@@ -47,9 +65,11 @@ bool view(PyObject *obj, scalekv_tensor *out) {
 bool floats(PyObject *obj, float **out) {
   *out = nullptr;
   if (obj == Py_None) return true;
-  if (!THPVariable_Check(obj)) {
-    PyErr_SetString(PyExc_TypeError, "expected a tensor or None");
-    return false;
+  if (!THPVariable_CheckExact(obj)) {
+    long long ptr;
+    if (!ask(obj, "data_ptr", -1, &ptr)) return false;
+    *out = reinterpret_cast<float *>((intptr_t)ptr);
+    return true;
   }
   return guarded([&] {
     *out = static_cast<float *>(THPVariable_Unpack(obj).data_ptr());

@@ -151,6 +151,17 @@ def native():
     return binding.load_call(), C.cast(fn, C.c_void_p).value, seen, fn, torch.arange(240.0).reshape(2, 3, 5, 8)
 
 
+def test_native_call_passes_views_and_the_status(native):
+    call, fn, seen, _, t = native
+
+    class Wrapped:                       # not a tensor, but it has what the library needs of one
+        dim, stride, data_ptr = t.dim, t.stride, t.data_ptr
+
+    part = t[:, 1:, ::2]
+    assert call.append(fn, 0, 4, 2, part, Wrapped()) == 7
+    assert seen == [(4, 2, [(part.data_ptr(), 120, 40, 16), (t.data_ptr(), 120, 40, 8)])]
+
+
 def test_native_call_raises_what_the_tensor_raises(native):
     import torch
 
@@ -161,4 +172,6 @@ def test_native_call_raises_what_the_tensor_raises(native):
         torch.func.vmap(lambda k: call.append(fn, 0, 0, 0, k, k))(t.unsqueeze(0))
     with pytest.raises(AssertionError):
         call.append(fn, 0, 0, 0, t.transpose(2, 3), t)
+    with pytest.raises(AttributeError):
+        call.append(fn, 0, 0, 0, None, t)
     assert not seen
