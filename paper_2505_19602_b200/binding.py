@@ -362,11 +362,16 @@ class ScaleKV:
         return O
 
     @staticmethod
-    def _window(window_pos):
-        """(array or None, its address, its length) of a window given as a sequence, as a prepared array or not at all."""
+    def _window(window_pos, prepared=False):
+        """(array or None, its address, its length) of a window given as a sequence, as a prepared array or not at all.  With
+        `prepared` a ctypes array of another type is refused, as ctypes does where it takes a pointer; else it is converted."""
         if window_pos is None:
             return None, 0, 0
-        wp = window_pos if isinstance(window_pos, C.Array) else _i32_array(window_pos)
+        wp = window_pos
+        if not isinstance(wp, C.Array) or wp._type_ is not C.c_int32:
+            if prepared and isinstance(wp, C.Array):
+                raise C.ArgumentError("a prepared window is an array of c_int32")
+            wp = _i32_array(wp)
         return wp, C.addressof(wp), len(wp)
 
     def scalekv_compress(self, layer, Qw, window_pos=None, qw_is_full_map=False):
@@ -392,7 +397,7 @@ class ScaleKV:
         if whole_map:
             wp, at, w = None, 0, -1
         else:
-            wp, at, w = self._window(window_pos)
+            wp, at, w = self._window(window_pos, prepared=True)
         self._check(self._call.step(self._fn["step"], self._handle, layer, scale, Q, K, V, O, lse, w, at))
 
     @staticmethod
@@ -404,7 +409,7 @@ class ScaleKV:
                         n_sink=0, head_shared=False, head_budgets=None, separate_kernels=False):
         """append + attend + scalekv_compress_ex (Q as the full current map) in one call; compress=False: no compress."""
         opts = self._select_opts(policy, pool_kernel, n_sink, head_shared, head_budgets, separate_kernels)
-        wp, at, w = self._window(window_pos)
+        wp, at, w = self._window(window_pos, prepared=True)
         self._check(self._call.step_ex(self._fn["step_ex"], self._handle, layer, scale, Q, K, V, O, lse, int(bool(compress)), w, at,
                                        C.addressof(opts)))
 

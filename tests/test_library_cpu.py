@@ -175,3 +175,25 @@ def test_native_call_raises_what_the_tensor_raises(native):
     with pytest.raises(AttributeError):
         call.append(fn, 0, 0, 0, None, t)
     assert not seen
+
+
+def test_windows_of_other_integer_types_are_never_read_as_int32():
+    windows = []
+
+    class Calls:                         # in the place of the native module: reads the window as the library does
+        def step(self, fn, ctx, layer, scale, Q, K, V, O, lse, w, at):
+            windows.append(list((C.c_int32 * w).from_address(at)))
+
+        def compress_ex(self, fn, ctx, layer, Qw, w, at, full, opts):
+            windows.append(list((C.c_int32 * w).from_address(at)))
+
+    kv = binding.ScaleKV.__new__(binding.ScaleKV)
+    kv._call, kv._fn, kv._handle = Calls(), {"step": 0, "compress_ex": 0}, 0
+    kv._check = lambda st: None
+    for window in ([1, 5, 9], np.array([1, 5, 9]), kv.window_array([1, 5, 9])):
+        kv.scalekv_step(0, 0, None, None, None, None, window_pos=window)
+        kv.scalekv_compress(0, None, window)
+    kv.scalekv_compress(0, None, (C.c_int64 * 3)(1, 5, 9))
+    assert windows == [[1, 5, 9]] * 7
+    with pytest.raises(C.ArgumentError):
+        kv.scalekv_step(0, 0, None, None, None, None, window_pos=(C.c_int64 * 3)(1, 5, 9))
