@@ -8,8 +8,10 @@ fallback: a missing or unloadable library raises.
 from __future__ import annotations
 
 import ctypes as C
+import hashlib
 import os
 import subprocess
+import sysconfig
 
 import torch
 
@@ -17,7 +19,6 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libscalekv.so")
 SOURCES = [os.path.join(_HERE, "csrc", f) for f in ("scalekv.cu", "select_static.cu", "kernels_simt.cuh", "attend_tc.cuh", "common.cuh")]
 HEADER = os.path.join(os.path.dirname(_HERE), "include", "scalekv.h")
-CALL_PATH = os.path.join(_HERE, "_scalekv_call.so")
 CALL_SOURCE = os.path.join(_HERE, "csrc", "call.cpp")
 
 KEEP_ALL = -1
@@ -76,24 +77,35 @@ def build_library(force=False, verbose=False):
     return LIB_PATH
 
 
-def build_call(force=False, verbose=False):
-    """Compiles the native module of the hot calls against PyTorch's headers."""
-    if not force and os.path.exists(CALL_PATH) and os.path.getmtime(CALL_PATH) >= max(os.path.getmtime(CALL_SOURCE), os.path.getmtime(HEADER)):
-        return CALL_PATH
-    import sysconfig
+def call_path():
+    """The native module's file.  Its name says what it was compiled from and against: a module of other sources, another PyTorch
+    (whose tensors it reads) or another Python is never taken for it."""
+    h = hashlib.sha256(f"{torch.__version__} {sysconfig.get_config_var('SOABI')}".encode())
+    for source in (CALL_SOURCE, HEADER):
+        with open(source, "rb") as f:
+            h.update(f.read())
+    return os.path.join(_HERE, f"_scalekv_call-{h.hexdigest()[:16]}.so")
 
+
+def build_call(force=False, verbose=False):
+    """Compiles the native module of the hot calls against PyTorch's headers, unless there is one of this state."""
+    path = call_path()
+    if not force and os.path.exists(path):
+        return path
     from torch.utils import cpp_extension
 
     libs = cpp_extension.library_paths()
+    part = f"{path[:-3]}.{os.getpid()}.so"         # moved into place whole: several processes may build, and load, at once
     cmd = ["g++", "-O2", "-shared", "-fPIC", "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           *(f"-isystem{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_path("include")]), CALL_SOURCE, "-o", CALL_PATH,
+           *(f"-isystem{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_path("include")]), CALL_SOURCE, "-o", part,
            *(f"-L{d}" for d in libs), *(f"-Wl,-rpath,{d}" for d in libs), "-lc10", "-ltorch_cpu", "-ltorch_python"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    os.replace(part, path)
     if verbose:
         print(res.stderr)
-    return CALL_PATH
+    return path
 
 
 _lib = None
@@ -101,15 +113,13 @@ _call = None
 
 
 def load_call():
-    """The native module of the hot calls (built when missing)."""
+    """The native module of the hot calls (built when there is none of this state)."""
     global _call
     if _call is None:
         import importlib.machinery
         import importlib.util
 
-        if not os.path.exists(CALL_PATH):
-            build_call()
-        loader = importlib.machinery.ExtensionFileLoader("_scalekv_call", CALL_PATH)
+        loader = importlib.machinery.ExtensionFileLoader("_scalekv_call", build_call())
         _call = importlib.util.module_from_spec(importlib.util.spec_from_loader("_scalekv_call", loader))
         loader.exec_module(_call)
     return _call

@@ -197,3 +197,18 @@ def test_windows_of_other_integer_types_are_never_read_as_int32():
     assert windows == [[1, 5, 9]] * 7
     with pytest.raises(C.ArgumentError):
         kv.scalekv_step(0, 0, None, None, None, None, window_pos=(C.c_int64 * 3)(1, 5, 9))
+
+
+def test_a_native_module_of_another_state_is_not_loaded(monkeypatch, tmp_path):
+    import torch
+
+    current = binding.call_path()
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", "0.0.0")
+        assert binding.call_path() != current
+    header = tmp_path / "scalekv.h"
+    header.write_text(open(binding.HEADER).read() + "\n// changed\n")
+    monkeypatch.setattr(binding, "HEADER", str(header))
+    assert binding.call_path() != current
+    monkeypatch.undo()
+    assert binding.call_path() == current == binding.build_call() and binding.load_call().__file__ == current
