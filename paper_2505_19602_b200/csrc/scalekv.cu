@@ -56,10 +56,10 @@ struct Plan {
   int ld_l = 0;                     // leading dimension of a logit row: room for the history rounded up to a key tile and a ragged last tile
   int n_max = 0;
   // pool layout (byte offsets)
-  size_t off_k, off_v, off_pos, off_pt, off_len, off_status, pool_bytes;
+  size_t off_k, off_v, off_pos, off_pt, off_len, off_status, off_count, count_bytes, pool_bytes;
   size_t pt_elems, logits_elems;
   // workspace layout
-  size_t off_logits, off_wlse, off_scores, off_keys, off_keep, off_kept, off_hbud, off_acc, off_count, off_stats, ws_bytes;
+  size_t off_logits, off_wlse, off_scores, off_keys, off_keep, off_kept, off_hbud, off_acc, off_stats, ws_bytes;
 };
 
 // Raster indices of the observation window of an h x w map (see scalekv_window_centroids).
@@ -168,6 +168,9 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
   // lengths before the even and before the odd scales: a scale's kernels read the one and write the other
   p.off_len = o; o = align_up(o + 2 * (size_t)p.n_layers * p.n_slices * 4, 1024);
   p.off_status = o; o = align_up(o + 256, 1024);
+  // layer_stats' counts of finished CTAs: zero between calls, so they stay with the store and not in the borrowed workspace
+  p.count_bytes = (size_t)p.n_slices * ((p.n_max + 63) / 64) * 4;
+  p.off_count = o; o = align_up(o + p.count_bytes, 1024);
   p.pool_bytes = o;
   o = 0;
   p.logits_elems = (size_t)p.n_slices * p.max_window * p.ld_l;   // one buffer per set
@@ -179,7 +182,6 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
   p.off_kept = o; o = align_up(o + (size_t)p.n_slices * 4, 1024);
   p.off_hbud = o; o = align_up(o + (size_t)p.n_slices * 4, 1024);
   p.off_acc = o; o = align_up(o + 16 + (size_t)p.n_slices * 24, 1024);
-  p.off_count = o; o = align_up(o + (size_t)p.n_slices * ((p.n_max + 63) / 64) * 4, 1024);
   p.off_stats = o; o = align_up(o + (size_t)kStatsMaxCtas * 64 * kStatsRec * 4, 1024);   // key-range partials of layer_stats
   p.ws_bytes = o;
   return SCALEKV_OK;
@@ -472,6 +474,7 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
   if (cudaMemset(ctx->pool + p.off_k, 0, p.off_pos - p.off_k) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
   if (cudaMemset(ctx->pool + p.off_len, 0, 2 * (size_t)p.n_layers * p.n_slices * 4) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
   if (cudaMemset(ctx->pool + p.off_status, 0, 256) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
+  if (cudaMemset(ctx->pool + p.off_count, 0, p.count_bytes) != cudaSuccess) return bail(SCALEKV_ERR_CUDA);
   ctx->next_scale.assign(p.n_layers, 0);
   ctx->hist.assign(p.n_layers, 0);
   ctx->pending.assign(p.n_layers, 0);
@@ -1088,7 +1091,6 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
       CU(cudaHostAlloc(reinterpret_cast<void **>(&ctx->stats_host), most * sizeof(double), cudaHostAllocMapped));
       CU(cudaHostGetDevicePointer(reinterpret_cast<void **>(&ctx->stats_host_dev), ctx->stats_host, 0));
       ctx->stats_host_doubles = most;
-      CU(cudaMemsetAsync(ctx->ws + p.off_count, 0, (size_t)p.n_slices * ((p.n_max + 63) / 64) * 4, ctx->s_main));
     }
     // (a programmatic launch: the kernel comes up while the one before it ends)
     cudaLaunchConfig_t cfg = {};
@@ -1102,7 +1104,7 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
     cfg.blockDim = dim3(256);
     Scope sc(ctx, ctx->s_main, kOther);
     CU(cudaLaunchKernelEx(&cfg, stats_mma_kernel, lv, tview(Q), nk, query_stride, rows, topk_prime, ctx->scale * 1.4426950408889634f, partial,
-                          reinterpret_cast<int *>(ctx->ws + p.off_count), ctx->stats_host_dev));
+                          reinterpret_cast<int *>(ctx->pool + p.off_count), ctx->stats_host_dev));
     sums = ctx->stats_host;
     ctx->len_written[layer] = 1;
   } else {

@@ -62,3 +62,22 @@ def test_rows_of_scores_near_the_lowest_number():
         L = sum(n[: k + 1])
         assert np.allclose(cs, nk / L, rtol=1e-5) and np.allclose(ts, min(topk, L - nk) / L, rtol=1e-5, atol=1e-7)
     kv.close()
+
+
+def test_nothing_is_expected_of_the_workspace_between_calls():
+    """The workspace is borrowed: its owner may have used it for something else between two calls."""
+    sides, heads, d = (4, 20), 2, 128
+    g = torch.Generator(device="cuda").manual_seed(23)
+    kv = binding.ScaleKV(1, 1, heads, d, "bf16", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    inputs = [tuple(torch.randn(1, heads, a * a, d, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(3)) for a in sides]
+    passes = []
+    for fill in (0, 0x2b):
+        kv.scalekv_reset()
+        passes.append([])
+        for k, (Q, K, V) in enumerate(inputs):
+            kv.workspace.fill_(fill)
+            torch.cuda.synchronize()
+            kv.scalekv_append(0, k, K, V)
+            passes[-1].append(kv.scalekv_layer_stats_ex(0, Q, 16, 1))
+    kv.close()
+    assert passes[0] == passes[1]
