@@ -421,8 +421,9 @@ __device__ __noinline__ Raised raise_reference(int valid, float c, float m, floa
   return {m_new, l_run * f, sum, o_landed, 1};
 }
 
-// Division of numbers below 2^21 by a divisor below 2^21 the quick way (the remainder of 2^42 costs less than one quotient):
+// Division of numbers below 2^21 (the plan sees to that) by a divisor below 2^21 the quick way (the remainder of 2^42 costs less than one quotient):
 // a CTA finds its item with three of these, and its first loads wait for it.
+constexpr long long kMaxItems = 1ll << 21;
 struct Divisor {
   unsigned long long mul;
   int d;

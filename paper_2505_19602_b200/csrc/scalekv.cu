@@ -110,6 +110,9 @@ scalekv_status make_plan(const scalekv_config *c, Plan &p, std::string &err) {
     p.N[k + 1] = p.N[k] + p.n[k];
     p.n_max = std::max(p.n_max, p.n[k]);
   }
+  if ((long long)c->batch * c->n_heads * ((p.n_max + 127) / 128) >= tc::kMaxItems) {
+    err = "a launch of more than 2^21 query tiles is not supported"; return SCALEKV_ERR_UNSUPPORTED;
+  }
   p.budgets.assign(c->budgets, c->budgets + (size_t)p.n_layers * p.K);
   if (c->window_patches < 0 || c->window_patches > c->max_window) { err = "window_patches must lie in [0, max_window]"; return SCALEKV_ERR_INVALID_ARG; }
   p.windows.assign(p.K, std::vector<int>());

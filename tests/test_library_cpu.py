@@ -135,6 +135,14 @@ def test_pass_work_counts_what_a_one_call_step_leaves_out():
     assert full["compress_bytes"] == step["compress_bytes"] and step["compress_launches"] == 1
 
 
+def test_schedules_with_too_many_query_tiles_are_refused(lib):
+    """The attention kernel finds its work by divisions that hold below 2^21 query tiles."""
+    pb, wb = C.c_size_t(), C.c_size_t()
+    for batch, side, status in ((2 ** 17 - 1, 11, "OK"), (2 ** 17, 11, "UNSUPPORTED"), (2 ** 16, 12, "UNSUPPORTED")):
+        cfg, keep = make_cfg(1, batch, 16, 128, binding.BF16, (side,), [[-1]], max_window=1, page_tokens=16)
+        assert lib.scalekv_query_sizes(C.byref(cfg), C.byref(pb), C.byref(wb)) == binding.STATUS_NAMES.index(status)
+
+
 # ---- the native module of the hot calls, driven with a stand-in for the library's function
 @pytest.fixture
 def native():
