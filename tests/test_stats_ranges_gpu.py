@@ -1,4 +1,5 @@
-"""scalekv_layer_stats_ex over its two kernels: few and many rows, splits that are no power of two, K' on either side of 16."""
+"""scalekv_layer_stats_ex over its two kernels: few and many rows, splits that are no power of two, K' on either side of 16, more rows
+than the scratch takes."""
 import numpy as np
 import pytest
 import torch
@@ -81,3 +82,25 @@ def test_nothing_is_expected_of_the_workspace_between_calls():
             passes[-1].append(kv.scalekv_layer_stats_ex(0, Q, 16, 1))
     kv.close()
     assert passes[0] == passes[1]
+
+
+def test_more_records_than_the_scratch_holds():
+    """33 slices x 4 096 rows: the tensor-core kernel's records do not fit, the other kernel takes the call although K' <= 16."""
+    sides, batch, heads, d, topk = (2, 64), 3, 11, 128, 5
+    g = torch.Generator(device="cuda").manual_seed(31)
+    kv = binding.ScaleKV(1, batch, heads, d, "bf16", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    keys = []
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(batch, heads, a * a, d, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+        keys.append(K)
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        _, _, cs, ts, _ = kv.scalekv_layer_stats_ex(0, Q, topk, 1)
+    for b in range(batch):
+        for h in range(heads):
+            A = (Q[b, h].double() @ torch.cat([K[b, h] for K in keys]).double().T / d ** 0.5).softmax(-1)
+            hist = sides[0] ** 2
+            # (the bound of the test above)
+            assert abs(cs[b][h] - A[:, hist:].sum(1).mean().item()) <= 1e-4 * cs[b][h] + 1e-7
+            assert abs(ts[b][h] - A[:, :hist].topk(min(topk, hist))[0].sum(1).mean().item()) <= 1e-4 * ts[b][h] + 1e-7
+    kv.close()
