@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, Tensor
 #pragma unroll
     for (int d = 8; d > 0; d >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], d);
 
+  // (lse: the logarithm of the sum taken to base e, one rounding behind it; to base 2 both are of larger numbers)
   if (n_split == 1) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, Tensor
         x[j] = ((i & 1) ? e.y : e.x) * inv;
       }
       *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, r)) + tx * 4) = make_float4(x[0], x[1], x[2], x[3]);
-      if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + r] = (m[i] + log2f(l[i])) * 0.6931471805599453f;
+      if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + r] = fmaf(m[i], 0.6931471805599453f, logf(l[i]));
     }
     return;
   }
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, Tensor
     }
     const float inv = 1.f / sum;
     *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, q0 + r)) + tx * 4) = make_float4(a0 * inv, a1 * inv, a2 * inv, a3 * inv);
-    if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + q0 + r] = (M + log2f(sum)) * 0.6931471805599453f;
+    if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + q0 + r] = fmaf(M, 0.6931471805599453f, logf(sum));
   }
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");

@@ -45,3 +45,26 @@ def test_f32_rows_of_scores_near_the_lowest_number(heads):
         want = torch.cat(values, 2).mean(2, keepdim=True)
         assert (O - want).abs().max().item() <= 1e-5
     kv.close()
+
+
+@pytest.mark.parametrize("heads", [2, 40])
+def test_f32_log_sum_exp_is_rounded_twice(heads):
+    """lse lies in [4, 8) and so does the logarithm of the sum, its largest part: two roundings of 2^-21 / sqrt(12) rms make 1.95e-7.  A
+    third, or one of numbers above 8, would show: 3e-7 where the logarithm is taken to base 2 and converted."""
+    sides = (5, 40)
+    g = torch.Generator(device="cuda").manual_seed(9)
+    kv = binding.ScaleKV(1, 1, heads, 64, "f32", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    keys = []
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(1, heads, a * a, 64, generator=g, device="cuda") for _ in range(3))
+        Q *= 0.25
+        keys.append(K)
+        lse = torch.empty(1, heads, a * a, device="cuda")
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        kv.scalekv_attend(0, Q, lse=lse)
+        kv.scalekv_sync()
+    want = (Q.double() @ torch.cat(keys, 2).double().transpose(2, 3) / 8).logsumexp(-1)
+    assert 4 < want.min().item() and want.max().item() < 8
+    assert (lse.double() - want).pow(2).mean().sqrt().item() <= 2.4e-7
+    kv.close()
