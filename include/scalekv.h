@@ -100,7 +100,7 @@ typedef struct {
  * are ignored).  The pool holds, per layer, ceil(cap_l / page_tokens) persistent pages per slice,
  * cap_l being the largest cache a compress leaves behind, plus four transient page sets (layer l
  * uses set l mod 4) that hold the part of the current map that exceeds cap_l until that layer's
- * compress; page tables; per-slice lengths.  No CUDA call is made. */
+ * compress; page tables; per-slice lengths; counters of layer_stats.  No CUDA call is made. */
 scalekv_status scalekv_query_sizes(const scalekv_config *cfg, size_t *pool_bytes, size_t *workspace_bytes);
 
 /* Creates a context: copies schedule and budgets, carves the pool, uploads the page tables and

@@ -1144,15 +1144,19 @@ struct AttendTc {
     return window ? (const void *)tc::attend_tc_kernel<true> : (const void *)tc::attend_tc_kernel<false>;
   }
 
-  // How a launch is cut.  Measured on a B200 (148 SMs), us per launch, averaged over a layer with a long and three with a short
-  // cache, against one CTA for every pair or odd tile, the odd ones by a single warpgroup:
-  //   16 slices, singles (split over clusters up to 400 queries): 256 / 400 / 576 / 1024 queries 22.0 -> 15.4, 26.8 -> 18.6,
-  //   30.3 -> 22.6, 37.3 -> 29.3;  two key tiles are not worth splitting;
-  //   128 slices x 1024 queries (512 pairs, 3.5 waves), the last 68 pairs as 136 singles: 135 -> 122.
+  // How a launch is cut.  us per launch on a B200 (148 SMs; attends of a map in the pages, back to back from a graph) behind
+  // 209 / 1 960 entries, one CTA for every pair or odd tile -> this rule:
+  //   16 slices, 64 queries 7.9 / 21.2 -> 8.0 / 10.5, 144: 9.9 / 34.5 -> 8.9 / 13.6, 256: 12.2 / 36.7 -> 8.9 / 13.8, 400: 14.1 / 38.7 ->
+  //   11.1 / 18.5, 576: 17.7 / 40.7 -> 13.4 / 27.5, 1 024: 23.9 / 48.8 -> 16.6 / 31.3;
+  //   128 slices x 1 024 queries (512 pairs, 3.5 waves), the last 68 pairs as 136 singles: 104.2 / 221.6 -> 98.6 / 214.1.
   // n_pair: items that are walked pair by pair; items: all of them; split: CTAs that share an item's keys.
   struct Cut { int n_pair, items, split; };
   Cut cut(int tiles, int slices, int key_tiles) const {
-    constexpr float kJoin = 0.9f;      // what combining over a cluster costs, in steps (of two key tiles) of a single
+    // What combining over a cluster costs, in steps (of two key tiles) of a single.  Behind 1 960 entries every split up to four
+    // CTAs gains (16 slices x 256 queries, 1 / 2 / 3 / 4 CTAs: 23.9 / 16.5 / 13.7 / 13.3 us); behind 209 a split of two mostly
+    // loses (unsplit / as here, 16 slices x 144, 256, 400 queries: 8.2 / 8.9, 9.3 / 8.9, 10.6 / 11.1; 32 slices x 144, 256: 8.4 /
+    // 10.1, 9.5 / 10.1), so 0.9 is too little for the shortest launches.
+    constexpr float kJoin = 0.9f;
     const int pairs = tiles / 2 * slices, odd = tiles % 2 * slices;
     auto steps = [&](int split) { const int per = (key_tiles + split - 1) / split; return (float)((per + 1) / 2); };
     if (2 * pairs + odd <= n_sm) {

@@ -1,6 +1,6 @@
 // The hot calls of the C ABI for Python callers: tensors are read through PyTorch's C++ interface and handed to the function
-// whose address the binding passes, in one native call.  Building four ctypes structures and converting them took 3.1 us
-// of the 11 us that a step costs the host; the small scales are bound by that.
+// whose address the binding passes, in one native call.  A step of a small map costs the host 5.9 us this way; with four ctypes
+// structures built for every call (and the launches and events that a step made then) it was 14.5 us, twice what the GPU takes.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <torch/csrc/Exceptions.h>

@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(256) score_logits_kernel(LayerView lv, TensorV
 // s_i = (1/w) sum_j 2^(y_ji - lse_j), lse_j the base-2 log-sum-exp of row j (recorded by attend, or
 // computed by row_lse_kernel).  Streaming and embarrassingly parallel: grid (ceil(L_max / 256),
 // n_slices), one entry per thread, the w loads of a thread independent and coalesced across the warp.
-// Besides the score (kept for inspection) it writes the entry's radix key: the bit pattern of the
+// Besides the score (kept for inspection) it writes the entry's key: the bit pattern of the
 // non-negative float, or a sentinel for window entries, which never take part in the selection.
 // ------------------------------------------------------------------------------------------
 constexpr uint32_t kWindowKey = 0xFFFFFFFFu;
@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(256) compact_kernel(LayerView lv, const int *k
 // CTA of 512 threads, the phases separated by block barriers - what score_kernel, select_kernel and
 // compact_kernel do in three launches, for every slice whose keys and keep list fit in shared memory.
 //   phase 1  policy 0: s_i = (1/w) sum_j 2^(y_ji * logit_scale - lse_j) from the window rows' logits (see
-//            score_kernel), two neighbouring columns per thread -> scores (global, kept for inspection) and radix keys
+//            score_kernel), two neighbouring columns per thread -> scores (global, kept for inspection) and keys
 //            (shared); the window entries, whose slots follow from the map's place behind the history, get the sentinel.
 //            policy 1: keys from the original positions (see recent_keys_kernel).
 //   phase 2  select_and_emit, ascending keep list in shared memory.

@@ -705,10 +705,14 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       ctx->logits_of[layer] = wl ? k : -1;
       ctx->logits_padded[layer] = fused ? 1 : 0;
     } else {
-      // CTAs that share a slice's keys: so that the SM with the most work has as little of it as possible
+      // CTAs that share a slice's keys: so that the SM with the most work has as little of it as possible, if its CTAs ran one after
+      // another.  us per launch, 16 slices behind 209 / 1 960 entries, unsplit -> as here (best of 1 to 8): 64 queries 43.8 / 251.5 ->
+      // 13.4 / 61.2 (13.0 / 51.7), 256: 67.4 / 276.9 -> 22.9 / 77.3 (22.9 / 77.2), 576: 106.3 / 315.6 -> 77.0 / 175.8 (the same), 1 600:
+      // 402.6 / 771.0 -> 318.8 / 584.3 (318.8 / 575.7).  Two CTAs of an SM do run together, so it is off where that decides: 16 slices
+      // x 1 024 160.7 / 370.1, unsplit (by two CTAs 146.8 / 336.9); 48 x 256 behind 209 73.4 (unsplit 67.4, by four 53.3).
       const int blocks = (nk + kF32Rows - 1) / kF32Rows, ctas = blocks * p.n_slices, tiles = (ctx->hist[layer] + nk + 63) / 64;
       int split = 1;
-      auto load = [&](int c) { return (float)((ctas * c + ctx->n_sm - 1) / ctx->n_sm) * ((float)((tiles + c - 1) / c) + 1.5f); };   // in key tiles; a CTA costs 1.5 more
+      auto load = [&](int c) { return (float)((ctas * c + ctx->n_sm - 1) / ctx->n_sm) * ((float)((tiles + c - 1) / c) + 1.5f); };   // in key tiles; its queries and its end cost a CTA 1.5 more
       for (int c = 2; c <= kF32MaxSplit && c <= tiles; ++c)
         if (load(c) < load(split)) split = c;
       cudaLaunchConfig_t cfg = {};
