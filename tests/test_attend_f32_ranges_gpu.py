@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("batch,heads,sides,budget", [
-    (1, 1, (1, 8, 9, 23), 30),           # 64 and 65 rows of keys and queries; clusters of up to 8 CTAs, some without a tile
+    (1, 1, (1, 8, 9, 23), 30),           # 64 and 65 rows of keys and queries; clusters of two to five CTAs
+    (1, 1, (2, 22), -1),                 # eight key tiles: clusters of eight
     (2, 3, (3, 16, 20), -1),             # full cache
     (4, 9, (2, 12, 27), 100),            # 36 slices: three CTAs per slice and tile of queries, then one
 ])

@@ -12,10 +12,10 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("heads,topk,stride,sides", [
     (1, 16, 1, (1, 3, 9)),            # fewer rows than a warp's 16, a history shorter than K', ragged key tiles
-    (3, 16, 1, (8, 16, 13)),          # tiles that are history, map and both
+    (3, 16, 1, (8, 16, 13)),          # tiles that are history, map and both; five and eight key ranges
     (2, 1, 3, (5, 31, 8)),
-    (16, 15, 2, (2, 20, 33)),         # key ranges that are no power of two
-    (5, 0, 4, (4, 11)),
+    (16, 15, 2, (2, 20, 33)),         # nine blocks of rows
+    (5, 0, 4, (4, 11)),               # three key ranges
     (2, 17, 1, (3, 18, 7)),           # K' > 16: the other kernel
 ])
 def test_statistics_match_the_oracle(heads, topk, stride, sides):
