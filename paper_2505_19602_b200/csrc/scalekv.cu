@@ -725,7 +725,7 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)split;
       cfg.attrs = attr;
       cfg.numAttrs = split > 1 ? 1 : 0;
-      CU(cudaLaunchKernelEx(&cfg, attend_f32_kernel, lv, tview(Q), tview(O), lse, nk, ctx->scale * 1.4426950408889634f));
+      CU(cudaLaunchKernelEx(&cfg, attend_f32_kernel, lv, tview(Q), tview(O), lse, nk, lv.pages_per_slice << lv.page_shift, ctx->scale * 1.4426950408889634f));
     }
   }
   ctx->attended[layer] = 1;
