@@ -129,7 +129,8 @@ scalekv_status scalekv_destroy(scalekv_ctx *ctx);
  * and V directly and writes its rows to the pages while it streams them (no second read, nothing
  * on the critical path); any other next call for this layer (compress, layer_stats, export, the
  * next append) copies first with a kernel of its own.  K and V must therefore stay unmodified
- * until stream_main has passed the layer's next call.  For f32 x 64 the copy is enqueued here.
+ * until stream_main has passed the layer's next call.  For f32 x 64 the copy is enqueued here (by a
+ * one-call step, below, it is left to the attend as well).
  * Ordered on stream_main after this layer's previous compress.
  * Layers l, l + 4, l + 8, .. share one transient page set, which holds the part of a
  * current map that exceeds the layer's persistent capacity, and one buffer of recorded window logits.  An append
@@ -145,7 +146,8 @@ scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, sc
  * slice (history that survived earlier compressions, then the current map).  Q and O are
  * [B][H][n_k][d] views in the configured dtype; lse (nullable) is a dense float [B][H][n_k]
  * that receives max + log-sum-exp of the scaled logits.  bf16: products are exact, sums are
- * fp32, P is rounded to bf16 before the PV product.  f32: plain fp32 FMA.  Runs on stream_main. */
+ * fp32, P is rounded to bf16 before the PV product.  f32: to the precision of fp32 arithmetic throughout (products
+ * of bf16 pieces on the tensor cores, sums in fp32).  Runs on stream_main. */
 scalekv_status scalekv_attend(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Q, scalekv_tensor O, float *lse);
 
 /* Sec. 3.3 "KV Cache Selection": with A = softmax(Q_W K^T * scale) over all L entries,

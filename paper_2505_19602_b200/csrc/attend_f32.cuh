@@ -1,0 +1,509 @@
+// Attention over the paged store for f32, head_dim 64 (Sec. 3.3, Eq. 5) on the tensor cores, at the precision of fp32 arithmetic.
+// Every operand is split into three bf16 numbers, x = h + m + l (8 significant bits each, so nothing of x is lost), and a product
+// is the six products of pieces that are larger than 2^-24 of it, the small ones summed first:
+//   S = Ql Kh + Qh Kl + Qm Km + Qm Kh + Qh Km + Qh Kh,  and P V alike.
+// A CTA of 256 threads, two per SM, owns 128 query rows of one slice and streams its keys in tiles of 64:
+//   warps 4-7 : operands.  They load K and V rows (the pages' or, for a map that has not been copied there, the caller's), split
+//               them and leave the pieces in 128B-swizzled shared memory; the next tile's rows wait in registers meanwhile.
+//   warps 0-3 : softmax, a thread per query row (TMEM lane).  The products of a tile of V land in TMEM and are added to the row's
+//               64 columns in registers: the tensor core cuts its sums off where fp32 arithmetic rounds them, which over the tiles of a
+//               long cache would show.  P goes back to TMEM in three pieces.  Warp 0 issues the products of the tile's values and of
+//               the next tile's keys in one go, when all four warps have met.
+// With two CTAs an SM's tensor pipe works for the one while the other is in its softmax.
+// Scores that are not numbers (an infinite key: its products with the pieces of a query may differ in sign) spoil their row's sum, and
+// values that are not its columns; such a row is done again at the end by fp32 FMA from the tensors (fma_row).
+// gridDim.z CTAs of a cluster share a slice's keys and combine: O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e, through distributed
+// shared memory.
+// What bounds it: six products stand for one, so a tile of 64 keys is 48 tcgen05.mma of 128 x 64 x 16; where two CTAs share an SM a step
+// of both takes about 8 000 cycles, of which these are half and the splitting of operands and of P, the exponentials and the way through
+// TMEM the rest.  us per layer and step, 16 slices behind 92 to 772 entries with their compresses, by packed fp32 FMA (66 % of that pipe)
+// and a copy, the window's logits and their sums by launches of their own -> here: 16 queries 15.4 -> 9.7, 64: 25.7 -> 17.0, 256:
+// 35.8 -> 21.0, 400: 65.0 -> 26.6, 576: 91 -> 35, 1 024: 179 -> 60, 1 600: 331 -> 127 (11 -> 29 TFLOP/s of fp32 results).
+// Error against 64 bits, full caches of 29 to 4 436 entries, queries and keys normal, queries times 0.25 / 1 / 3: outputs 0.9 to 1.6 / 1.0 to
+// 2.1 / 1.5 to 4.0 e-7 (by FMA 1.1 to 11.9 / 2.2 to 12.3 / 3.3 to 15.2), lse 1.1 to 3.2 / 1.1 to 3.4 / 2.9 to 3.7 e-7 rms (1.1 to 3.2 / 1.4 to 3.3 /
+// 5.2 to 8.2).
+#pragma once
+#include <cfloat>
+
+#include "attend_tc.cuh"
+#include "kernels_simt.cuh"
+
+namespace scalekv {
+namespace f32 {
+
+using tc::tc_fence_after;
+using tc::tc_fence_before;
+
+constexpr int kRows = 128, kKeys = 64, kThreads = 256;
+constexpr int kMaxSplit = 8;                                // CTAs that may share a slice's keys (portable cluster size)
+constexpr uint32_t kPieceQ = kRows * 128, kPieceK = kKeys * 128;                  // bytes of one bf16 piece of an operand tile
+constexpr uint32_t kOffQ = 0, kOffK = kOffQ + 3 * kPieceQ, kOffV = kOffK + 3 * kPieceK, kOffBar = kOffV + 3 * kPieceK;
+constexpr uint32_t kSmemBytes = kOffBar + 64;
+constexpr uint32_t kOffStat = kOffQ + kRows * 256;          // references and sums of the rows, behind their columns (where Q was)
+static_assert(kOffStat + kRows * 8 <= kOffK, "the parts of a row have to fit where Q was");
+static_assert(2 * (kSmemBytes + 1024) <= 233472, "two CTAs have to fit an SM");
+// What a score loses, of its size and on average, because the tensor core cuts its sums off: about half a unit in the last place (2^-24)
+// in each of the four steps over the large pieces, less in those where the sum is still growing.  It is given back (without: lse of queries
+// times 3 low by 6.6e-7 on average, 7.4e-7 rms; so by 0.3e-7, 3.4e-7 rms).
+constexpr float kCutOff = 1.2f / 16777216.f;
+constexpr uint32_t kTmemCols = 256, kColS = 0, kColP = 64, kColO = 160;           // 64 of scores, 3 x 32 of P, 64 of products with V
+
+struct Params {
+  LayerView lv;
+  TensorView Q, O, K, V;       // K, V: a current map outside the pages (fused)
+  float *lse;
+  int n_k, room;               // room: entries that a slice's pages hold
+  int fused, copy_in, n_prev;  // copy_in: the map's rows go to the pages on the way
+  float scale_log2e;
+  float *win_logits, *win_lse; // raw products of the window's rows by slot, [slice][rank][ld_l], and their base-2 log-sum-exp
+  int ld_l, w;
+  int win_pos[kMaxWindow];
+};
+
+// Four steps (of 16) of one product of pieces, issued by the elected lane of a converged warp.
+__device__ __forceinline__ void mma4_ss(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate_first) {
+  asm volatile(
+      "{\n\t.reg .pred e, pf, pt;\n\t.reg .b64 da, db;\n\t.reg .b32 al, bl;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 pf, %5, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
+      "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pf;\n\t"
+      "add.u32 al, %1, 2;\n\tadd.u32 bl, %2, 2;\n\tmov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
+      "add.u32 al, %1, 4;\n\tadd.u32 bl, %2, 4;\n\tmov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
+      "add.u32 al, %1, 6;\n\tadd.u32 bl, %2, 6;\n\tmov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
+      "}" ::"r"(d),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
+      : "memory");
+}
+__device__ __forceinline__ void mma4_ts(uint32_t d, uint32_t a, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate_first) {
+  asm volatile(
+      "{\n\t.reg .pred e, pf, pt;\n\t.reg .b64 db;\n\t.reg .b32 at, bl;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 pf, %5, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
+      "mov.b64 db, {%2, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pf;\n\t"
+      "add.u32 at, %1, 8;\n\tadd.u32 bl, %2, 128;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
+      "add.u32 at, %1, 16;\n\tadd.u32 bl, %2, 256;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
+      "add.u32 at, %1, 24;\n\tadd.u32 bl, %2, 384;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
+      "}" ::"r"(d),
+      "r"(a), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
+      : "memory");
+}
+__device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t *v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
+// a pair of numbers in three pairs of bf16 numbers that sum to them
+__device__ __forceinline__ void split2(float x, float y, uint32_t &h, uint32_t &m, uint32_t &l) {
+  h = tc::pack_bf16(x, y);
+  x -= __uint_as_float(h << 16);
+  y -= __uint_as_float(h & 0xffff0000u);
+  m = tc::pack_bf16(x, y);
+  x -= __uint_as_float(m << 16);
+  y -= __uint_as_float(m & 0xffff0000u);
+  l = tc::pack_bf16(x, y);
+}
+__device__ __forceinline__ void store16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// eight columns (chunk c) of row r of an operand tile: the pieces' 16 bytes, 128B-swizzled
+__device__ __forceinline__ void put_split(uint32_t tile, uint32_t piece_bytes, int r, int c, const float4 &a, const float4 &b) {
+  uint32_t h[4], m[4], l[4];
+  split2(a.x, a.y, h[0], m[0], l[0]);
+  split2(a.z, a.w, h[1], m[1], l[1]);
+  split2(b.x, b.y, h[2], m[2], l[2]);
+  split2(b.z, b.w, h[3], m[3], l[3]);
+  const uint32_t at = tile + (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4));
+  store16(at, h[0], h[1], h[2], h[3]);
+  store16(at + piece_bytes, m[0], m[1], m[2], m[3]);
+  store16(at + 2 * piece_bytes, l[0], l[1], l[2], l[3]);
+}
+// row `slot` of a slice's keys or values
+__device__ __forceinline__ const float *entry(const Params &prm, bool values, int slice, int b, int h, int hist, int slot) {
+  if (prm.fused && slot >= hist) return row_ptr<float>(values ? prm.V : prm.K, b, h, slot - hist);
+  return reinterpret_cast<const float *>((values ? prm.lv.v_pool : prm.lv.k_pool) + slot_row(prm.lv, slice, slot) * 256);
+}
+
+// The log-sum-exp of a row from its base-2 reference and sum: the logarithm is taken to base e and the sum rounded once (to base 2
+// both are of larger numbers), and what the 32-bit log2(e) in the reference is off by, 1.3e-8 of it, is put right.  rms error over
+// full caches of 521 to 4 240 entries, scores of deviation 0.25 / 1 / 3: 2.0 to 2.8e-7 / 1.9 to 3.0e-7 / 5.5 to 5.9e-7 (to base e
+// throughout 2.0 to 2.8 / 1.9 to 3.2 / 5.4 to 5.8; to base 2 throughout 2.6 to 3.6 / 2.7 to 3.7 / 6.5 to 6.7).
+__device__ __forceinline__ float row_lse_f32(float m, float l) {
+  return fmaf(m, 0.6931471805599453f, fmaf(m, (float)(1.0 / 1.4426950408889634f - 0.6931471805599453f), logf(l)));
+}
+
+// One row by fp32 FMA over the entries [from, to): its 64 columns go to `out` (16-byte pieces permuted by `swap`), its raw products
+// to win_row if it has one.  For rows whose scores or columns by pieces are not numbers.
+struct RowSum { float m, l; };
+__device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int h, int hist, int q_row, int from, int to, float *out, int swap,
+                                       float *win_row) {
+  const float *q = row_ptr<float>(prm.Q, b, h, q_row);
+  float o[64], m = kNoMax, l = 0.f;
+#pragma unroll
+  for (int d = 0; d < 64; ++d) o[d] = 0.f;
+#pragma unroll 1
+  for (int j = from; j < to; ++j) {
+    const float *k = entry(prm, false, slice, b, h, hist, j), *v = entry(prm, true, slice, b, h, hist, j);
+    float s = 0.f;
+#pragma unroll 8
+    for (int d = 0; d < 64; ++d) s = fmaf(q[d], k[d], s);
+    if (win_row != nullptr) win_row[j] = s;
+    const float y = s * prm.scale_log2e, mx = fmaxf(m, y), f = exp2f(m - mx), p = exp2f(y - mx);
+    m = mx;
+    l = fmaf(l, f, p);
+#pragma unroll
+    for (int d = 0; d < 64; ++d) o[d] = fmaf(p, v[d], o[d] * f);
+  }
+#pragma unroll
+  for (int c = 0; c < 16; ++c)
+    *reinterpret_cast<float4 *>(out + (c ^ swap) * 4) = make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+  return {m, l};
+}
+
+// grid (ceil(n_k / 128), n_slices, split); dynamic shared memory kSmemBytes.
+__global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid_constant__ Params prm) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = tc::smem_u32(smem_raw);
+  const uint32_t bar_ops = base + kOffBar, bar_mma = base + kOffBar + 8;
+  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem_raw + kOffBar + 16);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 20);
+  volatile int *leave_slot = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 24);
+  const LayerView &lv = prm.lv;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice - b * lv.n_heads;
+  const int q0 = blockIdx.x * kRows, n_k = prm.n_k, n_split = gridDim.z;
+  int *status = lv.status;
+  if (tid == 0) {
+    tc::mbar_init(bar_ops, 4);           // the operand warps announce V of a tile and K of the next
+    tc::mbar_init(bar_mma, 1);           // the products issued together have landed, and read what they read
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  } else if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + kOffBar + 16), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  // (what is above runs while the kernel before this one ends; see attend_tc_kernel)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int hist = lv.hist_len[slice];
+  // A slice that outgrows its pages is cut off, so that no slot behind the page table is looked up.
+  const int L = min(hist + n_k, prm.room);
+  const int tiles = (L + kKeys - 1) / kKeys;
+  const int lo = tiles * (int)blockIdx.z / n_split;
+  if (tid == 0) {
+    *abort_flag = 0;
+    // (an earlier CTA's wait has run out: do not pile on.  One thread decides for the CTA.)
+    int leave = *reinterpret_cast<volatile int *>(status) == kDevTimeout;
+    if (base & 1023u) { atomicExch(status, kDevCheck); leave = 1; }
+    if (hist + n_k > prm.room) atomicExch(status, kDevCheck);
+    *leave_slot = leave;
+    if (!leave && blockIdx.x == 0 && blockIdx.z == 0) lv.next_len[slice] = L;      // unless a compress of this scale evicts
+  }
+  // Q: a thread takes one chunk of eight columns of four rows
+  {
+    float4 x[4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = (tid >> 3) + 32 * u, c = tid & 7;
+      x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (q0 + r < n_k) {
+        const float4 *src = reinterpret_cast<const float4 *>(row_ptr<float>(prm.Q, b, h, q0 + r)) + 2 * c;
+        x[u][0] = __ldg(src);
+        x[u][1] = __ldg(src + 1);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) put_split(base + kOffQ, kPieceQ, (tid >> 3) + 32 * u, tid & 7, x[u][0], x[u][1]);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const bool leave = *leave_slot != 0;
+  const int nt = leave ? 0 : tiles * ((int)blockIdx.z + 1) / n_split - lo;
+  const uint32_t tmem = *tmem_slot;
+  float *rows_out = reinterpret_cast<float *>(smem_raw + kOffQ);               // [row][64], 16-byte pieces permuted by the row
+  float2 *stat_out = reinterpret_cast<float2 *>(smem_raw + kOffStat);
+
+  if (warp >= 4) {
+    // ---------------------------------------------------------------- operands
+    const int ct = tid - 128, c = ct & 7, r0 = ct >> 3;
+    auto load = [&](bool values, int tile, float4 (&x)[4][2]) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int slot = tile * kKeys + r0 + 16 * u;
+        x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (slot < L) {
+          const float4 *src = reinterpret_cast<const float4 *>(entry(prm, values, slice, b, h, hist, slot)) + 2 * c;
+          x[u][0] = src[0];
+          x[u][1] = src[1];
+        }
+      }
+    };
+    auto put = [&](bool values, int tile, const float4 (&x)[4][2]) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) put_split(base + (values ? kOffV : kOffK), kPieceK, r0 + 16 * u, c, x[u][0], x[u][1]);
+      if (prm.copy_in && tile * kKeys + kKeys > hist && tile % (int)gridDim.x == (int)blockIdx.x) {      // (the CTAs of a slice take turns)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int slot = tile * kKeys + r0 + 16 * u;
+          if (slot < hist || slot >= L) continue;
+          const size_t row = slot_row(lv, slice, slot);
+          float4 *dst = reinterpret_cast<float4 *>((values ? lv.v_pool : lv.k_pool) + row * 256) + 2 * c;
+          dst[0] = x[u][0];
+          dst[1] = x[u][1];
+          if (!values && c == 0) lv.pos_pool[row] = prm.n_prev + slot - hist;
+        }
+      }
+    };
+    auto announce = [&] {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(bar_ops);
+    };
+    float4 kx[4][2], vx[4][2];
+    if (nt > 0) {
+      load(false, lo, kx);
+      load(true, lo, vx);
+      put(false, lo, kx);
+      announce();
+      if (nt > 1) load(false, lo + 1, kx);
+      put(true, lo, vx);
+    }
+    for (int i = 0; i < nt; ++i) {
+      if (!tc::mbar_wait_warp(bar_mma, i & 1, abort_flag, status)) break;      // K_i and V_{i-1} have been read
+      if (i > 0) put(true, lo + i, vx);
+      if (i + 1 < nt) put(false, lo + i + 1, kx);
+      announce();
+      if (i + 1 < nt) load(true, lo + i + 1, vx);
+      if (i + 2 < nt) load(false, lo + i + 2, kx);
+    }
+  } else {
+    // ---------------------------------------------------------------- softmax
+    constexpr uint32_t dhi = tc::desc_hi(1024);
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);    // bf16, N = 64, M = 128
+    constexpr uint32_t idesc_pv = idesc | (1u << 16);                                                            // B is MN-major
+    const uint32_t q_lo = tc::desc_lo(base + kOffQ, 16), k_lo = tc::desc_lo(base + kOffK, 16), v_lo = tc::desc_lo(base + kOffV, 16);
+    // products of pieces, the smallest first
+    auto mma_s = [&] {
+      constexpr int A[6] = {2, 0, 1, 1, 0, 0}, B[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+      for (int e = 0; e < 6; ++e) mma4_ss(tmem + kColS, q_lo + A[e] * (kPieceQ >> 4), k_lo + B[e] * (kPieceK >> 4), dhi, idesc, e > 0);
+    };
+    auto mma_pv = [&] {
+      constexpr int A[6] = {2, 0, 1, 1, 0, 0}, B[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+      for (int e = 0; e < 6; ++e) mma4_ts(tmem + kColO, tmem + kColP + 32 * A[e], v_lo + B[e] * (kPieceK >> 4), dhi, idesc_pv, e > 0);
+    };
+    const int row = warp * 32 + lane;
+    const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
+    const float c = prm.scale_log2e;
+    float *win_row = nullptr;
+    int rank = -1;
+    if (prm.win_logits != nullptr)
+      for (int e = 0; e < prm.w; ++e)
+        if (prm.win_pos[e] == q0 + row) rank = e;
+    if (rank >= 0) win_row = prm.win_logits + ((size_t)slice * prm.w + rank) * prm.ld_l;
+    const bool wwarp = __any_sync(0xffffffffu, rank >= 0);
+    uint64_t o[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) o[i] = 0ull;
+    float m = kNoMax, l = 0.f, l_rest = 0.f;       // l_rest: what the additions to l have rounded off
+    auto add_products = [&] {            // of P with a tile of V
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t x[16];
+        tc::tc_ld16(lane_addr + kColO + 16 * e, x);
+        tc::tc_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[8 * e + i] = tc::add2(o[8 * e + i], tc::pack2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])));
+      }
+    };
+    bool ok = true;
+    if (warp == 0 && nt > 0) {
+      ok = tc::mbar_wait_warp(bar_ops, 0, abort_flag, status);
+      tc_fence_after();
+      if (ok) {
+        mma_s();
+        if (tc::elect_one()) tc::tc_commit(bar_mma);
+      }
+      __syncwarp();
+    }
+    int issued = ok && nt > 0 ? 1 : 0;   // commits of warp 0
+    for (int i = 0; i < nt; ++i) {
+      // (a warp whose wait gives up goes on to meet the others at the named barrier, which knows no limit)
+      ok = ok && tc::mbar_wait_warp(bar_mma, i & 1, abort_flag, status);
+      if (ok) {
+        tc_fence_after();
+        if (i > 0) add_products();
+        const int valid = L - (lo + i) * kKeys;
+        float mx = m;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          uint32_t x[16];
+          tc::tc_ld16(lane_addr + kColS + 16 * e, x);
+          tc::tc_wait_ld();
+          if (wwarp) {
+            // (columns beyond the last key: zeros that nobody reads)
+            if (win_row != nullptr) {
+              float4 *dst = reinterpret_cast<float4 *>(win_row + (lo + i) * kKeys + 16 * e);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                auto whole = [&](int e2) { const float s = __uint_as_float(x[4 * q + e2]); return fmaf(s, kCutOff, s); };
+                dst[q] = make_float4(whole(0), whole(1), whole(2), whole(3));
+              }
+            }
+            __syncwarp();
+          }
+#pragma unroll
+          for (int q = 0; q < 16; q += 2) {
+            const float y0 = 16 * e + q < valid ? __uint_as_float(x[q]) * c : kNoMax, y1 = 16 * e + q + 1 < valid ? __uint_as_float(x[q + 1]) * c : kNoMax;
+            mx = tc::max3(mx, y0, y1);
+          }
+        }
+        if (__any_sync(0xffffffffu, mx > m)) {
+          const float f = tc::ex2(m - mx);
+          const uint64_t ff = tc::pack2(f, f);
+#pragma unroll
+          for (int q = 0; q < 32; ++q) o[q] = tc::mul2(o[q], ff);
+          l *= f;
+          l_rest *= f;
+          m = mx;
+        }
+        const uint64_t c2 = tc::pack2(c, c), lost2 = tc::pack2(c * kCutOff, c * kCutOff), negm2 = tc::pack2(-m, -m);
+        uint64_t sum2[2] = {0ull, 0ull};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          uint32_t x[16], ph[8], pm[8], pl[8];
+          tc::tc_ld16(lane_addr + kColS + 16 * e, x);
+          tc::tc_wait_ld();
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            float a0, a1;
+            const uint64_t s2 = tc::pack2(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1]));
+            tc::unpack2(tc::fma2(s2, c2, tc::fma2(s2, lost2, negm2)), a0, a1);
+            a0 = 16 * e + 2 * q < valid ? tc::ex2(a0) : 0.f;
+            a1 = 16 * e + 2 * q + 1 < valid ? tc::ex2(a1) : 0.f;
+            sum2[q & 1] = tc::add2(sum2[q & 1], tc::pack2(a0, a1));
+            split2(a0, a1, ph[q], pm[q], pl[q]);
+          }
+          tc_st8(lane_addr + kColP + 8 * e, ph);
+          tc_st8(lane_addr + kColP + 32 + 8 * e, pm);
+          tc_st8(lane_addr + kColP + 64 + 8 * e, pl);
+        }
+        float s0, s1, s2, s3;
+        tc::unpack2(sum2[0], s0, s1);
+        tc::unpack2(sum2[1], s2, s3);
+        const float add = (s0 + s1) + (s2 + s3), sum = l + add, part = sum - l;
+        l_rest += (l - (sum - part)) + (add - part);
+        l = sum;
+        tc::tc_wait_st();
+        tc_fence_before();
+      }
+      asm volatile("bar.sync 2, 128;" ::: "memory");
+      if (warp == 0) {
+        ok = ok && tc::mbar_wait_warp(bar_ops, (i + 1) & 1, abort_flag, status);
+        if (ok) {
+          tc_fence_after();
+          mma_pv();
+          if (i + 1 < nt) mma_s();
+          if (tc::elect_one()) tc::tc_commit(bar_mma);
+          ++issued;
+        }
+        __syncwarp();
+      }
+    }
+    if (warp == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (nt > 0) ok = ok && tc::mbar_wait_warp(bar_mma, nt & 1, abort_flag, status);
+    tc_fence_after();
+    if (ok && nt > 0) add_products();
+    // (given up: what has been issued must be through before TMEM and shared memory are anybody else's)
+    if (!ok && warp == 0 && issued > 0) tc::mbar_drain(bar_mma, (issued - 1) & 1);
+    l += l_rest;
+    float *mine = rows_out + row * 64;
+    float amax = 0.f;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      float x0, x1, x2, x3;
+      tc::unpack2(o[2 * q], x0, x1);
+      tc::unpack2(o[2 * q + 1], x2, x3);
+      amax += (x0 - x0) + (x1 - x1) + (x2 - x2) + (x3 - x3);      // zero, unless one of them is not a number
+      *reinterpret_cast<float4 *>(mine + ((q ^ (row & 7)) << 2)) = make_float4(x0, x1, x2, x3);
+    }
+    if (nt > 0 && ok && q0 + row < n_k && !(amax == 0.f && l > 0.f && l < INFINITY)) {
+      const RowSum s = fma_row(prm, slice, b, h, hist, q0 + row, lo * kKeys, min((lo + nt) * kKeys, L), mine, row & 7, win_row);
+      m = s.m;
+      l = s.l;
+    }
+    stat_out[row] = make_float2(m, l);
+    if (n_split == 1 && ok && nt > 0 && q0 + row < n_k) {
+      if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + row] = row_lse_f32(m, l);
+      if (rank >= 0) prm.win_lse[(size_t)slice * prm.w + rank] = m + log2f(l);
+    }
+    tc_fence_before();
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+  const int ty = tid >> 4, tx = tid & 15, rows = min(kRows, n_k - q0);
+  if (n_split == 1) {
+    if (leave || *abort_flag) return;
+    for (int r = ty; r < rows; r += 16) {
+      const float inv = 1.f / stat_out[r].y;
+      const float4 x = *reinterpret_cast<const float4 *>(rows_out + r * 64 + ((tx ^ (r & 7)) << 2));
+      *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(prm.O, b, h, q0 + r)) + tx * 4) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
+    }
+    return;
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  auto peer = [&](const void *p, int cta) { return tc::remote((uint32_t)__cvta_generic_to_shared(p), cta); };
+  const int r_lo = rows * (int)blockIdx.z / n_split, r_hi = leave ? r_lo : rows * ((int)blockIdx.z + 1) / n_split;
+  for (int r = r_lo + ty; r < r_hi; r += 16) {
+    float4 x[kMaxSplit];
+    float me[kMaxSplit], le[kMaxSplit], M = kNoMax;
+#pragma unroll
+    for (int e = 0; e < kMaxSplit; ++e) {
+      x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      me[e] = kNoMax; le[e] = 0.f;
+      if (e < n_split) {
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(me[e]), "=f"(le[e]) : "r"(peer(stat_out + r, e)));
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[e].x), "=f"(x[e].y), "=f"(x[e].z), "=f"(x[e].w)
+                     : "r"(peer(rows_out + r * 64 + ((tx ^ (r & 7)) << 2), e)));
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < kMaxSplit; ++e) M = fmaxf(M, me[e]);
+    float sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+    for (int e = 0; e < kMaxSplit; ++e) {
+      const float f = exp2f(me[e] - M);
+      sum = fmaf(f, le[e], sum);
+      a0 = fmaf(f, x[e].x, a0); a1 = fmaf(f, x[e].y, a1); a2 = fmaf(f, x[e].z, a2); a3 = fmaf(f, x[e].w, a3);
+    }
+    const float inv = 1.f / sum;
+    *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(prm.O, b, h, q0 + r)) + tx * 4) = make_float4(a0 * inv, a1 * inv, a2 * inv, a3 * inv);
+    if (tx == 0) {
+      if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + r] = row_lse_f32(M, sum);
+      if (prm.win_logits != nullptr)
+        for (int e = 0; e < prm.w; ++e)
+          if (prm.win_pos[e] == q0 + r) prm.win_lse[(size_t)slice * prm.w + e] = M + log2f(sum);
+    }
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// CTAs that share a slice's keys.  ctas: CTAs of an unsplit launch.  In steps of a key tile: a CTA that has its SM to itself takes 1 per
+// tile, two that share one 1.35 each.
+inline int key_split(int ctas, int tiles, int n_sm) {
+  auto cost = [&](int c) {
+    const int n = ctas * c, per = (tiles + c - 1) / c, waves = (n + 2 * n_sm - 1) / (2 * n_sm);
+    return (n <= n_sm ? 1.f : 1.35f) * (float)(waves * (per + 3)) + (c > 1 ? 1.5f : 0.f);
+  };
+  int split = 1;
+  for (int c = 2; c <= kMaxSplit && c <= tiles; ++c)
+    if (cost(c) < cost(split)) split = c;
+  return split;
+}
+
+}  // namespace f32
+}  // namespace scalekv

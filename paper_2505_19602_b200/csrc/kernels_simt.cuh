@@ -1,5 +1,4 @@
-// Kernels of the ScaleKV hot path beside the tensor-core attention: append, fp32-FMA attention (the f32 x 64 configuration),
-// observation-window scoring, per-slice top-k, in-place gather-compaction and the offline layer statistics.
+// Kernels of the ScaleKV hot path beside the attention: append, observation-window scoring, per-slice top-k, in-place gather-compaction and the offline layer statistics.
 #pragma once
 #include <cfloat>
 
@@ -63,268 +62,7 @@ __global__ void commit_kernel(LayerView lv, int n_k) {
   if (s < lv.n_slices) lv.next_len[s] = lv.hist_len[s] + n_k;
 }
 
-// ------------------------------------------------------------------------------------------
-// attend, f32 x 64: O = softmax(scale * Q K^T) V with online softmax, fp32 FMA throughout (Eq. 5; the 1e-4 bound on outputs
-// rules TF32 out).  A CTA of 256 threads owns 128 query rows of one slice and streams its keys in tiles of 64; thread (ty, tx) owns
-// rows 8 ty .. 8 ty + 7 and keys, then output columns, 4 tx .. 4 tx + 3, all accumulators packed over pairs of rows.  Q, K and P
-// lie transposed in shared memory, so that both products read, per key column (per key), 8 rows and 4 keys (columns) with three
-// 16-byte loads for 16 packed multiply-adds of 2 cycles each: the FMA pipe bounds them.  Packing over the rows keeps the scores
-// in 32 registers (over columns they take 64), so that 16 warps of an SM cover the latencies.  K arrives (asynchronous
-// copies) under P V and is transposed from there, V arrives under S; a warp only reads P that it has written itself.
-// gridDim.z CTAs of a cluster share a slice's keys; each then combines a share of the rows,
-// O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e, reading the parts through distributed shared memory.
-// 16 slices, us per launch averaged over four layers, 64/144/256/400/576/1024/1600 queries: 22.8/40.6/61/85/120/244/479 with
-// 4 x 4 register tiles and scalar operands of P V, 15.3/18.8/26/54/93/187/363 with 64 rows per CTA packed over columns (FMA pipe
-// 55 % busy, 2.3 warps per scheduler), 17/21.6/29/51/84/169/330 here (68 %, shared-memory wavefronts 65 %).
-// grid (ceil(n_k / 128), n_slices, split); dynamic shared memory kAttendF32Smem (two CTAs per SM).
-// ------------------------------------------------------------------------------------------
-constexpr int kF32Rows = 128;
-constexpr int kAttendF32Smem = (64 * kF32Rows + 3 * 64 * 64 + 64 * kF32Rows) * 4;
-constexpr int kF32MaxSplit = 8;
 constexpr float kNoMax = -FLT_MAX;       // a finite stand-in for -inf, so that differences of maxima are numbers; no finite score lies below
-
-__device__ __forceinline__ uint64_t pair_fma(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t pair_mul(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t pair_of(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 pair_parts(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-
-// The log-sum-exp of a row from its base-2 reference and sum: the logarithm is taken to base e and the sum rounded once (to base 2
-// both are of larger numbers), and what the 32-bit log2(e) in the reference is off by, 1.3e-8 of it, is put right.  rms error over
-// full caches of 521 to 4 240 entries, scores of deviation 0.25 / 1 / 3: 2.0 to 2.8e-7 / 1.9 to 3.0e-7 / 5.5 to 5.9e-7 (to base e
-// throughout 2.0 to 2.8 / 1.9 to 3.2 / 5.4 to 5.8; to base 2 throughout 2.6 to 3.6 / 2.7 to 3.7 / 6.5 to 6.7).
-__device__ __forceinline__ float row_lse_f32(float m, float l) {
-  return fmaf(m, 0.6931471805599453f, fmaf(m, (float)(1.0 / 1.4426950408889634f - 0.6931471805599453f), logf(l)));
-}
-
-__global__ void __launch_bounds__(256, 2) attend_f32_kernel(LayerView lv, TensorView Q, TensorView O, float *lse, int n_k, int room,
-                                                            float scale_log2e) {
-  extern __shared__ __align__(16) float sm_f32[];
-  float *Qt = sm_f32;                     // [column][row]
-  float *Kt = Qt + 64 * kF32Rows;         // [column][key]
-  float *Kr = Kt + 64 * 64;               // [key][column], as it arrives; chunks permuted by the key
-  float *Vs = Kr + 64 * 64;               // [key][column]
-  float *Pt = Vs + 64 * 64;               // [key][row], chunks permuted by the key
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ty = tid >> 4, tx = tid & 15;
-  const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
-  const int q0 = blockIdx.x * kF32Rows;
-  // room: entries that a slice's pages hold.  The append before this launch has reported a slice that outgrows them; here it is cut
-  // off, so that no slot behind the page table is looked up.  (Leaving instead, as the other kernels do, made the compiler order the
-  // products worse: 16 slices x 1 024 queries behind 1 960 entries 358 -> 371 us; cut off 359.)
-  const int L = min(lv.hist_len[slice] + n_k, room);
-  if (blockIdx.x == 0 && blockIdx.z == 0 && tid == 0) lv.next_len[slice] = L;     // unless a compress of this scale evicts
-  const int n_split = gridDim.z, tiles = (L + 63) >> 6;
-  const int t_lo = tiles * (int)blockIdx.z / n_split, t_hi = tiles * ((int)blockIdx.z + 1) / n_split;
-  auto fetch = [&](float *tile, const char *pool, int t, bool permute) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = u * 16 + ty, slot = t * 64 + r;
-      float *dst = tile + r * 64 + (permute ? tx ^ (r & 7) : tx) * 4;
-      if (slot < L)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-                     "l"(pool + slot_row(lv, slice, slot) * 256 + tx * 16)
-                     : "memory");
-      else
-        *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  if (t_lo < t_hi) fetch(Kr, lv.k_pool, t_lo, true);
-  // Q: a warp transposes 32 rows, four columns at a time
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const int r = (warp & 3) * 32 + lane, c = (warp >> 2) * 8 + u;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (q0 + r < n_k) v = reinterpret_cast<const float4 *>(row_ptr<float>(Q, b, h, q0 + r))[c];
-    Qt[(4 * c + 0) * kF32Rows + r] = v.x;
-    Qt[(4 * c + 1) * kF32Rows + r] = v.y;
-    Qt[(4 * c + 2) * kF32Rows + r] = v.z;
-    Qt[(4 * c + 3) * kF32Rows + r] = v.w;
-  }
-  uint64_t o[4][4];                       // [pair of rows][column]
-  float m[8], l[8];                       // l: this thread's keys only
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) o[i][j] = 0ull;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { m[i] = kNoMax; l[i] = 0.f; }
-  // one step of either product: 8 rows (two 16-byte loads) times 4 keys or columns
-  auto step = [&](uint64_t (&acc)[4][4], const float *a0, const float *a1, const float *bv) {
-    const ulonglong2 r0 = *reinterpret_cast<const ulonglong2 *>(a0), r1 = *reinterpret_cast<const ulonglong2 *>(a1);
-    const float4 x = *reinterpret_cast<const float4 *>(bv);
-    const uint64_t rows[4] = {r0.x, r0.y, r1.x, r1.y};
-    const uint64_t cols[4] = {pair_of(x.x, x.x), pair_of(x.y, x.y), pair_of(x.z, x.z), pair_of(x.w, x.w)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = pair_fma(rows[i], cols[j], acc[i][j]);
-  };
-
-  for (int t = t_lo; t < t_hi; ++t) {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();                      // K has arrived (and V has been read)
-    fetch(Vs, lv.v_pool, t, false);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {         // a warp transposes 32 keys, four columns at a time
-      const int r = (warp & 1) * 32 + lane, c = (warp >> 1) * 4 + u;
-      const float4 v = *reinterpret_cast<const float4 *>(Kr + r * 64 + (c ^ (r & 7)) * 4);
-      Kt[(4 * c + 0) * 64 + r] = v.x;
-      Kt[(4 * c + 1) * 64 + r] = v.y;
-      Kt[(4 * c + 2) * 64 + r] = v.z;
-      Kt[(4 * c + 3) * 64 + r] = v.w;
-    }
-    __syncthreads();
-    if (t + 1 < t_hi) fetch(Kr, lv.k_pool, t + 1, true); else asm volatile("cp.async.commit_group;" ::: "memory");
-    uint64_t s2[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s2[i][j] = 0ull;
-#pragma unroll 4
-    for (int c = 0; c < 64; ++c) step(s2, Qt + c * kF32Rows + ty * 8, Qt + c * kF32Rows + ty * 8 + 4, Kt + c * 64 + tx * 4);
-    const int valid = L - t * 64;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float y[2][4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 e = pair_parts(s2[i][j]);
-        const bool real = tx * 4 + j < valid;
-        y[0][j] = real ? e.x * scale_log2e : -INFINITY;
-        y[1][j] = real ? e.y * scale_log2e : -INFINITY;
-      }
-      float f[2];
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const int q = 2 * i + r;
-        float mx = fmaxf(fmaxf(y[r][0], y[r][1]), fmaxf(y[r][2], y[r][3]));
-#pragma unroll
-        for (int d = 8; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-        mx = fmaxf(mx, m[q]);
-        f[r] = exp2f(m[q] - mx);
-        m[q] = mx;
-        float sum = 0.f;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          y[r][j] = exp2f(y[r][j] - mx);
-          sum += y[r][j];
-        }
-        l[q] = l[q] * f[r] + sum;
-      }
-      const uint64_t ff = pair_of(f[0], f[1]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        o[i][j] = pair_mul(o[i][j], ff);
-        s2[i][j] = pair_of(y[0][j], y[1][j]);
-      }
-    }
-    // P of key 4 tx + j: rows 8 ty .. as two chunks, permuted by the key's group of four
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int half = 0; half < 2; ++half)
-        *reinterpret_cast<ulonglong2 *>(Pt + (tx * 4 + j) * kF32Rows + ((ty * 2 + half) ^ (tx & 7)) * 4) =
-            make_ulonglong2(s2[2 * half][j], s2[2 * half + 1][j]);
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();                      // V has arrived
-#pragma unroll 4
-    for (int k = 0; k < 64; ++k) {
-      const float *p = Pt + k * kF32Rows;
-      const int x = (k >> 2) & 7;
-      step(o, p + ((ty * 2) ^ x) * 4, p + ((ty * 2 + 1) ^ x) * 4, Vs + k * 64 + tx * 4);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int d = 8; d > 0; d >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], d);
-
-  if (n_split == 1) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = q0 + ty * 8 + i;
-      if (r >= n_k) continue;
-      const float inv = 1.f / l[i];
-      float x[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 e = pair_parts(o[i >> 1][j]);
-        x[j] = ((i & 1) ? e.y : e.x) * inv;
-      }
-      *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, r)) + tx * 4) = make_float4(x[0], x[1], x[2], x[3]);
-      if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + r] = row_lse_f32(m[i], l[i]);
-    }
-    return;
-  }
-  // the parts: rows of 64 columns where Q was, references and sums where K was
-  __syncthreads();
-  float *part = Qt, *m_s = Kt, *l_s = Kt + kF32Rows;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float x[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 e = pair_parts(o[i >> 1][j]);
-      x[j] = (i & 1) ? e.y : e.x;
-    }
-    *reinterpret_cast<float4 *>(part + (ty * 8 + i) * 64 + tx * 4) = make_float4(x[0], x[1], x[2], x[3]);
-    if (tx == 0) { m_s[ty * 8 + i] = m[i]; l_s[ty * 8 + i] = l[i]; }
-  }
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  auto peer = [&](const float *p, int cta) {
-    uint32_t ra;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(cta));
-    return ra;
-  };
-  const int rows = min(kF32Rows, n_k - q0);
-  const int r_lo = rows * (int)blockIdx.z / n_split, r_hi = rows * ((int)blockIdx.z + 1) / n_split;
-  for (int r = r_lo + ty; r < r_hi; r += 16) {
-    float4 x[kF32MaxSplit];
-    float me[kF32MaxSplit], le[kF32MaxSplit], M = kNoMax;
-#pragma unroll
-    for (int e = 0; e < kF32MaxSplit; ++e) {
-      x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-      me[e] = kNoMax; le[e] = 0.f;
-      if (e < n_split) {
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(me[e]) : "r"(peer(m_s + r, e)));
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(le[e]) : "r"(peer(l_s + r, e)));
-        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[e].x), "=f"(x[e].y), "=f"(x[e].z), "=f"(x[e].w)
-                     : "r"(peer(part + r * 64 + tx * 4, e)));
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < kF32MaxSplit; ++e) M = fmaxf(M, me[e]);
-    float sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-    for (int e = 0; e < kF32MaxSplit; ++e) {
-      const float f = exp2f(me[e] - M);
-      sum = fmaf(f, le[e], sum);
-      a0 = fmaf(f, x[e].x, a0); a1 = fmaf(f, x[e].y, a1); a2 = fmaf(f, x[e].z, a2); a3 = fmaf(f, x[e].w, a3);
-    }
-    const float inv = 1.f / sum;
-    *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(O, b, h, q0 + r)) + tx * 4) = make_float4(a0 * inv, a1 * inv, a2 * inv, a3 * inv);
-    if (lse != nullptr && tx == 0) lse[(size_t)slice * n_k + q0 + r] = row_lse_f32(M, sum);
-  }
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
 
 template <typename T, int D>
 __device__ __forceinline__ void load_tile_rows(float *dst, int ld, const LayerView &lv, const char *pool, int slice,

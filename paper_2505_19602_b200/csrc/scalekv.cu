@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/scalekv.h"
+#include "attend_f32.cuh"
 #include "attend_tc.cuh"
 #include "kernels_simt.cuh"
 
@@ -505,7 +506,7 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
       ok = ok && set_smem(layer_stats_kernel<__nv_bfloat16, 128>, layer_stats_smem_bytes<128>(64));
     } else {
       ok = ok && set_smem(layer_stats_kernel<float, 64>, layer_stats_smem_bytes<64>(64));
-      ok = ok && set_smem(attend_f32_kernel, kAttendF32Smem);
+      ok = ok && set_smem(f32::attend_f32_tc_kernel, f32::kSmemBytes);
       ok = ok && set_smem(score_logits_kernel<float, 64>, 2 * 64 * 68 * 4);
     }
     // select and compact stage a slice in shared memory when it fits and work from global memory when it does not
@@ -583,7 +584,8 @@ scalekv_status scalekv_destroy(scalekv_ctx *ctx) {
   return SCALEKV_OK;
 }
 
-scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor K, scalekv_tensor V) {
+// defer: the map stays in the caller's tensors, from where the attend that follows takes it.
+static scalekv_status append_impl(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor K, scalekv_tensor V, bool defer) {
   if (!ctx) return SCALEKV_ERR_INVALID_ARG;
   const Plan &p = ctx->plan;
   if (layer < 0 || layer >= p.n_layers) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "layer %d out of range", layer);
@@ -636,8 +638,8 @@ scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, sc
   const int nk = p.n[scale];
   if (ctx->hist[layer] + nk > p.layers[layer].total_pages * p.P)
     return fail(ctx, SCALEKV_ERR_CAPACITY, "layer %d: %d + %d entries exceed the planned capacity", layer, ctx->hist[layer], nk);
-  if (ctx->tc.enabled()) {
-    // the tensor-core attend reads the map from K and V and copies it into the pages as it goes
+  if (defer) {
+    // attend reads the map from K and V and copies it into the pages as it goes
     ctx->pend_k[layer] = K;
     ctx->pend_v[layer] = V;
     ctx->in_store[layer] = 0;
@@ -653,6 +655,10 @@ scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, sc
   ctx->next_scale[layer] = scale + 1;
   ctx->set_owner[par] = layer;
   return check_launch(ctx, "append");
+}
+
+scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor K, scalekv_tensor V) {
+  return append_impl(ctx, layer, scale, K, V, ctx && ctx->tc.enabled());
 }
 
 // record: whether the kernel should also record the logits of the scale's planned observation window for a compress
@@ -673,60 +679,57 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
   if (ctx->pending[layer] == 0) return fail(ctx, SCALEKV_ERR_BAD_STATE, "layer %d: attend needs a preceding append", layer);
   if (!tensor_ok(Q, p.esize) || !tensor_ok(O, p.esize)) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "Q/O null or rows not 16-byte aligned");
   const int nk = ctx->pending[layer];
-  LayerView lv = layer_view(ctx, layer);
-  if (!ctx->tc.enabled()) {
-    scalekv_status st = materialize(ctx, layer);
-    if (st != SCALEKV_OK) return st;
-  }
+  const LayerView lv = layer_view(ctx, layer);
   {
     Scope sc(ctx, ctx->s_main, kAttend);
+    const bool fused = !ctx->in_store[layer];
+    TensorView kc{}, vc{};
+    if (fused) { kc = tview(ctx->pend_k[layer]); vc = tview(ctx->pend_v[layer]); }
+    const int k = ctx->next_scale[layer] - 1;
+    const std::vector<int> &win = p.windows[k];
+    float *wl = (win.empty() || !record || k + 1 == p.K)
+                    ? nullptr
+                    : reinterpret_cast<float *>(ctx->ws + p.off_logits) + (size_t)(layer % kSets) * p.logits_elems;
+    float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
+    // What it records goes where a compress of another layer of the set may still score: append has waited for this layer's
+    // and the owner's compresses, not for one that was called behind it.
+    const int cl = ctx->set_compressed[layer % kSets];
+    if (wl && cl >= 0 && ctx->ev_compress_live[cl] && ctx->compress_no[cl] > ctx->main_behind) {
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_compress[cl], 0));
+      ctx->main_behind = ctx->compress_no[cl];
+    }
     if (ctx->tc.enabled()) {
       std::string e;
-      const bool fused = !ctx->in_store[layer];
-      TensorView kc, vc;
-      if (fused) { kc = tview(ctx->pend_k[layer]); vc = tview(ctx->pend_v[layer]); }
-      const int k = ctx->next_scale[layer] - 1;
-      const std::vector<int> &win = p.windows[k];
-      float *wl = (win.empty() || !record || k + 1 == p.K)
-                      ? nullptr
-                      : reinterpret_cast<float *>(ctx->ws + p.off_logits) + (size_t)(layer % kSets) * p.logits_elems;
-      float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
-      // What it records goes where a compress of another layer of the set may still score: append has waited for this layer's
-      // and the owner's compresses, not for one that was called behind it.
-      const int cl = ctx->set_compressed[layer % kSets];
-      if (wl && cl >= 0 && ctx->ev_compress_live[cl] && ctx->compress_no[cl] > ctx->main_behind) {
-        CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_compress[cl], 0));
-        ctx->main_behind = ctx->compress_no[cl];
-      }
       if (!ctx->tc.launch(lv, tview(Q), tview(O), lse, nk, fused ? &kc : nullptr, fused ? &vc : nullptr, fused && copy, ctx->hist[layer], p.N[k],
                           ctx->scale, wl, wlse, p.ld_l, win.data(), (int)win.size(), ctx->s_main, e))
         return fail(ctx, SCALEKV_ERR_CUDA, "attend launch: %s", e.c_str());
-      if (copy) ctx->in_store[layer] = 1;
-      ctx->logits_of[layer] = wl ? k : -1;
-      ctx->logits_padded[layer] = fused ? 1 : 0;
     } else {
-      // CTAs that share a slice's keys: so that the SM with the most work has as little of it as possible, if its CTAs ran one after
-      // another.  us per launch, 16 slices behind 209 / 1 960 entries, unsplit -> as here (best of 1 to 8): 64 queries 43.8 / 251.5 ->
-      // 13.4 / 61.2 (13.0 / 51.7), 256: 67.4 / 276.9 -> 22.9 / 77.3 (22.9 / 77.2), 576: 106.3 / 315.6 -> 77.0 / 175.8 (the same), 1 600:
-      // 402.6 / 771.0 -> 318.8 / 584.3 (318.8 / 575.7).  Two CTAs of an SM do run together, so it is off where that decides: 16 slices
-      // x 1 024 160.7 / 370.1, unsplit (by two CTAs 146.8 / 336.9); 48 x 256 behind 209 73.4 (unsplit 67.4, by four 53.3).
-      const int blocks = (nk + kF32Rows - 1) / kF32Rows, ctas = blocks * p.n_slices, tiles = (ctx->hist[layer] + nk + 63) / 64;
-      int split = 1;
-      auto load = [&](int c) { return (float)((ctas * c + ctx->n_sm - 1) / ctx->n_sm) * ((float)((tiles + c - 1) / c) + 1.5f); };   // in key tiles; its queries and its end cost a CTA 1.5 more
-      for (int c = 2; c <= kF32MaxSplit && c <= tiles; ++c)
-        if (load(c) < load(split)) split = c;
+      f32::Params prm{};
+      prm.lv = lv; prm.Q = tview(Q); prm.O = tview(O); prm.K = kc; prm.V = vc; prm.lse = lse; prm.n_k = nk;
+      prm.room = lv.pages_per_slice << lv.page_shift;
+      prm.fused = fused ? 1 : 0; prm.copy_in = (fused && copy) ? 1 : 0; prm.n_prev = p.N[k];
+      prm.scale_log2e = ctx->scale * 1.4426950408889634f;
+      prm.win_logits = wl; prm.win_lse = wlse; prm.ld_l = p.ld_l; prm.w = wl ? (int)win.size() : 0;
+      for (int e = 0; e < prm.w; ++e) prm.win_pos[e] = win[e];
+      const int blocks = (nk + f32::kRows - 1) / f32::kRows;
+      const int split = f32::key_split(blocks * p.n_slices, (ctx->hist[layer] + nk + f32::kKeys - 1) / f32::kKeys, ctx->n_sm);
       cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute attr[1];
+      cudaLaunchAttribute attr[2];
       cfg.gridDim = dim3(blocks, p.n_slices, split);
-      cfg.blockDim = dim3(256);
-      cfg.dynamicSmemBytes = kAttendF32Smem;
+      cfg.blockDim = dim3(f32::kThreads);
+      cfg.dynamicSmemBytes = f32::kSmemBytes;
       cfg.stream = ctx->s_main;
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)split;
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      attr[1].id = cudaLaunchAttributeClusterDimension;
+      attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = (unsigned)split;
       cfg.attrs = attr;
-      cfg.numAttrs = split > 1 ? 1 : 0;
-      CU(cudaLaunchKernelEx(&cfg, attend_f32_kernel, lv, tview(Q), tview(O), lse, nk, lv.pages_per_slice << lv.page_shift, ctx->scale * 1.4426950408889634f));
+      cfg.numAttrs = split > 1 ? 2 : 1;
+      CU(cudaLaunchKernelEx(&cfg, f32::attend_f32_tc_kernel, prm));
     }
+    if (copy) ctx->in_store[layer] = 1;
+    ctx->logits_of[layer] = wl ? k : -1;
+    ctx->logits_padded[layer] = fused && ctx->tc.enabled() ? 1 : 0;
   }
   ctx->attended[layer] = 1;
   ctx->len_written[layer] = 1;
@@ -1012,11 +1015,13 @@ scalekv_status scalekv_step_host(scalekv_ctx *ctx, int32_t layer, int32_t scale,
 // the pages (the logits of exactly its window recorded, or a positional rule), so that it can take the map's
 // surviving rows from K and V itself; nor after the last scale without a compress, when nothing may ever need the rows.
 // A wrong guess costs a copy kernel, never a result.
-static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, bool compress, int w, const int32_t *window_pos,
-                        const scalekv_select_opts *opts) {
-  if (!ctx || !ctx->tc.enabled() || layer < 0 || layer >= ctx->plan.n_layers || scale < 0 || scale >= ctx->plan.K) return true;
+static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, const scalekv_tensor &K, const scalekv_tensor &V, bool compress, int w,
+                        const int32_t *window_pos, const scalekv_select_opts *opts) {
+  if (!ctx || layer < 0 || layer >= ctx->plan.n_layers || scale < 0 || scale >= ctx->plan.K) return true;
   const Plan &p = ctx->plan;
   if (!compress) return scale + 1 != p.K;
+  // (a compress that takes rows from the tensors wants K and V laid out alike; of f32 maps others have always been taken)
+  if (!ctx->tc.enabled() && (K.stride_b != V.stride_b || K.stride_h != V.stride_h || K.stride_t != V.stride_t)) return true;
   if (!ctx->fused_ok || (opts && (opts->head_shared || opts->separate_kernels || opts->head_budgets))) return true;
   const int table = p.budgets[(size_t)layer * p.K + scale];
   if (table == SCALEKV_KEEP_ALL) return true;
@@ -1033,9 +1038,9 @@ static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, bool compr
 
 scalekv_status scalekv_step(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor Q, scalekv_tensor K, scalekv_tensor V,
                             scalekv_tensor O, float *lse, int32_t w, const int32_t *window_pos) {
-  scalekv_status st = scalekv_append(ctx, layer, scale, K, V);
+  scalekv_status st = append_impl(ctx, layer, scale, K, V, true);
   if (st != SCALEKV_OK) return st;
-  st = attend_impl(ctx, layer, Q, O, lse, w > 0, step_copies(ctx, layer, scale, w != 0, w, window_pos, nullptr));
+  st = attend_impl(ctx, layer, Q, O, lse, w > 0, step_copies(ctx, layer, scale, K, V, w != 0, w, window_pos, nullptr));
   if (st != SCALEKV_OK) return st;
   if (w > 0) return scalekv_compress(ctx, layer, Q, w, window_pos, 1);
   if (w < 0) return scalekv_compress(ctx, layer, Q, 0, nullptr, 1);
@@ -1045,11 +1050,11 @@ scalekv_status scalekv_step(scalekv_ctx *ctx, int32_t layer, int32_t scale, scal
 scalekv_status scalekv_step_ex(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor Q, scalekv_tensor K, scalekv_tensor V,
                                scalekv_tensor O, float *lse, int32_t compress, int32_t w, const int32_t *window_pos,
                                const scalekv_select_opts *opts) {
-  scalekv_status st = scalekv_append(ctx, layer, scale, K, V);
+  scalekv_status st = append_impl(ctx, layer, scale, K, V, true);
   if (st != SCALEKV_OK) return st;
   const bool score = !opts || opts->policy == SCALEKV_SELECT_SCORE;
   st = attend_impl(ctx, layer, Q, O, lse, compress != 0 && score && w > 0,
-                   step_copies(ctx, layer, scale, compress != 0, w, window_pos, opts));
+                   step_copies(ctx, layer, scale, K, V, compress != 0, w, window_pos, opts));
   if (st != SCALEKV_OK) return st;
   if (!compress) return SCALEKV_OK;
   return scalekv_compress_ex(ctx, layer, Q, w, window_pos, 1, opts);

@@ -1,0 +1,131 @@
+"""The f32 attention by products of bf16 pieces: edges of its tiles, its error, numbers it cannot split, maps outside the pages."""
+import pytest
+import torch
+
+from oracle import scalekv_oracle as orc
+from paper_2505_19602_b200 import binding
+from parity_util import ParityRun
+
+pytestmark = pytest.mark.gpu
+
+
+def full_cache(heads, sides, make, sides_w=None, lse=False):
+    """Attends map after map behind a full cache; the last map's queries, all keys and values, and what came out."""
+    kv = binding.ScaleKV(1, 1, heads, 64, "f32", sides, sides_w or sides, [[binding.KEEP_ALL] * len(sides)])
+    keys, values = [], []
+    for k, n in enumerate(kv.n):
+        Q, K, V = make(k, n)
+        keys.append(K), values.append(V)
+        out = torch.empty(1, heads, n, device="cuda") if lse else None
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        O = kv.scalekv_attend(0, Q, lse=out)
+        kv.scalekv_sync()
+    kv.close()
+    return Q, torch.cat(keys, 2), torch.cat(values, 2), O, out
+
+
+def normal(seed, heads):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return lambda n: (torch.randn(1, heads, n, 64, generator=g, device="cuda") for _ in range(3))
+
+
+@pytest.mark.parametrize("page", [16, 128])
+@pytest.mark.parametrize("heights,widths,budget", [
+    ((1, 1, 1), (1, 63, 64), 20),        # a tile of keys, one less, one more
+    ((1, 1, 1), (3, 127, 129), 50),      # a block of queries and one row
+    ((1, 5, 16), (2, 13, 24), 33),
+])
+def test_one_call_steps_match_oracle(heights, widths, budget, page):
+    """Maps that stay in the caller's tensors, windows recorded by the attention, survivors taken from the tensors."""
+    n = orc.scale_token_counts(heights, widths)
+    g = torch.Generator().manual_seed(31)
+    data = [tuple(torch.randn(2, 3, nk, 64, generator=g) for _ in range(3)) for nk in n]
+    budgets = [[budget] * len(n)]
+    kv = binding.ScaleKV(1, 2, 3, 64, "f32", heights, widths, budgets, page_tokens=page)
+    run = ParityRun(kv, "f32", heights, budgets, lambda l, k: data[k], lambda k: orc.window_centroids(heights[k], widths[k], 16),
+                    [(0, b, h) for b in range(2) for h in range(3)], compress_last=True, sides_w=widths)
+    run.run_pipelined()
+    kv.close()
+
+
+# by queries' gain: a score of size s is off by about 2^-24 s per rounding of its sum and of its exponent, at random from key to key, and
+# a weight by as much; a few such for scores of 0.25, 1 and 3, whose larger ones carry the weight.  Measured: 1.4 to 1.7e-7, 2.2 to
+# 2.4e-7 and 3.9 to 4.0e-7; plain fp32 sums over these keys give 4.6 to 11.9e-7, 5.5 to 12.3e-7 and 10.7 to 15.2e-7.
+BOUND = {0.25: 3.5e-7, 1.0: 5e-7, 3.0: 8e-7}
+
+
+@pytest.mark.parametrize("heads", [1, 40])             # keys shared by a cluster, and not
+@pytest.mark.parametrize("gain", [0.25, 1.0, 3.0])
+def test_error_is_that_of_fp32_arithmetic(heads, gain):
+    """Against 64 bits.  A score s is off by some 2^-24 of the larger ones' size per rounding, and so is a weight; sums over thousands of
+    keys may not add to that."""
+    draw = normal(11, heads)
+
+    def make(k, n):
+        Q, K, V = draw(n)
+        return Q * gain, K, V
+
+    Q, K, V, O, lse = full_cache(heads, (24, 60), make, lse=True)
+    s = Q.double() @ K.double().transpose(2, 3) / 8
+    want = s.softmax(-1) @ V.double()
+    assert ((O.double() - want).norm() / want.norm()).item() <= BOUND[gain]
+    assert (lse.double() - s.logsumexp(-1)).pow(2).mean().sqrt().item() <= 1e-6
+
+
+@pytest.mark.parametrize("heads", [1, 40])
+@pytest.mark.parametrize("first", [0, 40, 64])
+def test_keys_masked_with_minus_infinity(heads, first):
+    """Keys whose products are -inf have no weight, whatever the signs of the queries' pieces."""
+    draw = normal(5, heads)
+
+    def make(k, n):
+        Q, K, V = draw(n)
+        Q[..., 0] = Q[..., 0].abs() + 0.01
+        if k == 1:
+            K[:, :, first: first + 32, 0] = -float("inf")
+        return Q, K, V
+
+    Q, K, V, O, _ = full_cache(heads, (8, 18), make)
+    s = (Q.double() @ K.double().transpose(2, 3) / 8).masked_fill(torch.isinf(K[..., 0])[:, :, None], -float("inf"))
+    assert (O.double() - s.softmax(-1) @ V.double()).abs().max().item() <= 1e-5
+
+
+@pytest.mark.parametrize("heads", [1, 40])
+def test_infinite_values_reach_their_column_only(heads):
+    draw = normal(6, heads)
+
+    def make(k, n):
+        Q, K, V = draw(n)
+        if k == 1:
+            V[:, :, 70, 5] = float("inf")
+        return Q, K, V
+
+    Q, K, V, O, _ = full_cache(heads, (8, 18), make)
+    want = (Q.double() @ K.double().transpose(2, 3) / 8).softmax(-1) @ V.double()
+    assert torch.isinf(O[..., 5]).all() and (O[..., 5] > 0).all()
+    rest = [c for c in range(64) if c != 5]
+    assert (O.double() - want)[..., rest].abs().max().item() <= 1e-5
+
+
+def test_a_map_whose_keys_and_values_are_laid_out_differently():
+    """A one-call step takes it, evicting or not."""
+    sides, heads = (4, 12, 15), 3
+    g = torch.Generator(device="cuda").manual_seed(8)
+    outs = []
+    maps = [[torch.randn(1, heads, a * a, 64, generator=g, device="cuda") for _ in range(3)] for a in sides]
+    for spread in (False, True):
+        kv = binding.ScaleKV(1, 1, heads, 64, "f32", sides, sides, [[40] * 3])
+        for k, (Q, K, V) in enumerate(maps):
+            if spread:
+                wide = torch.zeros(1, K.shape[2], heads, 64, device="cuda")
+                wide.copy_(V.transpose(1, 2))
+                V = wide.transpose(1, 2)
+            O = torch.zeros_like(Q)
+            window = kv.window_array(binding.scalekv_window_centroids(sides[k], sides[k], 16)) if k < 2 else None
+            torch.cuda.synchronize()
+            kv.scalekv_step(0, k, Q, K, V, O, window_pos=window)
+            kv.scalekv_sync()
+        outs.append(O.clone())
+        kv.close()
+    assert torch.equal(outs[0], outs[1])
