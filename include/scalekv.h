@@ -128,7 +128,7 @@ scalekv_status scalekv_destroy(scalekv_ctx *ctx);
  * For bf16 x 128 the copy is done by the scalekv_attend that follows, which reads the map from K
  * and V directly and writes its rows to the pages while it streams them (no second read, nothing
  * on the critical path); any other next call for this layer (compress, layer_stats, export, the
- * next append) copies first with a kernel of its own.  K and V must therefore stay unmodified
+ * next append) copies first with a kernel of its own, layer_stats of a small map in its own launch.  K and V must therefore stay unmodified
  * until stream_main has passed the layer's next call.  For f32 x 64 the copy is enqueued here (by a
  * one-call step, below, it is left to the attend as well).
  * Ordered on stream_main after this layer's previous compress.
@@ -250,7 +250,8 @@ scalekv_status scalekv_step_host(scalekv_ctx *ctx, int32_t layer, int32_t scale,
  * query row i = 0, query_stride, 2*query_stride, ... of Q and every slice, alpha_i = softmax row
  * over all entries; c_i = mass on the current map; t_i = sum of the min(K', |history|) largest
  * alpha_ij over the history.  *car and *htk (HOST) receive the means of c_i and t_i over rows and
- * slices; ASI = car * htk.  Synchronous; not part of the timed path.  topk_prime <= 64. */
+ * slices; ASI = car * htk.  Synchronous: when it returns Q, and K and V of the map, have been read (stream_main's own end may be known
+ * a little later).  topk_prime <= 64. */
 scalekv_status scalekv_layer_stats(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Q, int32_t topk_prime,
                                    int32_t query_stride, double *car, double *htk);
 

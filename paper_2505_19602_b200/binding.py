@@ -299,7 +299,7 @@ class ScaleKV:
         self.lib = load_library()
         self._call = load_call()
         self._fn = {f: C.cast(getattr(self.lib, "scalekv_" + f), C.c_void_p).value
-                    for f in ("step", "step_ex", "append", "attend", "compress_ex")}
+                    for f in ("step", "step_ex", "append", "attend", "compress_ex", "layer_stats_ex")}
         self.device = torch.device("cuda", device)
         self.n_layers, self.batch, self.n_heads, self.head_dim = n_layers, batch, n_heads, head_dim
         self.dtype = {"bf16": BF16, "f32": F32, BF16: BF16, F32: F32}[dtype]
@@ -442,14 +442,10 @@ class ScaleKV:
 
     def scalekv_layer_stats_ex(self, layer, Q, topk_prime=16, query_stride=1):
         """(car, htk, car per slice, htk per slice, normalized current attention per slice); lists are [B][H]."""
-        car, htk = C.c_double(0), C.c_double(0)
-        n = self.batch * self.n_heads
-        cs, ts, ns = (C.c_double * n)(), (C.c_double * n)(), (C.c_double * n)()
-        self._check(self.lib.scalekv_layer_stats_ex(self.ctx, layer, tensor_arg(Q), topk_prime, query_stride,
-                                                    C.byref(car), C.byref(htk), cs, ts, ns))
-        H = self.n_heads
-        shape = lambda a: [a[b * H:(b + 1) * H] for b in range(self.batch)]
-        return car.value, htk.value, shape(cs), shape(ts), shape(ns)
+        st, *stats = self._call.layer_stats_ex(self._fn["layer_stats_ex"], self._handle, layer, Q, topk_prime, query_stride,
+                                               self.batch, self.n_heads)
+        self._check(st)
+        return tuple(stats)
 
     def scalekv_lengths(self, layer):
         out = (C.c_int32 * (self.batch * self.n_heads))()

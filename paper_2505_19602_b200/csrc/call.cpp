@@ -7,6 +7,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <exception>
+#include <vector>
 
 #include "../../include/scalekv.h"
 
@@ -151,8 +152,50 @@ PyObject *compress_ex(PyObject *, PyObject *const *a, Py_ssize_t n) {
   CALL(fn(ctx, layer, q, w, window, full, opts));
 }
 
+// [batch][heads] of floats, as lists of lists
+PyObject *lists(const std::vector<double> &x, Py_ssize_t batch, Py_ssize_t heads) {
+  PyObject *out = PyList_New(batch);
+  for (Py_ssize_t b = 0; out && b < batch; ++b) {
+    PyObject *row = PyList_New(heads);
+    for (Py_ssize_t h = 0; row && h < heads; ++h) {
+      PyObject *v = PyFloat_FromDouble(x[(size_t)(b * heads + h)]);
+      if (!v) Py_CLEAR(row);
+      else PyList_SET_ITEM(row, h, v);
+    }
+    if (!row) Py_CLEAR(out);
+    else PyList_SET_ITEM(out, b, row);
+  }
+  return out;
+}
+
+// layer_stats_ex(function, ctx, layer, Q, topk_prime, query_stride, batch, heads) -> (status, car, htk and the three per slice)
+PyObject *layer_stats_ex(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  scalekv_tensor q;
+  if (!arguments(n, 8) || !view(a[3], &q)) return nullptr;
+  const auto fn = address<decltype(&scalekv_layer_stats_ex)>(a[0]);
+  const auto ctx = address<scalekv_ctx *>(a[1]);
+  const int layer = (int)PyLong_AsLong(a[2]), topk = (int)PyLong_AsLong(a[4]), stride = (int)PyLong_AsLong(a[5]);
+  const Py_ssize_t batch = PyLong_AsSsize_t(a[6]), heads = PyLong_AsSsize_t(a[7]);
+  if (PyErr_Occurred()) return nullptr;
+  double car = 0.0, htk = 0.0;
+  int st = 0;
+  std::vector<double> cs, ts, ns;
+  if (!guarded([&] {
+        cs.resize((size_t)(batch * heads)); ts.resize(cs.size()); ns.resize(cs.size());
+        return true;
+      })) return nullptr;
+  Py_BEGIN_ALLOW_THREADS
+  st = (int)fn(ctx, layer, q, topk, stride, &car, &htk, cs.data(), ts.data(), ns.data());
+  Py_END_ALLOW_THREADS
+  PyObject *c = lists(cs, batch, heads), *t = lists(ts, batch, heads), *m = lists(ns, batch, heads);
+  if (c && t && m) return Py_BuildValue("(iddNNN)", st, car, htk, c, t, m);
+  Py_XDECREF(c); Py_XDECREF(t); Py_XDECREF(m);
+  return nullptr;
+}
+
 #define METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {METHOD(step), METHOD(step_ex), METHOD(append), METHOD(attend), METHOD(compress_ex), {nullptr, nullptr, 0, nullptr}};
+PyMethodDef methods[] = {METHOD(step), METHOD(step_ex), METHOD(append), METHOD(attend), METHOD(compress_ex), METHOD(layer_stats_ex),
+                         {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_scalekv_call", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

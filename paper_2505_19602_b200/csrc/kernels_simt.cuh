@@ -983,10 +983,13 @@ __global__ void __launch_bounds__(64) layer_stats_merge_kernel(const float *part
 // exponential, an insertion where a list grows - and, at the small scales, the latency of a call.  Tensor-core products by
 // m16n8k16 leave the scores in registers and are a tenth of that time, so a TMEM pipeline would not shorten it.
 // One layer's 13 scales, one image, 16 slices: 2 048 us with the kernels above, 485 us here (4 096 queries, every 16th of them,
-// 10 521 keys: 921 + 19 -> 111 + 16 us); a call at the small scales 67 -> 32 us, sums in page-locked memory among the causes.
-// sums (host memory: the caller reads it when the stream is through): per slice and block of rows the sums of c_i and t_i, then
-// the slices' lengths.  counters: one per slice and block of rows, zero before and after.
-// grid (ceil(n_rows / 64), n_slices, n_split <= 16); static shared memory: two K tiles and the query tile.
+// 10 521 keys: 921 + 19 -> 111 + 16 us); a call at the small scales 67 -> 32 us, sums in page-locked memory among the causes. A pass of four layers 2 708 -> 2 145 us
+// since small maps are read where they are and the sums are watched (see the launch).
+// map_outside: the current map is still in the caller's tensors.  Its keys are read there, and CTAs of their own (blockIdx.z >=
+// n_split) copy its rows into the pages meanwhile.
+// sums (host memory, which the caller watches): per slice and block of rows the sums of c_i and t_i, then the slices' lengths, then a
+// word per copying CTA.  counters: one per slice and block of rows, zero before and after.
+// grid (ceil(n_rows / 64), n_slices, n_split <= 16 and as many again as copy); static shared memory: two K tiles and the query tile.
 // ------------------------------------------------------------------------------------------
 constexpr int kTop = 16;
 
@@ -1049,22 +1052,62 @@ struct RowStats {
     merge(m2, z2, cur2, t);
   }
 };
+// Rows part, part + parts, .. (in blocks of 128) of a bf16 map: K, V and positions to the pages.  256 threads, 16 pieces of 16 bytes in
+// flight per thread.
+__device__ __forceinline__ void copy_map_rows(const LayerView &lv, const TensorView &K, const TensorView &V, int slice, int hist, int n_k,
+                                              int n_prev, int part, int parts) {
+  const int b = slice / lv.n_heads, h = slice % lv.n_heads, c = threadIdx.x & 15, r = threadIdx.x >> 4;
+  for (int r0 = part * 128; r0 < n_k; r0 += parts * 128) {
+    uint4 x[2][8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = r0 + u * 16 + r;
+      if (i >= n_k) continue;
+      x[0][u] = __ldcs(reinterpret_cast<const uint4 *>(row_ptr<__nv_bfloat16>(K, b, h, i)) + c);
+      x[1][u] = __ldcs(reinterpret_cast<const uint4 *>(row_ptr<__nv_bfloat16>(V, b, h, i)) + c);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = r0 + u * 16 + r;
+      if (i >= n_k) continue;
+      const size_t row = slot_row(lv, slice, hist + i);
+      reinterpret_cast<uint4 *>(lv.k_pool + row * 256)[c] = x[0][u];
+      reinterpret_cast<uint4 *>(lv.v_pool + row * 256)[c] = x[1][u];
+      if (c == 0) lv.pos_pool[row] = n_prev + i;
+    }
+  }
+}
 constexpr int kStatsRec16 = 4 + kTop;    // floats per (split, row) record: m, z, cur, unused, the list
 
 __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorView Q, int n_k, int stride, int n_rows, int topk_prime,
-                                                           float scale_log2e, float *partial, int *counters, double *sums) {
+                                                           float scale_log2e, float *partial, int *counters, double *sums, int n_split,
+                                                           TensorView mapK, TensorView mapV, int map_outside, int n_prev) {
   __shared__ __align__(128) uint8_t sm[3 * 64 * 256];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wr = warp & 3, wc = warp >> 2;
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice % lv.n_heads;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int hist = lv.hist_len[slice], L = hist + n_k;
+  const bool copies = (int)blockIdx.z >= n_split;
+  const int parts = ((int)gridDim.z - n_split) * gridDim.x, part = ((int)blockIdx.z - n_split) * (int)gridDim.x + (int)blockIdx.x;
+  double *copied = sums + ((size_t)2 * gridDim.x + 1) * gridDim.y + (size_t)slice * parts + part;
   if (outgrown(lv, L)) {
-    if (tid < 2) sums[((size_t)slice * gridDim.x + blockIdx.x) * 2 + tid] = NAN;      // (not what an earlier call left there)
+    if (tid < 2) sums[((size_t)slice * gridDim.x + blockIdx.x) * 2 + tid] = NAN;      // (an answer all the same)
+    if (tid == 2 && blockIdx.x == 0) sums[(size_t)2 * gridDim.x * gridDim.y + slice] = NAN;
+    if (tid == 3 && copies) *copied = NAN;
+    return;
+  }
+  if (copies) {
+    copy_map_rows(lv, mapK, mapV, slice, hist, n_k, n_prev, part, parts);
+    __syncthreads();
+    if (tid == 0) {                      // (the caller may change the tensors when the call returns)
+      *copied = 0.0;
+      __threadfence_system();
+    }
     return;
   }
   const int r0 = blockIdx.x * 64;
-  const int tiles = (L + 63) >> 6, n_split = gridDim.z;
+  const int tiles = (L + 63) >> 6;
   const int t_lo = (int)((long long)tiles * blockIdx.z / n_split), t_hi = (int)((long long)tiles * (blockIdx.z + 1) / n_split);
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
   // 16-byte piece c of row r of a 64 x 256-byte tile
@@ -1073,8 +1116,11 @@ __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorV
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int r = u * 16 + (tid >> 4), c = tid & 15, slot = t * 64 + r;
-      if (slot < L)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at(t & 1, r, c)), "l"(lv.k_pool + slot_row(lv, slice, slot) * 256 + c * 16) : "memory");
+      if (slot < L) {
+        const char *src = map_outside && slot >= hist ? reinterpret_cast<const char *>(row_ptr<__nv_bfloat16>(mapK, b, h, slot - hist))
+                                                      : lv.k_pool + slot_row(lv, slice, slot) * 256;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at(t & 1, r, c)), "l"(src + c * 16) : "memory");
+      }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -1209,15 +1255,17 @@ __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorV
   int *last = reinterpret_cast<int *>(sm);
   __threadfence();
   __syncthreads();
-  if (tid == 0) {
-    int *count = counters + (size_t)slice * gridDim.x + blockIdx.x;
-    const int before = atomicAdd(count, 1);
-    *last = before == n_split - 1;
-    if (before == n_split - 1) *count = 0;             // as the next launch wants to find it
+  if (n_split > 1) {
+    if (tid == 0) {
+      int *count = counters + (size_t)slice * gridDim.x + blockIdx.x;
+      const int before = atomicAdd(count, 1);
+      *last = before == n_split - 1;
+      if (before == n_split - 1) *count = 0;           // as the next launch wants to find it
+    }
+    __syncthreads();
+    if (!*last) return;
+    __threadfence();
   }
-  __syncthreads();
-  if (!*last) return;
-  __threadfence();
   const int l = tid & 15, n_here = min(64, n_rows - r0);
   double c_sum = 0.0, t_sum = 0.0;
   for (int row0 = 0; row0 < n_here; row0 += 16) {
@@ -1252,10 +1300,12 @@ __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorV
     for (int d = 8; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
     double *out = sums + ((size_t)slice * gridDim.x + blockIdx.x) * 2;
     if (l == 0) out[tid >> 4] = v;
+    __threadfence_system();              // (on its way at once: the host is watching)
   }
   if (blockIdx.x == 0 && tid == 32) {
-    sums[(size_t)2 * gridDim.x * gridDim.y + slice] = (double)L;
     lv.next_len[slice] = L;              // what the next scale finds
+    sums[(size_t)2 * gridDim.x * gridDim.y + slice] = (double)L;
+    __threadfence_system();
   }
 }
 

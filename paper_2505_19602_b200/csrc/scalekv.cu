@@ -5,6 +5,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1060,6 +1061,25 @@ scalekv_status scalekv_step_ex(scalekv_ctx *ctx, int32_t layer, int32_t scale, s
   return scalekv_compress_ex(ctx, layer, Q, w, window_pos, 1, opts);
 }
 
+// What a sum that has not arrived looks like: a NaN that no arithmetic produces.
+static double no_sum() {
+  const uint64_t bits = 0x7ff8a5c35a3c17e9ull;
+  double x;
+  std::memcpy(&x, &bits, 8);
+  return x;
+}
+// Whether all of them arrive within half a millisecond.
+static bool sums_arrived(const double *sums, size_t n) {
+  const double none = no_sum();
+  uint64_t want;
+  std::memcpy(&want, &none, 8);
+  const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(500);
+  for (size_t i = 0; i < n; ++i)
+    for (int spins = 0; __atomic_load_n(reinterpret_cast<const uint64_t *>(sums) + i, __ATOMIC_ACQUIRE) == want; ++spins)
+      if ((spins & 63) == 63 && std::chrono::steady_clock::now() > until) return false;
+  return true;
+}
+
 scalekv_status scalekv_layer_stats(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Q, int32_t topk_prime,
                                    int32_t query_stride, double *car, double *htk) {
   return scalekv_layer_stats_ex(ctx, layer, Q, topk_prime, query_stride, car, htk, nullptr, nullptr, nullptr);
@@ -1075,8 +1095,6 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   if (ctx->map_lost[layer]) return fail(ctx, SCALEKV_ERR_BAD_STATE, "layer %d: the rows of its last map were handed to another layer after its attend", layer);
   if (topk_prime < 0 || topk_prime > 64 || query_stride < 1) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "topk_prime in [0,64], stride >= 1");
   if (!tensor_ok(Q, p.esize)) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "Q null or rows not 16-byte aligned");
-  scalekv_status st0 = materialize(ctx, layer);
-  if (st0 != SCALEKV_OK) return st0;
   const int nk = ctx->pending[layer];
   const int k = ctx->next_scale[layer] - 1;
   const int rows = (nk + query_stride - 1) / query_stride;
@@ -1090,20 +1108,40 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   float *partial = reinterpret_cast<float *>(ctx->ws + p.off_stats);
   // The tensor-core kernel: two CTAs per SM and no second wave (256 rows x 16 slices: 4 key ranges against 8).
   // (The records of a launch with very many rows may outgrow the scratch: then the other kernel.)
-  const int mma_split = std::max(1, std::min({16, 2 * ctx->n_sm / (row_blocks * p.n_slices), tiles}));
+  const int room = 2 * ctx->n_sm / (row_blocks * p.n_slices);
+  int mma_split = std::max(1, std::min({16, room, tiles}));
   const bool tensor = ctx->dtype == SCALEKV_BF16 && topk_prime <= kTop &&
                       (size_t)p.n_slices * rows * mma_split * kStatsRec16 <= (size_t)kStatsMaxCtas * 64 * kStatsRec;
+  if (!tensor) {
+    scalekv_status st = materialize(ctx, layer);
+    if (st != SCALEKV_OK) return st;
+  }
   const LayerView lv = layer_view(ctx, layer);
   const double *sums;      // sums of c_i and t_i over the rows and lengths: see the kernels
   std::vector<double> copied;
+  size_t words = 0;        // that the tensor-core kernel leaves in host memory
   if (tensor) {
-    const size_t need = (size_t)p.n_slices * (2 * row_blocks + 1);
-    if (ctx->stats_host_doubles < need) {      // (at the first call, sized for every row of the largest map)
-      const size_t most = (size_t)p.n_slices * (2 * ((p.n_max + 63) / 64) + 1);
+    // A map that still waits in the caller's tensors is read there and copied by CTAs of the same launch beside the others, for
+    // which those leave room - if it is so small that its copy is not what the call waits for in the end.  us per call, 16 slices, copied
+    // by a launch before this one -> so: 1 to 64 queries 31 -> 16, 256: 34 -> 20, 1 024: 46 -> 34; one CTA per 1 600 / 2 304 rows 61 ->
+    // 63, 86 -> 98.  (Of the gain at the small maps 8 us are the launch, the rest the wait for the stream and the way through ctypes.)
+    const int copy_z = std::max(1, std::min(4, room - mma_split));
+    const bool outside = !ctx->in_store[layer] && nk <= 512 * row_blocks * copy_z;
+    if (!outside) {
+      scalekv_status st = materialize(ctx, layer);
+      if (st != SCALEKV_OK) return st;
+    } else if (mma_split == room && mma_split > 1) {
+      --mma_split;
+    }
+    words = (size_t)p.n_slices * (2 * row_blocks + 1 + (outside ? row_blocks * copy_z : 0));
+    if (ctx->stats_host_doubles < words) {     // (at the first call, sized for every row of the largest map)
+      const size_t most = (size_t)p.n_slices * (6 * ((p.n_max + 63) / 64) + 1);
       CU(cudaHostAlloc(reinterpret_cast<void **>(&ctx->stats_host), most * sizeof(double), cudaHostAllocMapped));
       CU(cudaHostGetDevicePointer(reinterpret_cast<void **>(&ctx->stats_host_dev), ctx->stats_host, 0));
       ctx->stats_host_doubles = most;
     }
+    const TensorView mk = outside ? tview(ctx->pend_k[layer]) : TensorView{}, mv = outside ? tview(ctx->pend_v[layer]) : TensorView{};
+    std::fill(ctx->stats_host, ctx->stats_host + words, no_sum());
     // (a programmatic launch: the kernel comes up while the one before it ends)
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1112,11 +1150,12 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.stream = ctx->s_main;
-    cfg.gridDim = dim3(row_blocks, p.n_slices, mma_split);
+    cfg.gridDim = dim3(row_blocks, p.n_slices, mma_split + (outside ? copy_z : 0));
     cfg.blockDim = dim3(256);
     Scope sc(ctx, ctx->s_main, kOther);
     CU(cudaLaunchKernelEx(&cfg, stats_mma_kernel, lv, tview(Q), nk, query_stride, rows, topk_prime, ctx->scale * 1.4426950408889634f, partial,
-                          reinterpret_cast<int *>(ctx->pool + p.off_count), ctx->stats_host_dev));
+                          reinterpret_cast<int *>(ctx->pool + p.off_count), ctx->stats_host_dev, mma_split, mk, mv, outside ? 1 : 0, p.N[k]));
+    ctx->in_store[layer] = 1;
     sums = ctx->stats_host;
     ctx->len_written[layer] = 1;
   } else {
@@ -1143,7 +1182,9 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
     sums = copied.data();
     CU(cudaMemcpyAsync(copied.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, ctx->s_main));
   }
-  CU(cudaStreamSynchronize(ctx->s_main));
+  // The sums are watched as they arrive: the stream's own end is known several us later.  (Nothing for a while - work before this, a
+  // capture, a fault: the stream tells.)
+  if (!tensor || !sums_arrived(ctx->stats_host, words)) CU(cudaStreamSynchronize(ctx->s_main));
   double c_all = 0.0, t_all = 0.0;
   for (int s = 0; s < p.n_slices; ++s) {
     double c_sum = 0.0, t_sum = 0.0, len;
