@@ -1052,7 +1052,16 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       for (int cc = 0; cc < kChunks; ++cc) {
         uint32_t pk[16];
         const int vc = valid - cc * 32;
-        if (cc + 1 < kChunks) front(v[(cc + 1) & 1], vc - 32, masked);
+        // A ragged tile's chunks without keys: zeros, and no exponentials (the sweep is the larger part of a short CTA: small_image, maps of
+        // up to 256 queries, 249 -> 235 us; one image of 13 scales 12 347 -> 12 195, its graph 11 634 -> 11 477.  Leaving their steps out of
+        // the products as well needs a run-time number of them, which the MMA warp pays for in every tile: 3 to 4 % slower passes).
+        auto empty = [&](int left) { return decltype(masked)::value && left <= 0; };
+        if (empty(vc)) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) pk[i] = 0u;
+          tc_st16(s_addr + cc * 16, pk);
+        } else {
+        if (cc + 1 < kChunks && !empty(vc - 32)) front(v[(cc + 1) & 1], vc - 32, masked);
         const float lt = back(v[cc & 1], pk);
         if (cc + 2 < kChunks) tc_ld32(s_addr + (cc + 2) * 32, v[cc & 1]);
         if (__any_sync(0xffffffffu, !(lt <= 8192.f))) {
@@ -1066,7 +1075,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           if (!ok) return;
           m = r.m; l = r.l + r.sum;
           if (r.o_landed) o_landed = late ? 2 : 1;
-          if (cc + 1 < kChunks) {
+          if (cc + 1 < kChunks && !empty(vc - 32)) {
             // the next chunk's exponentials were taken against the old reference: once more, from its raw products
             tc_ld32(s_addr + (cc + 1) * 32, v[(cc + 1) & 1]);
             tc_wait_ld();
@@ -1075,6 +1084,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         } else {
           tc_st16(s_addr + cc * 16, pk);
           l += lt;
+        }
         }
         if (cc == kEarlyChunks - 1) {
           // P of the first chunks is complete: that part of the PV product may start under the rest of the sweep
