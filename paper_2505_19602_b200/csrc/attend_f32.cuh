@@ -17,8 +17,7 @@
 // What bounds it: six products stand for one, so a tile of 64 keys is 48 tcgen05.mma of 128 x 64 x 16; where two CTAs share an SM a step
 // of both takes about 8 000 cycles, of which these are half and the splitting of operands and of P, the exponentials and the way through
 // TMEM the rest.  us per layer and step, 16 slices behind 92 to 772 entries with their compresses, by packed fp32 FMA (66 % of that pipe)
-// and a copy, the window's logits and their sums by launches of their own -> here: 16 queries 15.4 -> 9.7, 64: 25.7 -> 17.0, 256:
-// 35.8 -> 21.0, 400: 65.0 -> 26.6, 576: 91 -> 35, 1 024: 179 -> 60, 1 600: 331 -> 127 (11 -> 29 TFLOP/s of fp32 results).
+// and a copy of the map -> here: 16 queries 15.4 -> 9.7, 256: 35.8 -> 26.6, 400: 65 -> 46, 576: 91 -> 55, 1 024: 179 -> 76, 1 600: 331 -> 139.
 // Error against 64 bits, full caches of 29 to 4 436 entries, queries and keys normal, queries times 0.25 / 1 / 3: outputs 0.9 to 1.6 / 1.0 to
 // 2.1 / 1.5 to 4.0 e-7 (by FMA 1.1 to 11.9 / 2.2 to 12.3 / 3.3 to 15.2), lse 1.1 to 3.2 / 1.1 to 3.4 / 2.9 to 3.7 e-7 rms (1.1 to 3.2 / 1.4 to 3.3 /
 // 5.2 to 8.2).
@@ -55,9 +54,6 @@ struct Params {
   int n_k, room;               // room: entries that a slice's pages hold
   int fused, copy_in, n_prev;  // copy_in: the map's rows go to the pages on the way
   float scale_log2e;
-  float *win_logits, *win_lse; // raw products of the window's rows by slot, [slice][rank][ld_l], and their base-2 log-sum-exp
-  int ld_l, w;
-  int win_pos[kMaxWindow];
 };
 
 // Four steps (of 16) of one product of pieces, issued by the elected lane of a converged warp.
@@ -130,11 +126,10 @@ __device__ __forceinline__ float row_lse_f32(float m, float l) {
   return fmaf(m, 0.6931471805599453f, fmaf(m, (float)(1.0 / 1.4426950408889634f - 0.6931471805599453f), logf(l)));
 }
 
-// One row by fp32 FMA over the entries [from, to): its 64 columns go to `out` (16-byte pieces permuted by `swap`), its raw products
-// to win_row if it has one.  For rows whose scores or columns by pieces are not numbers.
+// One row by fp32 FMA over the entries [from, to): its 64 columns go to `out` (16-byte pieces permuted by `swap`).  For
+// rows whose scores or columns by pieces are not numbers.
 struct RowSum { float m, l; };
-__device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int h, int hist, int q_row, int from, int to, float *out, int swap,
-                                       float *win_row) {
+__device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int h, int hist, int q_row, int from, int to, float *out, int swap) {
   const float *q = row_ptr<float>(prm.Q, b, h, q_row);
   float o[64], m = kNoMax, l = 0.f;
 #pragma unroll
@@ -145,7 +140,6 @@ __device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int 
     float s = 0.f;
 #pragma unroll 8
     for (int d = 0; d < 64; ++d) s = fmaf(q[d], k[d], s);
-    if (win_row != nullptr) win_row[j] = s;
     const float y = s * prm.scale_log2e, mx = fmaxf(m, y), f = exp2f(m - mx), p = exp2f(y - mx);
     m = mx;
     l = fmaf(l, f, p);
@@ -294,13 +288,6 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     const int row = warp * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
     const float c = prm.scale_log2e;
-    float *win_row = nullptr;
-    int rank = -1;
-    if (prm.win_logits != nullptr)
-      for (int e = 0; e < prm.w; ++e)
-        if (prm.win_pos[e] == q0 + row) rank = e;
-    if (rank >= 0) win_row = prm.win_logits + ((size_t)slice * prm.w + rank) * prm.ld_l;
-    const bool wwarp = __any_sync(0xffffffffu, rank >= 0);
     uint64_t o[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) o[i] = 0ull;
@@ -339,18 +326,6 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
           uint32_t x[16];
           tc::tc_ld16(lane_addr + kColS + 16 * e, x);
           tc::tc_wait_ld();
-          if (wwarp) {
-            // (columns beyond the last key: zeros that nobody reads)
-            if (win_row != nullptr) {
-              float4 *dst = reinterpret_cast<float4 *>(win_row + (lo + i) * kKeys + 16 * e);
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                auto whole = [&](int e2) { const float s = __uint_as_float(x[4 * q + e2]); return fmaf(s, kCutOff, s); };
-                dst[q] = make_float4(whole(0), whole(1), whole(2), whole(3));
-              }
-            }
-            __syncwarp();
-          }
 #pragma unroll
           for (int q = 0; q < 16; q += 2) {
             const float y0 = 16 * e + q < valid ? __uint_as_float(x[q]) * c : kNoMax, y1 = 16 * e + q + 1 < valid ? __uint_as_float(x[q + 1]) * c : kNoMax;
@@ -427,14 +402,13 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       *reinterpret_cast<float4 *>(mine + ((q ^ (row & 7)) << 2)) = make_float4(x0, x1, x2, x3);
     }
     if (nt > 0 && ok && q0 + row < n_k && !(amax == 0.f && l > 0.f && l < INFINITY)) {
-      const RowSum s = fma_row(prm, slice, b, h, hist, q0 + row, lo * kKeys, min((lo + nt) * kKeys, L), mine, row & 7, win_row);
+      const RowSum s = fma_row(prm, slice, b, h, hist, q0 + row, lo * kKeys, min((lo + nt) * kKeys, L), mine, row & 7);
       m = s.m;
       l = s.l;
     }
     stat_out[row] = make_float2(m, l);
     if (n_split == 1 && ok && nt > 0 && q0 + row < n_k) {
       if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + row] = row_lse_f32(m, l);
-      if (rank >= 0) prm.win_lse[(size_t)slice * prm.w + rank] = m + log2f(l);
     }
     tc_fence_before();
   }
@@ -481,12 +455,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     }
     const float inv = 1.f / sum;
     *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(prm.O, b, h, q0 + r)) + tx * 4) = make_float4(a0 * inv, a1 * inv, a2 * inv, a3 * inv);
-    if (tx == 0) {
-      if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + r] = row_lse_f32(M, sum);
-      if (prm.win_logits != nullptr)
-        for (int e = 0; e < prm.w; ++e)
-          if (prm.win_pos[e] == q0 + r) prm.win_lse[(size_t)slice * prm.w + e] = M + log2f(sum);
-    }
+    if (tx == 0 && prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + r] = row_lse_f32(M, sum);
   }
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");

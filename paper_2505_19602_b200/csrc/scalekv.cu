@@ -688,7 +688,9 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
     if (fused) { kc = tview(ctx->pend_k[layer]); vc = tview(ctx->pend_v[layer]); }
     const int k = ctx->next_scale[layer] - 1;
     const std::vector<int> &win = p.windows[k];
-    float *wl = (win.empty() || !record || k + 1 == p.K)
+    // (f32: the compress takes the window's logits from K, in plain fp32 sums.  Importances a few 1e-7 apart decide what is kept, so that
+    // logits of another rounding, as exact as they may be, keep another entry in one pass of some.)
+    float *wl = (win.empty() || !record || k + 1 == p.K || !ctx->tc.enabled())
                     ? nullptr
                     : reinterpret_cast<float *>(ctx->ws + p.off_logits) + (size_t)(layer % kSets) * p.logits_elems;
     float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
@@ -710,8 +712,6 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       prm.room = lv.pages_per_slice << lv.page_shift;
       prm.fused = fused ? 1 : 0; prm.copy_in = (fused && copy) ? 1 : 0; prm.n_prev = p.N[k];
       prm.scale_log2e = ctx->scale * 1.4426950408889634f;
-      prm.win_logits = wl; prm.win_lse = wlse; prm.ld_l = p.ld_l; prm.w = wl ? (int)win.size() : 0;
-      for (int e = 0; e < prm.w; ++e) prm.win_pos[e] = win[e];
       const int blocks = (nk + f32::kRows - 1) / f32::kRows;
       const int split = f32::key_split(blocks * p.n_slices, (ctx->hist[layer] + nk + f32::kKeys - 1) / f32::kKeys, ctx->n_sm);
       cudaLaunchConfig_t cfg = {};
@@ -1031,7 +1031,7 @@ static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, const scal
     const int sinks = std::min(std::max(opts->n_sink, 0), p.N[scale + 1]);
     return !(std::max(table - sinks, 0) < L - sinks);
   }
-  if (w <= 0) return true;
+  if (w <= 0 || !ctx->tc.enabled()) return true;
   bool planned = scale + 1 != p.K && window_pos && (int)p.windows[scale].size() == w;
   for (int j = 0; planned && j < w; ++j) planned = p.windows[scale][j] == window_pos[j];
   return !(planned && table < L - w);

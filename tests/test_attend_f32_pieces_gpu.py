@@ -37,7 +37,7 @@ def normal(seed, heads):
     ((1, 5, 16), (2, 13, 24), 33),
 ])
 def test_one_call_steps_match_oracle(heights, widths, budget, page):
-    """Maps that stay in the caller's tensors, windows recorded by the attention, survivors taken from the tensors."""
+    """Maps that the attention reads in the caller's tensors and copies into the pages."""
     n = orc.scale_token_counts(heights, widths)
     g = torch.Generator().manual_seed(31)
     data = [tuple(torch.randn(2, 3, nk, 64, generator=g) for _ in range(3)) for nk in n]
