@@ -5,24 +5,30 @@
 // A CTA of 256 threads, two per SM, owns 128 query rows of one slice and streams its keys in tiles of 64:
 //   warps 4-7 : operands.  They load K and V rows (the pages' or, for a map that has not been copied there, the caller's), split
 //               them and leave the pieces in 128B-swizzled shared memory; the next tile's rows wait in registers meanwhile.
+//               Warp 4 issues S of a tile as soon as its keys lie there, into the other of two buffers, under the softmax of
+//               the tile before.
 //   warps 0-3 : softmax, a thread per query row (TMEM lane).  The products of a tile of V land in TMEM and are added to the row's
 //               64 columns in registers: the tensor core cuts its sums off where fp32 arithmetic rounds them, which over the tiles of a
-//               long cache would show.  P goes back to TMEM in three pieces.  Warp 0 issues the products of the tile's values and of
-//               the next tile's keys in one go, when all four warps have met.
+//               long cache would show.  P goes back to TMEM in three pieces, over the scores it comes from.  Warp 0 issues P V when all
+//               four warps have met; its result is added behind the softmax of the next tile.
 // With two CTAs an SM's tensor pipe works for the one while the other is in its softmax.
 // Scores that are not numbers (an infinite key: its products with the pieces of a query may differ in sign) spoil their row's sum, and
 // values that are not its columns; such a row is done again at the end by fp32 FMA from the tensors (fma_row).
+// The observation window's logits are taken by CTAs of their own beside the others, in plain fp32 (see the launch).
 // gridDim.z CTAs of a cluster share a slice's keys and combine: O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e, through distributed
 // shared memory.
-// What bounds it: six products stand for one, so a tile of 64 keys is 48 tcgen05.mma of 128 x 64 x 16; where two CTAs share an SM a step
-// of both takes about 8 000 cycles, of which these are half and the splitting of operands and of P, the exponentials and the way through
-// TMEM the rest.  us per layer and step, 16 slices behind 92 to 772 entries with their compresses, by packed fp32 FMA (66 % of that pipe)
-// and a copy of the map -> here: 16 queries 15.4 -> 9.7, 256: 35.8 -> 26.6, 400: 65 -> 46, 576: 91 -> 55, 1 024: 179 -> 76, 1 600: 331 -> 139.
+// What bounds it: the instructions of the softmax and of the splitting, and the tensor pipe, six products standing for one; a step of two
+// CTAs that share an SM takes about 8 000 cycles.  (Working copies that skip work, us per layer, 16 slices x 1 600 queries: whole 130; one
+// product of six 102; P not split 115; K and V not split 112.)  S of the next tile under the softmax of this one, from two buffers, and
+// fewer instructions: 139 -> 123.  us per layer and step, 16 slices behind 92 to 772 entries with their compresses, by packed fp32 FMA (66 %
+// of that pipe), a copy of the map and three launches per compress -> here: 16 queries 15.4 -> 10, 64: 25.7 -> 20, 256: 35.8 -> 26,
+// 400: 65 -> 40, 576: 91 -> 55, 1 024: 179 -> 80, 1 600: 331 -> 123.
 // Error against 64 bits, full caches of 29 to 4 436 entries, queries and keys normal, queries times 0.25 / 1 / 3: outputs 0.9 to 1.6 / 1.0 to
 // 2.1 / 1.5 to 4.0 e-7 (by FMA 1.1 to 11.9 / 2.2 to 12.3 / 3.3 to 15.2), lse 1.1 to 3.2 / 1.1 to 3.4 / 2.9 to 3.7 e-7 rms (1.1 to 3.2 / 1.4 to 3.3 /
 // 5.2 to 8.2).
 #pragma once
 #include <cfloat>
+#include <type_traits>
 
 #include "attend_tc.cuh"
 #include "kernels_simt.cuh"
@@ -45,7 +51,10 @@ static_assert(2 * (kSmemBytes + 1024) <= 233472, "two CTAs have to fit an SM");
 // in each of the four steps over the large pieces, less in those where the sum is still growing.  It is given back (without: lse of queries
 // times 3 low by 6.6e-7 on average, 7.4e-7 rms; so by 0.3e-7, 3.4e-7 rms).
 constexpr float kCutOff = 1.2f / 16777216.f;
-constexpr uint32_t kTmemCols = 256, kColS = 0, kColP = 64, kColO = 160;           // 64 of scores, 3 x 32 of P, 64 of products with V
+// TMEM: two buffers of 96 columns for scores and P, 64 columns for products with V.  The 16 keys of step kk have their scores in columns
+// 16 kk .. of a buffer, and their P there (h in the first eight, m in the next) and in columns 64 + 8 kk .. (l).
+constexpr uint32_t kTmemCols = 256, kBufCols = 96, kColPm = 8, kColPl = 64, kColO = 192;
+enum { bV = 0, bPv = 1, bS = 2 };                           // barriers: V is there; P V has landed; S has, by buffer
 
 struct Params {
   LayerView lv;
@@ -53,7 +62,11 @@ struct Params {
   float *lse;
   int n_k, room;               // room: entries that a slice's pages hold
   int fused, copy_in, n_prev;  // copy_in: the map's rows go to the pages on the way
-  float scale_log2e;
+  float scale, scale_log2e;
+  int blocks;                  // blocks of query rows; the CTAs behind them (blockIdx.x) take the logits of the window's w rows
+  float *win_logits;           // base-2 logits by slot, [slice][rank][ld_l]
+  int ld_l, w;
+  int win_pos[kMaxWindow];
 };
 
 // Four steps (of 16) of one product of pieces, issued by the elected lane of a converged warp.
@@ -69,16 +82,17 @@ __device__ __forceinline__ void mma4_ss(uint32_t d, uint32_t a_lo, uint32_t b_lo
       "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
       : "memory");
 }
+template <int STEP>              // columns of P from one step to the next
 __device__ __forceinline__ void mma4_ts(uint32_t d, uint32_t a, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate_first) {
   asm volatile(
       "{\n\t.reg .pred e, pf, pt;\n\t.reg .b64 db;\n\t.reg .b32 at, bl;\n\t"
       "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 pf, %5, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
       "mov.b64 db, {%2, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pf;\n\t"
-      "add.u32 at, %1, 8;\n\tadd.u32 bl, %2, 128;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, 16;\n\tadd.u32 bl, %2, 256;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
-      "add.u32 at, %1, 24;\n\tadd.u32 bl, %2, 384;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
+      "add.u32 at, %1, %6;\n\tadd.u32 bl, %2, 128;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
+      "add.u32 at, %1, %7;\n\tadd.u32 bl, %2, 256;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
+      "add.u32 at, %1, %8;\n\tadd.u32 bl, %2, 384;\n\tmov.b64 db, {bl, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, pt;\n\t"
       "}" ::"r"(d),
-      "r"(a), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
+      "r"(a), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first), "n"(STEP), "n"(2 * STEP), "n"(3 * STEP)
       : "memory");
 }
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t *v) {
@@ -87,15 +101,15 @@ __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t *v) {
                : "memory");
 }
 
-// a pair of numbers in three pairs of bf16 numbers that sum to them
+// A pair of numbers in three pairs of bf16 numbers that sum to them.  (What h and m leave of 24 bits fits the eight of l, so l is the
+// upper half of what is left.)
 __device__ __forceinline__ void split2(float x, float y, uint32_t &h, uint32_t &m, uint32_t &l) {
+  const uint64_t minus = tc::pack2(-1.f, -1.f);
   h = tc::pack_bf16(x, y);
-  x -= __uint_as_float(h << 16);
-  y -= __uint_as_float(h & 0xffff0000u);
+  tc::unpack2(tc::fma2(tc::pack2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), minus, tc::pack2(x, y)), x, y);
   m = tc::pack_bf16(x, y);
-  x -= __uint_as_float(m << 16);
-  y -= __uint_as_float(m & 0xffff0000u);
-  l = tc::pack_bf16(x, y);
+  tc::unpack2(tc::fma2(tc::pack2(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u)), minus, tc::pack2(x, y)), x, y);
+  l = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
 }
 __device__ __forceinline__ void store16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -152,25 +166,49 @@ __device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int 
   return {m, l};
 }
 
-// grid (ceil(n_k / 128), n_slices, split); dynamic shared memory kSmemBytes.
+// The window's logits against the 64 entries of a tile, as score_logits_kernel takes them from the pages.
+__device__ __noinline__ void window_logits(const Params &prm, float *sm, int slice, int b, int h, int hist, int L, int tile) {
+  constexpr int LD = 68;
+  float *Qs = sm, *Ks = sm + 64 * LD;
+  const int c = threadIdx.x & 15, j0 = tile * kKeys;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = (threadIdx.x >> 4) + 16 * u;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 q = r < prm.w ? reinterpret_cast<const float4 *>(row_ptr<float>(prm.Q, b, h, prm.win_pos[r]))[c] : zero;
+    const float4 k = j0 + r < L ? reinterpret_cast<const float4 *>(entry(prm, false, slice, b, h, hist, j0 + r))[c] : zero;
+    *reinterpret_cast<float4 *>(Qs + r * LD + 4 * c) = q;
+    *reinterpret_cast<float4 *>(Ks + r * LD + 4 * c) = k;
+  }
+  __syncthreads();
+  tile_logits<64>(Qs, Ks, prm.w, j0, L, prm.win_logits + (size_t)slice * prm.w * prm.ld_l, prm.ld_l, prm.scale);
+}
+
+// grid (ceil(n_k / 128) and, where the window is recorded, the key tiles over split, n_slices, split); dynamic shared memory kSmemBytes.
 __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid_constant__ Params prm) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = tc::smem_u32(smem_raw);
-  const uint32_t bar_ops = base + kOffBar, bar_mma = base + kOffBar + 8;
-  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem_raw + kOffBar + 16);
-  volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 20);
-  volatile int *leave_slot = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 24);
+  auto bar = [&](int i) { return base + kOffBar + 8u * (uint32_t)i; };
+  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem_raw + kOffBar + 32);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 36);
+  volatile int *leave_slot = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 40);
   const LayerView &lv = prm.lv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice - b * lv.n_heads;
   const int q0 = blockIdx.x * kRows, n_k = prm.n_k, n_split = gridDim.z;
   int *status = lv.status;
+  if ((int)blockIdx.x >= prm.blocks) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int hist = lv.hist_len[slice], L = min(hist + n_k, prm.room), tile = ((int)blockIdx.x - prm.blocks) * n_split + (int)blockIdx.z;
+    if (tile * kKeys < L) window_logits(prm, reinterpret_cast<float *>(smem_raw), slice, b, h, hist, L, tile);
+    return;
+  }
   if (tid == 0) {
-    tc::mbar_init(bar_ops, 4);           // the operand warps announce V of a tile and K of the next
-    tc::mbar_init(bar_mma, 1);           // the products issued together have landed, and read what they read
+    tc::mbar_init(bar(bV), 4);           // (one lane of each operand warp)
+    for (int i = bPv; i <= bS + 1; ++i) tc::mbar_init(bar(i), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   } else if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + kOffBar + 16), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + kOffBar + 32), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   // (what is above runs while the kernel before this one ends; see attend_tc_kernel)
@@ -189,7 +227,9 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     *leave_slot = leave;
     if (!leave && blockIdx.x == 0 && blockIdx.z == 0) lv.next_len[slice] = L;      // unless a compress of this scale evicts
   }
-  // Q: a thread takes one chunk of eight columns of four rows
+  // Q: a thread takes one chunk of eight columns of four rows.  (Of a negative scale Q takes the sign, so that the largest product is
+  // the largest score.)
+  const float sign = prm.scale_log2e < 0.f ? -1.f : 1.f;
   {
     float4 x[4][2];
 #pragma unroll
@@ -198,8 +238,9 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (q0 + r < n_k) {
         const float4 *src = reinterpret_cast<const float4 *>(row_ptr<float>(prm.Q, b, h, q0 + r)) + 2 * c;
-        x[u][0] = __ldg(src);
-        x[u][1] = __ldg(src + 1);
+        const float4 x0 = __ldg(src), x1 = __ldg(src + 1);
+        x[u][0] = make_float4(x0.x * sign, x0.y * sign, x0.z * sign, x0.w * sign);
+        x[u][1] = make_float4(x1.x * sign, x1.y * sign, x1.z * sign, x1.w * sign);
       }
     }
 #pragma unroll
@@ -214,26 +255,36 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   const uint32_t tmem = *tmem_slot;
   float *rows_out = reinterpret_cast<float *>(smem_raw + kOffQ);               // [row][64], 16-byte pieces permuted by the row
   float2 *stat_out = reinterpret_cast<float2 *>(smem_raw + kOffStat);
+  constexpr uint32_t dhi = tc::desc_hi(1024);
+  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);    // bf16, N = 64, M = 128
+  constexpr uint32_t idesc_pv = idesc | (1u << 16);                                                            // B is MN-major
+  // S of tile i and P V of tile i have landed (waits)
+  auto s_landed = [&](int i) { return tc::mbar_wait_warp(bar(bS + (i & 1)), (i >> 1) & 1, abort_flag, status); };
+  auto pv_landed = [&](int i) { return tc::mbar_wait_warp(bar(bPv), i & 1, abort_flag, status); };
 
   if (warp >= 4) {
     // ---------------------------------------------------------------- operands
     const int ct = tid - 128, c = ct & 7, r0 = ct >> 3;
-    auto load = [&](bool values, int tile, float4 (&x)[4][2]) {
+    long long at[4];                     // where the rows of the tile whose keys were loaded last lie in the pages, in bytes
+    auto load = [&](bool values, int tile, float4 (&x)[4][2]) {      // (the keys of a tile before its values)
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int slot = tile * kKeys + r0 + 16 * u;
+        const bool outside = prm.fused && slot >= hist;
         x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (slot < L) {
-          const float4 *src = reinterpret_cast<const float4 *>(entry(prm, values, slice, b, h, hist, slot)) + 2 * c;
-          x[u][0] = src[0];
-          x[u][1] = src[1];
+          if (!values && !outside) at[u] = (long long)slot_row(lv, slice, slot) * 256;
+          const char *row = outside ? reinterpret_cast<const char *>(row_ptr<float>(values ? prm.V : prm.K, b, h, slot - hist))
+                                    : (values ? lv.v_pool : lv.k_pool) + at[u];
+          x[u][0] = reinterpret_cast<const float4 *>(row)[2 * c];
+          x[u][1] = reinterpret_cast<const float4 *>(row)[2 * c + 1];
         }
       }
     };
     auto put = [&](bool values, int tile, const float4 (&x)[4][2]) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) put_split(base + (values ? kOffV : kOffK), kPieceK, r0 + 16 * u, c, x[u][0], x[u][1]);
-      if (prm.copy_in && tile * kKeys + kKeys > hist && tile % (int)gridDim.x == (int)blockIdx.x) {      // (the CTAs of a slice take turns)
+      if (prm.copy_in && tile * kKeys + kKeys > hist && tile % prm.blocks == (int)blockIdx.x) {      // (the CTAs of a slice take turns)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int slot = tile * kKeys + r0 + 16 * u;
@@ -246,53 +297,86 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
         }
       }
     };
-    auto announce = [&] {
+    const uint32_t q_lo = tc::desc_lo(base + kOffQ, 16), k_lo = tc::desc_lo(base + kOffK, 16);
+    int issued = 0;                      // products S issued by warp 4
+    auto mma_s = [&](int i) {            // products of pieces, the smallest first
+      constexpr int A[6] = {2, 0, 1, 1, 0, 0}, B[6] = {0, 2, 1, 0, 1, 0};
+      tc_fence_after();
+#pragma unroll
+      for (int e = 0; e < 6; ++e) mma4_ss(tmem + kBufCols * (i & 1), q_lo + A[e] * (kPieceQ >> 4), k_lo + B[e] * (kPieceK >> 4), dhi, idesc, e > 0);
+      if (tc::elect_one()) tc::tc_commit(bar(bS + (i & 1)));
+      __syncwarp();
+      issued = i + 1;
+    };
+    auto keys_there = [&] {              // all four warps have left their part
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("bar.sync 3, 128;" ::: "memory");
+    };
+    auto announce_v = [&] {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(bar_ops);
+      if (lane == 0) tc::mbar_arrive(bar(bV));
     };
     float4 kx[4][2], vx[4][2];
     if (nt > 0) {
       load(false, lo, kx);
       load(true, lo, vx);
       put(false, lo, kx);
-      announce();
-      if (nt > 1) load(false, lo + 1, kx);
+      keys_there();
+      if (warp == 4) mma_s(0);
       put(true, lo, vx);
+      announce_v();
+      if (nt > 1) {
+        load(false, lo + 1, kx);
+        load(true, lo + 1, vx);
+      }
     }
+    bool ok = true;
+    // (a warp whose wait gives up goes on to meet the others at the named barrier, which knows no limit)
     for (int i = 0; i < nt; ++i) {
-      if (!tc::mbar_wait_warp(bar_mma, i & 1, abort_flag, status)) break;      // K_i and V_{i-1} have been read
-      if (i > 0) put(true, lo + i, vx);
-      if (i + 1 < nt) put(false, lo + i + 1, kx);
-      announce();
-      if (i + 1 < nt) load(true, lo + i + 1, vx);
-      if (i + 2 < nt) load(false, lo + i + 2, kx);
+      const bool more = i + 1 < nt;
+      ok = ok && s_landed(i);                                 // K_i has been read
+      if (more) {
+        if (ok) put(false, lo + i + 1, kx);
+        keys_there();
+      }
+      ok = ok && (i == 0 || pv_landed(i - 1));                // V_{i-1} has been read, and P_{i-1}
+      if (warp == 4 && more && ok) mma_s(i + 1);
+      if (ok && i > 0) {
+        put(true, lo + i, vx);
+        announce_v();
+        if (more) load(true, lo + i + 1, vx);
+      }
+      if (ok && i + 2 < nt) load(false, lo + i + 2, kx);
     }
+    // (given up: what has been issued must be through before TMEM and shared memory are anybody else's)
+    if (!ok && issued > 0) tc::mbar_drain(bar(bS + ((issued - 1) & 1)), ((issued - 1) >> 1) & 1);
   } else {
     // ---------------------------------------------------------------- softmax
-    constexpr uint32_t dhi = tc::desc_hi(1024);
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);    // bf16, N = 64, M = 128
-    constexpr uint32_t idesc_pv = idesc | (1u << 16);                                                            // B is MN-major
-    const uint32_t q_lo = tc::desc_lo(base + kOffQ, 16), k_lo = tc::desc_lo(base + kOffK, 16), v_lo = tc::desc_lo(base + kOffV, 16);
-    // products of pieces, the smallest first
-    auto mma_s = [&] {
-      constexpr int A[6] = {2, 0, 1, 1, 0, 0}, B[6] = {0, 2, 1, 0, 1, 0};
-#pragma unroll
-      for (int e = 0; e < 6; ++e) mma4_ss(tmem + kColS, q_lo + A[e] * (kPieceQ >> 4), k_lo + B[e] * (kPieceK >> 4), dhi, idesc, e > 0);
-    };
-    auto mma_pv = [&] {
-      constexpr int A[6] = {2, 0, 1, 1, 0, 0}, B[6] = {0, 2, 1, 0, 1, 0};
-#pragma unroll
-      for (int e = 0; e < 6; ++e) mma4_ts(tmem + kColO, tmem + kColP + 32 * A[e], v_lo + B[e] * (kPieceK >> 4), dhi, idesc_pv, e > 0);
+    const uint32_t v_lo = tc::desc_lo(base + kOffV, 16);
+    auto mma_pv = [&](int i) {
+      const uint32_t p = tmem + kBufCols * (i & 1);
+      constexpr uint32_t step_v = kPieceK >> 4;
+      tc_fence_after();
+      mma4_ts<8>(tmem + kColO, p + kColPl, v_lo, dhi, idesc_pv, 0);
+      mma4_ts<16>(tmem + kColO, p, v_lo + 2 * step_v, dhi, idesc_pv, 1);
+      mma4_ts<16>(tmem + kColO, p + kColPm, v_lo + step_v, dhi, idesc_pv, 1);
+      mma4_ts<16>(tmem + kColO, p + kColPm, v_lo, dhi, idesc_pv, 1);
+      mma4_ts<16>(tmem + kColO, p, v_lo + step_v, dhi, idesc_pv, 1);
+      mma4_ts<16>(tmem + kColO, p, v_lo, dhi, idesc_pv, 1);
+      if (tc::elect_one()) tc::tc_commit(bar(bPv));
+      __syncwarp();
     };
     const int row = warp * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-    const float c = prm.scale_log2e;
+    const float c = prm.scale_log2e * sign;
     uint64_t o[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) o[i] = 0ull;
     float m = kNoMax, l = 0.f, l_rest = 0.f;       // l_rest: what the additions to l have rounded off
-    auto add_products = [&] {            // of P with a tile of V
+    // (o + P V of the tile before) f
+    auto add_products = [&](float f, bool scale) {
+      const uint64_t ff = tc::pack2(f, f);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         uint32_t x[16];
@@ -301,95 +385,95 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[8 * e + i] = tc::add2(o[8 * e + i], tc::pack2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])));
       }
+      if (scale) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) o[i] = tc::mul2(o[i], ff);
+      }
+    };
+    // The softmax of tile i (masked: a ragged one).  f: what the sums so far are to be scaled by; returns whether any is not 1.
+    auto sweep = [&](int i, float &f, auto masked) {
+      const int valid = L - (lo + i) * kKeys;
+      const uint32_t buf = lane_addr + kBufCols * (i & 1);
+      auto real = [&](int key) { return !decltype(masked)::value || key < valid; };
+      float mx = -INFINITY;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t x[16];
+        tc::tc_ld16(buf + 16 * e, x);
+        tc::tc_wait_ld();
+#pragma unroll
+        for (int q = 0; q < 16; q += 2)
+          mx = tc::max3(mx, real(16 * e + q) ? __uint_as_float(x[q]) : -INFINITY, real(16 * e + q + 1) ? __uint_as_float(x[q + 1]) : -INFINITY);
+      }
+      mx = fmaxf(m, mx * c);
+      const bool scale = __any_sync(0xffffffffu, mx > m);
+      if (scale) {
+        f = tc::ex2(m - mx);
+        l *= f;
+        l_rest *= f;
+        m = mx;
+      }
+      const uint64_t c2 = tc::pack2(c, c), lost2 = tc::pack2(c * kCutOff, c * kCutOff), negm2 = tc::pack2(-m, -m);
+      uint64_t sum2[2] = {0ull, 0ull};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t x[16], ph[8], pm[8], pl[8];
+        tc::tc_ld16(buf + 16 * e, x);
+        tc::tc_wait_ld();
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float a0, a1;
+          const uint64_t s2 = tc::pack2(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1]));
+          tc::unpack2(tc::fma2(s2, c2, tc::fma2(s2, lost2, negm2)), a0, a1);
+          a0 = real(16 * e + 2 * q) ? tc::ex2(a0) : 0.f;
+          a1 = real(16 * e + 2 * q + 1) ? tc::ex2(a1) : 0.f;
+          sum2[q & 1] = tc::add2(sum2[q & 1], tc::pack2(a0, a1));
+          split2(a0, a1, ph[q], pm[q], pl[q]);
+        }
+        tc_st8(buf + 16 * e, ph);
+        tc_st8(buf + 16 * e + kColPm, pm);
+        tc_st8(buf + 8 * e + kColPl, pl);
+      }
+      float s0, s1, s2, s3;
+      tc::unpack2(sum2[0], s0, s1);
+      tc::unpack2(sum2[1], s2, s3);
+      const float add = (s0 + s1) + (s2 + s3), sum = l + add, part = sum - l;
+      l_rest += (l - (sum - part)) + (add - part);
+      l = sum;
+      return scale;
     };
     bool ok = true;
-    if (warp == 0 && nt > 0) {
-      ok = tc::mbar_wait_warp(bar_ops, 0, abort_flag, status);
-      tc_fence_after();
-      if (ok) {
-        mma_s();
-        if (tc::elect_one()) tc::tc_commit(bar_mma);
-      }
-      __syncwarp();
-    }
-    int issued = ok && nt > 0 ? 1 : 0;   // commits of warp 0
+    int issued = 0;                      // products P V issued by warp 0
     for (int i = 0; i < nt; ++i) {
       // (a warp whose wait gives up goes on to meet the others at the named barrier, which knows no limit)
-      ok = ok && tc::mbar_wait_warp(bar_mma, i & 1, abort_flag, status);
+      ok = ok && s_landed(i);
       if (ok) {
         tc_fence_after();
-        if (i > 0) add_products();
-        const int valid = L - (lo + i) * kKeys;
-        float mx = m;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          uint32_t x[16];
-          tc::tc_ld16(lane_addr + kColS + 16 * e, x);
-          tc::tc_wait_ld();
-#pragma unroll
-          for (int q = 0; q < 16; q += 2) {
-            const float y0 = 16 * e + q < valid ? __uint_as_float(x[q]) * c : kNoMax, y1 = 16 * e + q + 1 < valid ? __uint_as_float(x[q + 1]) * c : kNoMax;
-            mx = tc::max3(mx, y0, y1);
-          }
+        float f = 1.f;
+        const bool scale = L - (lo + i) * kKeys < kKeys ? sweep(i, f, std::true_type{}) : sweep(i, f, std::false_type{});
+        if (i > 0) {
+          ok = pv_landed(i - 1);
+          tc_fence_after();
+          if (ok) add_products(f, scale);
         }
-        if (__any_sync(0xffffffffu, mx > m)) {
-          const float f = tc::ex2(m - mx);
-          const uint64_t ff = tc::pack2(f, f);
-#pragma unroll
-          for (int q = 0; q < 32; ++q) o[q] = tc::mul2(o[q], ff);
-          l *= f;
-          l_rest *= f;
-          m = mx;
-        }
-        const uint64_t c2 = tc::pack2(c, c), lost2 = tc::pack2(c * kCutOff, c * kCutOff), negm2 = tc::pack2(-m, -m);
-        uint64_t sum2[2] = {0ull, 0ull};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          uint32_t x[16], ph[8], pm[8], pl[8];
-          tc::tc_ld16(lane_addr + kColS + 16 * e, x);
-          tc::tc_wait_ld();
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            float a0, a1;
-            const uint64_t s2 = tc::pack2(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1]));
-            tc::unpack2(tc::fma2(s2, c2, tc::fma2(s2, lost2, negm2)), a0, a1);
-            a0 = 16 * e + 2 * q < valid ? tc::ex2(a0) : 0.f;
-            a1 = 16 * e + 2 * q + 1 < valid ? tc::ex2(a1) : 0.f;
-            sum2[q & 1] = tc::add2(sum2[q & 1], tc::pack2(a0, a1));
-            split2(a0, a1, ph[q], pm[q], pl[q]);
-          }
-          tc_st8(lane_addr + kColP + 8 * e, ph);
-          tc_st8(lane_addr + kColP + 32 + 8 * e, pm);
-          tc_st8(lane_addr + kColP + 64 + 8 * e, pl);
-        }
-        float s0, s1, s2, s3;
-        tc::unpack2(sum2[0], s0, s1);
-        tc::unpack2(sum2[1], s2, s3);
-        const float add = (s0 + s1) + (s2 + s3), sum = l + add, part = sum - l;
-        l_rest += (l - (sum - part)) + (add - part);
-        l = sum;
         tc::tc_wait_st();
         tc_fence_before();
       }
       asm volatile("bar.sync 2, 128;" ::: "memory");
       if (warp == 0) {
-        ok = ok && tc::mbar_wait_warp(bar_ops, (i + 1) & 1, abort_flag, status);
+        ok = ok && tc::mbar_wait_warp(bar(bV), i & 1, abort_flag, status);
         if (ok) {
-          tc_fence_after();
-          mma_pv();
-          if (i + 1 < nt) mma_s();
-          if (tc::elect_one()) tc::tc_commit(bar_mma);
+          mma_pv(i);
           ++issued;
         }
-        __syncwarp();
       }
     }
     if (warp == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (nt > 0) ok = ok && tc::mbar_wait_warp(bar_mma, nt & 1, abort_flag, status);
+    if (nt > 0) ok = ok && pv_landed(nt - 1);
     tc_fence_after();
-    if (ok && nt > 0) add_products();
-    // (given up: what has been issued must be through before TMEM and shared memory are anybody else's)
-    if (!ok && warp == 0 && issued > 0) tc::mbar_drain(bar_mma, (issued - 1) & 1);
+    if (ok && nt > 0) add_products(1.f, false);
+    // (given up: as above)
+    if (!ok && issued > 0) tc::mbar_drain(bar(bPv), (issued - 1) & 1);
     l += l_rest;
     float *mine = rows_out + row * 64;
     float amax = 0.f;

@@ -84,6 +84,48 @@ __device__ __forceinline__ void load_tile_rows(float *dst, int ld, const LayerVi
   }
 }
 
+// The base-2 logits of w window rows (Qs, 64 rows of D + 4 columns) against the 64 entries from j0 on (Ks alike): every one a chain of
+// multiply-adds in the order of the columns, whichever kernel asks.  256 threads; `out`: the rows' logits by slot.
+template <int D>
+__device__ __forceinline__ void tile_logits(const float *Qs, const float *Ks, int w, int j0, int L, float *out, int ld_l, float scale) {
+  constexpr int LD = D + 4;
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  const int ni = (w + 15) >> 4;  // active 16-row groups
+  float s[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+  for (int c = 0; c < D; c += 4) {
+    float4 k[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const float4 *>(&Ks[(tx + 16 * j) * LD + c]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i < ni) {
+        const float4 q = *reinterpret_cast<const float4 *>(&Qs[(ty + 16 * i) * LD + c]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s[i][j] = fmaf(q.x, k[j].x, s[i][j]);
+          s[i][j] = fmaf(q.y, k[j].y, s[i][j]);
+          s[i][j] = fmaf(q.z, k[j].z, s[i][j]);
+          s[i][j] = fmaf(q.w, k[j].w, s[i][j]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = ty + 16 * i;
+    if (r >= w) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int col = j0 + tx + 16 * j;
+      if (col < L) out[(size_t)r * ld_l + col] = s[i][j] * (scale * 1.4426950408889634f);
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------------
 // score, step 1 (only when attend did not record them): logits of the window rows against a tile of
 // 64 cache entries (Eq. 5), in base-2 units: y = scale * log2(e) * <q, k>.
@@ -119,40 +161,7 @@ __global__ void __launch_bounds__(256) score_logits_kernel(LayerView lv, TensorV
   }
   load_tile_rows<T, D>(Ks, LD, lv, lv.k_pool, slice, j0, L);
   __syncthreads();
-  const int ni = (wa.w + 15) >> 4;  // active 16-row groups
-  float s[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-  for (int c = 0; c < D; c += 4) {
-    float4 k[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const float4 *>(&Ks[(tx + 16 * j) * LD + c]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (i < ni) {
-        const float4 q = *reinterpret_cast<const float4 *>(&Qs[(ty + 16 * i) * LD + c]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s[i][j] = fmaf(q.x, k[j].x, s[i][j]);
-          s[i][j] = fmaf(q.y, k[j].y, s[i][j]);
-          s[i][j] = fmaf(q.z, k[j].z, s[i][j]);
-          s[i][j] = fmaf(q.w, k[j].w, s[i][j]);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = ty + 16 * i;
-    if (r >= wa.w) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int col = j0 + tx + 16 * j;
-      if (col < L) logits[((size_t)slice * wa.w + r) * ld_l + col] = s[i][j] * (scale * 1.4426950408889634f);
-    }
-  }
+  tile_logits<D>(Qs, Ks, wa.w, j0, L, logits + (size_t)slice * wa.w * ld_l, ld_l, scale);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -265,55 +274,59 @@ __global__ void __launch_bounds__(256) recent_keys_kernel(LayerView lv, int n_k,
   keys[(size_t)slice * ld_s + i] = pos < n_sink ? kWindowKey : (uint32_t)pos + 1u;
 }
 
-// Base-2 log-sum-exp of every window row of y[w][L] when attend did not record it: one CTA of 1024
-// threads per slice, 16 rows per round, a maximum sweep and a sum sweep.  lse is [n_slices][w].
+// Base-2 log-sum-exp of every window row of y[w][L] when attend did not record it: a CTA of 1024 threads per slice and four
+// rows, a maximum sweep and a sum sweep.  What bounds it is the latency of its reductions: 16 slices behind 92 to 772 entries, us per layer and
+// step of the f32 attention with 16 rows per CTA -> so: 64 queries 20.5 -> 19.5, 576: 55.3 -> 53.8.  lse is [n_slices][w].
+// grid (n_slices, ceil(w / 4)).
 __global__ void __launch_bounds__(1024) row_lse_kernel(LayerView lv, WindowArg wa, const float *logits, int ld_l, float *lse) {
-  __shared__ float part[32][16];
-  __shared__ float m_row[16];
+  constexpr int R = 4;
+  __shared__ float part[32][R];
+  __shared__ float m_row[R];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (the compress comes up and waits)
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int slice = blockIdx.x;
   const int L = lv.hist_len[slice] + wa.n_k;
   if (outgrown(lv, L)) return;
   const int w = wa.w;
   const float *y = logits + (size_t)slice * w * ld_l;
-  for (int g0 = 0; g0 < w; g0 += 16) {
-    const int nr = w - g0 < 16 ? w - g0 : 16;
-    float acc[16];
+  for (int g0 = R * (int)blockIdx.y; g0 < w; g0 += R * (int)gridDim.y) {
+    const int nr = w - g0 < R ? w - g0 : R;
+    float acc[R];
 #pragma unroll
-    for (int r = 0; r < 16; ++r) acc[r] = -INFINITY;
+    for (int r = 0; r < R; ++r) acc[r] = -INFINITY;
     for (int i = tid; i < L; i += 1024) {
 #pragma unroll
-      for (int r = 0; r < 16; ++r)
+      for (int r = 0; r < R; ++r)
         if (r < nr) acc[r] = fmaxf(acc[r], y[(size_t)(g0 + r) * ld_l + i]);
     }
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < R; ++r) {
       float v = acc[r];
       for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
       if (lane == 0) part[wid][r] = v;
     }
     __syncthreads();
-    if (tid < 16) {
+    if (tid < R) {
       float v = part[0][tid];
       for (int k = 1; k < 32; ++k) v = fmaxf(v, part[k][tid]);
       m_row[tid] = v;
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < 16; ++r) acc[r] = 0.f;
+    for (int r = 0; r < R; ++r) acc[r] = 0.f;
     for (int i = tid; i < L; i += 1024) {
 #pragma unroll
-      for (int r = 0; r < 16; ++r)
+      for (int r = 0; r < R; ++r)
         if (r < nr) acc[r] += exp2f(y[(size_t)(g0 + r) * ld_l + i] - m_row[r]);
     }
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < R; ++r) {
       float v = acc[r];
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) part[wid][r] = v;
     }
     __syncthreads();
-    if (tid < 16) {
+    if (tid < R) {
       float v = 0.f;
       for (int k = 0; k < 32; ++k) v += part[k][tid];     // fixed order: deterministic
       if (tid < nr) lse[(size_t)slice * w + g0 + tid] = m_row[tid] + log2f(v);
@@ -619,10 +632,11 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int slice = blockIdx.x;
   const int w = wa.w;
+  for (int i = tid; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(lv.page_table + (size_t)slice * lv.pages_per_slice + i);
+  asm volatile("griddepcontrol.wait;" ::: "memory");                        // (behind a kernel of the same call it comes up while that ends)
   const int dev_status = *reinterpret_cast<volatile int *>(lv.status);      // (all of this is under way before any of it is needed)
   const int hist = *reinterpret_cast<volatile int *>(lv.hist_len + slice);
   if (slice_budget != nullptr) budget = slice_budget[slice];
-  for (int i = tid; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(lv.page_table + (size_t)slice * lv.pages_per_slice + i);
   if (policy == 0 && tid < w) lse_row[tid] = lse[(size_t)slice * w + tid];
   const int L = hist + wa.n_k;
   if (dev_status != 0 || outgrown(lv, L)) return;   // a failed check, an earlier kernel's or this one's: leave the store alone

@@ -688,9 +688,7 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
     if (fused) { kc = tview(ctx->pend_k[layer]); vc = tview(ctx->pend_v[layer]); }
     const int k = ctx->next_scale[layer] - 1;
     const std::vector<int> &win = p.windows[k];
-    // (f32: the compress takes the window's logits from K, in plain fp32 sums.  Importances a few 1e-7 apart decide what is kept, so that
-    // logits of another rounding, as exact as they may be, keep another entry in one pass of some.)
-    float *wl = (win.empty() || !record || k + 1 == p.K || !ctx->tc.enabled())
+    float *wl = (win.empty() || !record || k + 1 == p.K)
                     ? nullptr
                     : reinterpret_cast<float *>(ctx->ws + p.off_logits) + (size_t)(layer % kSets) * p.logits_elems;
     float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
@@ -711,12 +709,19 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       prm.lv = lv; prm.Q = tview(Q); prm.O = tview(O); prm.K = kc; prm.V = vc; prm.lse = lse; prm.n_k = nk;
       prm.room = lv.pages_per_slice << lv.page_shift;
       prm.fused = fused ? 1 : 0; prm.copy_in = (fused && copy) ? 1 : 0; prm.n_prev = p.N[k];
-      prm.scale_log2e = ctx->scale * 1.4426950408889634f;
+      prm.scale = ctx->scale; prm.scale_log2e = ctx->scale * 1.4426950408889634f;
+      // The window's logits: plain fp32 sums, as the compress would take them from K by a launch of its own, 16 rows of every key tile by a
+      // CTA beside the others.  (Not from the tensor core's scores: importances a few 1e-7 apart decide what is kept, so that logits of
+      // another rounding, as exact as they may be, keep another entry in one pass of some.)
+      prm.win_logits = wl; prm.ld_l = p.ld_l; prm.w = wl ? (int)win.size() : 0;
+      for (int e = 0; e < prm.w; ++e) prm.win_pos[e] = win[e];
       const int blocks = (nk + f32::kRows - 1) / f32::kRows;
       const int split = f32::key_split(blocks * p.n_slices, (ctx->hist[layer] + nk + f32::kKeys - 1) / f32::kKeys, ctx->n_sm);
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[2];
-      cfg.gridDim = dim3(blocks, p.n_slices, split);
+      prm.blocks = blocks;
+      const int key_tiles = (ctx->hist[layer] + nk + f32::kKeys - 1) / f32::kKeys;
+      cfg.gridDim = dim3(blocks + (wl ? (key_tiles + split - 1) / split : 0), p.n_slices, split);
       cfg.blockDim = dim3(f32::kThreads);
       cfg.dynamicSmemBytes = f32::kSmemBytes;
       cfg.stream = ctx->s_main;
@@ -874,12 +879,13 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     }
     ctx->logits_of[layer] = -1;
     float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
-    if (!recorded) {
+    const bool summed = recorded && ctx->tc.enabled();          // (the f32 attention leaves what the logits kernel would)
+    if (!recent && !summed) {
       Scope sc(ctx, s, kScore);
-      row_lse_kernel<<<p.n_slices, 1024, 0, s>>>(lv, wa, logits, p.ld_l, wlse);
+      row_lse_kernel<<<dim3(p.n_slices, (wa.w + 3) / 4), 1024, 0, s>>>(lv, wa, logits, p.ld_l, wlse);
     }
     // logits recorded by attend are raw products in the tile-aligned layout; the logits kernel writes base-2 logits by slot
-    const float logit_scale = recorded ? ctx->scale * 1.4426950408889634f : 1.f;
+    const float logit_scale = summed ? ctx->scale * 1.4426950408889634f : 1.f;
     const int tile_padded = (recorded && ctx->logits_padded[layer]) ? 1 : 0;
     // keys are the bits of non-negative floats, or positions: what has to be shifted out to leave 11 bits
     int shift = 20;
@@ -903,9 +909,18 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
       // and a compress that is quicker alone is slower among them (16 slices, 1 944 of 4 248 entries kept, by one CTA, a
       // cluster of two or of four: alone 35, 25, 20 us; a pass of one image, 32 layers, 13.31, 13.57, 13.87 ms called layer
       // by layer, replayed from a graph 12.30, 12.47, 12.5).
-      compress_fused_kernel<<<p.n_slices, kCompressThreads, ctx->fused_smem, s>>>(lv, wa, recent ? 1 : 0, n_sink, logits, wlse, p.ld_l,
-                                                                                 logit_scale, tile_padded, budget, slice_budget, pool,
-                                                                                 shift, scores, p.ld_s, kept, ext);
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr[1];
+      cfg.gridDim = dim3(p.n_slices);
+      cfg.blockDim = dim3(kCompressThreads);
+      cfg.dynamicSmemBytes = ctx->fused_smem;
+      cfg.stream = s;
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = recent || summed ? 0 : 1;   // (behind a kernel of this call)
+      CU(cudaLaunchKernelEx(&cfg, compress_fused_kernel, lv, wa, recent ? 1 : 0, n_sink, (const float *)logits, (const float *)wlse, p.ld_l,
+                            logit_scale, tile_padded, budget, (const int *)slice_budget, pool, shift, scores, p.ld_s, kept, ext));
       if (external) ctx->in_store[layer] = 1;
     } else {
       if (!recent) {
@@ -1031,7 +1046,7 @@ static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, const scal
     const int sinks = std::min(std::max(opts->n_sink, 0), p.N[scale + 1]);
     return !(std::max(table - sinks, 0) < L - sinks);
   }
-  if (w <= 0 || !ctx->tc.enabled()) return true;
+  if (w <= 0) return true;
   bool planned = scale + 1 != p.K && window_pos && (int)p.windows[scale].size() == w;
   for (int j = 0; planned && j < w; ++j) planned = p.windows[scale][j] == window_pos[j];
   return !(planned && table < L - w);
