@@ -1173,6 +1173,9 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
     ctx->in_store[layer] = 1;
     sums = ctx->stats_host;
     ctx->len_written[layer] = 1;
+    // The call does not wait for the stream's end: a compress that follows does, not only for the attend (the kernel writes the
+    // length and the map's rows).
+    ctx->attend_marked[layer] = 0;
   } else {
     CU(cudaMemsetAsync(acc, 0, acc_bytes, ctx->s_main));
     {

@@ -1,4 +1,6 @@
 """Compresses that run beside later layers' attends: the same values, bit for bit, as with everything on one stream."""
+import time
+
 import pytest
 import torch
 
@@ -77,4 +79,38 @@ def test_layers_that_share_a_logit_buffer_wait_for_each_other(order):
     windows = [orc.window_centroids(a, a, 16) for a in sides]
     beside, alone = (_shared_buffer_pass(order, data, windows, sides, s) for s in (True, False))
     for x, y in zip(beside, alone, strict=True):
+        assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("calls", ["attend", "step"])        # a map that the attend has copied, one that the statistics copy
+def test_a_compress_waits_for_the_statistics_before_it(calls):
+    """layer_stats returns when its sums have arrived, before stream_main's end is known: the compress waits for what stream_main
+    has been given since the attend, as work behind the statistics shows."""
+    sides, heads = (4, 12), 16
+    n = orc.scale_token_counts(sides)
+    gen = torch.Generator(device="cuda").manual_seed(37)
+    data = [tuple(torch.randn(1, heads, nk, 128, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(3)) for nk in n]
+    kept = []
+    for side_stream in (True, False):
+        kv = binding.ScaleKV(1, 1, heads, 128, "bf16", sides, sides, [[30] * len(n)], side_stream=side_stream)
+        torch.cuda.synchronize()
+        for k, (Q, K, V) in enumerate(data):
+            if calls == "attend" or k + 1 < len(n):
+                kv.scalekv_append(0, k, K, V)
+                kv.scalekv_attend(0, Q)
+            else:
+                kv.scalekv_step(0, k, Q, K, V, torch.empty_like(Q))
+            kv.scalekv_layer_stats_ex(0, Q)
+            with torch.cuda.stream(kv.stream_main):
+                torch.cuda._sleep(200_000_000)                # about a tenth of a second
+            kv.scalekv_compress(0, Q, orc.window_centroids(sides[k], sides[k], 16), qw_is_full_map=True)
+            done = torch.cuda.Event()
+            done.record(kv.stream_side)
+            time.sleep(0.02)
+            evicts = n[k] > 30 + 16
+            assert not (evicts and done.query())
+            kv.scalekv_sync()
+        kept.append([torch.cat([x.float().reshape(len(x), -1) for x in kv.scalekv_export_slice(0, 0, h, with_kv=True)], 1) for h in range(heads)])
+        kv.close()
+    for x, y in zip(*kept, strict=True):
         assert torch.equal(x, y)
