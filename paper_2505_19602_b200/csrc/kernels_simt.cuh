@@ -1106,8 +1106,9 @@ __global__ void __launch_bounds__(256, 2) stats_mma_kernel(LayerView lv, TensorV
   const int parts = ((int)gridDim.z - n_split) * gridDim.x, part = ((int)blockIdx.z - n_split) * (int)gridDim.x + (int)blockIdx.x;
   double *copied = sums + ((size_t)2 * gridDim.x + 1) * gridDim.y + (size_t)slice * parts + part;
   if (outgrown(lv, L)) {
-    if (tid < 2) sums[((size_t)slice * gridDim.x + blockIdx.x) * 2 + tid] = NAN;      // (an answer all the same)
-    if (tid == 2 && blockIdx.x == 0) sums[(size_t)2 * gridDim.x * gridDim.y + slice] = NAN;
+    // (an answer all the same, and every word of it by one CTA: behind the last of them the host may prepare the words for another call)
+    if (tid < 2 && blockIdx.z == 0) sums[((size_t)slice * gridDim.x + blockIdx.x) * 2 + tid] = NAN;
+    if (tid == 2 && blockIdx.z == 0 && blockIdx.x == 0) sums[(size_t)2 * gridDim.x * gridDim.y + slice] = NAN;
     if (tid == 3 && copies) *copied = NAN;
     return;
   }

@@ -38,3 +38,24 @@ def test_a_map_outside_the_pages(heads, height, width, stride):
         kv.close()
     # (the keys may be split over another number of CTAs: sums of fp32 weights in another order)
     assert torch.allclose(answers[0], answers[1], rtol=1e-5, atol=0)
+
+
+def test_every_word_of_an_answer_has_one_writer():
+    """Behind a refused selection the device's slices outgrow their pages, and every call answers that it has no numbers - at once, with
+    many CTAs per block of rows still to come: none of them may write into the next call's words."""
+    sides, heads = (2, 5, 9, 24), 3
+    kv = binding.ScaleKV(1, 1, heads, 128, "bf16", sides, sides, [[10] * 4], page_tokens=16)
+    g = torch.Generator(device="cuda").manual_seed(43)
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(1, heads, a * a, 128, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        if k < 3:                                                            # the heads part at scale 1; their common selection is refused at scale 2
+            kv.scalekv_attend(0, Q)
+            kv.scalekv_compress_ex(0, Q, binding.scalekv_window_centroids(a, a, 16), qw_is_full_map=True, head_shared=k == 2)
+    for _ in range(200):
+        car, htk, cars, htks, ncas = kv.scalekv_layer_stats_ex(0, Q, 16, 1)
+        assert all(x != x for x in [car, htk] + cars[0] + htks[0] + ncas[0])
+    with pytest.raises(binding.ScaleKVError):
+        kv.scalekv_sync()
+    kv.close()
