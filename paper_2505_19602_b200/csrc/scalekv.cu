@@ -308,6 +308,10 @@ bool tensor_ok(const scalekv_tensor &t, int esize) {
   return ((t.stride_b * esize) % 16 == 0) && ((t.stride_h * esize) % 16 == 0) && ((t.stride_t * esize) % 16 == 0);
 }
 
+bool same_strides(const scalekv_tensor &a, const scalekv_tensor &b) {
+  return a.stride_b == b.stride_b && a.stride_h == b.stride_h && a.stride_t == b.stride_t;
+}
+
 const char *const kClassNames[kNumClasses] = {"scalekv.append", "scalekv.attend", "scalekv.score", "scalekv.select",
                                                "scalekv.compact", "scalekv.other", "scalekv.compress"};
 
@@ -828,8 +832,10 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
   for (int j = 0; !recent && recorded && j < wa.w; ++j) recorded = p.windows[k][j] == wa.pos[j];
   const bool fused = ctx->fused_ok && !head_shared && !(opts && opts->separate_kernels);
   // A map that attend left in the caller's tensors stays there when the one-launch compress can do without the pages:
-  // it needs no K (the logits are recorded) and takes the surviving rows from the tensors.  Everything else copies first.
-  const bool external = !ctx->in_store[layer] && ctx->attended[layer] && evict && fused && recorded;
+  // it needs no K (the logits are recorded) and takes the surviving rows from the tensors, where K and V lie alike.  Everything
+  // else copies first.
+  const bool external = !ctx->in_store[layer] && ctx->attended[layer] && evict && fused && recorded &&
+                        same_strides(ctx->pend_k[layer], ctx->pend_v[layer]);
   const bool copy_now = !ctx->in_store[layer] && !external;
   if (!external) {
     st = materialize(ctx, layer);
@@ -903,7 +909,6 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
       if (external) {
         const TensorView kc = tview(ctx->pend_k[layer]), vc = tview(ctx->pend_v[layer]);
         ext.on = 1; ext.k = kc.ptr; ext.v = vc.ptr; ext.sb = kc.sb; ext.sh = kc.sh; ext.st = kc.st; ext.esize = p.esize;
-        if (vc.sb != kc.sb || vc.sh != kc.sh || vc.st != kc.st) return fail(ctx, SCALEKV_ERR_INVALID_ARG, "K and V of a map must have the same strides");
       }
       // One CTA per slice, however few the slices: every CTA keeps an attention CTA of the layers that follow off its SM,
       // and a compress that is quicker alone is slower among them (16 slices, 1 944 of 4 248 entries kept, by one CTA, a
@@ -1028,17 +1033,15 @@ scalekv_status scalekv_step_host(scalekv_ctx *ctx, int32_t layer, int32_t scale,
 
 // Whether the attend of a one-call step copies the current map into the pages (see attend_impl).  It does not when
 // the step's own compress will evict - the test scalekv_compress_ex makes - and will find what it needs without K in
-// the pages (the logits of exactly its window recorded, or a positional rule), so that it can take the map's
-// surviving rows from K and V itself; nor after the last scale without a compress, when nothing may ever need the rows.
+// the pages (the logits of exactly its window recorded, or a positional rule) and K and V laid out alike, so that it can take the
+// map's surviving rows from the tensors itself; nor after the last scale without a compress, when nothing may ever need the rows.
 // A wrong guess costs a copy kernel, never a result.
 static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, const scalekv_tensor &K, const scalekv_tensor &V, bool compress, int w,
                         const int32_t *window_pos, const scalekv_select_opts *opts) {
   if (!ctx || layer < 0 || layer >= ctx->plan.n_layers || scale < 0 || scale >= ctx->plan.K) return true;
   const Plan &p = ctx->plan;
   if (!compress) return scale + 1 != p.K;
-  // (a compress that takes rows from the tensors wants K and V laid out alike; of f32 maps others have always been taken)
-  if (!ctx->tc.enabled() && (K.stride_b != V.stride_b || K.stride_h != V.stride_h || K.stride_t != V.stride_t)) return true;
-  if (!ctx->fused_ok || (opts && (opts->head_shared || opts->separate_kernels || opts->head_budgets))) return true;
+  if (!same_strides(K, V) || !ctx->fused_ok || (opts && (opts->head_shared || opts->separate_kernels || opts->head_budgets))) return true;
   const int table = p.budgets[(size_t)layer * p.K + scale];
   if (table == SCALEKV_KEEP_ALL) return true;
   const int L = ctx->hist[layer] + p.n[scale];

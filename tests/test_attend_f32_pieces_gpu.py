@@ -129,3 +129,33 @@ def test_a_map_whose_keys_and_values_are_laid_out_differently():
         outs.append(O.clone())
         kv.close()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("policy", ["recent", "score"])
+def test_maps_laid_out_differently_are_pruned_like_others(dtype, policy):
+    """In the steps, and by a compress of its own behind the last one, which leaves its map in the caller's tensors."""
+    sides, heads, d = (4, 12, 15), 3, 64 if dtype == "f32" else 128
+    g = torch.Generator(device="cuda").manual_seed(8)
+    maps = [[torch.randn(1, heads, a * a, d, generator=g, device="cuda") for _ in range(3)] for a in sides]
+    left = []
+    for spread in (False, True):
+        kv = binding.ScaleKV(1, 1, heads, d, dtype, sides, sides, [[40] * 3])
+        for k, tensors in enumerate(maps):
+            Q, K, V = (x.to(kv.torch_dtype) for x in tensors)
+            if spread:
+                V = V.transpose(1, 2).contiguous().transpose(1, 2)
+            O = torch.zeros_like(Q)
+            window = binding.scalekv_window_centroids(sides[k], sides[k], 16)
+            torch.cuda.synchronize()
+            kv.scalekv_step_ex(0, k, Q, K, V, O, compress=k < 2, window_pos=kv.window_array(window), policy=policy)
+            if k == 2:
+                kv.scalekv_compress_ex(0, Q, window, qw_is_full_map=True, policy=policy)
+            kv.scalekv_sync()
+            left.append(O.clone())
+        left.append([kv.scalekv_export_slice(0, 0, h, with_kv=True) for h in range(heads)])
+        kv.close()
+    for x, y in zip(left[:3], left[4:7]):
+        assert torch.equal(x, y)
+    for x, y in zip(left[3], left[7]):
+        assert all(torch.equal(a, b) for a, b in zip(x, y))
