@@ -670,7 +670,9 @@ scalekv_status scalekv_append(scalekv_ctx *ctx, int32_t layer, int32_t scale, sc
 // that follows.  Recording costs the kernel 3-13 % (the threads that own window rows store 512 bytes per key tile and
 // their tile waits for them), so it is left out where no compress can use it: after the last scale of the schedule
 // (Sec. 3.3: nothing is generated after it, so the method prunes nothing there; a compress called all the same takes
-// its logits from K) and in a one-call step that names no window.
+// its logits from K) and in a one-call step that names no window.  The f32 kernel has CTAs of their own for it, which read the window's
+// queries while the others write outputs, so it does it only in a step, where that is known to be wanted: an f32 attend by itself takes an O
+// that lies over its Q, waits for nobody's compress, and the compress behind it takes its logits from K.
 // copy: whether a current map that is still in the caller's tensors is also copied into the pages while the kernel
 // streams it.  A one-call step leaves the copy out when its own compress will evict (the compress then takes the
 // surviving rows of the map straight from the caller's tensors: in a refiner layer 19 of 20 rows of a map would be
@@ -752,7 +754,7 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
 }
 
 scalekv_status scalekv_attend(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Q, scalekv_tensor O, float *lse) {
-  return attend_impl(ctx, layer, Q, O, lse, true, true);
+  return attend_impl(ctx, layer, Q, O, lse, ctx && ctx->tc.enabled(), true);
 }
 
 scalekv_status scalekv_compress(scalekv_ctx *ctx, int32_t layer, scalekv_tensor Qw, int32_t w, const int32_t *window_pos,
@@ -1014,7 +1016,7 @@ scalekv_status scalekv_step_host(scalekv_ctx *ctx, int32_t layer, int32_t scale,
   };
   scalekv_status st = scalekv_append(ctx, layer, scale, dense(dk), dense(dv));
   if (st != SCALEKV_OK) return st;
-  st = scalekv_attend(ctx, layer, dense(dq), dense(dout), nullptr);
+  st = attend_impl(ctx, layer, dense(dq), dense(dout), nullptr, ctx->tc.enabled() || w > 0, true);
   if (st != SCALEKV_OK) return st;
   CU(cudaEventRecord(ctx->ev_att[set], ctx->s_main));
   CU(cudaStreamWaitEvent(ctx->s_d2h, ctx->ev_att[set], 0));

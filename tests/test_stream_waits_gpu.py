@@ -114,3 +114,37 @@ def test_a_compress_waits_for_the_statistics_before_it(calls):
         kv.close()
     for x, y in zip(*kept, strict=True):
         assert torch.equal(x, y)
+
+
+def test_an_f32_attend_records_no_window():
+    """It does not know what compress follows, if any: it waits for no other layer's compress, and writes O over Q where it is asked to."""
+    sides, heads = (8, 32), 16
+    gen = torch.Generator(device="cuda").manual_seed(41)
+    data = [tuple(torch.randn(1, heads, a * a, 64, generator=gen, device="cuda") for _ in range(3)) for a in sides]
+    window = orc.window_centroids(32, 32, 16)
+    kept = []
+    for in_place in (True, False):
+        kv = binding.ScaleKV(5, 1, heads, 64, "f32", sides, sides, [[5, 50]] * 5, page_tokens=4096)
+        torch.cuda.synchronize()
+        for l in (0, 4):
+            kv.scalekv_step(l, 0, *data[0], torch.empty_like(data[0][0]), window_pos=orc.window_centroids(8, 8, 16))
+        kv.scalekv_sync()
+        Q, K, V = data[1]
+        kv.scalekv_append(0, 1, K, V)
+        kv.scalekv_attend(0, Q)
+        kv.scalekv_append(4, 1, K, V)
+        out, done = Q.clone(), torch.cuda.Event()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(kv.stream_side):
+            torch.cuda._sleep(200_000_000)                    # about a tenth of a second
+        kv.scalekv_compress(0, Q, window, qw_is_full_map=True)
+        O = kv.scalekv_attend(4, out if in_place else Q, out)
+        done.record(kv.stream_main)
+        time.sleep(0.02)
+        assert done.query()
+        kv.scalekv_compress(4, Q, window, qw_is_full_map=True)
+        kv.scalekv_sync()
+        kept.append([O] + [kv.scalekv_export_slice(l, 0, h) for l in (0, 4) for h in range(heads)])
+        kv.close()
+    for x, y in zip(*kept, strict=True):
+        assert torch.equal(x, y)
