@@ -632,12 +632,18 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int slice = blockIdx.x;
   const int w = wa.w;
-  for (int i = tid; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(lv.page_table + (size_t)slice * lv.pages_per_slice + i);
-  asm volatile("griddepcontrol.wait;" ::: "memory");                        // (behind a kernel of the same call it comes up while that ends)
-  const int dev_status = *reinterpret_cast<volatile int *>(lv.status);      // (all of this is under way before any of it is needed)
+  // All of this is under way before any of it is needed.  (Behind a kernel of the same call the CTA comes up while that ends: only the page
+  // table is there before the wait.)
+  const int *pages = lv.page_table + (size_t)slice * lv.pages_per_slice;
+  const int page = tid < lv.pages_per_slice ? __ldg(pages + tid) : 0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int dev_status = *reinterpret_cast<volatile int *>(lv.status);
   const int hist = *reinterpret_cast<volatile int *>(lv.hist_len + slice);
   if (slice_budget != nullptr) budget = slice_budget[slice];
-  if (policy == 0 && tid < w) lse_row[tid] = lse[(size_t)slice * w + tid];
+  const float row_lse = policy == 0 && tid < w ? lse[(size_t)slice * w + tid] : 0.f;
+  if (tid < lv.pages_per_slice) pt[tid] = page;
+  for (int i = tid + NT; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(pages + i);
+  if (policy == 0 && tid < w) lse_row[tid] = row_lse;
   const int L = hist + wa.n_k;
   if (dev_status != 0 || outgrown(lv, L)) return;   // a failed check, an earlier kernel's or this one's: leave the store alone
   __syncthreads();
