@@ -131,7 +131,7 @@ def test_an_f32_attend_records_no_window():
         kv.scalekv_sync()
         Q, K, V = data[1]
         kv.scalekv_append(0, 1, K, V)
-        kv.scalekv_attend(0, Q)
+        beside = kv.scalekv_attend(0, Q)                      # (held: what it is written to must not be given to `out`)
         kv.scalekv_append(4, 1, K, V)
         out, done = Q.clone(), torch.cuda.Event()
         torch.cuda.synchronize()
@@ -144,7 +144,7 @@ def test_an_f32_attend_records_no_window():
         assert done.query()
         kv.scalekv_compress(4, Q, window, qw_is_full_map=True)
         kv.scalekv_sync()
-        kept.append([O] + [kv.scalekv_export_slice(l, 0, h) for l in (0, 4) for h in range(heads)])
+        kept.append([O, beside] + [kv.scalekv_export_slice(l, 0, h) for l in (0, 4) for h in range(heads)])
         kv.close()
     for x, y in zip(*kept, strict=True):
         assert torch.equal(x, y)
