@@ -15,7 +15,7 @@
 // Scores that are not numbers (an infinite key: its products with the pieces of a query may differ in sign) spoil their row's sum, and
 // values that are not its columns; such a row is done again at the end by fp32 FMA from the tensors (fma_row).
 // The observation window's logits are taken by CTAs of their own beside the others, in plain fp32 (see the launch).
-// gridDim.z CTAs of a cluster share a slice's keys and combine: O = sum_e 2^(m_e - M) O_e / sum_e 2^(m_e - M) l_e, through distributed
+// gridDim.z CTAs of a cluster share a slice's keys and combine: O = sum_e 2^(c (m_e - M)) O_e / sum_e 2^(c (m_e - M)) l_e, through distributed
 // shared memory.
 // What bounds it: the instructions of the softmax and of the splitting, and the tensor pipe, six products standing for one; a step of two
 // CTAs that share an SM takes about 8 000 cycles.  (Working copies that skip work, us per layer, 16 slices x 1 600 queries: whole 130; one
@@ -49,7 +49,9 @@ static_assert(kOffStat + kRows * 8 <= kOffK, "the parts of a row have to fit whe
 static_assert(2 * (kSmemBytes + 1024) <= 233472, "two CTAs have to fit an SM");
 // What a score loses, of its size and on average, because the tensor core cuts its sums off: about half a unit in the last place (2^-24)
 // in each of the four steps over the large pieces, less in those where the sum is still growing.  It is given back (without: lse of queries
-// times 3 low by 6.6e-7 on average, 7.4e-7 rms; so by 0.3e-7, 3.4e-7 rms).
+// times 3 low by 6.6e-7 on average, 7.4e-7 rms; so by 0.1 to 0.5e-7, 3.2 to 3.4e-7 rms): to the differences between a row's products and their
+// reference, and to the reference where it enters a log-sum-exp.  (Given to the products alone, it would leave the largest weight at 2^(7e-8 m),
+// m its exponent: of scores near -1e9 the weights would lie where their pieces run out of range.)
 constexpr float kCutOff = 1.2f / 16777216.f;
 // TMEM: two buffers of 96 columns for scores and P, 64 columns for products with V.  The 16 keys of step kk have their scores in columns
 // 16 kk .. of a buffer, and their P there (h in the first eight, m in the next) and in columns 64 + 8 kk .. (l).
@@ -62,7 +64,8 @@ struct Params {
   float *lse;
   int n_k, room;               // room: entries that a slice's pages hold
   int fused, copy_in, n_prev;  // copy_in: the map's rows go to the pages on the way
-  float scale, scale_log2e;
+  float scale;
+  float weight_scale;          // what a difference of two rows' products is multiplied with to make a weight's exponent: |scale| log2(e), and kCutOff
   int blocks;                  // blocks of query rows; the CTAs behind them (blockIdx.x) take the logits of the window's w rows
   float *win_logits;           // base-2 logits by slot, [slice][rank][ld_l]
   int ld_l, w;
@@ -132,12 +135,13 @@ __device__ __forceinline__ const float *entry(const Params &prm, bool values, in
   return reinterpret_cast<const float *>((values ? prm.lv.v_pool : prm.lv.k_pool) + slot_row(prm.lv, slice, slot) * 256);
 }
 
-// The log-sum-exp of a row from its base-2 reference and sum: the logarithm is taken to base e and the sum rounded once (to base 2
-// both are of larger numbers), and what the 32-bit log2(e) in the reference is off by, 1.3e-8 of it, is put right.  rms error over
-// full caches of 521 to 4 240 entries, scores of deviation 0.25 / 1 / 3: 2.0 to 2.8e-7 / 1.9 to 3.0e-7 / 5.5 to 5.9e-7 (to base e
-// throughout 2.0 to 2.8 / 1.9 to 3.2 / 5.4 to 5.8; to base 2 throughout 2.6 to 3.6 / 2.7 to 3.7 / 6.5 to 6.7).
-__device__ __forceinline__ float row_lse_f32(float m, float l) {
-  return fmaf(m, 0.6931471805599453f, fmaf(m, (float)(1.0 / 1.4426950408889634f - 0.6931471805599453f), logf(l)));
+// The log-sum-exp of a row from its reference, the largest of its products, and its sum: the logarithm is taken to base e (to base 2 both are
+// of larger numbers), and what the sum of the two is rounded by is put right together with kCutOff's part, which by itself would be lost in it.
+__device__ __forceinline__ float row_lse_f32(float m, float l, float scale) {
+  const float lg = logf(l), sum = fmaf(m, scale, lg);
+  if (!(fabsf(sum) < INFINITY)) return sum;
+  const float rest = fabsf(m * scale) > fabsf(lg) ? fmaf(m, scale, -sum) + lg : fmaf(m, scale, lg - sum);      // (exact: the larger first)
+  return sum + fmaf(m, scale * kCutOff, rest);
 }
 
 // One row by fp32 FMA over the entries [from, to): its 64 columns go to `out` (16-byte pieces permuted by `swap`).  For
@@ -145,6 +149,7 @@ __device__ __forceinline__ float row_lse_f32(float m, float l) {
 struct RowSum { float m, l; };
 __device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int h, int hist, int q_row, int from, int to, float *out, int swap) {
   const float *q = row_ptr<float>(prm.Q, b, h, q_row);
+  const float cut = copysignf(1.f - kCutOff, prm.scale);                 // (products as the tensor core would leave them)
   float o[64], m = kNoMax, l = 0.f;
 #pragma unroll
   for (int d = 0; d < 64; ++d) o[d] = 0.f;
@@ -154,7 +159,8 @@ __device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int 
     float s = 0.f;
 #pragma unroll 8
     for (int d = 0; d < 64; ++d) s = fmaf(q[d], k[d], s);
-    const float y = s * prm.scale_log2e, mx = fmaxf(m, y), f = exp2f(m - mx), p = exp2f(y - mx);
+    s *= cut;
+    const float mx = fmaxf(m, s), f = exp2f((m - mx) * prm.weight_scale), p = exp2f((s - mx) * prm.weight_scale);
     m = mx;
     l = fmaf(l, f, p);
 #pragma unroll
@@ -229,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   }
   // Q: a thread takes one chunk of eight columns of four rows.  (Of a negative scale Q takes the sign, so that the largest product is
   // the largest score.)
-  const float sign = prm.scale_log2e < 0.f ? -1.f : 1.f;
+  const float sign = prm.scale < 0.f ? -1.f : 1.f;
   {
     float4 x[4][2];
 #pragma unroll
@@ -369,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     };
     const int row = warp * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-    const float c = prm.scale_log2e * sign;
+    const float c = prm.weight_scale;
     uint64_t o[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) o[i] = 0ull;
@@ -405,15 +411,15 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
         for (int q = 0; q < 16; q += 2)
           mx = tc::max3(mx, real(16 * e + q) ? __uint_as_float(x[q]) : -INFINITY, real(16 * e + q + 1) ? __uint_as_float(x[q + 1]) : -INFINITY);
       }
-      mx = fmaxf(m, mx * c);
+      mx = fmaxf(m, mx);
       const bool scale = __any_sync(0xffffffffu, mx > m);
       if (scale) {
-        f = tc::ex2(m - mx);
+        f = tc::ex2((m - mx) * c);
         l *= f;
         l_rest *= f;
         m = mx;
       }
-      const uint64_t c2 = tc::pack2(c, c), lost2 = tc::pack2(c * kCutOff, c * kCutOff), negm2 = tc::pack2(-m, -m);
+      const uint64_t c2 = tc::pack2(c, c), negm2 = tc::pack2(-m, -m);
       uint64_t sum2[2] = {0ull, 0ull};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -424,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
         for (int q = 0; q < 8; ++q) {
           float a0, a1;
           const uint64_t s2 = tc::pack2(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1]));
-          tc::unpack2(tc::fma2(s2, c2, tc::fma2(s2, lost2, negm2)), a0, a1);
+          tc::unpack2(tc::mul2(tc::add2(s2, negm2), c2), a0, a1);
           a0 = real(16 * e + 2 * q) ? tc::ex2(a0) : 0.f;
           a1 = real(16 * e + 2 * q + 1) ? tc::ex2(a1) : 0.f;
           sum2[q & 1] = tc::add2(sum2[q & 1], tc::pack2(a0, a1));
@@ -492,7 +498,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     }
     stat_out[row] = make_float2(m, l);
     if (n_split == 1 && ok && nt > 0 && q0 + row < n_k) {
-      if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + row] = row_lse_f32(m, l);
+      if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + row] = row_lse_f32(m, l, fabsf(prm.scale));
     }
     tc_fence_before();
   }
@@ -533,13 +539,13 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     float sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
     for (int e = 0; e < kMaxSplit; ++e) {
-      const float f = exp2f(me[e] - M);
+      const float f = exp2f((me[e] - M) * prm.weight_scale);
       sum = fmaf(f, le[e], sum);
       a0 = fmaf(f, x[e].x, a0); a1 = fmaf(f, x[e].y, a1); a2 = fmaf(f, x[e].z, a2); a3 = fmaf(f, x[e].w, a3);
     }
     const float inv = 1.f / sum;
     *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(prm.O, b, h, q0 + r)) + tx * 4) = make_float4(a0 * inv, a1 * inv, a2 * inv, a3 * inv);
-    if (tx == 0 && prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + r] = row_lse_f32(M, sum);
+    if (tx == 0 && prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + r] = row_lse_f32(M, sum, fabsf(prm.scale));
   }
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");

@@ -715,7 +715,8 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       prm.lv = lv; prm.Q = tview(Q); prm.O = tview(O); prm.K = kc; prm.V = vc; prm.lse = lse; prm.n_k = nk;
       prm.room = lv.pages_per_slice << lv.page_shift;
       prm.fused = fused ? 1 : 0; prm.copy_in = (fused && copy) ? 1 : 0; prm.n_prev = p.N[k];
-      prm.scale = ctx->scale; prm.scale_log2e = ctx->scale * 1.4426950408889634f;
+      prm.scale = ctx->scale;
+      prm.weight_scale = (float)(std::fabs((double)ctx->scale) * 1.4426950408889634 * (1.0 + (double)f32::kCutOff));
       // The window's logits: plain fp32 sums, as the compress would take them from K by a launch of its own, 16 rows of every key tile by a
       // CTA beside the others.  (Not from the tensor core's scores: importances a few 1e-7 apart decide what is kept, so that logits of
       // another rounding, as exact as they may be, keep another entry in one pass of some.)

@@ -69,3 +69,28 @@ def test_f32_log_sum_exp_is_rounded_twice(heads):
     assert 4 < want.min().item() and want.max().item() < 8
     assert (lse.double() - want).pow(2).mean().sqrt().item() <= 2.4e-7
     kv.close()
+
+
+@pytest.mark.parametrize("heads", [1, 40])
+@pytest.mark.parametrize("key", [-2.0 ** 33, -1.125 * 2.0 ** 33, 1.125 * 2.0 ** 33, -2.0 ** 40, -2.0 ** 100])
+def test_f32_rows_of_equal_scores_far_from_zero(heads, key):
+    """Equal scores, exact in 32 bits: equal weights, however far from zero they lie, to the roundings of sums over 340 values."""
+    sides = (4, 18)
+    g = torch.Generator(device="cuda").manual_seed(13)
+    kv = binding.ScaleKV(1, 1, heads, 64, "f32", sides, sides, [[binding.KEEP_ALL] * len(sides)])
+    values = []
+    for k, a in enumerate(sides):
+        Q, K, V = (torch.randn(1, heads, a * a, 64, generator=g, device="cuda") for _ in range(3))
+        Q[...], K[..., 0] = 0.0, key
+        Q[..., 0] = 1.0
+        values.append(V)
+        lse = torch.empty(1, heads, a * a, device="cuda")
+        torch.cuda.synchronize()
+        kv.scalekv_append(0, k, K, V)
+        O = kv.scalekv_attend(0, Q, lse=lse)
+        kv.scalekv_sync()
+    want = torch.cat(values, 2).double().mean(2, keepdim=True)
+    # means of size 1/18 of values of size 1, whose sums are rounded by a few 2^-24 of their size: 2e-7 sqrt(a few) of the means
+    assert ((O.double() - want).norm() / (O.shape[2] ** 0.5 * want.norm())).item() <= 2e-6
+    assert (lse.double() - (key / 8 + torch.log(torch.tensor(340.0, dtype=torch.float64)).item())).abs().max().item() <= abs(key) / 8 * 2e-7 + 1e-6
+    kv.close()
