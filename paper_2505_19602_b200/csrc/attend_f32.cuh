@@ -12,8 +12,8 @@
 //               long cache would show.  P goes back to TMEM in three pieces, over the scores it comes from.  Warp 0 issues P V when all
 //               four warps have met; its result is added behind the softmax of the next tile.
 // With two CTAs an SM's tensor pipe works for the one while the other is in its softmax.
-// Scores that are not numbers (an infinite key: its products with the pieces of a query may differ in sign) spoil their row's sum, and
-// values that are not its columns; such a row is done again at the end by fp32 FMA from the tensors (fma_row).
+// Scores that are not numbers (an infinite key: its products with the pieces of a query may differ in sign) are taken again, by signs or fp32 FMA
+// (repair_scores).  Rows whose sum or columns are none all the same, an infinite value's, are done again at the end by fp32 FMA (redo_rows).
 // The observation window's logits are taken by CTAs of their own beside the others, in plain fp32 (see the launch).
 // gridDim.z CTAs of a cluster share a slice's keys and combine: O = sum_e 2^(c (m_e - M)) O_e / sum_e 2^(c (m_e - M)) l_e, through distributed
 // shared memory.
@@ -104,6 +104,13 @@ __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t *v) {
                : "memory");
 }
 
+// the largest, or no number where one of them is none
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // A pair of numbers in three pairs of bf16 numbers that sum to them.  (What h and m leave of 24 bits fits the eight of l, so l is the
 // upper half of what is left.)
 __device__ __forceinline__ void split2(float x, float y, uint32_t &h, uint32_t &m, uint32_t &l) {
@@ -144,32 +151,220 @@ __device__ __forceinline__ float row_lse_f32(float m, float l, float scale) {
   return sum + fmaf(m, scale * kCutOff, rest);
 }
 
-// One row by fp32 FMA over the entries [from, to): its 64 columns go to `out` (16-byte pieces permuted by `swap`).  For
-// rows whose scores or columns by pieces are not numbers.
-struct RowSum { float m, l; };
-__device__ __noinline__ RowSum fma_row(const Params &prm, int slice, int b, int h, int hist, int q_row, int from, int to, float *out, int swap) {
-  const float *q = row_ptr<float>(prm.Q, b, h, q_row);
-  const float cut = copysignf(1.f - kCutOff, prm.scale);                 // (products as the tensor core would leave them)
-  float o[64], m = kNoMax, l = 0.f;
+// Scores that are not numbers, for they are the sums of products with a query's pieces that differ in sign: an infinite key's, or those of numbers near
+// the range's end.  A warp takes them again, a thread its row's, 32 keys at a time.  A score with an infinite column is decided by signs: a lane reads
+// one key's and hands its masks round.  The others are taken by fp32 FMA, four keys at a time: two columns of each in a lane, handed round likewise,
+// and the query put together from its pieces eight columns at a time.  (Few registers, so that the softmax around it spills no more than it did: with
+// the query in 64 of them every launch took 4 % longer.  us per launch of 16 slices x 1 600 queries behind 772
+// entries, of keys masked by -inf in a column: none 142, one 164, 32 in a row 179, 32 apart 316, 300 in a row 403; with fp32 FMA for each 142, 171,
+// 248, 334, 1 038; fp32 FMA throughout 398.)
+struct Repaired { float max; int hopeless; };      // hopeless: the row has a score that is +inf or no number all the same, and so no output that is one
+__device__ __noinline__ Repaired repair_scores(const Params &prm, const uint8_t *q_tile, uint32_t buf, int row, int slice, int b, int h, int hist,
+                                               int key0, int valid) {
+  const int lane = threadIdx.x & 31;
+  auto query = [&](int c, float (&q)[8]) {         // columns 8 c ..
+    const uint8_t *at = q_tile + row * 128 + ((c ^ (row & 7)) << 4);
+    const uint4 h4 = *reinterpret_cast<const uint4 *>(at), m4 = *reinterpret_cast<const uint4 *>(at + kPieceQ), l4 = *reinterpret_cast<const uint4 *>(at + 2 * kPieceQ);
+    const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, mw[4] = {m4.x, m4.y, m4.z, m4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
-  for (int d = 0; d < 64; ++d) o[d] = 0.f;
+    for (int i = 0; i < 4; ++i) {
+      q[2 * i] = (__uint_as_float(hw[i] << 16) + __uint_as_float(mw[i] << 16)) + __uint_as_float(lw[i] << 16);
+      q[2 * i + 1] = (__uint_as_float(hw[i] & 0xffff0000u) + __uint_as_float(mw[i] & 0xffff0000u)) + __uint_as_float(lw[i] & 0xffff0000u);
+    }
+  };
+  float over = 0.f;
+  uint64_t q_pos = 0, q_neg = 0;         // by column
 #pragma unroll 1
-  for (int j = from; j < to; ++j) {
-    const float *k = entry(prm, false, slice, b, h, hist, j), *v = entry(prm, true, slice, b, h, hist, j);
-    float s = 0.f;
-#pragma unroll 8
-    for (int d = 0; d < 64; ++d) s = fmaf(q[d], k[d], s);
-    s *= cut;
-    const float mx = fmaxf(m, s), f = exp2f((m - mx) * prm.weight_scale), p = exp2f((s - mx) * prm.weight_scale);
-    m = mx;
-    l = fmaf(l, f, p);
+  for (int c = 0; c < 8; ++c) {
+    float q[8];
+    uint32_t pos = 0, neg = 0;
+    query(c, q);
 #pragma unroll
-    for (int d = 0; d < 64; ++d) o[d] = fmaf(p, v[d], o[d] * f);
+    for (int i = 0; i < 8; ++i) {
+      over += q[i] - q[i];
+      if (q[i] > 0.f) pos |= 1u << i;
+      if (q[i] < 0.f) neg |= 1u << i;
+    }
+    q_pos |= (uint64_t)pos << (8 * c);
+    q_neg |= (uint64_t)neg << (8 * c);
   }
+  const bool row_ok = over == 0.f;       // (a query that cannot be split spoils all its scores: its row is done again in the end)
+  Repaired r{-INFINITY, 0};
+#pragma unroll 1
+  for (int j0 = 0; j0 < valid; j0 += 32) {
+    uint32_t bad = 0;
+#pragma unroll 1
+    for (int j = 0; j < 32; j += 8) {
+      uint32_t x[8];
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]),
+                   "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]) : "r"(buf + j0 + j));
+      tc::tc_wait_ld();
 #pragma unroll
-  for (int c = 0; c < 16; ++c)
-    *reinterpret_cast<float4 *>(out + (c ^ swap) * 4) = make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
-  return {m, l};
+      for (int e = 0; e < 8; ++e) {
+        const float y = __uint_as_float(x[e]);
+        if (j0 + j + e >= valid) continue;
+        if (__any_sync(0xffffffffu, y != y && row_ok)) bad |= 1u << (j + e);
+        r.max = fmaxf(r.max, y);
+      }
+    }
+    if (bad == 0) continue;
+    const uint64_t key = (uint64_t)entry(prm, false, slice, b, h, hist, key0 + min(j0 + lane, valid - 1));
+    uint64_t k_pos = 0, k_neg = 0;       // the lane's key: its infinite columns
+    bool nan = false;
+    if ((bad >> lane) & 1u) {
+#pragma unroll 1
+      for (int c = 0; c < 16; c += 4) {
+        float4 z[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = reinterpret_cast<const float4 *>(key)[c + i];
+        uint32_t pos = 0, neg = 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float y = i % 4 == 0 ? z[i / 4].x : i % 4 == 1 ? z[i / 4].y : i % 4 == 2 ? z[i / 4].z : z[i / 4].w;
+          if (y == INFINITY) pos |= 1u << i;
+          if (y == -INFINITY) neg |= 1u << i;
+          nan = nan || y != y;
+        }
+        k_pos |= (uint64_t)pos << (4 * c);
+        k_neg |= (uint64_t)neg << (4 * c);
+      }
+    }
+    const uint32_t signs = __ballot_sync(0xffffffffu, nan || (k_pos | k_neg) != 0), nans = __ballot_sync(0xffffffffu, nan);
+    // a score, not lifted, to its column in TMEM
+    auto put = [&](int j, float y) {
+      uint32_t x;
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(x) : "r"(buf + j0 + j));
+      tc::tc_wait_ld();
+      if (row_ok && __uint_as_float(x) != __uint_as_float(x)) {
+        if (!(y < INFINITY)) r.hopeless = 1;
+        x = __float_as_uint(y);
+        r.max = fmaxf(r.max, y);
+      }
+      __syncwarp();
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(buf + j0 + j), "r"(x) : "memory");
+    };
+#pragma unroll 1
+    for (uint32_t left = signs; left != 0; left &= left - 1) {
+      const int j = __ffs(left) - 1;
+      const uint64_t pos = __shfl_sync(0xffffffffu, k_pos, j), neg = __shfl_sync(0xffffffffu, k_neg, j);
+      const bool up = ((pos & q_pos) | (neg & q_neg)) != 0, down = ((pos & q_neg) | (neg & q_pos)) != 0;
+      const bool none = ((nans >> j) & 1u) || (up && down) || ((pos | neg) & ~(q_pos | q_neg)) != 0;
+      put(j, none ? NAN : up ? INFINITY : -INFINITY);
+    }
+    bad &= ~signs;
+#pragma unroll 1
+    while (bad != 0) {
+      uint32_t rest = bad;
+      float2 k[4];
+      float s[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int j = rest != 0 ? __ffs(rest) - 1 : 0;
+        rest &= rest - 1;
+        k[e] = reinterpret_cast<const float2 *>(__shfl_sync(0xffffffffu, key, j))[lane];
+        s[e] = 0.f;
+      }
+#pragma unroll 1
+      for (int c = 0; c < 8; ++c) {
+        float q[8];
+        query(c, q);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) s[e] = fmaf(q[i], __shfl_sync(0xffffffffu, i & 1 ? k[e].y : k[e].x, 4 * c + (i >> 1)), s[e]);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (bad == 0) break;
+        put(__ffs(bad) - 1, s[e] * (1.f - kCutOff));       // (as the tensor core would leave it)
+        bad &= bad - 1;
+      }
+    }
+  }
+  tc::tc_wait_st();
+  return r;
+}
+
+// Rows whose sums or columns by pieces are no numbers all the same (an infinite value's all, an infinite query's own), by fp32 FMA over the entries
+// [from, to): two threads per row, which share its columns by 16-byte pieces, keys and values in tiles of 64 where their pieces lay.  For rows that few
+// will ever need, so without pipelining: 16 slices x 1 600 queries behind 772 entries, all rows, 683 us.
+__device__ __noinline__ void redo_rows(const Params &prm, uint8_t *smem, const uint32_t *marks) {
+  const int tid = threadIdx.x, row = tid >> 1, half = tid & 1;
+  // (worked out once more: passed, they would have to outlive the softmax)
+  const int slice = blockIdx.y, b = slice / prm.lv.n_heads, h = slice - b * prm.lv.n_heads, q0 = blockIdx.x * kRows;
+  const int hist = prm.lv.hist_len[slice], L = min(hist + prm.n_k, prm.room), tiles = (L + kKeys - 1) / kKeys;
+  const int from = tiles * (int)blockIdx.z / (int)gridDim.z * kKeys, to = min(tiles * ((int)blockIdx.z + 1) / (int)gridDim.z * kKeys, L);
+  float *Ks = reinterpret_cast<float *>(smem + kOffK), *Vs = reinterpret_cast<float *>(smem + kOffV);
+  const float cut = copysignf(1.f - kCutOff, prm.scale), c = prm.weight_scale;       // (products as the tensor core would leave them)
+  float4 q[8], o[8];
+  const float4 *qp = reinterpret_cast<const float4 *>(row_ptr<float>(prm.Q, b, h, min(q0 + row, prm.n_k - 1)));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { q[i] = qp[2 * i + half]; o[i] = make_float4(0.f, 0.f, 0.f, 0.f); }
+  float m = kNoMax, l = 0.f;
+#pragma unroll 1
+  for (int t0 = from; t0 < to; t0 += kKeys) {
+    __syncthreads();                     // the tile before has been read
+    {
+      const int r = tid >> 2;
+      const bool there = t0 + r < to;
+      const float4 *k = reinterpret_cast<const float4 *>(entry(prm, false, slice, b, h, hist, there ? t0 + r : from));
+      const float4 *v = reinterpret_cast<const float4 *>(entry(prm, true, slice, b, h, hist, there ? t0 + r : from));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int piece = (tid & 3) + 4 * u;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f), x = there ? k[piece] : zero, y = there ? v[piece] : zero;
+        reinterpret_cast<float4 *>(Ks)[r * 16 + piece] = x;
+        reinterpret_cast<float4 *>(Vs)[r * 16 + piece] = y;
+      }
+    }
+    __syncthreads();
+    const int n = min(kKeys, to - t0);
+#pragma unroll 1
+    for (int j = 0; j < n; j += 8) {
+      float s[8], mx = m;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        float a = 0.f, a2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 z = reinterpret_cast<const float4 *>(Ks)[(j + e) * 16 + 2 * i + half];
+          a = fmaf(q[i].x, z.x, a);
+          a2 = fmaf(q[i].y, z.y, a2);
+          a = fmaf(q[i].z, z.z, a);
+          a2 = fmaf(q[i].w, z.w, a2);
+        }
+        a += a2;
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        s[e] = j + e < n ? a * cut : -INFINITY;
+        mx = fmaxf(mx, s[e]);
+      }
+      const float f = exp2f((m - mx) * c);
+      float sum = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) o[i] = make_float4(o[i].x * f, o[i].y * f, o[i].z * f, o[i].w * f);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float p = exp2f((s[e] - mx) * c);
+        sum += p;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 z = reinterpret_cast<const float4 *>(Vs)[(j + e) * 16 + 2 * i + half];
+          o[i] = make_float4(fmaf(p, z.x, o[i].x), fmaf(p, z.y, o[i].y), fmaf(p, z.z, o[i].z), fmaf(p, z.w, o[i].w));
+        }
+      }
+      l = fmaf(l, f, sum);
+      m = mx;
+    }
+  }
+  if ((marks[row >> 5] >> (row & 31)) & 1u) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<float4 *>(smem + kOffQ + row * 256 + (((2 * i + half) ^ (row & 7)) << 4)) = o[i];
+    if (half == 0) {
+      reinterpret_cast<float2 *>(smem + kOffStat)[row] = make_float2(m, l);
+      if (gridDim.z == 1 && prm.lse != nullptr) prm.lse[(size_t)slice * prm.n_k + q0 + row] = row_lse_f32(m, l, fabsf(prm.scale));
+    }
+  }
 }
 
 // The window's logits against the 64 entries of a tile, as score_logits_kernel takes them from the pages.
@@ -198,6 +393,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem_raw + kOffBar + 32);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 36);
   volatile int *leave_slot = reinterpret_cast<volatile int *>(smem_raw + kOffBar + 40);
+  uint32_t *marks = reinterpret_cast<uint32_t *>(smem_raw + kOffBar + 44);      // rows that are to be done again, by warp
   const LayerView &lv = prm.lv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice - b * lv.n_heads;
@@ -235,7 +431,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   }
   // Q: a thread takes one chunk of eight columns of four rows.  (Of a negative scale Q takes the sign, so that the largest product is
   // the largest score.)
-  const float sign = prm.scale < 0.f ? -1.f : 1.f;
+  const float sign = copysignf(1.f, prm.scale);
   {
     float4 x[4][2];
 #pragma unroll
@@ -380,6 +576,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
 #pragma unroll
     for (int i = 0; i < 32; ++i) o[i] = 0ull;
     float m = kNoMax, l = 0.f, l_rest = 0.f;       // l_rest: what the additions to l have rounded off
+    int hopeless = 0;                              // the row has a score that makes its output no number
     // (o + P V of the tile before) f
     auto add_products = [&](float f, bool scale) {
       const uint64_t ff = tc::pack2(f, f);
@@ -409,7 +606,12 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
         tc::tc_wait_ld();
 #pragma unroll
         for (int q = 0; q < 16; q += 2)
-          mx = tc::max3(mx, real(16 * e + q) ? __uint_as_float(x[q]) : -INFINITY, real(16 * e + q + 1) ? __uint_as_float(x[q + 1]) : -INFINITY);
+          mx = max3_nan(mx, real(16 * e + q) ? __uint_as_float(x[q]) : -INFINITY, real(16 * e + q + 1) ? __uint_as_float(x[q + 1]) : -INFINITY);
+      }
+      if (__any_sync(0xffffffffu, mx != mx)) {
+        const Repaired r = repair_scores(prm, smem_raw + kOffQ, buf, row, slice, b, h, hist, (lo + i) * kKeys, min(valid, kKeys));
+        mx = r.max;
+        hopeless |= r.hopeless;
       }
       mx = fmaxf(m, mx);
       const bool scale = __any_sync(0xffffffffu, mx > m);
@@ -491,11 +693,8 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       amax += (x0 - x0) + (x1 - x1) + (x2 - x2) + (x3 - x3);      // zero, unless one of them is not a number
       *reinterpret_cast<float4 *>(mine + ((q ^ (row & 7)) << 2)) = make_float4(x0, x1, x2, x3);
     }
-    if (nt > 0 && ok && q0 + row < n_k && !(amax == 0.f && l > 0.f && l < INFINITY)) {
-      const RowSum s = fma_row(prm, slice, b, h, hist, q0 + row, lo * kKeys, min((lo + nt) * kKeys, L), mine, row & 7);
-      m = s.m;
-      l = s.l;
-    }
+    const unsigned spoiled = __ballot_sync(0xffffffffu, nt > 0 && ok && q0 + row < n_k && !hopeless && !(amax == 0.f && l > 0.f && l < INFINITY));
+    if (lane == 0) marks[warp] = spoiled;
     stat_out[row] = make_float2(m, l);
     if (n_split == 1 && ok && nt > 0 && q0 + row < n_k) {
       if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + row] = row_lse_f32(m, l, fabsf(prm.scale));
@@ -506,6 +705,10 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+  if ((marks[0] | marks[1] | marks[2] | marks[3]) != 0u) {
+    redo_rows(prm, smem_raw, marks);
+    __syncthreads();
   }
   const int ty = tid >> 4, tx = tid & 15, rows = min(kRows, n_k - q0);
   if (n_split == 1) {

@@ -108,6 +108,78 @@ def test_infinite_values_reach_their_column_only(heads):
     assert (O.double() - want)[..., rest].abs().max().item() <= 1e-5
 
 
+@pytest.mark.parametrize("heads", [1, 40])
+@pytest.mark.parametrize("masked", [1, 3, 64, 1500])
+def test_masked_keys_among_thousands(heads, masked):
+    """-inf in one of their columns, here and there: the others' weights are those of fp32 arithmetic."""
+    draw = normal(14, heads)
+    g = torch.Generator(device="cuda").manual_seed(15)
+
+    def make(k, n):
+        Q, K, V = draw(n)
+        Q[..., 7] = Q[..., 7].abs() + 0.01
+        K[:, :, torch.randperm(n, generator=g, device="cuda")[:masked if k == 0 else 1], 7] = -float("inf")
+        return Q, K, V
+
+    Q, K, V, O, lse = full_cache(heads, (60, 12), make, lse=True)
+    s = (Q.double() @ K.double().transpose(2, 3) / 8).masked_fill(torch.isinf(K[..., 7])[:, :, None], -float("inf"))
+    want = s.softmax(-1) @ V.double()
+    assert ((O.double() - want).norm() / want.norm()).item() <= BOUND[1.0]
+    assert (lse.double() - s.logsumexp(-1)).pow(2).mean().sqrt().item() <= 1e-6
+
+
+@pytest.mark.parametrize("heads", [1, 40])
+def test_infinite_columns_of_either_sign(heads):
+    """The sign of a score with infinite columns is its query's, or it has none: where both signs meet, and where the query is zero."""
+    draw = normal(20, heads)
+
+    def make(k, n):
+        Q, K, V = draw(n)
+        Q[..., 3], Q[..., 40], Q[..., 63] = Q[..., 3].abs() + 0.01, -Q[..., 40].abs() - 0.01, Q[..., 63].abs() + 0.01
+        for first, second in ((5, 6), (n - 1, n - 2)):
+            K[:, :, first, 3], K[:, :, first, 40] = -float("inf"), float("inf")
+            K[:, :, second, 3], K[:, :, second, 63] = -float("inf"), -float("inf")
+        K[:, 0, 9, 40] = float("inf")
+        Q[:, :, 2, 3] = 0.0
+        Q[:, :, 4, 40] = 1e-30
+        Q[:, :, 6, 3], Q[:, :, 6, 40], Q[:, :, 6, 63] = -1.0, 1.0, -1.0
+        return Q, K, V
+
+    Q, K, V, O, lse = full_cache(heads, (60, 12), make, lse=True)
+    s = Q.double() @ K.double().transpose(2, 3) / 8
+    want = s.softmax(-1) @ V.double()
+    assert torch.isnan(want).any(-1).sum().item() == 3 * heads and (torch.isnan(O) == torch.isnan(want)).all()
+    there = torch.isfinite(want)
+    assert ((O.double() - want)[there].norm() / want[there].norm()).item() <= BOUND[1.0]
+    assert (lse.double() - s.logsumexp(-1))[there[..., 0]].pow(2).mean().sqrt().item() <= 1e-6
+
+
+@pytest.mark.parametrize("heads", [1, 40])
+def test_rows_that_are_done_again_are_as_exact_as_plain_sums(heads):
+    """An infinite value spoils all rows, an infinite query its own, a key that is no number all of its head's."""
+    draw = normal(16, heads)
+
+    def make(k, n):
+        Q, K, V = draw(n)
+        if k == 0:
+            V[:, 0, 70, 5] = float("inf")
+            if heads > 1:
+                K[:, 1, 3000, 9] = float("nan")
+        else:
+            Q[:, -1, 3, 2] = float("inf")
+        return Q, K, V
+
+    Q, K, V, O, lse = full_cache(heads, (60, 12), make, lse=True)
+    s = Q.double() @ K.double().transpose(2, 3) / 8
+    want = s.softmax(-1) @ V.double()
+    assert (torch.isnan(O) == torch.isnan(want)).all() and (torch.isinf(O) == torch.isinf(want)).all()
+    there = torch.isfinite(want)
+    # sums of 3 744 terms one behind the other: half a unit of 2^-24 each of a growing sum, at random, sqrt(3744 / 3) / 2 of them
+    assert ((O.double() - want)[there].norm() / want[there].norm()).item() <= 2e-6
+    finite = torch.isfinite(s).all(-1)
+    assert (lse.double() - s.logsumexp(-1))[finite].abs().max().item() <= 2e-6
+
+
 def test_a_map_whose_keys_and_values_are_laid_out_differently():
     """A one-call step takes it, evicting or not."""
     sides, heads = (4, 12, 15), 3
