@@ -1,5 +1,5 @@
 // Attention over the paged store for f32, head_dim 64 (Sec. 3.3, Eq. 5) on the tensor cores, at the precision of fp32 arithmetic.
-// Every operand is split into three bf16 numbers, x = h + m + l (8 significant bits each, so nothing of x is lost), and a product
+// Every operand is split into three bf16 numbers, x = h + m + l (8 significant bits each, so nothing of x is lost, see kLift), and a product
 // is the six products of pieces that are larger than 2^-24 of it, the small ones summed first:
 //   S = Ql Kh + Qh Kl + Qm Km + Qm Kh + Qh Km + Qh Kh,  and P V alike.
 // A CTA of 256 threads, two per SM, owns 128 query rows of one slice and streams its keys in tiles of 64:
@@ -53,6 +53,11 @@ static_assert(2 * (kSmemBytes + 1024) <= 233472, "two CTAs have to fit an SM");
 // reference, and to the reference where it enters a log-sum-exp.  (Given to the products alone, it would leave the largest weight at 2^(7e-8 m),
 // m its exponent: of scores near -1e9 the weights would lie where their pieces run out of range.)
 constexpr float kCutOff = 1.2f / 16777216.f;
+// Queries and values are lifted by 2^24 before they are split, and products and outputs taken down again, so that the pieces of small ones
+// are not bf16's subnormal numbers (of values near 1e-36 the output would be off by 1e-5 of it): every query and value of normal size is held
+// whole.  Keys are not: theirs below 2^-110 lose up to 2^-134, which the largest query that can be split, 2^103, does not make 2^-30 of a score.  What
+// the lift takes beyond the range - queries and values from 2^103, products from 2^104 - is an infinity and done by fp32 FMA, as those are.
+constexpr float kLift = 16777216.f;
 // TMEM: two buffers of 96 columns for scores and P, 64 columns for products with V.  The 16 keys of step kk have their scores in columns
 // 16 kk .. of a buffer, and their P there (h in the first eight, m in the next) and in columns 64 + 8 kk .. (l).
 constexpr uint32_t kTmemCols = 256, kBufCols = 96, kColPm = 8, kColPl = 64, kColO = 192;
@@ -124,6 +129,13 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t &h, uint32_t &
 __device__ __forceinline__ void store16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+__device__ __forceinline__ float4 times(const float4 &x, float f) {
+  const uint64_t ff = tc::pack2(f, f);
+  float4 y;
+  tc::unpack2(tc::mul2(tc::pack2(x.x, x.y), ff), y.x, y.y);
+  tc::unpack2(tc::mul2(tc::pack2(x.z, x.w), ff), y.z, y.w);
+  return y;
+}
 // eight columns (chunk c) of row r of an operand tile: the pieces' 16 bytes, 128B-swizzled
 __device__ __forceinline__ void put_split(uint32_t tile, uint32_t piece_bytes, int r, int c, const float4 &a, const float4 &b) {
   uint32_t h[4], m[4], l[4];
@@ -162,7 +174,7 @@ struct Repaired { float max; int hopeless; };      // hopeless: the row has a sc
 __device__ __noinline__ Repaired repair_scores(const Params &prm, const uint8_t *q_tile, uint32_t buf, int row, int slice, int b, int h, int hist,
                                                int key0, int valid) {
   const int lane = threadIdx.x & 31;
-  auto query = [&](int c, float (&q)[8]) {         // columns 8 c ..
+  auto query = [&](int c, float (&q)[8]) {         // columns 8 c .., lifted
     const uint8_t *at = q_tile + row * 128 + ((c ^ (row & 7)) << 4);
     const uint4 h4 = *reinterpret_cast<const uint4 *>(at), m4 = *reinterpret_cast<const uint4 *>(at + kPieceQ), l4 = *reinterpret_cast<const uint4 *>(at + 2 * kPieceQ);
     const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, mw[4] = {m4.x, m4.y, m4.z, m4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
@@ -237,8 +249,8 @@ __device__ __noinline__ Repaired repair_scores(const Params &prm, const uint8_t 
       tc::tc_wait_ld();
       if (row_ok && __uint_as_float(x) != __uint_as_float(x)) {
         if (!(y < INFINITY)) r.hopeless = 1;
-        x = __float_as_uint(y);
-        r.max = fmaxf(r.max, y);
+        x = __float_as_uint(y * kLift);
+        r.max = fmaxf(r.max, y * kLift);
       }
       __syncwarp();
       asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(buf + j0 + j), "r"(x) : "memory");
@@ -270,8 +282,9 @@ __device__ __noinline__ Repaired repair_scores(const Params &prm, const uint8_t 
         query(c, q);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
+          const float x = q[i] * (1.f / kLift);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) s[e] = fmaf(q[i], __shfl_sync(0xffffffffu, i & 1 ? k[e].y : k[e].x, 4 * c + (i >> 1)), s[e]);
+          for (int e = 0; e < 4; ++e) s[e] = fmaf(x, __shfl_sync(0xffffffffu, i & 1 ? k[e].y : k[e].x, 4 * c + (i >> 1)), s[e]);
         }
       }
 #pragma unroll
@@ -431,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   }
   // Q: a thread takes one chunk of eight columns of four rows.  (Of a negative scale Q takes the sign, so that the largest product is
   // the largest score.)
-  const float sign = copysignf(1.f, prm.scale);
+  const float lift = copysignf(kLift, prm.scale);
   {
     float4 x[4][2];
 #pragma unroll
@@ -440,9 +453,8 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (q0 + r < n_k) {
         const float4 *src = reinterpret_cast<const float4 *>(row_ptr<float>(prm.Q, b, h, q0 + r)) + 2 * c;
-        const float4 x0 = __ldg(src), x1 = __ldg(src + 1);
-        x[u][0] = make_float4(x0.x * sign, x0.y * sign, x0.z * sign, x0.w * sign);
-        x[u][1] = make_float4(x1.x * sign, x1.y * sign, x1.z * sign, x1.w * sign);
+        x[u][0] = times(__ldg(src), lift);
+        x[u][1] = times(__ldg(src + 1), lift);
       }
     }
 #pragma unroll
@@ -485,7 +497,10 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     };
     auto put = [&](bool values, int tile, const float4 (&x)[4][2]) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) put_split(base + (values ? kOffV : kOffK), kPieceK, r0 + 16 * u, c, x[u][0], x[u][1]);
+      for (int u = 0; u < 4; ++u) {
+        if (values) put_split(base + kOffV, kPieceK, r0 + 16 * u, c, times(x[u][0], kLift), times(x[u][1], kLift));
+        else put_split(base + kOffK, kPieceK, r0 + 16 * u, c, x[u][0], x[u][1]);
+      }
       if (prm.copy_in && tile * kKeys + kKeys > hist && tile % prm.blocks == (int)blockIdx.x) {      // (the CTAs of a slice take turns)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -571,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     };
     const int row = warp * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-    const float c = prm.weight_scale;
+    const float c = prm.weight_scale * (1.f / kLift);
     uint64_t o[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) o[i] = 0ull;
@@ -683,6 +698,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     // (given up: as above)
     if (!ok && issued > 0) tc::mbar_drain(bar(bPv), (issued - 1) & 1);
     l += l_rest;
+    if (m != kNoMax) m *= 1.f / kLift;
     float *mine = rows_out + row * 64;
     float amax = 0.f;
 #pragma unroll
@@ -691,7 +707,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       tc::unpack2(o[2 * q], x0, x1);
       tc::unpack2(o[2 * q + 1], x2, x3);
       amax += (x0 - x0) + (x1 - x1) + (x2 - x2) + (x3 - x3);      // zero, unless one of them is not a number
-      *reinterpret_cast<float4 *>(mine + ((q ^ (row & 7)) << 2)) = make_float4(x0, x1, x2, x3);
+      *reinterpret_cast<float4 *>(mine + ((q ^ (row & 7)) << 2)) = times(make_float4(x0, x1, x2, x3), 1.f / kLift);
     }
     const unsigned spoiled = __ballot_sync(0xffffffffu, nt > 0 && ok && q0 + row < n_k && !hopeless && !(amax == 0.f && l > 0.f && l < INFINITY));
     if (lane == 0) marks[warp] = spoiled;

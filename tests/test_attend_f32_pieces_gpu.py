@@ -74,6 +74,23 @@ def test_error_is_that_of_fp32_arithmetic(heads, gain):
 
 
 @pytest.mark.parametrize("heads", [1, 40])
+@pytest.mark.parametrize("q,k,v", [(0, 0, -118), (0, 0, 99), (0, 0, 110), (-118, 118, 0), (118, -118, 0), (-118, 95, 0), (95, -105, 0), (100, -100, 0)])
+def test_numbers_at_the_ends_of_the_range(heads, q, k, v):
+    """Gains of 2^q, 2^k and 2^v: pieces that would be subnormal, operands that cannot be lifted.  The bound of scores of size 1."""
+    draw = normal(12, heads)
+
+    def make(_, n):
+        Q, K, V = draw(n)
+        return Q * 2.0 ** q, K * 2.0 ** k, V * 2.0 ** v
+
+    Q, K, V, O, lse = full_cache(heads, (8, 18), make, lse=True)
+    s = Q.double() @ K.double().transpose(2, 3) / 8
+    want = s.softmax(-1) @ V.double()
+    assert ((O.double() - want).norm() / want.norm()).item() <= BOUND[1.0]
+    assert (lse.double() - s.logsumexp(-1)).pow(2).mean().sqrt().item() <= 1e-6
+
+
+@pytest.mark.parametrize("heads", [1, 40])
 @pytest.mark.parametrize("first", [0, 40, 64])
 def test_keys_masked_with_minus_infinity(heads, first):
     """Keys whose products are -inf have no weight, whatever the signs of the queries' pieces."""
