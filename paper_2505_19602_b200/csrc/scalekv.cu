@@ -1058,15 +1058,20 @@ static bool step_copies(const scalekv_ctx *ctx, int layer, int scale, const scal
   return !(planned && table < L - w);
 }
 
+// What a step that has appended its map ends with.  An f32 step that was refused half-way leaves the map in the pages, where an append by
+// itself puts it: the caller goes on from there, without the tensors.
+static scalekv_status step_ends(scalekv_ctx *ctx, int layer, scalekv_status st) {
+  if (st != SCALEKV_OK && !ctx->tc.enabled()) materialize(ctx, layer);
+  return st;
+}
+
 scalekv_status scalekv_step(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor Q, scalekv_tensor K, scalekv_tensor V,
                             scalekv_tensor O, float *lse, int32_t w, const int32_t *window_pos) {
   scalekv_status st = append_impl(ctx, layer, scale, K, V, true);
   if (st != SCALEKV_OK) return st;
   st = attend_impl(ctx, layer, Q, O, lse, w > 0, step_copies(ctx, layer, scale, K, V, w != 0, w, window_pos, nullptr));
-  if (st != SCALEKV_OK) return st;
-  if (w > 0) return scalekv_compress(ctx, layer, Q, w, window_pos, 1);
-  if (w < 0) return scalekv_compress(ctx, layer, Q, 0, nullptr, 1);
-  return SCALEKV_OK;
+  if (st == SCALEKV_OK && w != 0) st = scalekv_compress(ctx, layer, Q, std::max(w, 0), w > 0 ? window_pos : nullptr, 1);
+  return step_ends(ctx, layer, st);
 }
 
 scalekv_status scalekv_step_ex(scalekv_ctx *ctx, int32_t layer, int32_t scale, scalekv_tensor Q, scalekv_tensor K, scalekv_tensor V,
@@ -1077,9 +1082,8 @@ scalekv_status scalekv_step_ex(scalekv_ctx *ctx, int32_t layer, int32_t scale, s
   const bool score = !opts || opts->policy == SCALEKV_SELECT_SCORE;
   st = attend_impl(ctx, layer, Q, O, lse, compress != 0 && score && w > 0,
                    step_copies(ctx, layer, scale, K, V, compress != 0, w, window_pos, opts));
-  if (st != SCALEKV_OK) return st;
-  if (!compress) return SCALEKV_OK;
-  return scalekv_compress_ex(ctx, layer, Q, w, window_pos, 1, opts);
+  if (st == SCALEKV_OK && compress) st = scalekv_compress_ex(ctx, layer, Q, w, window_pos, 1, opts);
+  return step_ends(ctx, layer, st);
 }
 
 // What a sum that has not arrived looks like: a NaN that no arithmetic produces.

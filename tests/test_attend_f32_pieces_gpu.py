@@ -37,7 +37,8 @@ def normal(seed, heads):
     ((1, 5, 16), (2, 13, 24), 33),
 ])
 def test_one_call_steps_match_oracle(heights, widths, budget, page):
-    """Maps that the attention reads in the caller's tensors and copies into the pages."""
+    """Maps that the attention reads in the caller's tensors: a step that evicts nothing copies them into the pages, from one that does the
+    compress takes the rows that stay."""
     n = orc.scale_token_counts(heights, widths)
     g = torch.Generator().manual_seed(31)
     data = [tuple(torch.randn(2, 3, nk, 64, generator=g) for _ in range(3)) for nk in n]
@@ -248,3 +249,34 @@ def test_maps_laid_out_differently_are_pruned_like_others(dtype, policy):
         assert torch.equal(x, y)
     for x, y in zip(left[3], left[7]):
         assert all(torch.equal(a, b) for a, b in zip(x, y))
+
+
+@pytest.mark.parametrize("refused", ["attend", "compress"])
+def test_a_step_that_is_refused_half_way_keeps_its_map(refused):
+    """In the pages, as an append by itself would have: the caller goes on without the tensors."""
+    heads, n = 3, (20, 150)
+    draw = normal(18, heads)
+    kv = binding.ScaleKV(1, 1, heads, 64, "f32", [1, 1], n, [[30] * 2], page_tokens=16)
+    Q, K, V = draw(n[0])
+    torch.cuda.synchronize()
+    kv.scalekv_append(0, 0, K, V)
+    kv.scalekv_attend(0, Q)
+    kv.scalekv_sync()
+    keys, values = [K], [V]
+    Q, K, V = draw(n[1])
+    keys.append(K.clone()), values.append(V.clone())
+    O = torch.empty_like(Q)
+    torch.cuda.synchronize()
+    with pytest.raises(binding.ScaleKVError):
+        if refused == "attend":                            # rows that start between 16-byte boundaries
+            kv.scalekv_step(0, 1, torch.empty(Q.numel() + 1, device="cuda")[1:].view_as(Q), K, V, O, window_pos=[3, 70])
+        else:                                              # more sinks than the pages were planned for
+            kv.scalekv_step_ex(0, 1, Q, K, V, O, policy="recent", n_sink=140)
+    kv.scalekv_sync()
+    K.zero_(), V.zero_()
+    torch.cuda.synchronize()
+    O = kv.scalekv_attend(0, Q)
+    kv.scalekv_sync()
+    want = (Q.double() @ torch.cat(keys, 2).double().transpose(2, 3) / 8).softmax(-1) @ torch.cat(values, 2).double()
+    assert (O.double() - want).abs().max().item() <= 1e-5
+    kv.close()
