@@ -12,9 +12,9 @@ pytestmark = pytest.mark.gpu
 SIDES = (2, 6, 12, 20, 24)
 
 
-def _pass(budgets, heads, data, side_stream):
+def _pass(budgets, heads, data, side_stream, dtype="bf16"):
     n = orc.scale_token_counts(SIDES)
-    kv = binding.ScaleKV(len(budgets), 1, heads, 128, "bf16", SIDES, SIDES, budgets, side_stream=side_stream)
+    kv = binding.ScaleKV(len(budgets), 1, heads, data[0][0][0].shape[-1], dtype, SIDES, SIDES, budgets, side_stream=side_stream)
     out = [[torch.empty_like(data[l][k][0]) for l in range(len(budgets))] for k in range(len(n))]
     torch.cuda.synchronize()
     for _ in range(2):                     # the second pass finds every layer's and every page set's last compress to wait for
@@ -39,6 +39,20 @@ def test_overlapped_compresses_change_nothing(layers, budget_of):
     data = [[tuple(torch.randn(1, heads, nk, 128, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(3))
              for nk in orc.scale_token_counts(SIDES)] for _ in range(layers)]
     beside, alone = (_pass(budgets, heads, data, s) for s in (True, False))
+    for k in range(len(SIDES)):
+        for l in range(layers):
+            assert torch.equal(beside[k][l], alone[k][l]), (k, l)
+
+
+# f32 steps record into the sets' buffers by CTAs of the attend's launch, and their compresses take rows from the caller's tensors
+@pytest.mark.parametrize("layers,budget_of", [(5, (40, 200)), (9, (40,)), (8, (-1, 40, 40, -1))])
+def test_overlapped_f32_compresses_change_nothing(layers, budget_of):
+    heads = 16
+    budgets = [[budget_of[l % len(budget_of)]] * len(SIDES) for l in range(layers)]
+    gen = torch.Generator(device="cuda").manual_seed(19)
+    data = [[tuple(torch.randn(1, heads, nk, 64, generator=gen, device="cuda") for _ in range(3)) for nk in orc.scale_token_counts(SIDES)]
+            for _ in range(layers)]
+    beside, alone = (_pass(budgets, heads, data, s, "f32") for s in (True, False))
     for k in range(len(SIDES)):
         for l in range(layers):
             assert torch.equal(beside[k][l], alone[k][l]), (k, l)
