@@ -569,7 +569,7 @@ def run_scalekv(args):
                        "window": wl.window, "parallelism": f"replica x{world} (batch-sharded, no collective)",
                        "l2_policy": f"inputs larger than L2: {inputs.bytes() / 1e9:.1f} GB of Q/K/V per pass",
                        "side_stream": not args.no_side_stream, "cuda_graph": graph_note, "calibration_s": round(calib_s, 1),
-                       "attend_kernel": "tcgen05" if (wl.dtype == "bf16" and wl.head_dim == 128) else "fp32 FMA"},
+                       "attend_kernel": "tcgen05" if (wl.dtype == "bf16" and wl.head_dim == 128) else "tcgen05 (products of bf16 pieces)"},
             "roofline": roofline, "kernels": kernels, "per_scale": per_scale, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
             "clocks": clocks, "work_per_pass": {k: v for k, v in work.items() if k != "per_scale_flop"},
         }

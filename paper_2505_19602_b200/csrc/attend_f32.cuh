@@ -166,7 +166,7 @@ __device__ __forceinline__ float row_lse_f32(float m, float l, float scale) {
 // Scores that are not numbers, for they are the sums of products with a query's pieces that differ in sign: an infinite key's, or those of numbers near
 // the range's end.  A warp takes them again, a thread its row's, 32 keys at a time.  A score with an infinite column is decided by signs: a lane reads
 // one key's and hands its masks round.  The others are taken by fp32 FMA, four keys at a time: two columns of each in a lane, handed round likewise,
-// and the query put together from its pieces eight columns at a time.  (Few registers, so that the softmax around it spills no more than it did: with
+// and the query put together from its pieces eight columns at a time.  (Few registers, so that the softmax around it spills hardly more than without: with
 // the query in 64 of them every launch took 4 % longer.  us per launch of 16 slices x 1 600 queries behind 772
 // entries, of keys masked by -inf in a column: none 142, one 164, 32 in a row 179, 32 apart 316, 300 in a row 403; with fp32 FMA for each 142, 171,
 // 248, 334, 1 038; fp32 FMA throughout 398.)
@@ -771,7 +771,8 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
 }
 
 // CTAs that share a slice's keys.  ctas: CTAs of an unsplit launch.  In steps of a key tile: a CTA that has its SM to itself takes 1 per
-// tile, two that share one 1.35 each.
+// tile, two that share one 1.35 each.  (The CTAs of a recorded window, one per key tile and slice, are not counted: they hold an SM for about a tile's
+// time, and with them counted as others the split at mid sizes would be smaller.  Not measured.)
 inline int key_split(int ctas, int tiles, int n_sm) {
   auto cost = [&](int c) {
     const int n = ctas * c, per = (tiles + c - 1) / c, waves = (n + 2 * n_sm - 1) / (2 * n_sm);

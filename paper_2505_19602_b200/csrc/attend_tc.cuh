@@ -1061,30 +1061,30 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           for (int i = 0; i < 16; ++i) pk[i] = 0u;
           tc_st16(s_addr + cc * 16, pk);
         } else {
-        if (cc + 1 < kChunks && !empty(vc - 32)) front(v[(cc + 1) & 1], vc - 32, masked);
-        const float lt = back(v[cc & 1], pk);
-        if (cc + 2 < kChunks) tc_ld32(s_addr + (cc + 2) * 32, v[cc & 1]);
-        if (__any_sync(0xffffffffu, !(lt <= 8192.f))) {
-          // Once the early chunks' P is with the tensor core, their product has to land before O is scaled, and only
-          // the later chunks' P is still this thread's to scale.
-          const bool late = cc >= kEarlyChunks;
-          const Raised r = raise_reference(vc, c, m, l, s_addr, cc, late ? kEarlyChunks : 0, o_addr, (late || j > 0) ? 1 : 0,
-                                           late ? (o_landed == 2) : (o_landed >= 1), bar((late ? bPvEarly : bPvDone) + qt),
-                                           (late ? j : j - 1) & 1, abort_flag, status);
-          ok = __all_sync(0xffffffffu, r.ok != 0);
-          if (!ok) return;
-          m = r.m; l = r.l + r.sum;
-          if (r.o_landed) o_landed = late ? 2 : 1;
-          if (cc + 1 < kChunks && !empty(vc - 32)) {
-            // the next chunk's exponentials were taken against the old reference: once more, from its raw products
-            tc_ld32(s_addr + (cc + 1) * 32, v[(cc + 1) & 1]);
-            tc_wait_ld();
-            front(v[(cc + 1) & 1], vc - 32, masked);
+          if (cc + 1 < kChunks && !empty(vc - 32)) front(v[(cc + 1) & 1], vc - 32, masked);
+          const float lt = back(v[cc & 1], pk);
+          if (cc + 2 < kChunks) tc_ld32(s_addr + (cc + 2) * 32, v[cc & 1]);
+          if (__any_sync(0xffffffffu, !(lt <= 8192.f))) {
+            // Once the early chunks' P is with the tensor core, their product has to land before O is scaled, and only
+            // the later chunks' P is still this thread's to scale.
+            const bool late = cc >= kEarlyChunks;
+            const Raised r = raise_reference(vc, c, m, l, s_addr, cc, late ? kEarlyChunks : 0, o_addr, (late || j > 0) ? 1 : 0,
+                                             late ? (o_landed == 2) : (o_landed >= 1), bar((late ? bPvEarly : bPvDone) + qt),
+                                             (late ? j : j - 1) & 1, abort_flag, status);
+            ok = __all_sync(0xffffffffu, r.ok != 0);
+            if (!ok) return;
+            m = r.m; l = r.l + r.sum;
+            if (r.o_landed) o_landed = late ? 2 : 1;
+            if (cc + 1 < kChunks && !empty(vc - 32)) {
+              // the next chunk's exponentials were taken against the old reference: once more, from its raw products
+              tc_ld32(s_addr + (cc + 1) * 32, v[(cc + 1) & 1]);
+              tc_wait_ld();
+              front(v[(cc + 1) & 1], vc - 32, masked);
+            }
+          } else {
+            tc_st16(s_addr + cc * 16, pk);
+            l += lt;
           }
-        } else {
-          tc_st16(s_addr + cc * 16, pk);
-          l += lt;
-        }
         }
         if (cc == kEarlyChunks - 1) {
           // P of the first chunks is complete: that part of the PV product may start under the rest of the sweep
@@ -1190,7 +1190,7 @@ struct AttendTc {
 
   bool init(int dtype, int head_dim, void *k_pool, void *v_pool, long long n_pages, int page_tokens, std::string &err) {
     on = false;
-    if (dtype != 0 || head_dim != 128) return true;   // f32 x 64 is served by the FMA kernel
+    if (dtype != 0 || head_dim != 128) return true;   // f32 x 64 has a kernel of its own (attend_f32.cuh)
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || !fn) {

@@ -37,7 +37,7 @@ __device__ __forceinline__ size_t slot_row(const LayerView &lv, int slice, int s
 
 // Whether a slice's L entries outgrow its page table: reports, and the caller leaves before it looks up a slot.  Behind a
 // refused compress the device keeps the uncompressed length while the host goes on with the compressed one, so every kernel
-// that walks a slice to the device's length asks (the f32 attention, behind its append, cuts the length off).  The answer is the same in
+// that walks a slice to the device's length asks (the f32 attention reports too, and cuts the length off).  The answer is the same in
 // all CTAs of a slice: no cluster loses a part.
 __device__ __forceinline__ bool outgrown(const LayerView &lv, int L) {
   if (L <= (lv.pages_per_slice << lv.page_shift)) return false;

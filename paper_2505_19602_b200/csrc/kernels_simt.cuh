@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256) score_logits_kernel(LayerView lv, TensorV
   extern __shared__ float smem[];
   float *Qs = smem;             // [64][LD], rows >= w zero
   float *Ks = Qs + 64 * LD;     // [64][LD]
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int tid = threadIdx.x;
   const int slice = blockIdx.y;
   const int b = slice / lv.n_heads, h = slice % lv.n_heads;
   const int L = lv.hist_len[slice] + wa.n_k;

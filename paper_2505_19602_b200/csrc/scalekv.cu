@@ -1148,7 +1148,7 @@ scalekv_status scalekv_layer_stats_ex(scalekv_ctx *ctx, int32_t layer, scalekv_t
   if (tensor) {
     // A map that still waits in the caller's tensors is read there and copied by CTAs of the same launch beside the others, for
     // which those leave room - if it is so small that its copy is not what the call waits for in the end.  us per call, 16 slices, copied
-    // by a launch before this one -> so: 1 to 64 queries 31 -> 16, 256: 34 -> 20, 1 024: 46 -> 34; one CTA per 1 600 / 2 304 rows 61 ->
+    // by a launch before this one -> so: 1 to 64 queries 31 -> 17, 256: 34 -> 22, 1 024: 46 -> 30; one CTA per 1 600 / 2 304 rows 61 ->
     // 63, 86 -> 98.  (Of the gain at the small maps 8 us are the launch, the rest the wait for the stream and the way through ctypes.)
     const int copy_z = std::max(1, std::min(4, room - mma_split));
     const bool outside = !ctx->in_store[layer] && nk <= 512 * row_blocks * copy_z;
