@@ -464,56 +464,56 @@ __device__ __forceinline__ uint32_t remote(uint32_t addr, int cta) {
   return ra;
 }
 
-// The end of a softmax warp's work: its 32 rows of the O accumulator at o_addr, with references m and sums l, are normalised
-// and stored (have: there were keys for this tile).  A function of its own so that the sweep's registers are not allocated
-// around it.  window: this thread's row belongs to the observation window.
-__device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, uint32_t o_addr, int slice, int first_row, int qt, bool pair,
-                                         bool shared, bool have, int n_split, float m, float l, bool window) {
+// The end of a softmax warp's work, behind its last sweep: 32 rows of O with references m and sums l are normalised and stored
+// (have: there were keys for this tile).  A function of its own so that the sweep's registers are not allocated around it.
+// window: this thread's row belongs to the observation window.
+// What a row needs besides its columns (log-sum-exp, addresses, the place of a window row) is worked out before the last product is
+// waited for, and the two parts of a shared single are read from TMEM at once (a step of 16 slices x 36 / 144 / 576 / 1 024 queries behind
+// 21 / 80 / 209 / 209 entries: 5.8 / 7.5 / 13.5 / 18.1 -> 5.5 / 7.0 / 13.0 / 17.6 us; 128 x 1 600: 206.1 -> 204.7).  A pair's last tile
+// shared by both warpgroups, or 64 columns at a time there, gave the instance that records a window another schedule of
+// the sweep, 1-2 % slower throughout.
+__device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, uint32_t lane_addr, int slice, int first_row, int qt, bool pair,
+                                         bool shared, bool have, int n_split, float m, float l, bool window, volatile int *abort_flag,
+                                         int *status) {
   const int n_k = prm.n_k;
   const int lane = threadIdx.x & 31, quarter = (threadIdx.x >> 5) & 3, row = quarter * 32 + lane;
-  // Output rows leave through shared memory, 32 columns of the warp's 32 rows at a time (128 of a row's 256 bytes there), so that a store instruction
-  // writes eight whole 64-byte pieces (a row written by its own thread straight from the registers touches 32 lines per
-  // instruction) and neither another warp nor an asynchronous copy has to be waited for.  16-byte pieces are permuted by
-  // the row's index against bank conflicts. 
+  // Output rows leave through shared memory, so that a store instruction writes whole 64- or 128-byte pieces (a row written by its own
+  // thread straight from the registers touches 32 lines per instruction) and neither another warp nor an asynchronous copy has
+  // to be waited for.  16-byte pieces are permuted by the row's index against bank conflicts.
   const int b = prm.per_heads.div(slice), h = slice - b * prm.per_heads.d;
-  const int w0 = first_row + (pair ? qt * 128 : 0) + quarter * 32;       // the warp's first row
-  const int sub = lane >> 2, piece = lane & 3;
-  char *out = const_cast<char *>(prm.O.ptr) +
-              ((long long)b * prm.O.sb + (long long)h * prm.O.sh + (long long)(w0 + sub) * prm.O.st) * 2 + piece * 16;
-  auto slot = [](int r, int i) { return (uint32_t)r * 256 + (uint32_t)(((i ^ ((r >> 1) & 3)) + 4 * (r & 1)) << 4); };
-  auto emit = [&](const uint32_t *pk, uint32_t stage, int col) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + slot(lane, i)), "r"(pk[4 * i]),
-                   "r"(pk[4 * i + 1]), "r"(pk[4 * i + 2]), "r"(pk[4 * i + 3])
-                   : "memory");
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = 8 * i + sub;
-      uint4 val;
-      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
-                   : "r"(stage + slot(r, piece)) : "memory");
-      if (w0 + r < n_k) *reinterpret_cast<uint4 *>(out + i * prm.O.st * 16 + col * 2) = val;
-    }
+  const int r_own = first_row + (pair ? qt * 128 : 0) + row;             // this thread's row of its own tile
+  const uint32_t stage0 = base + kOffQ + qt * kTileBytes + quarter * 8192;     // (the last product has read the query tile before it is used)
+  char *obase = const_cast<char *>(prm.O.ptr) + ((long long)b * prm.O.sb + (long long)h * prm.O.sh) * 2;
+  // a barrier that completes exactly once, after a tile's last PV product: the per-tile PV barrier will not do, a parity wait
+  // cannot tell phases two apart and this warp may be that far behind it
+  auto final_product = [&](int t) {
+    const bool ok = mbar_wait_warp(base + kOffBar + 8 * (bFinal + t), 0, abort_flag, status);
+    tc_fence_after();
+    return ok;
   };
   auto window_rank = [&] {
     int rank = -1;
     if (window)
       for (int e = 0; e < prm.w; ++e)
-        if (prm.win_pos[e] == w0 + lane) rank = e;
+        if (prm.win_pos[e] == r_own) rank = e;
     return rank;
   };
   auto row_sums = [&](float mr, float lr) {              // what is kept of a row besides its output
     const float y = mr + log2f(lr);
-    if (prm.lse != nullptr && w0 + lane < n_k) prm.lse[(size_t)slice * n_k + w0 + lane] = y * 0.6931471805599453f;
+    if (prm.lse != nullptr && r_own < n_k) prm.lse[(size_t)slice * n_k + r_own] = y * 0.6931471805599453f;
     const int rank = window_rank();
     if (rank >= 0) prm.win_lse[(size_t)slice * prm.w + rank] = y;
   };
+  const uint32_t stat = base + kOffStat + (uint32_t)row * 8;             // of this row in tile A; tile B's lie 1024 bytes further
   if (!shared) {
-    if (have) {
+    if (have) row_sums(m, l);
+    if (have && final_product(qt)) {
+      // 32 columns of the warp's 32 rows at a time (128 of a row's 256 bytes there), eight 64-byte pieces a store instruction
       const float inv = 1.f / l;
-      const uint32_t stage = base + kOffQ + qt * kTileBytes + quarter * 8192;    // (no product reads the query tile any more)
+      const uint32_t o_addr = lane_addr + kColO + qt * 128;
+      const int sub = lane >> 2, piece = lane & 3, w0 = r_own - lane;
+      char *out = obase + (long long)(w0 + sub) * prm.O.st * 2 + piece * 16;
+      auto slot = [](int r, int i) { return (uint32_t)r * 256 + (uint32_t)(((i ^ ((r >> 1) & 3)) + 4 * (r & 1)) << 4); };
       float o[2][32];
       tc_ld32(o_addr, o[0]);
 #pragma unroll
@@ -523,9 +523,22 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
         if (cc + 1 < kChunks) tc_ld32(o_addr + (cc + 1) * 32, o[(cc + 1) & 1]);
 #pragma unroll
         for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(o[cc & 1][2 * i] * inv, o[cc & 1][2 * i + 1] * inv);
-        emit(pk, stage + (cc & 1) * 128, cc * 32);
+        const uint32_t stage = stage0 + (cc & 1) * 128;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + slot(lane, i)), "r"(pk[4 * i]),
+                       "r"(pk[4 * i + 1]), "r"(pk[4 * i + 2]), "r"(pk[4 * i + 3])
+                       : "memory");
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = 8 * i + sub;
+          uint4 val;
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
+                       : "r"(stage + slot(r, piece)) : "memory");
+          if (w0 + r < n_k) *reinterpret_cast<uint4 *>(out + i * prm.O.st * 16 + cc * 64) = val;
+        }
       }
-      row_sums(m, l);
     }
   } else {
     // ---- the two parts of a shared single are merged, half of the columns by each warpgroup: the rows of both lie in the
@@ -534,59 +547,79 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     // (with the parts handed over in shared memory, one row at a time per warp in finish_cluster and pushes of single pieces, a
     // step of 16 slices x 144 / 256 / 400 / 576 queries took 13.7 / 14.3 / 16.9 / 19.1 us; now 10.7 / 11.3 / 14.4 / 18.4).
     if (!have) { m = -INFINITY; l = 0.f; }
-    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(base + kOffStat + (uint32_t)(qt * 128 + row) * 8), "f"(m), "f"(l) : "memory");
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(stat + (uint32_t)qt * 1024), "f"(m), "f"(l) : "memory");
     // of a cluster the rows' owner: it gets this CTA's merged part, unnormalised, with its reference and sum
     const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(small_div(row, own_rows), n_split - 1);   // (rows beyond the map go nowhere)
     const int at = (int)blockIdx.z * own_rows + row - owner * own_rows;      // and the row's place there
     const uint32_t dst = n_split > 1 ? remote(base + kOffRing + (uint32_t)at * 512 + (uint32_t)qt * 256, owner) : 0;
-    const int rank = window_rank();
+    const int rank = n_split > 1 ? window_rank() : -1;
+    if (have) final_product(qt);
+    if (n_split > 1) cluster_arrive_relaxed();             // this CTA's ring is free (this warp has never touched it)
     tc_fence_before();
     asm volatile("bar.sync 2, 256;" ::: "memory");         // both accumulators are complete, no product reads the query tile any more
     tc_fence_after();
+    float o[64], other[64];
+    const uint32_t o_addr = lane_addr + kColO + qt * 64;
+#pragma unroll
+    for (int cc = 0; cc < 2; ++cc) {
+      tc_ld32(o_addr + qt * 128 + cc * 32, o + cc * 32);
+      tc_ld32(o_addr + (qt ^ 1) * 128 + cc * 32, other + cc * 32);
+    }
     float m2, l2;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(base + kOffStat + (uint32_t)((qt ^ 1) * 128 + row) * 8) : "memory");
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(stat + (uint32_t)(qt ^ 1) * 1024) : "memory");
     const float M = fmaxf(m, m2);
     float f1 = l > 0.f ? ex2(m - M) : 0.f, f2 = l2 > 0.f ? ex2(m2 - M) : 0.f;
     const float both = l * f1 + l2 * f2;
-    if (n_split == 1) { const float inv = 1.f / both; f1 *= inv; f2 *= inv; }
+    if (n_split == 1) {
+      const float inv = 1.f / both;
+      f1 *= inv; f2 *= inv;
+      if (qt == 0) row_sums(M, both);
+    }
     const bool none1 = !__any_sync(0xffffffffu, l > 0.f), none2 = !__any_sync(0xffffffffu, l2 > 0.f);   // a part without keys left garbage
     const uint64_t ff1 = pack2(f1, f1), ff2 = pack2(f2, f2);
-    // (of a cluster) the warpgroup's half of the row, 16-byte pieces permuted by its index
-    const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256;
-#pragma unroll 1
-    for (int cc = 0; cc < 2; ++cc) {
-      float o[32], other[32];
-      uint32_t pk[16];
-      tc_ld32(o_addr + qt * 64 + cc * 32, o);
-      tc_ld32((qt == 0 ? o_addr + 128 : o_addr - 128) + qt * 64 + cc * 32, other);
-      tc_wait_ld();
-      if (none1) {
+    tc_wait_ld();
+    if (none1) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = 0.f;
-      }
-      if (none2) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) other[i] = 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        unpack2(fma2(pack2(o[2 * i], o[2 * i + 1]), ff1, mul2(pack2(other[2 * i], other[2 * i + 1]), ff2)), o[2 * i], o[2 * i + 1]);
-        pk[i] = pack_bf16(o[2 * i], o[2 * i + 1]);
-      }
-      if (n_split > 1) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((cc * 8 + (i ^ (row & 7))) << 4)), "f"(o[4 * i]),
-                       "f"(o[4 * i + 1]), "f"(o[4 * i + 2]), "f"(o[4 * i + 3]) : "memory");
-      }
-      __syncwarp();
-      if (n_split == 1) emit(pk, base + kOffQ + qt * kTileBytes + quarter * 8192 + cc * 128, qt * 64 + cc * 32);   // (where it has read)
+      for (int i = 0; i < 64; ++i) o[i] = 0.f;
     }
-    if (n_split > 1) {
+    if (none2) {
+#pragma unroll
+      for (int i = 0; i < 64; ++i) other[i] = 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      unpack2(fma2(pack2(o[2 * i], o[2 * i + 1]), ff1, mul2(pack2(other[2 * i], other[2 * i + 1]), ff2)), o[2 * i], o[2 * i + 1]);
+    if (n_split == 1) {
+      // four 128-byte pieces a store instruction
+      const uint32_t stage = stage0 + qt * 4096, mine = stage + lane * 128;
+      const int w0 = first_row + quarter * 32 + (lane >> 3);
+      char *out = obase + (long long)w0 * prm.O.st * 2 + qt * 128 + (lane & 7) * 16;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((i ^ (lane & 7)) << 4)), "r"(pack_bf16(o[8 * i], o[8 * i + 1])),
+                     "r"(pack_bf16(o[8 * i + 2], o[8 * i + 3])), "r"(pack_bf16(o[8 * i + 4], o[8 * i + 5])), "r"(pack_bf16(o[8 * i + 6], o[8 * i + 7]))
+                     : "memory");
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int r = 4 * i + (lane >> 3);
+        uint4 val;
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
+                     : "r"(stage + (uint32_t)r * 128 + (uint32_t)(((lane & 7) ^ (r & 7)) << 4)) : "memory");
+        if (w0 + 4 * i < n_k) *reinterpret_cast<uint4 *>(out + i * prm.O.st * 8) = val;
+      }
+    } else {
+      // the warpgroup's half of the row, 16-byte pieces permuted by its index
+      const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256;
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((i & 8) << 4) + (uint32_t)(((i & 7) ^ (row & 7)) << 4)), "f"(o[4 * i]),
+                     "f"(o[4 * i + 1]), "f"(o[4 * i + 2]), "f"(o[4 * i + 3]) : "memory");
+      __syncwarp();
       // Off to the owners: 256 contiguous bytes (this warpgroup's half of a row) by 16 lanes at a time; stores of 16-byte
       // pieces of 32 rows travel between SMs piece by piece.
       cluster_wait();                                     // every CTA of the cluster is through with its ring
-      if (qt == 0 && first_row + row < n_k)
+      if (qt == 0 && r_own < n_k)
         asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(remote(base + kOffPartStat + (uint32_t)at * 8, owner)), "f"(M), "f"(both)
                      : "memory");
       const int half = lane >> 4, p16 = lane & 15;
@@ -597,14 +630,12 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
         float4 x;
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
                      : "r"(mine + (uint32_t)((r - lane) * 256) + (uint32_t)((p16 ^ (r & 7)) << 4)) : "memory");
-        if (w0 + r < n_k)
+        if (r_own - lane + r < n_k)
           asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(to), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
       }
       __syncwarp();
       if (qt == 0)                                        // (for the row's owner to find after the cluster's barrier)
         asm volatile("st.shared.s32 [%0], %1;" ::"r"(mine), "r"(rank) : "memory");
-    } else if (qt == 0) {
-      row_sums(M, both);
     }
   }
 }
@@ -1113,14 +1144,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(bPFull + qt));
     }
-    if (ok && steps > 0) {
-      // a barrier that completes exactly once, after the last PV product: the per-tile PV barrier will
-      // not do, a parity wait cannot tell phases two apart and this warp may be that far behind it
-      ok = mbar_wait_warp(bar(bFinal + qt), 0, abort_flag, status);
-    }
-    if (n_split > 1) cluster_arrive_relaxed();             // this CTA's ring is free (this warp has never touched it)
-    tc_fence_after();
-    finish_rows(prm, base, o_addr, item_slot[0], item_slot[1], qt, pair, shared, ok && steps > 0, n_split, m, l, kWindow && win_row != nullptr);
+    finish_rows(prm, base, lane_addr, item_slot[0], item_slot[1], qt, pair, shared, ok && steps > 0, n_split, m, l, kWindow && win_row != nullptr,
+                abort_flag, status);
     tc_fence_before();
   }
   __syncthreads();
