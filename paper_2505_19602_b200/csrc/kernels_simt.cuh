@@ -174,32 +174,6 @@ __global__ void __launch_bounds__(256) score_logits_kernel(LayerView lv, TensorV
 // ------------------------------------------------------------------------------------------
 constexpr uint32_t kWindowKey = 0xFFFFFFFFu;
 
-__device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int *total) {
-  // returns exclusive prefix of v over the block (thread order); *total = block sum
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int incl = v;
-  for (int o = 1; o < 32; o <<= 1) {
-    int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  __syncthreads();
-  if (lane == 31) warp_sums[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    int ws = (lane < (int)(blockDim.x >> 5)) ? warp_sums[lane] : 0;
-    int wi = ws;
-    for (int o = 1; o < 32; o <<= 1) {
-      int t = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += t;
-    }
-    warp_sums[lane] = wi - ws;        // exclusive warp offsets
-    if (lane == 31) warp_sums[32] = wi;  // block total
-  }
-  __syncthreads();
-  *total = warp_sums[32];
-  return warp_sums[wid] + incl - v;
-}
-
 // logit_scale: what turns a stored logit into a base-2 logit (1 when the logits kernel wrote them, softmax scale *
 // log2(e) when attend recorded raw products).  tile_padded: attend recorded them while the current map was
 // not in the store yet, so its entries sit behind the history rounded up to a multiple of 128 columns.
@@ -358,44 +332,111 @@ struct SelectShared {
   int hist[kSelectBins];
   int warp_sums[33];
   int keeps[32], ties[32];
+  uint32_t lowest[32], highest[32];
+  int first_gap;
   int bin, need, in_bin, n_cand, n_ties;
   uint32_t tie_key;
 };
 
 // The selection proper, run by a whole CTA of NT threads: key[0 .. L) (shared or global memory) -> out[] = the
 // ascending slots of the survivors (the `budget` largest keys, equal keys by lowest slot, plus every sentinel
-// entry).  Returns the number of survivors; *kprime_plus_win receives the count the rule demands.  Keys other than the
-// sentinel are below 2^(shift + 11); out has room for L entries and serves as scratch before it is written.
-//   A histogram over the keys' upper 11 bits says in which bin the budget runs out; when the bin holds no more keys than there
-//   are threads they are gathered and every one is ranked against all, else the next 11 bits decide in the same way.
-//   The emit gives every warp a run of consecutive entries and orders them by ballots, twice: to count, and behind one
-//   exclusive sum over the warps to write.
-// What bounds it is the latency of its rounds of block barriers.  Four 8-bit radix passes with warp-aggregated updates and
-// three block scans took 11 000 cycles for 265 entries and 23 000 for 4 248 (1 024 threads).
+// entry).  Returns the number of survivors; *kprime_plus_win receives the count the rule demands, sh.first_gap the lowest slot that
+// does not survive (L: all do).  lowest / highest: bounds of the keys, other than the sentinel, that this thread has seen; every key has
+// been seen by one.  Its first barrier ends its callers' writes of keys; out has room for L entries and serves as scratch before it is
+// written.
+//   Up to kRankAll entries: every key is ranked against all.
+//   More: a histogram of 2 048 bins between the lowest and the highest key says in which bin the budget runs out; when the bin
+//   holds no more keys than there are threads they are gathered and every one is ranked against all, else the next 11 bits
+//   decide in the same way.  The emit gives every warp a run of consecutive entries and orders them by ballots, twice: to count, and
+//   behind one exclusive sum over the warps to write.
+// What bounds it is the latency of its rounds of block barriers, and updates of one bin, which take turns.  512 threads, 56 / 224 /
+// 785 / 1 233 / 4 248 entries: 1 870 / 3 170 / 3 930 / 5 400 / 8 900 cycles.  (Bins of the keys' upper 11 bits, eight to an octave of importance,
+// and no ranking of all: 4 050 / 4 140 / 5 370 / 6 240 / 13 870.  Ranking 144 entries against all takes 3 900, hence the line at 128.)
+constexpr int kRankAll = 128;
 template <int NT>
-__device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int budget, int shift, int *out, SelectShared &sh,
-                                                int *kprime_plus_win) {
+__device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int budget, uint32_t lowest, uint32_t highest, int *out,
+                                                SelectShared &sh, int *kprime_plus_win) {
   constexpr int NW = NT / 32, PER = kSelectBins / NT;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  lowest = __reduce_min_sync(0xffffffffu, lowest);
+  highest = __reduce_max_sync(0xffffffffu, highest);
+  if (lane == 0) { sh.lowest[wid] = lowest; sh.highest[wid] = highest; }
+  for (int i = tid; i < kSelectBins; i += NT) sh.hist[i] = 0;
+  if (tid == 0) { sh.n_cand = 0; sh.first_gap = L; }
+  __syncthreads();
+  const uint32_t lower = (1u << lane) - 1u;
+  if (L <= kRankAll) {
+    // entry i by the threads i, i + 128, ..: how many candidates of their share of the entries stand before it (sentinels are
+    // zeros here, and stand before nothing)
+    constexpr int kParts = NT / kRankAll;
+    const int i = tid % kRankAll, part = tid / kRankAll, share = (L + kParts - 1) / kParts, lo = part * share, hi = min(lo + share, L);
+    const uint32_t k = i < L ? key[i] + 1u : 0u;
+    int before = 0;
+    if ((i & ~31) < L) {
+#pragma unroll 8
+      for (int j = lo; j < hi; ++j) {
+        const uint32_t o = key[j] + 1u;
+        before += o > k || (o == k && j < i);
+      }
+    }
+    if (part > 0) sh.hist[tid] = before;
+    const int all = __syncthreads_count(part == 0 && k != 0u);
+    kprime_plus_win[0] = (budget < 0 || budget > all ? all : budget) + (L - all);
+    bool keep = false;
+    if (part == 0) {
+#pragma unroll
+      for (int p = 1; p < kParts; ++p) before += sh.hist[p * kRankAll + i];
+      keep = i < L && (k == 0u || budget < 0 || before < budget);
+      const uint32_t kept = __ballot_sync(0xffffffffu, keep), gaps = __ballot_sync(0xffffffffu, i < L && !keep);
+      if (lane == 0) {
+        sh.keeps[wid] = __popc(kept);
+        if (gaps) atomicMin(&sh.first_gap, wid * 32 + __ffs(gaps) - 1);
+      }
+    }
+    __syncthreads();
+    const int keeps = lane < kRankAll / 32 ? sh.keeps[lane] : 0;
+    const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+    const int at = __reduce_add_sync(0xffffffffu, lane < wid ? keeps : 0) + __popc(kept & lower);
+    if (keep) out[at] = i;
+    return __reduce_add_sync(0xffffffffu, keeps);
+  }
+  lowest = __reduce_min_sync(0xffffffffu, lane < NW ? sh.lowest[lane] : 0xffffffffu);
+  highest = __reduce_max_sync(0xffffffffu, lane < NW ? sh.highest[lane] : 0u);
+  if (lowest > highest) lowest = highest = 0;          // nothing but sentinels
+  const int shift = max(21 - __clz((highest - lowest) | 1u), 0);       // the range of keys in 11 bits
   int kprime = 0;
   uint32_t above_min = kWindowKey, tie_key = kWindowKey;     // the smallest key of which every entry stays; the key of which
   int n_ties = 0;                                            // the first n_ties entries stay as well
+  // (keys less the lowest from here on)
   uint32_t prefix = 0;                                       // the keys in question: those with key >> above_shift == prefix
   for (int above_shift = shift + 11, s = shift, need = 0;; above_shift = s, s = s > 11 ? s - 11 : 0) {
     const bool first = above_shift == shift + 11;
-    for (int i = tid; i < kSelectBins; i += NT) sh.hist[i] = 0;
-    if (tid == 0) sh.n_cand = 0;
-    __syncthreads();
+    if (!first) {
+      for (int i = tid; i < kSelectBins; i += NT) sh.hist[i] = 0;
+      __syncthreads();
+    }
     for (int i = tid; i < L; i += NT) {
       const uint32_t k = key[i];
-      if (k != kWindowKey && (k >> above_shift) == prefix) atomicAdd(&sh.hist[(k >> s) - (prefix << (above_shift - s))], 1);
+      if (k != kWindowKey && ((k - lowest) >> above_shift) == prefix) atomicAdd(&sh.hist[((k - lowest) >> s) - (prefix << (above_shift - s))], 1);
     }
     __syncthreads();
     // thread t counts the bins 2047 - PER t, .. downwards, so that the exclusive sum is what lies above them
     int c[PER], mine = 0, all;
 #pragma unroll
     for (int e = 0; e < PER; ++e) { c[e] = sh.hist[kSelectBins - 1 - (tid * PER + e)]; mine += c[e]; }
-    const int above = block_exclusive_scan(mine, sh.warp_sums, &all);
+    int above = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, above, o);
+      if (lane >= o) above += x;
+    }
+    if (lane == 31) sh.warp_sums[wid] = above;
+    __syncthreads();
+    {
+      const int sums = lane < NW ? sh.warp_sums[lane] : 0;
+      all = __reduce_add_sync(0xffffffffu, sums);
+      above += __reduce_add_sync(0xffffffffu, lane < wid ? sums : 0) - mine;
+    }
     if (first) {
       kprime = (budget < 0 || budget > all) ? all : budget;
       *kprime_plus_win = kprime + (L - all);
@@ -418,19 +459,19 @@ __device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int b
     need = sh.need;
     const int m = sh.in_bin;
     if (m == need) {                             // the whole bin stays
-      above_min = prefix << s;
+      above_min = (prefix << s) + lowest;
       break;
     }
     if (s == 0) {                                // equal keys
-      tie_key = prefix;
+      tie_key = prefix + lowest;
       n_ties = need;
-      above_min = prefix + 1;
+      above_min = tie_key + 1;
       break;
     }
     if (m <= NT) {
       for (int i = tid; i < L; i += NT) {
         const uint32_t k = key[i];
-        if (k != kWindowKey && (k >> s) == prefix) out[atomicAdd(&sh.n_cand, 1)] = (int)k;
+        if (k != kWindowKey && ((k - lowest) >> s) == prefix) out[atomicAdd(&sh.n_cand, 1)] = (int)k;
       }
       __syncthreads();
       const int v = tid < m ? out[tid] : -1;     // (keys are below 2^31)
@@ -454,7 +495,6 @@ __device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int b
 
   // ordered emit: warp w owns entries [w * run, (w + 1) * run)
   const int run = ((L + NW - 1) / NW + 31) & ~31, lo = wid * run, hi = min(lo + run, L);
-  const uint32_t lower = (1u << lane) - 1u;
   int n_keep = 0, n_tie = 0;
   for (int i0 = lo; i0 < hi; i0 += 32) {
     const int i = i0 + lane;
@@ -467,18 +507,20 @@ __device__ __forceinline__ int select_and_emit(const uint32_t *key, int L, int b
   const int keeps = lane < NW ? sh.keeps[lane] : 0, ties = lane < NW ? sh.ties[lane] : 0;
   const int total = __reduce_add_sync(0xffffffffu, keeps) + min(__reduce_add_sync(0xffffffffu, ties), n_ties);
   int tie_at = __reduce_add_sync(0xffffffffu, lane < wid ? ties : 0);
-  int at = __reduce_add_sync(0xffffffffu, lane < wid ? keeps : 0) + min(tie_at, n_ties);
+  int at = __reduce_add_sync(0xffffffffu, lane < wid ? keeps : 0) + min(tie_at, n_ties), gap = L;
   for (int i0 = lo; i0 < hi; i0 += 32) {
     const int i = i0 + lane;
     const uint32_t k = i < hi ? key[i] : 0u;
     const bool tie = i < hi && k == tie_key && k != kWindowKey;
     const uint32_t tied = __ballot_sync(0xffffffffu, tie);
     const bool keep = (i < hi && (k >= above_min || k == kWindowKey)) || (tie && tie_at + __popc(tied & lower) < n_ties);
-    const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+    const uint32_t kept = __ballot_sync(0xffffffffu, keep), gaps = __ballot_sync(0xffffffffu, i < hi && !keep);
     if (keep) out[at + __popc(kept & lower)] = i;
+    if (gap == L && gaps) gap = i0 + __ffs(gaps) - 1;
     at += __popc(kept);
     tie_at += __popc(tied);
   }
+  if (lane == 0 && gap < L) atomicMin(&sh.first_gap, gap);
   return total;
 }
 
@@ -496,7 +538,7 @@ __device__ __forceinline__ uint32_t pooled_key(const float *sc, int i, int L, in
 // that is selected from the global key array as it stands (with pool > 1 the pooled keys are first written back
 // there), every pass streaming the keys through L2.
 __global__ void __launch_bounds__(1024) select_kernel(LayerView lv, WindowArg wa, int budget, const int *slice_budget, uint32_t *keys,
-                                                      const float *scores, int pool, int ld_s, int in_smem, int shift, int *keep_list,
+                                                      const float *scores, int pool, int ld_s, int in_smem, int *keep_list,
                                                       int *kept_count) {
   extern __shared__ uint32_t key_sm[];         // [L] when in_smem
   __shared__ SelectShared sh;
@@ -508,16 +550,17 @@ __global__ void __launch_bounds__(1024) select_kernel(LayerView lv, WindowArg wa
   int *out = keep_list + (size_t)slice * ld_s;
   uint32_t *gkey = keys + (size_t)slice * ld_s;
   const float *sc = scores + (size_t)slice * ld_s;
+  uint32_t lowest = 0xffffffffu, highest = 0u;
   for (int i = tid; i < L; i += 1024) {
     uint32_t k = gkey[i];
     if (pool > 1 && k != kWindowKey) k = pooled_key(sc, i, L, pool);
+    if (k != kWindowKey) { lowest = min(lowest, k); highest = max(highest, k); }
     if (in_smem) key_sm[i] = k;
     else if (pool > 1) gkey[i] = k;
   }
-  __syncthreads();
   if (slice_budget != nullptr) budget = slice_budget[slice];
   int want;
-  const int keep_total = select_and_emit<1024>(in_smem ? key_sm : gkey, L, budget, shift, out, sh, &want);
+  const int keep_total = select_and_emit<1024>(in_smem ? key_sm : gkey, L, budget, lowest, highest, out, sh, &want);
   if (tid == 0) {
     kept_count[slice] = keep_total;
     // the count rule of the selection: k' candidates and every sentinel entry survive
@@ -620,8 +663,8 @@ constexpr int kCompressThreads = 512;
 __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(LayerView lv, WindowArg wa, int policy, int n_sink,
                                                                           const float *logits, const float *lse, int ld_l,
                                                                           float logit_scale, int tile_padded, int budget,
-                                                                          const int *slice_budget, int pool, int shift, float *scores,
-                                                                          int ld_s, int *kept_count, ExternalMap ext) {
+                                                                          const int *slice_budget, int pool, float *scores, int ld_s,
+                                                                          int *kept_count, ExternalMap ext) {
   constexpr int NT = kCompressThreads;
   extern __shared__ __align__(16) uint32_t fsm[];
   int *list = reinterpret_cast<int *>(fsm);              // [ld_s]
@@ -651,6 +694,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   const long long ext_base = ext.on ? (long long)(slice / lv.n_heads) * ext.sb + (long long)(slice % lv.n_heads) * ext.sh : 0;
 
   // ---- phase 1: keys
+  uint32_t lowest = 0xffffffffu, highest = 0u;
   if (policy == 0) {
     float *sc_out = scores + (size_t)slice * ld_s;
     // columns of a logit row: the history's, then the current map's from map_col on
@@ -682,14 +726,23 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
         const int i = col < hist ? col : (col >= map_col && col < cols ? col - map_col + hist : -1);   // (the padding between them is nobody's)
         if (i >= 0) {
           const float sc = (e == 0 ? s0 : s1) * inv_w;
+          const uint32_t k = __float_as_uint(sc) & 0x7FFFFFFFu;
           sc_out[i] = sc;
-          key[i] = __float_as_uint(sc) & 0x7FFFFFFFu;
+          key[i] = k;
+          lowest = min(lowest, k);
+          highest = max(highest, k);
         }
       }
     }
     __syncthreads();
     if (pool > 1) {
-      for (int i = tid; i < L; i += NT) list[i] = (int)pooled_key(reinterpret_cast<const float *>(key), i, L, pool);
+      lowest = 0xffffffffu; highest = 0u;
+      for (int i = tid; i < L; i += NT) {
+        const uint32_t k = pooled_key(reinterpret_cast<const float *>(key), i, L, pool);
+        list[i] = (int)k;
+        lowest = min(lowest, k);
+        highest = max(highest, k);
+      }
       __syncthreads();
       for (int i = tid; i < L; i += NT) key[i] = (uint32_t)list[i];
       __syncthreads();
@@ -699,13 +752,13 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
     for (int i = tid; i < L; i += NT) {
       const int pos = i >= hist ? wa.n_prev + (i - hist) : lv.pos_pool[row_of(i)];
       key[i] = pos < n_sink ? kWindowKey : (uint32_t)pos + 1u;
+      if (pos >= n_sink) { lowest = min(lowest, (uint32_t)pos + 1u); highest = max(highest, (uint32_t)pos + 1u); }
     }
   }
-  __syncthreads();
 
   // ---- phase 2: selection
   int want;
-  const int kept = select_and_emit<NT>(key, L, budget, shift, list, sh, &want);
+  const int kept = select_and_emit<NT>(key, L, budget, lowest, highest, list, sh, &want);
   if (kept != want) {                          // the count rule of the selection (block-uniform)
     if (tid == 0) atomicExch(lv.status, kDevCheck);
     return;
@@ -713,42 +766,50 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   __syncthreads();
 
   // ---- phase 3: in-place gather of K, V and pos (a row of K or V is 256 bytes for either data type)
-  int lo = 0, hi = kept;                       // first j with keep[j] != j
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (list[mid] == mid) lo = mid + 1; else hi = mid;
-  }
+  int lo = min(sh.first_gap, kept);            // first j with keep[j] != j
   if (ext.on && lo > hist) lo = hist;          // kept rows of the current map are not where they belong yet, whatever their index
   const int piece = lane;                      // of a row's 32 16-byte pieces (16 of K, 16 of V)
   const char *ext_ptr = (piece < 16 ? ext.k : ext.v) + (piece & 15) * 16;
   char *pool_ptr = (piece < 16 ? lv.k_pool : lv.v_pool) + (piece & 15) * 16;
-  constexpr int kRows = NT / 32, C = 8 * kRows;  // rows per chunk, at most one per thread
-  for (int c0 = lo; c0 < kept; c0 += C) {
-    uint4 buf[8];
+  // Chunks of 128 rows, eight to a warp; a lane looks up where one row of four chunks comes from and goes, and the warp learns it
+  // by shuffles (16 slices, 1 944 rows: 61 700 -> 51 100 cycles, 26 a row; look-ups by every lane for every row cost as many issue slots
+  // as the copies take).  Copies of the next chunk under the stores of this one, in registers or by cp.async, gave nothing: loads
+  // queue behind the stores.
+  constexpr int kUnits = 8, C = kUnits * NT / 32;
+  for (int j0 = lo; j0 < kept; j0 += NT) {
+    const int mine = j0 + (lane / kUnits) * C + wid * kUnits + lane % kUnits;
+    unsigned long long from = 0;               // offset of the row in its array; odd: in the caller's
+    unsigned to = 0;
     int pos = 0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int j = c0 + wid + u * kRows;
-      if (j < kept) {
-        const int src = list[j];
-        const char *from = ext.on && src >= hist ? ext_ptr + (ext_base + (long long)(src - hist) * ext.st) * ext.esize
-                                                 : pool_ptr + row_of(src) * 256;
-        buf[u] = __ldcg(reinterpret_cast<const uint4 *>(from));
+    if (mine < kept) {
+      const int src = list[mine];
+      to = (unsigned)row_of(mine);
+      if (ext.on && src >= hist) {
+        from = (unsigned long long)((ext_base + (long long)(src - hist) * ext.st) * ext.esize) + 1;
+        pos = wa.n_prev + (src - hist);
+      } else {
+        const size_t row = row_of(src);
+        from = (unsigned long long)row * 256;
+        pos = lv.pos_pool[row];
       }
     }
-    const int jp = c0 + tid;
-    const bool has_pos = tid < C && jp < kept;
-    if (has_pos) {
-      const int src = list[jp];
-      pos = ext.on && src >= hist ? wa.n_prev + (src - hist) : lv.pos_pool[row_of(src)];
-    }
-    __syncthreads();
+#pragma unroll 1
+    for (int e = 0; e < 32 / kUnits && j0 + e * C < kept; ++e) {
+      const int n = kept - (j0 + e * C + wid * kUnits);      // rows of this warp in the chunk, if less than kUnits
+      uint4 buf[kUnits];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int j = c0 + wid + u * kRows;
-      if (j < kept) *reinterpret_cast<uint4 *>(pool_ptr + row_of(j) * 256) = buf[u];
+      for (int u = 0; u < kUnits; ++u) {
+        const unsigned long long f = __shfl_sync(0xffffffffu, from, e * kUnits + u);
+        if (u < n) buf[u] = __ldcg(reinterpret_cast<const uint4 *>(f & 1 ? ext_ptr + (f - 1) : pool_ptr + f));
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < kUnits; ++u) {
+        const unsigned t = __shfl_sync(0xffffffffu, to, e * kUnits + u);
+        if (u < n) *reinterpret_cast<uint4 *>(pool_ptr + (size_t)t * 256) = buf[u];
+      }
+      if (e == 0 && mine < kept) lv.pos_pool[to] = pos;      // (of all four chunks: their sources have been read)
     }
-    if (has_pos) lv.pos_pool[row_of(jp)] = pos;
   }
   if (tid == 0) {
     lv.next_len[slice] = kept;

@@ -896,9 +896,6 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     // logits recorded by attend are raw products in the tile-aligned layout; the logits kernel writes base-2 logits by slot
     const float logit_scale = summed ? ctx->scale * 1.4426950408889634f : 1.f;
     const int tile_padded = (recorded && ctx->logits_padded[layer]) ? 1 : 0;
-    // keys are the bits of non-negative floats, or positions: what has to be shifted out to leave 11 bits
-    int shift = 20;
-    if (recent) for (shift = 0; ((p.N[k + 1] + 1) >> shift) >= kSelectBins;) ++shift;
     int *slice_budget = nullptr;
     if (hb_on) {
       slice_budget = reinterpret_cast<int *>(ctx->ws + p.off_hbud);
@@ -928,7 +925,7 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
       cfg.attrs = attr;
       cfg.numAttrs = recent || summed ? 0 : 1;   // (behind a kernel of this call)
       CU(cudaLaunchKernelEx(&cfg, compress_fused_kernel, lv, wa, recent ? 1 : 0, n_sink, (const float *)logits, (const float *)wlse, p.ld_l,
-                            logit_scale, tile_padded, budget, (const int *)slice_budget, pool, shift, scores, p.ld_s, kept, ext));
+                            logit_scale, tile_padded, budget, (const int *)slice_budget, pool, scores, p.ld_s, kept, ext));
       if (external) ctx->in_store[layer] = 1;
     } else {
       if (!recent) {
@@ -943,7 +940,7 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
       {
         Scope sc(ctx, s, kSelect);
         select_kernel<<<p.n_slices, 1024, ctx->select_smem_ok ? (size_t)p.ld_s * 4 : 0, s>>>(
-            lv, wa, budget, slice_budget, keys, recent ? nullptr : scores, pool, p.ld_s, ctx->select_smem_ok ? 1 : 0, shift, keep, kept);
+            lv, wa, budget, slice_budget, keys, recent ? nullptr : scores, pool, p.ld_s, ctx->select_smem_ok ? 1 : 0, keep, kept);
       }
       {
         Scope sc(ctx, s, kCompact);

@@ -44,6 +44,27 @@ def test_ties_at_every_level(distinct, budget, heads, separate):
     kv.close()
 
 
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("distinct", [3, 4096])           # ties through the whole slice; hardly any
+@pytest.mark.parametrize("entries,budget", [
+    (127, 60), (128, 60), (129, 60),                       # every key ranked against all, up to 128 entries
+    (128, 0), (128, 112), (40, 23),                        # nothing but the window; all but none; a block mostly idle
+    (700, 112), (700, 113),                                # 128 and 129 rows: one chunk of the gather, and one row more
+    (1200, 496), (1200, 497),                              # 512 and 513: one round of look-ups, and one row more
+])
+def test_edges_of_ranking_and_gather(entries, budget, distinct, separate):
+    n = [24, entries - 24, 1]
+    budgets = [[binding.KEEP_ALL, budget, binding.KEEP_ALL]]
+    window = list(range(0, n[1], max(1, n[1] // 16)))[:16]
+    kv = binding.ScaleKV(1, 1, 3, 128, "bf16", [1, 1, 1], n, budgets)
+    run = ParityRun(kv, "bf16", [1, 1, 1], budgets, levels_inputs(1, 3, 128, n, distinct, entries),
+                    lambda k: window if k == 1 else [0], [(0, 0, 0), (0, 0, 2)], max_rows=16, sides_w=n)
+    run.separate_kernels = separate
+    run.run()
+    assert run.resyncs == 0
+    kv.close()
+
+
 @pytest.mark.parametrize("heads", [2, 17])
 @pytest.mark.parametrize("separate", [False, True])
 @pytest.mark.parametrize("budget", [5, 129, 2100])         # around the sinks, a chunk of rows, everything but a few
