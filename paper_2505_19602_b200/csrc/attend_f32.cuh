@@ -21,8 +21,8 @@
 // CTAs that share an SM takes about 8 000 cycles.  (Working copies that skip work, us per layer, 16 slices x 1 600 queries: whole 130; one
 // product of six 102; P not split 115; K and V not split 112.)  S of the next tile under the softmax of this one, from two buffers, and
 // fewer instructions: 139 -> 123.  us per layer and step, 16 slices behind 92 to 772 entries with their compresses, by packed fp32 FMA (66 %
-// of that pipe), a copy of the map and three launches per compress -> here: 16 queries 15.4 -> 10, 64: 25.7 -> 20, 256: 35.8 -> 26,
-// 400: 65 -> 40, 576: 91 -> 55, 1 024: 179 -> 80, 1 600: 331 -> 123.
+// of that pipe), a copy of the map and three launches per compress -> here: 16 queries 15.4 -> 10, 64: 25.7 -> 20, 256: 35.8 -> 21,
+// 400: 65 -> 32, 576: 91 -> 42, 1 024: 179 -> 66, 1 600: 331 -> 122.
 // Error against 64 bits, full caches of 29 to 4 436 entries, queries and keys normal, queries times 0.25 / 1 / 3: outputs 0.9 to 1.6 / 1.0 to
 // 2.1 / 1.5 to 4.0 e-7 (by FMA 1.1 to 11.9 / 2.2 to 12.3 / 3.3 to 15.2), lse 1.1 to 3.2 / 1.1 to 3.4 / 2.9 to 3.7 e-7 rms (1.1 to 3.2 / 1.4 to 3.3 /
 // 5.2 to 8.2).
@@ -71,7 +71,7 @@ struct Params {
   int fused, copy_in, n_prev;  // copy_in: the map's rows go to the pages on the way
   float scale;
   float weight_scale;          // what a difference of two rows' products is multiplied with to make a weight's exponent: |scale| log2(e), and kCutOff
-  int blocks;                  // blocks of query rows; the CTAs behind them (blockIdx.x) take the logits of the window's w rows
+  int win_tiles;               // key tiles of a slice whose logits with the window's w rows the CTAs behind the slices' (blockIdx.y) take
   float *win_logits;           // base-2 logits by slot, [slice][rank][ld_l]
   int ld_l, w;
   int win_pos[kMaxWindow];
@@ -398,7 +398,7 @@ __device__ __noinline__ void window_logits(const Params &prm, float *sm, int sli
   tile_logits<64>(Qs, Ks, prm.w, j0, L, prm.win_logits + (size_t)slice * prm.w * prm.ld_l, prm.ld_l, prm.scale);
 }
 
-// grid (ceil(n_k / 128) and, where the window is recorded, the key tiles over split, n_slices, split); dynamic shared memory kSmemBytes.
+// grid (ceil(n_k / 128), n_slices and, where the window is recorded, as many as its key tiles take, split); dynamic shared memory kSmemBytes.
 __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid_constant__ Params prm) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = tc::smem_u32(smem_raw);
@@ -412,10 +412,13 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   const int slice = blockIdx.y, b = slice / lv.n_heads, h = slice - b * lv.n_heads;
   const int q0 = blockIdx.x * kRows, n_k = prm.n_k, n_split = gridDim.z;
   int *status = lv.status;
-  if ((int)blockIdx.x >= prm.blocks) {
+  if (slice >= lv.n_slices) {
+    const int e = ((slice - lv.n_slices) * (int)gridDim.x + (int)blockIdx.x) * n_split + (int)blockIdx.z;
+    const int sl = e / prm.win_tiles, tile = e - sl * prm.win_tiles;
+    if (sl >= lv.n_slices) return;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int hist = lv.hist_len[slice], L = min(hist + n_k, prm.room), tile = ((int)blockIdx.x - prm.blocks) * n_split + (int)blockIdx.z;
-    if (tile * kKeys < L) window_logits(prm, reinterpret_cast<float *>(smem_raw), slice, b, h, hist, L, tile);
+    const int hist = lv.hist_len[sl], L = min(hist + n_k, prm.room);
+    if (tile * kKeys < L) window_logits(prm, reinterpret_cast<float *>(smem_raw), sl, sl / lv.n_heads, sl % lv.n_heads, hist, L, tile);
     return;
   }
   if (tid == 0) {
@@ -501,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
         if (values) put_split(base + kOffV, kPieceK, r0 + 16 * u, c, times(x[u][0], kLift), times(x[u][1], kLift));
         else put_split(base + kOffK, kPieceK, r0 + 16 * u, c, x[u][0], x[u][1]);
       }
-      if (prm.copy_in && tile * kKeys + kKeys > hist && tile % prm.blocks == (int)blockIdx.x) {      // (the CTAs of a slice take turns)
+      if (prm.copy_in && tile * kKeys + kKeys > hist && tile % (int)gridDim.x == (int)blockIdx.x) {      // (the CTAs of a slice take turns)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int slot = tile * kKeys + r0 + 16 * u;

@@ -94,3 +94,35 @@ def test_f32_rows_of_equal_scores_far_from_zero(heads, key):
     assert ((O.double() - want).norm() / (O.shape[2] ** 0.5 * want.norm())).item() <= 2e-6
     assert (lse.double() - (key / 8 + torch.log(torch.tensor(340.0, dtype=torch.float64)).item())).abs().max().item() <= abs(key) / 8 * 2e-7 + 1e-6
     kv.close()
+
+
+@pytest.mark.parametrize("batch,heads,hist,n", [
+    (1, 3, 300, 1),            # one block of queries, more key tiles than that: rows of the grid behind the slices'
+    (1, 3, 70, 129),           # a last row of the grid that is not full
+    (2, 40, 500, 300),         # clusters of none, more CTAs than SMs
+    (128, 128, 300, 1),        # more rows than a grid has: the compress scores from K
+])
+def test_window_logits_behind_the_slices(batch, heads, hist, n):
+    sides_w, budget = [hist, n, 1], 40
+    kv = binding.ScaleKV(1, batch, heads, 64, "f32", [1, 1, 1], sides_w, [[binding.KEEP_ALL, budget, binding.KEEP_ALL]], window_patches=16,
+                         window_kind="last")
+    g = torch.Generator().manual_seed(hist + n)
+    slices = sorted({(0, 0), (batch - 1, heads - 1), (batch // 2, heads // 2)})
+    caches = {s: orc.SliceCache(sides_w, 64) for s in slices}
+    for k, nk in enumerate(sides_w):
+        base = [torch.randn(1, 3, nk, 64, generator=g) for _ in range(3)]          # head h of any image has what head h mod 3 has here
+        Q, K, V = (x.cuda()[:, torch.arange(heads) % 3].repeat(batch, 1, 1, 1) for x in base)
+        O = torch.empty_like(Q)
+        window = list(range(max(0, nk - 16), nk))
+        torch.cuda.synchronize()
+        kv.scalekv_step(0, k, Q, K, V, O, window_pos=window if k == 1 else None)
+        kv.scalekv_sync()
+        for b, h in slices:
+            q, key, value = (x[0, h % 3].double().numpy() for x in base)
+            caches[b, h].append(key, value)
+            want, _ = caches[b, h].attend(q)
+            assert abs(want - O[b, h].double().cpu().numpy()).max() <= 1e-4
+            if k == 1:
+                pos, _ = caches[b, h].compress(q[window], window, budget)
+                assert (kv.scalekv_export_slice(0, b, h).numpy() == pos).all()
+    kv.close()
