@@ -20,9 +20,10 @@
 // What bounds it: the instructions of the softmax and of the splitting, and the tensor pipe, six products standing for one; a step of two
 // CTAs that share an SM takes about 8 000 cycles.  (Working copies that skip work, us per layer, 16 slices x 1 600 queries: whole 130; one
 // product of six 102; P not split 115; K and V not split 112.)  S of the next tile under the softmax of this one, from two buffers, and
-// fewer instructions: 139 -> 123.  us per layer and step, 16 slices behind 92 to 772 entries with their compresses, by packed fp32 FMA (66 %
-// of that pipe), a copy of the map and three launches per compress -> here: 16 queries 15.4 -> 10, 64: 25.7 -> 20, 256: 35.8 -> 21,
-// 400: 65 -> 32, 576: 91 -> 42, 1 024: 179 -> 66, 1 600: 331 -> 122.
+// fewer instructions: 139 -> 123.  The softmax's loops over a tile's 16-column pieces and the operands' part of a step are compiled once, not unrolled or
+// copied: 123 -> 113 (fewer spills, less code to fetch in short launches).  us per layer and step, 16 slices behind 92 to 772 entries with their compresses,
+// by packed fp32 FMA (66 % of that pipe), a copy of the map and three launches per compress -> here: 16 queries 15.4 -> 8.7, 64: 25.7 -> 16, 256: 35.8 -> 20,
+// 400: 65 -> 31, 576: 91 -> 40, 1 024: 179 -> 63, 1 600: 331 -> 113.
 // Error against 64 bits, full caches of 29 to 4 436 entries, queries and keys normal, queries times 0.25 / 1 / 3: outputs 0.9 to 1.6 / 1.0 to
 // 2.1 / 1.5 to 4.0 e-7 (by FMA 1.1 to 11.9 / 2.2 to 12.3 / 3.3 to 15.2), lse 1.1 to 3.2 / 1.1 to 3.4 / 2.9 to 3.7 e-7 rms (1.1 to 3.2 / 1.4 to 3.3 /
 // 5.2 to 8.2).
@@ -445,6 +446,29 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     *leave_slot = leave;
     if (!leave && blockIdx.x == 0 && blockIdx.z == 0) lv.next_len[slice] = L;      // unless a compress of this scale evicts
   }
+  const int c = tid & 7, r0 = (tid & 127) >> 3;
+  // The operand warps' part of a tile: chunk c of rows r0, r0 + 16, ..
+  long long at[4];                     // where the rows of the tile whose keys were loaded last lie in the pages, in bytes
+  auto load = [&](bool values, int tile, float4 (&x)[4][2]) {      // (the keys of a tile before its values)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int slot = tile * kKeys + r0 + 16 * u;
+      const bool outside = prm.fused && slot >= hist;
+      x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (slot < L) {
+        if (!values && !outside) at[u] = (long long)slot_row(lv, slice, slot) * 256;
+        const char *row = outside ? reinterpret_cast<const char *>(row_ptr<float>(values ? prm.V : prm.K, b, h, slot - hist))
+                                  : (values ? lv.v_pool : lv.k_pool) + at[u];
+        x[u][0] = reinterpret_cast<const float4 *>(row)[2 * c];
+        x[u][1] = reinterpret_cast<const float4 *>(row)[2 * c + 1];
+      }
+    }
+  };
+  float4 kx[4][2], vx[4][2];
+  if (warp >= 4 && lo < tiles * ((int)blockIdx.z + 1) / n_split) {       // (on their way while Q is split)
+    load(false, lo, kx);
+    load(true, lo, vx);
+  }
   // Q: a thread takes one chunk of eight columns of four rows.  (Of a negative scale Q takes the sign, so that the largest product is
   // the largest score.)
   const float lift = copysignf(kLift, prm.scale);
@@ -481,23 +505,6 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
 
   if (warp >= 4) {
     // ---------------------------------------------------------------- operands
-    const int ct = tid - 128, c = ct & 7, r0 = ct >> 3;
-    long long at[4];                     // where the rows of the tile whose keys were loaded last lie in the pages, in bytes
-    auto load = [&](bool values, int tile, float4 (&x)[4][2]) {      // (the keys of a tile before its values)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int slot = tile * kKeys + r0 + 16 * u;
-        const bool outside = prm.fused && slot >= hist;
-        x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (slot < L) {
-          if (!values && !outside) at[u] = (long long)slot_row(lv, slice, slot) * 256;
-          const char *row = outside ? reinterpret_cast<const char *>(row_ptr<float>(values ? prm.V : prm.K, b, h, slot - hist))
-                                    : (values ? lv.v_pool : lv.k_pool) + at[u];
-          x[u][0] = reinterpret_cast<const float4 *>(row)[2 * c];
-          x[u][1] = reinterpret_cast<const float4 *>(row)[2 * c + 1];
-        }
-      }
-    };
     auto put = [&](bool values, int tile, const float4 (&x)[4][2]) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -537,37 +544,27 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(bar(bV));
     };
-    float4 kx[4][2], vx[4][2];
-    if (nt > 0) {
-      load(false, lo, kx);
-      load(true, lo, vx);
-      put(false, lo, kx);
-      keys_there();
-      if (warp == 4) mma_s(0);
-      put(true, lo, vx);
-      announce_v();
-      if (nt > 1) {
-        load(false, lo + 1, kx);
-        load(true, lo + 1, vx);
-      }
-    }
     bool ok = true;
     // (a warp whose wait gives up goes on to meet the others at the named barrier, which knows no limit)
-    for (int i = 0; i < nt; ++i) {
+#pragma unroll 1
+    for (int i = -1; i < nt; ++i) {
       const bool more = i + 1 < nt;
-      ok = ok && s_landed(i);                                 // K_i has been read
+      ok = ok && (i < 0 || s_landed(i));                      // K_i has been read
       if (more) {
         if (ok) put(false, lo + i + 1, kx);
+        if (i < 0 && nt > 1) load(false, lo + 1, kx);
         keys_there();
       }
-      ok = ok && (i == 0 || pv_landed(i - 1));                // V_{i-1} has been read, and P_{i-1}
+      ok = ok && (i <= 0 || pv_landed(i - 1));                // V_{i-1} has been read, and P_{i-1}
       if (warp == 4 && more && ok) mma_s(i + 1);
-      if (ok && i > 0) {
-        put(true, lo + i, vx);
+      if (ok && i != 0 && nt > 0) {                           // (V_0 before the softmax of tile 0)
+        put(true, lo + max(i, 0), vx);
         announce_v();
-        if (more) load(true, lo + i + 1, vx);
       }
-      if (ok && i + 2 < nt) load(false, lo + i + 2, kx);
+      if (ok && i >= 0) {
+        if (more) load(true, lo + i + 1, vx);
+        if (i + 2 < nt) load(false, lo + i + 2, kx);
+      }
     }
     // (given up: what has been issued must be through before TMEM and shared memory are anybody else's)
     if (!ok && issued > 0) tc::mbar_drain(bar(bS + ((issued - 1) & 1)), ((issued - 1) >> 1) & 1);
@@ -617,7 +614,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       const uint32_t buf = lane_addr + kBufCols * (i & 1);
       auto real = [&](int key) { return !decltype(masked)::value || key < valid; };
       float mx = -INFINITY;
-#pragma unroll
+#pragma unroll 4
       for (int e = 0; e < 4; ++e) {
         uint32_t x[16];
         tc::tc_ld16(buf + 16 * e, x);
@@ -641,7 +638,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       }
       const uint64_t c2 = tc::pack2(c, c), negm2 = tc::pack2(-m, -m);
       uint64_t sum2[2] = {0ull, 0ull};
-#pragma unroll
+#pragma unroll 1
       for (int e = 0; e < 4; ++e) {
         uint32_t x[16], ph[8], pm[8], pl[8];
         tc::tc_ld16(buf + 16 * e, x);
