@@ -683,13 +683,35 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   const int dev_status = *reinterpret_cast<volatile int *>(lv.status);
   const int hist = *reinterpret_cast<volatile int *>(lv.hist_len + slice);
   if (slice_budget != nullptr) budget = slice_budget[slice];
-  const float row_lse = policy == 0 && tid < w ? lse[(size_t)slice * w + tid] : 0.f;
+  const float row_lse = policy == 0 && lse != nullptr && tid < w ? lse[(size_t)slice * w + tid] : 0.f;
   if (tid < lv.pages_per_slice) pt[tid] = page;
   for (int i = tid + NT; i < lv.pages_per_slice; i += NT) pt[i] = __ldg(pages + i);
-  if (policy == 0 && tid < w) lse_row[tid] = row_lse;
+  if (policy == 0 && lse != nullptr && tid < w) lse_row[tid] = row_lse;
   const int L = hist + wa.n_k;
   if (dev_status != 0 || outgrown(lv, L)) return;   // a failed check, an earlier kernel's or this one's: leave the store alone
   __syncthreads();
+  if (policy == 0 && lse == nullptr) {
+    // The rows' log-sum-exps, a warp a row, to the bit those of row_lse_kernel: there a thread adds up every 1 024th entry, a warp its threads' sums
+    // crosswise and one thread the 32 warps' in turn.
+    for (int j = wid; j < w; j += NT / 32) {
+      const float *y = logits + ((size_t)slice * w + j) * ld_l;
+      float top = -INFINITY, sum = 0.f;
+#pragma unroll 8
+      for (int i = lane; i < L; i += 32) top = fmaxf(top, __ldg(y + i));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+#pragma unroll 4
+      for (int k0 = 0; k0 < min(L, 1024); k0 += 32) {
+        float v = 0.f;
+        for (int i = k0 + lane; i < L; i += 1024) v += exp2f(__ldg(y + i) - top);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        sum += v;
+      }
+      if (lane == 0) lse_row[j] = top + log2f(sum);
+    }
+    __syncthreads();
+  }
   auto row_of = [&](int slot) { return ((size_t)pt[slot >> lv.page_shift] << lv.page_shift) + (size_t)(slot & lv.page_mask); };
   const long long ext_base = ext.on ? (long long)(slice / lv.n_heads) * ext.sb + (long long)(slice % lv.n_heads) * ext.sh : 0;
 

@@ -31,6 +31,10 @@ constexpr int kSets = 4;
 // layer_stats splits a slice's keys over several CTAs while the launch would otherwise leave SMs idle; this many CTAs
 // bound the scratch of their partial results (about 10 MB)
 constexpr int kStatsMaxCtas = 592;
+// Up to how many entries of a slice the one-launch compress takes the log-sum-exps of the window's rows itself where attend has not left them: a
+// launch less on the way from an f32 attend to its layer's next.  us per layer and step, 16 slices x 64 / 144 / 256 / 400 queries: a launch of its own
+// 17.0 / 17.9 / 20.5 / 31.2; none up to 256 entries 16.0 / 17.4 / 20.0 / 30.7; none up to 1 024 16.4 / 17.4 / 20.0 / 33.8.
+constexpr int kSumsInCompress = 512;
 constexpr int kNumClasses = 7;
 enum KernelClass { kAppend = 0, kAttend = 1, kScore = 2, kSelect = 3, kCompact = 4, kOther = 5, kCompress = 6 };
 
@@ -892,7 +896,8 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     ctx->logits_of[layer] = -1;
     float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
     const bool summed = recorded && ctx->tc.enabled();          // (the f32 attention leaves what the logits kernel would)
-    if (!recent && !summed) {
+    const bool sums = !recent && !summed && !(fused && L <= kSumsInCompress);
+    if (sums) {
       Scope sc(ctx, s, kScore);
       row_lse_kernel<<<dim3(p.n_slices, (wa.w + 3) / 4), 1024, 0, s>>>(lv, wa, logits, p.ld_l, wlse);
     }
@@ -926,8 +931,9 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr[0].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
-      cfg.numAttrs = recent || summed ? 0 : 1;   // (behind a kernel of this call)
-      CU(cudaLaunchKernelEx(&cfg, compress_fused_kernel, lv, wa, recent ? 1 : 0, n_sink, (const float *)logits, (const float *)wlse, p.ld_l,
+      cfg.numAttrs = sums || !recorded ? 1 : 0;   // (behind a kernel of this call)
+      CU(cudaLaunchKernelEx(&cfg, compress_fused_kernel, lv, wa, recent ? 1 : 0, n_sink, (const float *)logits,
+                            (const float *)(summed || sums ? wlse : nullptr), p.ld_l,
                             logit_scale, tile_padded, budget, (const int *)slice_budget, pool, scores, p.ld_s, kept, ext));
       if (external) ctx->in_store[layer] = 1;
     } else {
