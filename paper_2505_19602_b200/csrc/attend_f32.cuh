@@ -773,10 +773,12 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
 // CTAs that share a slice's keys.  ctas: CTAs of an unsplit launch.  In steps of a key tile: a CTA that has its SM to itself takes 1 per
 // tile, two that share one 1.35 each.  (The CTAs of a recorded window, one per key tile and slice, are not counted: they hold an SM for about a tile's
 // time, and with them counted as others the split at mid sizes would be smaller.  Not measured.)
+// What combining costs is set by slices of two tiles, which gain by a split (64 queries behind 57 entries, 4 / 16 / 32 / 64 / 73 slices, us per launch, one CTA ->
+// two: 10.4 / 10.6 / 10.6 / 10.6 / 10.8 -> 8.7 / 9.0 / 9.0 / 9.7 / 9.9); at 1.5 they had none.  Longer ones split as they did.
 inline int key_split(int ctas, int tiles, int n_sm) {
   auto cost = [&](int c) {
     const int n = ctas * c, per = (tiles + c - 1) / c, waves = (n + 2 * n_sm - 1) / (2 * n_sm);
-    return (n <= n_sm ? 1.f : 1.35f) * (float)(waves * (per + 3)) + (c > 1 ? 1.5f : 0.f);
+    return (n <= n_sm ? 1.f : 1.35f) * (float)(waves * (per + 3)) + (c > 1 ? 0.8f : 0.f);
   };
   int split = 1;
   for (int c = 2; c <= kMaxSplit && c <= tiles; ++c)
