@@ -465,16 +465,17 @@ __device__ __forceinline__ uint32_t remote(uint32_t addr, int cta) {
 }
 
 // The end of a softmax warp's work, behind its last sweep: 32 rows of O with references m and sums l are normalised and stored
-// (have: there were keys for this tile).  A function of its own so that the sweep's registers are not allocated around it.
-// window: this thread's row belongs to the observation window.
+// (have: there were keys for this tile; whole: nothing has been given up so far).  A function of its own so that the sweep's registers are not
+// allocated around it.  window: this thread's row belongs to the observation window.
+// A row that lacks a product, because some wait for it has run out, is left as it is: its accumulator and its query tile may still be in use.
 // What a row needs besides its columns (log-sum-exp, addresses, the place of a window row) is worked out before the last product is
 // waited for, and the two parts of a shared single are read from TMEM at once (a step of 16 slices x 36 / 144 / 576 / 1 024 queries behind
 // 21 / 80 / 209 / 209 entries: 5.8 / 7.5 / 13.5 / 18.1 -> 5.5 / 7.0 / 13.0 / 17.6 us; 128 x 1 600: 206.1 -> 204.7).  A pair's last tile
 // shared by both warpgroups, or 64 columns at a time there, gave the instance that records a window another schedule of
 // the sweep, 1-2 % slower throughout.
 __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, uint32_t lane_addr, int slice, int first_row, int qt, bool pair,
-                                         bool shared, bool have, int n_split, float m, float l, bool window, volatile int *abort_flag,
-                                         int *status) {
+                                         bool shared, bool have, bool whole, int n_split, float m, float l, bool window,
+                                         volatile int *abort_flag, int *status) {
   const int n_k = prm.n_k;
   const int lane = threadIdx.x & 31, quarter = (threadIdx.x >> 5) & 3, row = quarter * 32 + lane;
   // Output rows leave through shared memory, so that a store instruction writes whole 64- or 128-byte pieces (a row written by its own
@@ -498,16 +499,17 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
         if (prm.win_pos[e] == r_own) rank = e;
     return rank;
   };
-  auto row_sums = [&](float mr, float lr) {              // what is kept of a row besides its output
-    const float y = mr + log2f(lr);
+  auto keep_sums = [&](float y, int rank) {              // what is kept of a row besides its output: its base-2 log-sum-exp
     if (prm.lse != nullptr && r_own < n_k) prm.lse[(size_t)slice * n_k + r_own] = y * 0.6931471805599453f;
-    const int rank = window_rank();
     if (rank >= 0) prm.win_lse[(size_t)slice * prm.w + rank] = y;
   };
   const uint32_t stat = base + kOffStat + (uint32_t)row * 8;             // of this row in tile A; tile B's lie 1024 bytes further
   if (!shared) {
-    if (have) row_sums(m, l);
-    if (have && final_product(qt)) {
+    if (!have || !whole) return;
+    const float y = m + log2f(l);
+    const int rank = window_rank();
+    if (final_product(qt)) {
+      keep_sums(y, rank);
       // 32 columns of the warp's 32 rows at a time (128 of a row's 256 bytes there), eight 64-byte pieces a store instruction
       const float inv = 1.f / l;
       const uint32_t o_addr = lane_addr + kColO + qt * 128;
@@ -552,8 +554,11 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(small_div(row, own_rows), n_split - 1);   // (rows beyond the map go nowhere)
     const int at = (int)blockIdx.z * own_rows + row - owner * own_rows;      // and the row's place there
     const uint32_t dst = n_split > 1 ? remote(base + kOffRing + (uint32_t)at * 512 + (uint32_t)qt * 256, owner) : 0;
-    const int rank = n_split > 1 ? window_rank() : -1;
-    if (have) final_product(qt);
+    const int rank = window_rank();
+    if (!whole || (have && !final_product(qt))) {          // (no sum is negative)
+      l = -1.f;
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(stat + (uint32_t)qt * 1024 + 4), "f"(l) : "memory");
+    }
     if (n_split > 1) cluster_arrive_relaxed();             // this CTA's ring is free (this warp has never touched it)
     tc_fence_before();
     asm volatile("bar.sync 2, 256;" ::: "memory");         // both accumulators are complete, no product reads the query tile any more
@@ -567,13 +572,14 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     }
     float m2, l2;
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(stat + (uint32_t)(qt ^ 1) * 1024) : "memory");
+    whole = !(l < 0.f || l2 < 0.f);                        // (the same for the warp's rows)
     const float M = fmaxf(m, m2);
     float f1 = l > 0.f ? ex2(m - M) : 0.f, f2 = l2 > 0.f ? ex2(m2 - M) : 0.f;
     const float both = l * f1 + l2 * f2;
     if (n_split == 1) {
       const float inv = 1.f / both;
       f1 *= inv; f2 *= inv;
-      if (qt == 0) row_sums(M, both);
+      if (qt == 0 && whole) keep_sums(M + log2f(both), rank);
     }
     const bool none1 = !__any_sync(0xffffffffu, l > 0.f), none2 = !__any_sync(0xffffffffu, l2 > 0.f);   // a part without keys left garbage
     const uint64_t ff1 = pack2(f1, f1), ff2 = pack2(f2, f2);
@@ -590,6 +596,7 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     for (int i = 0; i < 32; ++i)
       unpack2(fma2(pack2(o[2 * i], o[2 * i + 1]), ff1, mul2(pack2(other[2 * i], other[2 * i + 1]), ff2)), o[2 * i], o[2 * i + 1]);
     if (n_split == 1) {
+      if (!whole) return;
       // four 128-byte pieces a store instruction
       const uint32_t stage = stage0 + qt * 4096, mine = stage + lane * 128;
       const int w0 = first_row + quarter * 32 + (lane >> 3);
@@ -611,17 +618,20 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     } else {
       // the warpgroup's half of the row, 16-byte pieces permuted by its index
       const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256;
+      if (whole) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
-        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((i & 8) << 4) + (uint32_t)(((i & 7) ^ (row & 7)) << 4)), "f"(o[4 * i]),
-                     "f"(o[4 * i + 1]), "f"(o[4 * i + 2]), "f"(o[4 * i + 3]) : "memory");
+        for (int i = 0; i < 16; ++i)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((i & 8) << 4) + (uint32_t)(((i & 7) ^ (row & 7)) << 4)), "f"(o[4 * i]),
+                       "f"(o[4 * i + 1]), "f"(o[4 * i + 2]), "f"(o[4 * i + 3]) : "memory");
+      }
       __syncwarp();
       // Off to the owners: 256 contiguous bytes (this warpgroup's half of a row) by 16 lanes at a time; stores of 16-byte
       // pieces of 32 rows travel between SMs piece by piece.
       cluster_wait();                                     // every CTA of the cluster is through with its ring
       if (qt == 0 && r_own < n_k)
-        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(remote(base + kOffPartStat + (uint32_t)at * 8, owner)), "f"(M), "f"(both)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(remote(base + kOffPartStat + (uint32_t)at * 8, owner)), "f"(M), "f"(whole ? both : -1.f)
                      : "memory");
+      if (!whole) return;
       const int half = lane >> 4, p16 = lane & 15;
 #pragma unroll 8
       for (int e = 0; e < 16; ++e) {
@@ -659,6 +669,7 @@ __device__ __forceinline__ void finish_cluster(const Params &prm, uint32_t base,
     float m = -INFINITY, sum = 0.f;
     if (part < n_split)
       asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m), "=f"(sum) : "r"(base + kOffPartStat + (uint32_t)(part * own_rows + at) * 8));
+    const bool whole = !(__ballot_sync(0xffffffffu, sum < 0.f) & (0xffu << (8 * sub)));       // no part has been given up
     float M = m;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
@@ -682,7 +693,7 @@ __device__ __forceinline__ void finish_cluster(const Params &prm, uint32_t base,
         a[4 * i + 2] = fmaf(x.z, f, a[4 * i + 2]); a[4 * i + 3] = fmaf(x.w, f, a[4 * i + 3]);
       }
     }
-    if (live) {
+    if (live && whole) {
       const float inv = 1.f / sum;
       const int qi = q_first + r;
 #pragma unroll
@@ -1144,8 +1155,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(bPFull + qt));
     }
-    finish_rows(prm, base, lane_addr, item_slot[0], item_slot[1], qt, pair, shared, ok && steps > 0, n_split, m, l, kWindow && win_row != nullptr,
-                abort_flag, status);
+    finish_rows(prm, base, lane_addr, item_slot[0], item_slot[1], qt, pair, shared, steps > 0, ok && !leave, n_split, m, l,
+                kWindow && win_row != nullptr, abort_flag, status);
     tc_fence_before();
   }
   __syncthreads();
