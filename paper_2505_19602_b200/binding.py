@@ -17,7 +17,8 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libscalekv.so")
-SOURCES = [os.path.join(_HERE, "csrc", f) for f in ("scalekv.cu", "select_static.cu", "kernels_simt.cuh", "attend_tc.cuh", "attend_f32.cuh", "common.cuh")]
+SOURCES = [os.path.join(_HERE, "csrc", f) for f in ("scalekv.cu", "select_static.cu", "kernels_simt.cuh", "attend_tc.cuh", "attend_f32.cuh", "key_split.h",
+                                                 "common.cuh")]
 HEADER = os.path.join(os.path.dirname(_HERE), "include", "scalekv.h")
 CALL_SOURCE = os.path.join(_HERE, "csrc", "call.cpp")
 

@@ -33,6 +33,7 @@
 
 #include "attend_tc.cuh"
 #include "kernels_simt.cuh"
+#include "key_split.h"
 
 namespace scalekv {
 namespace f32 {
@@ -41,7 +42,6 @@ using tc::tc_fence_after;
 using tc::tc_fence_before;
 
 constexpr int kRows = 128, kKeys = 64, kThreads = 256;
-constexpr int kMaxSplit = 8;                                // CTAs that may share a slice's keys (portable cluster size)
 constexpr uint32_t kPieceQ = kRows * 128, kPieceK = kKeys * 128;                  // bytes of one bf16 piece of an operand tile
 constexpr uint32_t kOffQ = 0, kOffK = kOffQ + 3 * kPieceQ, kOffV = kOffK + 3 * kPieceK, kOffBar = kOffV + 3 * kPieceK;
 constexpr uint32_t kSmemBytes = kOffBar + 64;
@@ -768,22 +768,6 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   }
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // nobody leaves while a peer still reads here
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// CTAs that share a slice's keys.  ctas: CTAs of an unsplit launch.  In steps of a key tile: a CTA that has its SM to itself takes 1 per
-// tile, two that share one 1.35 each.  (The CTAs of a recorded window, one per key tile and slice, are not counted: they hold an SM for about a tile's
-// time, and with them counted as others the split at mid sizes would be smaller.  Not measured.)
-// What combining costs is set by slices of two tiles, which gain by a split (64 queries behind 57 entries, 4 / 16 / 32 / 64 / 73 slices, us per launch, one CTA ->
-// two: 10.4 / 10.6 / 10.6 / 10.6 / 10.8 -> 8.7 / 9.0 / 9.0 / 9.7 / 9.9); at 1.5 they had none.  Longer ones split as they did.
-inline int key_split(int ctas, int tiles, int n_sm) {
-  auto cost = [&](int c) {
-    const int n = ctas * c, per = (tiles + c - 1) / c, waves = (n + 2 * n_sm - 1) / (2 * n_sm);
-    return (n <= n_sm ? 1.f : 1.35f) * (float)(waves * (per + 3)) + (c > 1 ? 0.8f : 0.f);
-  };
-  int split = 1;
-  for (int c = 2; c <= kMaxSplit && c <= tiles; ++c)
-    if (cost(c) < cost(split)) split = c;
-  return split;
 }
 
 }  // namespace f32
