@@ -6,21 +6,23 @@ namespace f32 {
 
 constexpr int kMaxSplit = 8;                                // CTAs that may share a slice's keys (portable cluster size)
 
-// CTAs that share a slice's keys.  ctas: CTAs of an unsplit launch.  In steps of a key tile: a CTA that has its SM to itself takes 1 per
-// tile, two that share one 1.35 each.  (The CTAs of a recorded window, one per key tile and slice, are not counted: they hold an SM for about a tile's
-// time, and with them counted as others the split at mid sizes would be smaller.  Not measured.)
-// Combining costs 1.5; 0.8 for slices of two tiles, which gain by a split wherever two CTAs for one find an SM each (64 queries behind 57
-// entries, 4 / 16 / 32 / 64 / 73 slices, us per launch, one CTA -> two: 10.4 / 10.6 / 10.6 / 10.6 / 10.8 -> 8.7 / 9.0 / 9.0 / 9.7 / 9.9) and at
-// 1.5 had none.  0.8 would cut longer slices into more pieces as well, where nobody has measured it (3 tiles and 50 CTAs, 8 and 300, 14 and 740).
-inline int key_split(int ctas, int tiles, int n_sm) {
-  const float join = tiles == 2 ? 0.8f : 1.5f;
+// CTAs that share a slice's keys.  ctas: CTAs of an unsplit launch.  fit: clusters of c CTAs that the device runs at once (0: none).  In steps of a
+// key tile: a CTA that has its SM to itself takes 1 per tile, two that share one 1.35 each.
+// A cluster has to fit one GPC: of 296 places on 148 SMs clusters of 2 .. 8 use 148, 93, 71, 56, 45, 37, 33 times c.  With waves of 296 CTAs instead, a launch
+// whose clusters just did not fit ran a second wave for the last few (us, 296 places / those that fit; key tiles x CTAs: 13 x 96, three for one 50.3 /
+// two 38.7; 28 x 41, seven 51.0 / six 36.8; 35 x 46, six 63.5 / five 44.5; 20 x 192, three 102 / one 87.5; 14 x 190, three 85 / one 70).
+// Combining costs 0.8 where the unsplit launch is no more than a wave (one CTA / as here: 2 x 64 10.6 / 9.7, 3 x 64 17.9 / 16.9, 5 x 90 26.4 /
+// 23.4, 9 x 148 43.6 / 39.4, 12 x 149 58.9 / 55.8, 34 x 198 139 / 133).  CTAs of longer launches follow on one another, not in waves, and a split loses
+// what the model takes the last wave for: 1.5 (8 x 360 81.2, at 0.8 83.8; 11 x 396 94.7, 103.7; 14 x 740 208, 214).
+inline int key_split(int ctas, int tiles, int n_sm, const int *fit) {
+  const float join = ctas <= 2 * n_sm ? 0.8f : 1.5f;
   auto cost = [&](int c) {
-    const int n = ctas * c, per = (tiles + c - 1) / c, waves = (n + 2 * n_sm - 1) / (2 * n_sm);
+    const int n = ctas * c, per = (tiles + c - 1) / c, at_once = c > 1 ? fit[c] : 2 * n_sm, waves = (ctas + at_once - 1) / at_once;
     return (n <= n_sm ? 1.f : 1.35f) * (float)(waves * (per + 3)) + (c > 1 ? join : 0.f);
   };
   int split = 1;
   for (int c = 2; c <= kMaxSplit && c <= tiles; ++c)
-    if (cost(c) < cost(split)) split = c;
+    if (fit[c] > 0 && cost(c) < cost(split)) split = c;
   return split;
 }
 

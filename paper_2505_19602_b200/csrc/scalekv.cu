@@ -241,6 +241,7 @@ struct scalekv_ctx {
   bool select_smem_ok = false;     // the separate select kernel can stage a slice's keys in shared memory
   bool compact_smem_ok = false;    // the separate compact kernel can stage a slice's keep list in shared memory
   size_t fused_smem = 0;
+  int f32_clusters[f32::kMaxSplit + 1] = {0};   // clusters of c CTAs of the f32 attention that the device runs at once
   bool side_dirty = false;         // stream_side has work that stream_main has not joined yet
   int set_owner[kSets] = {-1, -1, -1, -1};   // layer that last appended into each transient page set / logit buffer
   int set_compressed[kSets] = {-1, -1, -1, -1};   // layer whose compress on stream_side last used the set's logit buffer
@@ -359,6 +360,34 @@ template <typename F> bool set_smem(F *f, size_t bytes) {
   if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) return true;
   cudaGetLastError();
   return false;
+}
+
+// What stands for the f32 attention where the runtime is asked how many of its clusters fit the device: of a kernel that allocates TMEM it counts
+// one CTA to an SM, whatever that allocates, and two of the attention's share one.  Never launched.
+__global__ void __launch_bounds__(f32::kThreads, 2) f32_cluster_size_kernel() {}
+
+// Clusters of c CTAs of the f32 attention that the device runs at once (0: none).  It takes the runtime about a millisecond to tell, so it is
+// asked once per device.
+void f32_cluster_counts(int *counts) {
+  struct Counts { int v[f32::kMaxSplit + 1] = {0}; };
+  static std::mutex lock;
+  static std::map<int, Counts> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return; }
+  std::lock_guard<std::mutex> hold(lock);
+  const bool asked = known.count(dev) != 0;
+  Counts &k = known[dev];
+  if (!asked && set_smem(f32_cluster_size_kernel, f32::kSmemBytes))
+    for (int c = 2; c <= f32::kMaxSplit; ++c) {
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr[1];
+      cfg.gridDim = dim3(1, 1, c); cfg.blockDim = dim3(f32::kThreads); cfg.dynamicSmemBytes = f32::kSmemBytes;
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = c;
+      cfg.attrs = attr; cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&k.v[c], f32_cluster_size_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); k.v[c] = 0; }
+    }
+  std::copy(k.v, k.v + f32::kMaxSplit + 1, counts);
 }
 
 scalekv_status check_launch(scalekv_ctx *ctx, const char *what) {
@@ -516,6 +545,7 @@ scalekv_status scalekv_init(const scalekv_config *cfg, scalekv_ctx **out) {
     } else {
       ok = ok && set_smem(layer_stats_kernel<float, 64>, layer_stats_smem_bytes<64>(64));
       ok = ok && set_smem(f32::attend_f32_tc_kernel, f32::kSmemBytes);
+      if (ok) f32_cluster_counts(ctx->f32_clusters);
       ok = ok && set_smem(score_logits_kernel<float, 64>, 2 * 64 * 68 * 4);
     }
     // select and compact stage a slice in shared memory when it fits and work from global memory when it does not
@@ -727,7 +757,7 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       prm.win_logits = wl; prm.ld_l = p.ld_l; prm.w = wl ? (int)win.size() : 0;
       for (int e = 0; e < prm.w; ++e) prm.win_pos[e] = win[e];
       const int blocks = (nk + f32::kRows - 1) / f32::kRows;
-      const int split = f32::key_split(blocks * p.n_slices, (ctx->hist[layer] + nk + f32::kKeys - 1) / f32::kKeys, ctx->n_sm);
+      const int split = f32::key_split(blocks * p.n_slices, (ctx->hist[layer] + nk + f32::kKeys - 1) / f32::kKeys, ctx->n_sm, ctx->f32_clusters);
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[2];
       // (they come behind all the others, in rows of the grid of their own, so that none of those waits for an SM: 16 slices x 400 / 576 / 1 024

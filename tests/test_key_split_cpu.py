@@ -6,39 +6,43 @@ import subprocess
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2505_19602_b200", "csrc")
-SMS = 148
+SMS, FIT = 148, (0, 0, 148, 93, 71, 56, 45, 37, 33)         # what a B200 has room for: clusters of 2, 3, .. CTAs, two CTAs to an SM
 
 
 @pytest.fixture(scope="module")
 def split(tmp_path_factory):
     at = tmp_path_factory.mktemp("key_split")
-    (at / "rule.cpp").write_text('#include "key_split.h"\nextern "C" int rule(int ctas, int tiles, int n_sm) { return scalekv::f32::key_split(ctas, tiles, n_sm); }\n')
+    (at / "rule.cpp").write_text('#include "key_split.h"\nextern "C" int rule(int ctas, int tiles, int n_sm, const int *fit) '
+                                 '{ return scalekv::f32::key_split(ctas, tiles, n_sm, fit); }\n')
     subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I", CSRC, str(at / "rule.cpp"), "-o", str(at / "rule.so")], check=True)
     rule = ctypes.CDLL(str(at / "rule.so")).rule
-    return lambda ctas, tiles: rule(ctas, tiles, SMS)
+    return lambda tiles, ctas, fit=FIT: rule(ctas, tiles, SMS, (ctypes.c_int * 9)(*fit))
 
 
 def test_slices_of_two_tiles_are_shared_where_every_cta_finds_an_sm(split):
-    assert [split(ctas, 2) for ctas in (1, 4, 73, 74, 75, 148, 149, 296, 297, 5000)] == [2, 2, 2, 2, 1, 1, 1, 1, 1, 1]
+    assert [split(2, ctas) for ctas in (1, 4, 73, 74, 75, 148, 149, 296, 297, 5000)] == [2, 2, 2, 2, 1, 1, 1, 1, 1, 1]
 
 
-@pytest.mark.parametrize("tiles,first,last", [
-    # key tiles, CTAs of the unsplit launch: sizes that are not shared, since nobody has measured that they should be
-    (3, 50, 74), (5, 75, 98), (6, 99, 148), (9, 99, 148), (8, 297, 444), (11, 297, 444), (12, 149, 197), (16, 149, 197),
-    (14, 149, 197), (14, 593, 740), (28, 198, 222), (31, 198, 222), (34, 198, 222), (37, 198, 222), (50, 223, 236), (54, 223, 236), (58, 223, 236), (62, 223, 236),
+@pytest.mark.parametrize("tiles,ctas,more", [
+    (5, 91, 3), (14, 189, 3), (13, 94, 3), (28, 216, 4), (24, 72, 4), (29, 57, 5), (50, 234, 5), (35, 46, 6), (28, 41, 7), (32, 36, 8),
 ])
-def test_longer_slices_are_not_shared_on_the_model_s_word_alone(split, tiles, first, last):
-    assert {split(ctas, tiles) for ctas in range(first, last + 1)} == {1}
+def test_no_wave_of_clusters_for_the_last_few(split, tiles, ctas, more):
+    """`more` CTAs for one fit 296 places, but not as clusters."""
+    assert ctas * more <= 2 * SMS * -(-ctas * more // (2 * SMS))
+    chosen = split(tiles, ctas)
+    assert chosen != more or -(-ctas // FIT[more]) == -(-ctas * more // (2 * SMS))
 
 
-def test_a_split_charges_one_and_a_half_tiles_above_two(split):
-    def charged(ctas, tiles):
-        def cost(c):
-            n, per = ctas * c, -(-tiles // c)
-            return (1 if n <= SMS else 1.35) * (-(-n // (2 * SMS)) * (per + 3)) + (1.5 if c > 1 else 0)
-        costs = [cost(c) for c in range(1, min(8, tiles) + 1)]
-        near = [c + 1 for c in range(len(costs)) if costs[c] <= min(costs) + 1e-3]       # (32 bits may break a tie either way)
-        return near
-    for tiles in list(range(3, 40)) + [50, 62, 80, 165]:
-        for ctas in list(range(1, 760, 7)) + [1000, 1199, 4096]:
-            assert split(ctas, tiles) in charged(ctas, tiles), (tiles, ctas)
+@pytest.mark.parametrize("tiles,ctas,want", [
+    (3, 74, 2), (5, 75, 3), (5, 90, 3), (6, 148, 2), (9, 100, 2), (12, 149, 3), (16, 178, 3), (34, 198, 4), (28, 213, 4),
+    (8, 297, 1), (8, 444, 1), (11, 360, 1), (14, 600, 1), (14, 740, 1), (27, 972, 1),            # more than a wave, one CTA each
+])
+def test_sizes_with_both_sides_measured(split, tiles, ctas, want):
+    assert split(tiles, ctas) == want
+
+
+def test_bounds(split):
+    for tiles in list(range(1, 24)) + [80, 165, 1000]:
+        for ctas in (1, 7, 33, 37, 38, 148, 149, 296, 297, 4096):
+            assert 1 <= split(tiles, ctas) <= min(8, tiles)
+            assert split(tiles, ctas, (0,) * 9) == 1        # a device that cannot run clusters
