@@ -659,6 +659,7 @@ __global__ void __launch_bounds__(256) compact_kernel(LayerView lv, const int *k
 // Dynamic shared memory: 4 * (2 * ld_s + pages_per_slice) bytes.  grid (n_slices).
 // ------------------------------------------------------------------------------------------
 constexpr int kCompressThreads = 512;
+constexpr int kSumsInCompress = 512;      // entries of a slice up to which it can take the window rows' log-sum-exps itself: a warp's lanes hold a row
 
 __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(LayerView lv, WindowArg wa, int policy, int n_sink,
                                                                           const float *logits, const float *lse, int ld_l,
@@ -691,22 +692,33 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_fused_kernel(Lay
   if (dev_status != 0 || outgrown(lv, L)) return;   // a failed check, an earlier kernel's or this one's: leave the store alone
   __syncthreads();
   if (policy == 0 && lse == nullptr) {
-    // The rows' log-sum-exps, a warp a row, to the bit those of row_lse_kernel: there a thread adds up every 1 024th entry, a warp its threads' sums
-    // crosswise and one thread the 32 warps' in turn.
+    if (L > kSumsInCompress) {                 // (no caller asks for it)
+      if (tid == 0) atomicExch(lv.status, kDevCheck);
+      return;
+    }
+    // The rows' log-sum-exps, a warp a row at a time, to the bit those of row_lse_kernel: there a thread takes the exponential of one entry (of
+    // up to 1 024), a warp adds its threads' crosswise and one thread the warps' in turn.
+    const int mine = L - lane;                 // (this lane's entries are 32 u, 32 u below it)
     for (int j = wid; j < w; j += NT / 32) {
-      const float *y = logits + ((size_t)slice * w + j) * ld_l;
-      float top = -INFINITY, sum = 0.f;
-#pragma unroll 8
-      for (int i = lane; i < L; i += 32) top = fmaxf(top, __ldg(y + i));
+      const float *y = logits + ((size_t)slice * w + j) * ld_l + lane;
+      float x[kSumsInCompress / 32], top = -INFINITY, sum = 0.f;
+#pragma unroll
+      for (int u = 0; u < kSumsInCompress / 32; ++u) x[u] = 32 * u < mine ? __ldg(y + 32 * u) : -INFINITY;
+#pragma unroll
+      for (int u = 0; u < kSumsInCompress / 32; ++u) top = fmaxf(top, x[u]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-#pragma unroll 4
-      for (int k0 = 0; k0 < min(L, 1024); k0 += 32) {
-        float v = 0.f;
-        for (int i = k0 + lane; i < L; i += 1024) v += exp2f(__ldg(y + i) - top);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        sum += v;
+      for (int u0 = 0; u0 < kSumsInCompress / 32; u0 += 4) {
+        if (32 * u0 >= L) break;
+#pragma unroll
+        for (int u = u0; u < u0 + 4; ++u) x[u] = 32 * u < mine ? exp2f(x[u] - top) : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int u = u0; u < u0 + 4; ++u) x[u] += __shfl_xor_sync(0xffffffffu, x[u], o);
+#pragma unroll
+        for (int u = u0; u < u0 + 4; ++u) sum += x[u];
       }
       if (lane == 0) lse_row[j] = top + log2f(sum);
     }

@@ -31,10 +31,6 @@ constexpr int kSets = 4;
 // layer_stats splits a slice's keys over several CTAs while the launch would otherwise leave SMs idle; this many CTAs
 // bound the scratch of their partial results (about 10 MB)
 constexpr int kStatsMaxCtas = 592;
-// Up to how many entries of a slice the one-launch compress takes the log-sum-exps of the window's rows itself where attend has not left them: a
-// launch less on the way from an f32 attend to its layer's next.  us per layer and step, 16 slices x 64 / 144 / 256 / 400 queries: a launch of its own
-// 17.0 / 17.9 / 20.5 / 31.2; none up to 256 entries 16.0 / 17.4 / 20.0 / 30.7; none up to 1 024 16.4 / 17.4 / 20.0 / 33.8.
-constexpr int kSumsInCompress = 512;
 constexpr int kNumClasses = 7;
 enum KernelClass { kAppend = 0, kAttend = 1, kScore = 2, kSelect = 3, kCompact = 4, kOther = 5, kCompress = 6 };
 
@@ -926,7 +922,14 @@ scalekv_status scalekv_compress_ex(scalekv_ctx *ctx, int32_t layer, scalekv_tens
     ctx->logits_of[layer] = -1;
     float *wlse = reinterpret_cast<float *>(ctx->ws + p.off_wlse) + (size_t)(layer % kSets) * p.n_slices * p.max_window;
     const bool summed = recorded && ctx->tc.enabled();          // (the f32 attention leaves what the logits kernel would)
-    const bool sums = !recent && !summed && !(fused && L <= kSumsInCompress);
+    // The log-sum-exps of rows that attend has not summed: by the compress itself, 16 rows at a time, or by a launch of their own in front of it, four rows a
+    // CTA, which is the quicker for long rows in more than two rounds, as long as it has an SM for every CTA.  us per layer and step, a launch / here, f32
+    // recorded by attend, bf16 behind an attend that has not: 16 slices x 16 rows of 512 entries 25.2 / 23.2, 26.8 / 25.3, of 256 17.2 / 15.1, 22.9 / 19.8; 4 x 32
+    // of 512 16.4 / 16.5, 25.9 / 25.1; 128 x 64 161 / 129, 140 / 111; 12 x 64 24.5 / 24.3, 35.1 / 34.3; 8 x 64 21.8 / 22.3, 31.2 / 33.1; 4 x 40 17.0 / 18.9,
+    // 28.1 / 28.4, 4 x 64 19.1 / 21.4, 30.7 / 32.7; of 256 entries 1 x 64 16.0 / 17.2, 28.1 / 27.1, 4 x 64 17.0 / 17.0, 28.7 / 29.1, 8 x 64 18.9 / 17.4,
+    // 29.8 / 29.1; of 128 4 x 64 15.4 / 14.8, 27.6 / 27.5.
+    const bool sums_here = fused && L <= kSumsInCompress && (wa.w <= 32 || L <= 256 || p.n_slices > 8);
+    const bool sums = !recent && !summed && !sums_here;
     if (sums) {
       Scope sc(ctx, s, kScore);
       row_lse_kernel<<<dim3(p.n_slices, (wa.w + 3) / 4), 1024, 0, s>>>(lv, wa, logits, p.ld_l, wlse);
