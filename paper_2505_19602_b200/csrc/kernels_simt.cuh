@@ -330,9 +330,9 @@ __global__ void head_budget_kernel(HeadBudgets hb, int n_heads, int n_slices, in
 constexpr int kSelectBins = 2048;
 struct SelectShared {
   int hist[kSelectBins];
-  int warp_sums[33];
-  int keeps[32], ties[32];
-  uint32_t lowest[32], highest[32];
+  int warp_sums[32];
+  union { uint32_t lowest[32]; int keeps[32]; };           // bounds first, counts behind several barriers (every byte here is one that a
+  union { uint32_t highest[32]; int ties[32]; };           // slice's keys and keep list cannot have)
   int first_gap;
   int bin, need, in_bin, n_cand, n_ties;
   uint32_t tie_key;
