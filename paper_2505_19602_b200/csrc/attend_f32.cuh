@@ -711,7 +711,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
     }
     const unsigned spoiled = __ballot_sync(0xffffffffu, nt > 0 && ok && q0 + row < n_k && !hopeless && !(amax == 0.f && l > 0.f && l < INFINITY));
     if (lane == 0) marks[warp] = spoiled;
-    stat_out[row] = make_float2(m, l);
+    stat_out[row] = make_float2(m, ok && !leave ? l : -1.f);             // (no sum is negative: a part that has been given up)
     if (n_split == 1 && ok && nt > 0 && q0 + row < n_k) {
       if (prm.lse != nullptr) prm.lse[(size_t)slice * n_k + q0 + row] = row_lse_f32(m, l, fabsf(prm.scale));
     }
@@ -743,6 +743,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   for (int r = r_lo + ty; r < r_hi; r += 16) {
     float4 x[kMaxSplit];
     float me[kMaxSplit], le[kMaxSplit], M = kNoMax;
+    bool whole = true;
 #pragma unroll
     for (int e = 0; e < kMaxSplit; ++e) {
       x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -754,7 +755,11 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       }
     }
 #pragma unroll
-    for (int e = 0; e < kMaxSplit; ++e) M = fmaxf(M, me[e]);
+    for (int e = 0; e < kMaxSplit; ++e) {
+      M = fmaxf(M, me[e]);
+      whole = whole && !(le[e] < 0.f);
+    }
+    if (!whole) continue;
     float sum = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
     for (int e = 0; e < kMaxSplit; ++e) {

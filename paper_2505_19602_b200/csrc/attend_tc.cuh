@@ -128,7 +128,10 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
   while (true) {
     for (int i = 0; i < 64; ++i)
       if (mbar_try(bar, parity)) return true;
-    if (*abort_flag || *reinterpret_cast<volatile int *>(status) != 0) return false;
+    if (*abort_flag || *reinterpret_cast<volatile int *>(status) != 0) {
+      *abort_flag = 1;                                     // (whoever gives up, for whatever reason: the CTA knows)
+      return false;
+    }
     if (globaltimer() - t0 > limit_ns) {
       *abort_flag = 1;
       atomicExch(status, kDevTimeout);
