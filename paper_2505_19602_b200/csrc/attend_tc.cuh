@@ -472,11 +472,9 @@ __device__ __forceinline__ uint32_t remote(uint32_t addr, int cta) {
 // allocated around it.  window: this thread's row belongs to the observation window.
 // A row that lacks a product, because some wait for it has run out, is left as it is: its accumulator and its query tile may still be in use.
 // What a row needs besides its columns (log-sum-exp, addresses, the place of a window row) is worked out before the last product is
-// waited for.  The two parts of a shared single are read from TMEM at once where one CTA has all of its keys, 32 columns at a time where a
-// cluster shares them: a loop there is less code to fetch.  us per launch of 16 slices, a map in the pages, averages over sizes (worked out
-// behind the wait, 32 columns at a time / before it, at once everywhere / as it is): 16-128 queries behind 21 entries 10.89 / 10.58 / 10.61,
-// 520-1 024 behind 210 20.84 / 20.46 / 20.52, 130-512 behind 209 (clusters) 16.05 / 16.07 / 15.83; of 32 slices x 130-512 16.68 / 16.57 /
-// 16.46.  A pair's last tile shared by both warpgroups, or 64 columns at a time there, gave the instance that records a window another schedule of
+// waited for, and the two parts of a shared single are read from TMEM at once (a step of 16 slices x 36 / 144 / 576 / 1 024 queries behind
+// 21 / 80 / 209 / 209 entries: 5.8 / 7.5 / 13.5 / 18.1 -> 5.5 / 7.0 / 13.0 / 17.6 us; 128 x 1 600: 206.1 -> 204.7).  A pair's last tile
+// shared by both warpgroups, or 64 columns at a time there, gave the instance that records a window another schedule of
 // the sweep, 1-2 % slower throughout.
 __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, uint32_t lane_addr, int slice, int first_row, int qt, bool pair,
                                          bool shared, bool have, bool whole, int n_split, float m, float l, bool window,
@@ -559,7 +557,7 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(small_div(row, own_rows), n_split - 1);   // (rows beyond the map go nowhere)
     const int at = (int)blockIdx.z * own_rows + row - owner * own_rows;      // and the row's place there
     const uint32_t dst = n_split > 1 ? remote(base + kOffRing + (uint32_t)at * 512 + (uint32_t)qt * 256, owner) : 0;
-    const int rank = n_split > 1 ? window_rank() : -1;
+    const int rank = window_rank();
     if (!whole || (have && !final_product(qt))) {          // (no sum is negative)
       l = -1.f;
       asm volatile("st.shared.f32 [%0], %1;" ::"r"(stat + (uint32_t)qt * 1024 + 4), "f"(l) : "memory");
@@ -568,49 +566,40 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     tc_fence_before();
     asm volatile("bar.sync 2, 256;" ::: "memory");         // both accumulators are complete, no product reads the query tile any more
     tc_fence_after();
+    float o[64], other[64];
     const uint32_t o_addr = lane_addr + kColO + qt * 64;
-    auto load = [&](int c0, float *o, float *other) {      // 32 columns of both parts
-      tc_ld32(o_addr + qt * 128 + c0, o);
-      tc_ld32(o_addr + (qt ^ 1) * 128 + c0, other);
-    };
-    float M, both, f1, f2;
-    bool none1, none2;                                     // a part without keys left garbage
-    auto weights = [&] {
-      float m2, l2;
-      asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(stat + (uint32_t)(qt ^ 1) * 1024) : "memory");
-      whole = !(l < 0.f || l2 < 0.f);                      // (the same for the warp's rows)
-      M = fmaxf(m, m2);
-      f1 = l > 0.f ? ex2(m - M) : 0.f; f2 = l2 > 0.f ? ex2(m2 - M) : 0.f;
-      both = l * f1 + l2 * f2;
-      none1 = !__any_sync(0xffffffffu, l > 0.f); none2 = !__any_sync(0xffffffffu, l2 > 0.f);
-    };
-    auto merge = [&](float *o, float *other) {
-      const uint64_t ff1 = pack2(f1, f1), ff2 = pack2(f2, f2);
-      if (none1) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = 0.f;
-      }
-      if (none2) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) other[i] = 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 16; ++i)
-        unpack2(fma2(pack2(o[2 * i], o[2 * i + 1]), ff1, mul2(pack2(other[2 * i], other[2 * i + 1]), ff2)), o[2 * i], o[2 * i + 1]);
-    };
+    for (int cc = 0; cc < 2; ++cc) {
+      tc_ld32(o_addr + qt * 128 + cc * 32, o + cc * 32);
+      tc_ld32(o_addr + (qt ^ 1) * 128 + cc * 32, other + cc * 32);
+    }
+    float m2, l2;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m2), "=f"(l2) : "r"(stat + (uint32_t)(qt ^ 1) * 1024) : "memory");
+    whole = !(l < 0.f || l2 < 0.f);                        // (the same for the warp's rows)
+    const float M = fmaxf(m, m2);
+    float f1 = l > 0.f ? ex2(m - M) : 0.f, f2 = l2 > 0.f ? ex2(m2 - M) : 0.f;
+    const float both = l * f1 + l2 * f2;
     if (n_split == 1) {
-      // all columns at once, under the weights
-      float o[64], other[64];
-      load(0, o, other);
-      load(32, o + 32, other + 32);
-      weights();
       const float inv = 1.f / both;
       f1 *= inv; f2 *= inv;
-      if (qt == 0 && whole) keep_sums(M + log2f(both), window_rank());
-      tc_wait_ld();
+      if (qt == 0 && whole) keep_sums(M + log2f(both), rank);
+    }
+    const bool none1 = !__any_sync(0xffffffffu, l > 0.f), none2 = !__any_sync(0xffffffffu, l2 > 0.f);   // a part without keys left garbage
+    const uint64_t ff1 = pack2(f1, f1), ff2 = pack2(f2, f2);
+    tc_wait_ld();
+    if (none1) {
+#pragma unroll
+      for (int i = 0; i < 64; ++i) o[i] = 0.f;
+    }
+    if (none2) {
+#pragma unroll
+      for (int i = 0; i < 64; ++i) other[i] = 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      unpack2(fma2(pack2(o[2 * i], o[2 * i + 1]), ff1, mul2(pack2(other[2 * i], other[2 * i + 1]), ff2)), o[2 * i], o[2 * i + 1]);
+    if (n_split == 1) {
       if (!whole) return;
-      merge(o, other);
-      merge(o + 32, other + 32);
       // four 128-byte pieces a store instruction
       const uint32_t stage = stage0 + qt * 4096, mine = stage + lane * 128;
       const int w0 = first_row + quarter * 32 + (lane >> 3);
@@ -632,16 +621,10 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     } else {
       // the warpgroup's half of the row, 16-byte pieces permuted by its index
       const uint32_t mine = base + kOffQ + qt * kTileBytes + row * 256;
-      weights();
-#pragma unroll 1
-      for (int c0 = 0; c0 < 64 && whole; c0 += 32) {
-        float o[32], other[32];
-        load(c0, o, other);
-        tc_wait_ld();
-        merge(o, other);
+      if (whole) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)(c0 << 2) + (uint32_t)((i ^ (row & 7)) << 4)), "f"(o[4 * i]),
+        for (int i = 0; i < 16; ++i)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(mine + (uint32_t)((i & 8) << 4) + (uint32_t)(((i & 7) ^ (row & 7)) << 4)), "f"(o[4 * i]),
                        "f"(o[4 * i + 1]), "f"(o[4 * i + 2]), "f"(o[4 * i + 3]) : "memory");
       }
       __syncwarp();
