@@ -14,14 +14,15 @@
 // With two CTAs an SM's tensor pipe works for the one while the other is in its softmax.
 // Scores that are not numbers (an infinite key: its products with the pieces of a query may differ in sign) are taken again, by signs or fp32 FMA
 // (repair_scores).  Rows whose sum or columns are none all the same, an infinite value's, are done again at the end by fp32 FMA (redo_rows).
-// The observation window's logits are taken by CTAs of their own beside the others, in plain fp32 (see the launch).
+// The observation window's logits are taken by CTAs of their own behind those of all slices, in plain fp32 (see the launch).
 // gridDim.z CTAs of a cluster share a slice's keys and combine: O = sum_e 2^(c (m_e - M)) O_e / sum_e 2^(c (m_e - M)) l_e, through distributed
 // shared memory.
-// What bounds it: the instructions of the softmax and of the splitting, and the tensor pipe, six products standing for one; a step of two
-// CTAs that share an SM takes about 8 000 cycles.  (Working copies that skip work, us per layer, 16 slices x 1 600 queries: whole 130; one
+// What bounds it: the issue of MMAs, six products standing for one (48 a tile and CTA; one of N = 64 holds the path for 65 cycles, as long as one of
+// N = 128, though its work is half of that: the pipe counts 37 % at 1 600 queries), and the instructions of the softmax and of the splitting (issue slots
+// 48 %); a step of two CTAs that share an SM takes about 8 000 cycles.  (Working copies that skip work, us per layer, 16 slices x 1 600 queries: whole 130; one
 // product of six 102; P not split 115; K and V not split 112.)  S of the next tile under the softmax of this one, from two buffers, and
-// fewer instructions: 139 -> 123.  The softmax's loops over a tile's 16-column pieces and the operands' part of a step are compiled once, not unrolled or
-// copied: 123 -> 113 (fewer spills, less code to fetch in short launches).  us per layer and step, 16 slices behind 92 to 772 entries with their compresses,
+// fewer instructions: 139 -> 123.  The loop of exponentials and splitting over a tile's 16-column pieces is not unrolled (that of the maximum is), and the
+// operands' part of a step stands once: 123 -> 113 (fewer spills, less code to fetch in short launches).  us per layer and step, 16 slices behind 92 to 772 entries with their compresses,
 // by packed fp32 FMA (66 % of that pipe), a copy of the map and three launches per compress -> here: 16 queries 15.4 -> 8.7, 64: 25.7 -> 16, 256: 35.8 -> 20,
 // 400: 65 -> 31, 576: 91 -> 40, 1 024: 179 -> 63, 1 600: 331 -> 113.
 // Error against 64 bits, full caches of 29 to 4 436 entries, queries and keys normal, queries times 0.25 / 1 / 3: outputs 0.9 to 1.6 / 1.0 to
@@ -614,7 +615,7 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
       const uint32_t buf = lane_addr + kBufCols * (i & 1);
       auto real = [&](int key) { return !decltype(masked)::value || key < valid; };
       float mx = -INFINITY;
-#pragma unroll 4
+#pragma unroll 4                       // (all of it; a plain unroll is scheduled otherwise, with 20 bytes more of spills)
       for (int e = 0; e < 4; ++e) {
         uint32_t x[16];
         tc::tc_ld16(buf + 16 * e, x);
@@ -728,9 +729,11 @@ __global__ void __launch_bounds__(kThreads, 2) attend_f32_tc_kernel(const __grid
   }
   const int ty = tid >> 4, tx = tid & 15, rows = min(kRows, n_k - q0);
   if (n_split == 1) {
-    if (leave || *abort_flag) return;
+    if (leave) return;
     for (int r = ty; r < rows; r += 16) {
-      const float inv = 1.f / stat_out[r].y;
+      const float sum = stat_out[r].y;
+      if (sum < 0.f) continue;
+      const float inv = 1.f / sum;
       const float4 x = *reinterpret_cast<const float4 *>(rows_out + r * 64 + ((tx ^ (r & 7)) << 2));
       *reinterpret_cast<float4 *>(const_cast<float *>(row_ptr<float>(prm.O, b, h, q0 + r)) + tx * 4) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
     }

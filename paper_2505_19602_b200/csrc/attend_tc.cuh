@@ -128,10 +128,7 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
   while (true) {
     for (int i = 0; i < 64; ++i)
       if (mbar_try(bar, parity)) return true;
-    if (*abort_flag || *reinterpret_cast<volatile int *>(status) != 0) {
-      *abort_flag = 1;                                     // (whoever gives up, for whatever reason: the CTA knows)
-      return false;
-    }
+    if (*abort_flag || *reinterpret_cast<volatile int *>(status) != 0) return false;
     if (globaltimer() - t0 > limit_ns) {
       *abort_flag = 1;
       atomicExch(status, kDevTimeout);
@@ -468,17 +465,20 @@ __device__ __forceinline__ uint32_t remote(uint32_t addr, int cta) {
 }
 
 // The end of a softmax warp's work, behind its last sweep: 32 rows of O with references m and sums l are normalised and stored
-// (have: there were keys for this tile; whole: nothing has been given up so far).  A function of its own so that the sweep's registers are not
-// allocated around it.  window: this thread's row belongs to the observation window.
+// (have: there were keys for this tile and all have been swept; whole: nothing has been given up so far).  A function of its own so that the sweep's
+// registers are not allocated around it.  window: this thread's row belongs to the observation window.
 // A row that lacks a product, because some wait for it has run out, is left as it is: its accumulator and its query tile may still be in use.
 // What a row needs besides its columns (log-sum-exp, addresses, the place of a window row) is worked out before the last product is
-// waited for, and the two parts of a shared single are read from TMEM at once (a step of 16 slices x 36 / 144 / 576 / 1 024 queries behind
-// 21 / 80 / 209 / 209 entries: 5.8 / 7.5 / 13.5 / 18.1 -> 5.5 / 7.0 / 13.0 / 17.6 us; 128 x 1 600: 206.1 -> 204.7).  A pair's last tile
-// shared by both warpgroups, or 64 columns at a time there, gave the instance that records a window another schedule of
-// the sweep, 1-2 % slower throughout.
+// waited for, which a row's log-sum-exp does not depend on, and the two parts of a shared single are read from TMEM at once.  us per launch of 16
+// slices, a map in the pages, averages over sizes, worked out behind the wait and 32 columns at a time / so: 16-128 queries behind 21 entries 10.89 /
+// 10.58, 520-1 024 behind 210 20.84 / 20.46; where a cluster shares the keys the code that runs once costs what it saves, 130-512 behind 209
+// 16.05 / 16.07 (single sizes up to 3 % longer: 400 queries with their step 11.9 / 12.3), of 32 slices 16.68 / 16.57; 128 x 1 600: 206.1 / 204.7.
+// The instance that records a window is scheduled anew with every change here: 32 columns at a time in clusters alone (15.83, 16.46) made its
+// sweep 2-3 % slower at 4 096 queries and more, as did a pair's last tile shared by both warpgroups, the sums kept behind the wait 0.4 %, and
+// a flag set in mbar_wait_slow for waits that end by the status 1 %.
 __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, uint32_t lane_addr, int slice, int first_row, int qt, bool pair,
-                                         bool shared, bool have, bool whole, int n_split, float m, float l, bool window,
-                                         volatile int *abort_flag, int *status) {
+                                         bool shared, bool have, bool whole, int n_split, float m, float l, bool window, volatile int *abort_flag,
+                                         int *status) {
   const int n_k = prm.n_k;
   const int lane = threadIdx.x & 31, quarter = (threadIdx.x >> 5) & 3, row = quarter * 32 + lane;
   // Output rows leave through shared memory, so that a store instruction writes whole 64- or 128-byte pieces (a row written by its own
@@ -502,17 +502,16 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
         if (prm.win_pos[e] == r_own) rank = e;
     return rank;
   };
-  auto keep_sums = [&](float y, int rank) {              // what is kept of a row besides its output: its base-2 log-sum-exp
+  auto row_sums = [&](float mr, float lr) {              // what is kept of a row besides its output
+    const float y = mr + log2f(lr);
     if (prm.lse != nullptr && r_own < n_k) prm.lse[(size_t)slice * n_k + r_own] = y * 0.6931471805599453f;
+    const int rank = window_rank();
     if (rank >= 0) prm.win_lse[(size_t)slice * prm.w + rank] = y;
   };
   const uint32_t stat = base + kOffStat + (uint32_t)row * 8;             // of this row in tile A; tile B's lie 1024 bytes further
   if (!shared) {
-    if (!have || !whole) return;
-    const float y = m + log2f(l);
-    const int rank = window_rank();
-    if (final_product(qt)) {
-      keep_sums(y, rank);
+    if (have) row_sums(m, l);
+    if (have && final_product(qt)) {
       // 32 columns of the warp's 32 rows at a time (128 of a row's 256 bytes there), eight 64-byte pieces a store instruction
       const float inv = 1.f / l;
       const uint32_t o_addr = lane_addr + kColO + qt * 128;
@@ -557,7 +556,7 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     const int own_rows = n_split > 1 ? cluster_share(n_k, first_row, n_split) : 128, owner = min(small_div(row, own_rows), n_split - 1);   // (rows beyond the map go nowhere)
     const int at = (int)blockIdx.z * own_rows + row - owner * own_rows;      // and the row's place there
     const uint32_t dst = n_split > 1 ? remote(base + kOffRing + (uint32_t)at * 512 + (uint32_t)qt * 256, owner) : 0;
-    const int rank = window_rank();
+    const int rank = n_split > 1 ? window_rank() : -1;
     if (!whole || (have && !final_product(qt))) {          // (no sum is negative)
       l = -1.f;
       asm volatile("st.shared.f32 [%0], %1;" ::"r"(stat + (uint32_t)qt * 1024 + 4), "f"(l) : "memory");
@@ -582,7 +581,7 @@ __device__ __forceinline__ void finish_rows(const Params &prm, uint32_t base, ui
     if (n_split == 1) {
       const float inv = 1.f / both;
       f1 *= inv; f2 *= inv;
-      if (qt == 0 && whole) keep_sums(M + log2f(both), rank);
+      if (qt == 0 && whole) row_sums(M, both);
     }
     const bool none1 = !__any_sync(0xffffffffu, l > 0.f), none2 = !__any_sync(0xffffffffu, l2 > 0.f);   // a part without keys left garbage
     const uint64_t ff1 = pack2(f1, f1), ff2 = pack2(f2, f2);
@@ -1158,8 +1157,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(bPFull + qt));
     }
-    finish_rows(prm, base, lane_addr, item_slot[0], item_slot[1], qt, pair, shared, steps > 0, ok && !leave, n_split, m, l,
-                kWindow && win_row != nullptr, abort_flag, status);
+    finish_rows(prm, base, lane_addr, item_slot[0], item_slot[1], qt, pair, shared, ok && steps > 0, ok && !leave, n_split, m, l, kWindow && win_row != nullptr,
+                abort_flag, status);
     tc_fence_before();
   }
   __syncthreads();

@@ -747,8 +747,8 @@ static scalekv_status attend_impl(scalekv_ctx *ctx, int32_t layer, scalekv_tenso
       prm.fused = fused ? 1 : 0; prm.copy_in = (fused && copy) ? 1 : 0; prm.n_prev = p.N[k];
       prm.scale = ctx->scale;
       prm.weight_scale = (float)(std::fabs((double)ctx->scale) * 1.4426950408889634 * (1.0 + (double)f32::kCutOff));
-      // The window's logits: plain fp32 sums, as the compress would take them from K by a launch of its own, 16 rows of every key tile by a
-      // CTA beside the others.  (Not from the tensor core's scores: importances a few 1e-7 apart decide what is kept, so that logits of
+      // The window's logits: plain fp32 sums, as the compress would take them from K by a launch of its own, all rows of a key tile by a
+      // CTA behind the others.  (Not from the tensor core's scores: importances a few 1e-7 apart decide what is kept, so that logits of
       // another rounding, as exact as they may be, keep another entry in one pass of some.)
       prm.win_logits = wl; prm.ld_l = p.ld_l; prm.w = wl ? (int)win.size() : 0;
       for (int e = 0; e < prm.w; ++e) prm.win_pos[e] = win[e];
