@@ -28,13 +28,13 @@ if ROOT not in sys.path:
 
 METRIC = "scale_steps_per_sec"
 # DRAM traffic of the attend kernel: (dram__bytes_read.sum + dram__bytes_write.sum) / algorithmic bytes over the two
-# launches of an ncu capture of one layer of the headline workload, its two largest scales (455.7 + 654.6 = 1110.3 MB
+# launches of an ncu capture of one layer of the headline workload, its two largest scales (454.6 + 654.3 = 1108.9 MB
 # measured against 1128.4 MB algorithmic).  The capture runs
 # one layer of the workload; traffic grows in proportion to the bytes a launch must move, so the roofline object reports
 # this ratio times the average algorithmic bytes per launch.  Captured on the kernel as of the commit named below
 # (profiles/attend_tc_kernel_pass2b_1layer.md); set ATTEND_TRAFFIC_RATIO to None when attend_tc.cuh changes after it.
-ATTEND_TRAFFIC_RATIO = 1110.3 / 1128.4
-ATTEND_TRAFFIC_SOURCE = ("ncu capture of attend_tc_kernel at commit 1967c54 (one layer, scales 12 and 13), scaled to the "
+ATTEND_TRAFFIC_RATIO = 1108.9 / 1128.4
+ATTEND_TRAFFIC_SOURCE = ("ncu capture of attend_tc_kernel at commit a12feed (one layer, scales 12 and 13), scaled to the "
                          "average launch by algorithmic bytes")
 UNIT = "scale-steps/s"
 E2E_HOST_LAYERS = 4
